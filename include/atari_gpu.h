@@ -94,9 +94,9 @@ typedef struct {
                              2 = bank-aware: re-sorted at every step by the bank their state holds at the
                              step's start (stable in env order), so a warp's lanes start in one bank of an
                              banked cartridge; 0 = autotune */
-    int dispatch;         /* batched form, the interpreter's hot opcode switch: 1 = every common opcode inline;
-                             2 = compact (indirect forms, BIT, stack pushes and pulls, indexed and absolute
-                             read-modify-writes through the general decoder: a smaller hot loop); 0 = autotune */
+    int dispatch;         /* batched form: 0, 1 or 2.  Kept for callers: it chose between two opcode switches;
+                             the interpreter's hot loop has no switch any more, and every value runs the same
+                             code (launch_shape reports 2 as before) */
     int idle_skip;        /* batched form: 1 = a RIOT-timer wait loop (LDA INTIM at PC, BNE back to PC) retires
                              the iterations that read a nonzero timer value at once (cycles and instruction
                              counts advanced exactly; same results), 0 = every iteration runs.  Default 1;

@@ -135,14 +135,15 @@ std::vector<uint32_t> build_decode_table() {
 }
 
 // The batched console's decode bytes: per opcode, operation | page-cross
-// penalty << 7, then mode | cycles << 4.
+// penalty << 7, then mode | cycles << 4, then the control words.
 std::vector<uint8_t> build_dec_op(const std::vector<uint32_t> &dec) {
-  std::vector<uint8_t> d(512, 0);
+  std::vector<uint8_t> d(DEC_BYTES, 0);
   for (int o = 0; o < 256; ++o) {
     const uint32_t t = dec[o];
     d[o] = (uint8_t)((t & 0x7F) | ((t >> 16) & 1u) << 7);
     d[256 + o] = (uint8_t)(((t >> 8) & 0xFu) | ((t >> 12) & 0xFu) << 4);
   }
+  build_ctl(dec.data(), d.data() + 512);
   return d;
 }
 
@@ -192,50 +193,50 @@ __device__ void reset_from_cache(uint8_t *st, const uint8_t *cache, const uint32
 // memory), which steps the same machine as the plain console and is far
 // faster than it for one sequential trajectory; the block stages the
 // cartridge.  rom_stage = bytes of the largest cartridge.
+struct CacheHook {
+  uint8_t *st, *snaps;
+  int startup, max_noops, f;  // f: frames run
+  __device__ void keep(FastConsoleT<false> &m) {
+    m.drain();  // the queued TIA writes belong to the state
+    m.store(st);
+    const uint4 *s4 = reinterpret_cast<const uint4 *>(st);
+    uint4 *d4 = reinterpret_cast<uint4 *>(snaps + (size_t)(f - startup) * 256);
+    for (int q = 0; q < 16; ++q) d4[q] = s4[q];
+  }
+  __device__ bool frame_done(FastConsoleT<false> &m) {
+    ++f;
+    if (f >= startup) keep(m);
+    if (f == startup + max_noops) return false;
+    m.apply_action(0);
+    return true;
+  }
+};
 __global__ void __launch_bounds__(128) k_cache_run(uint8_t *work, uint8_t *snaps, const uint8_t *roms,
                                                     const uint32_t *info, const uint8_t *dec_op_g, int rom_stage,
                                                     int startup, int max_noops) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  uint8_t *rom8 = smem;                                   // rom_stage bytes, then 16 of padding
-  uint8_t *dec_op = smem + (size_t)rom_stage + 16;
-  uint8_t *ram = dec_op + 512;
-  uint32_t *iow = reinterpret_cast<uint32_t *>(ram + RAM_BYTES);
-  uint8_t *tia = reinterpret_cast<uint8_t *>(iow + IO_STRIDE);
   const int r = blockIdx.x;
   const uint32_t inf = info[r];
   const uint32_t banks = inf >> 24;
   const uint4 *src = reinterpret_cast<const uint4 *>(roms + (size_t)r * ROM_SLOT);
-  uint4 *dst = reinterpret_cast<uint4 *>(rom8);
+  uint4 *dst = reinterpret_cast<uint4 *>(g_smem);
   for (uint32_t q = threadIdx.x; q < banks * 256u; q += blockDim.x) dst[q] = src[q];
   if (threadIdx.x == 0) dst[banks * 256u] = make_uint4(0, 0, 0, 0);
-  for (int t = threadIdx.x; t < 512; t += blockDim.x) dec_op[t] = dec_op_g[t];
+  for (uint32_t t = threadIdx.x; t < DEC_BYTES; t += blockDim.x) sm8(rom_stage + 16 + t) = dec_op_g[t];
   __syncthreads();
   if (threadIdx.x != 0) return;
   uint8_t *st = work + (size_t)r * 256;
-  FastConsoleT<false, false> m;
-  m.rom8 = rom8;
-  m.dec_op = dec_op;
-  m.ram = ram;
-  m.io = IoCtx{tia, iow};
+  const EnvOff off = env_off((uint32_t)rom_stage, 1, 0);
+  FastConsoleT<false> m;
+  m.attach(off);
   m.scheme = inf & 0xFF;
   m.wmask = 1u;
   m.idle = 1u;
+  m.to = TiaOut{nullptr, nullptr, nullptr, nullptr, 0};
   m.load(st);
-  m.set_log(nullptr, 0, nullptr);
-  for (int f = 0; f < startup; ++f) {
-    m.apply_action(0);
-    m.run_frame();
-  }
-  for (int j = 0; j <= max_noops; ++j) {
-    m.store(st);
-    const uint4 *s4 = reinterpret_cast<const uint4 *>(st);
-    uint4 *d4 = reinterpret_cast<uint4 *>(snaps + ((size_t)r * (max_noops + 1) + j) * 256);
-    for (int q = 0; q < 16; ++q) d4[q] = s4[q];
-    if (j < max_noops) {
-      m.apply_action(0);
-      m.run_frame();
-    }
-  }
+  m.apply_action(0);
+  CacheHook h{st, snaps + (size_t)r * (max_noops + 1) * 256, startup, max_noops, 0};
+  if (startup == 0) h.keep(m);
+  if (startup + max_noops > 0) m.run(h);
 }
 
 __global__ void k_cache_pick(uint8_t *cache, const uint8_t *snaps, int n_roms, int n_cache, int max_noops,
@@ -523,7 +524,7 @@ struct atari_env {
   uint8_t *d_obs_tmp = nullptr;
   // batched form
   uint8_t *d_romb = nullptr;        // [n_roms][ROMB_SLOT] cartridge bytes for the batched stage
-  uint8_t *d_dec_op = nullptr;      // 512 bytes
+  uint8_t *d_dec_op = nullptr;      // DEC_BYTES
   int32_t *d_grp = nullptr;         // rom, start, count per work item (3 * n_groups) then perm (n)
   int32_t *d_seg = nullptr;         // first env-list position of each cartridge (n_roms + 1)
   int32_t *d_perm_dyn = nullptr;    // bank-aware grouping: the env list re-sorted at every step
@@ -532,7 +533,7 @@ struct atari_env {
   int *d_queue = nullptr;
   int n_groups = 0, lanes = 32, warps = 4, wpf = 4, grid = 0, rom_stage = 4096, max_blocks = 1;
   bool split = false;   // paired CPU / TIA warps (k_interp_split)
-  bool compact = false; // the interpreter with the compact hot opcode switch
+  bool compact = false; // cfg.dispatch == 2, reported by atari_env_launch_shape; no effect on the kernels
   std::vector<int32_t> h_env_rom;
   std::vector<uint32_t> h_banks;
   cudaStream_t cap_stream = nullptr;
@@ -585,6 +586,10 @@ int validate(const atari_config &c) {
 
 namespace {
 
+size_t interp_smem(const atari_env *E) {
+  return (size_t)E->rom_stage + 16 + DEC_BYTES + (size_t)E->lanes * E->warps * ENV_SMEM;
+}
+
 // Envs grouped by cartridge into work items of E envs (ascending env index
 // within a cartridge); uploads rom/start/count per item and the permutation.
 int build_groups(atari_env *E, int lanes, int warps, bool split) {
@@ -625,16 +630,14 @@ int build_groups(atari_env *E, int lanes, int warps, bool split) {
   E->lanes = lanes;
   E->warps = warps;
   E->split = split;
-  const size_t smem = (size_t)E->rom_stage + 16 + 512 + (size_t)lanes * warps * (ENV_SMEM + (split ? 4 * QSTRIDE : 0));
+  const size_t smem = interp_smem(E);
   int per_sm = 0;
   if (split) {
-    CUDA_TRY(cudaFuncSetAttribute(k_interp_split<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    CUDA_TRY(cudaFuncSetAttribute(k_interp_split<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp_split<false>, 2 * warps * 32, smem));
+    CUDA_TRY(cudaFuncSetAttribute(k_interp_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp_split, 2 * warps * 32, smem));
   } else {
-    CUDA_TRY(cudaFuncSetAttribute(k_interp_batched<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    CUDA_TRY(cudaFuncSetAttribute(k_interp_batched<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp_batched<false>, warps * 32, smem));
+    CUDA_TRY(cudaFuncSetAttribute(k_interp_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp_batched, warps * 32, smem));
   }
   int sms = 0;
   CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, E->device));
@@ -684,19 +687,11 @@ BatchArgs batch_args(atari_env *E, const uint8_t *d_actions, int32_t *d_rewards,
   return a;
 }
 
-size_t interp_smem(const atari_env *E) {
-  return (size_t)E->rom_stage + 16 + 512 + (size_t)E->lanes * E->warps * (ENV_SMEM + (E->split ? 4 * QSTRIDE : 0));
-}
 // The batched interpreter in the env's current form and shape.
 void launch_interp(atari_env *E, const BatchArgs &a, int grid, cudaStream_t s) {
   const unsigned th = (E->split ? 2 : 1) * E->warps * 32;
-  if (E->split) {
-    if (E->compact) k_interp_split<true><<<grid, th, interp_smem(E), s>>>(a);
-    else k_interp_split<false><<<grid, th, interp_smem(E), s>>>(a);
-  } else {
-    if (E->compact) k_interp_batched<true><<<grid, th, interp_smem(E), s>>>(a);
-    else k_interp_batched<false><<<grid, th, interp_smem(E), s>>>(a);
-  }
+  if (E->split) k_interp_split<<<grid, th, interp_smem(E), s>>>(a);
+  else k_interp_batched<<<grid, th, interp_smem(E), s>>>(a);
 }
 
 size_t fused_smem() { return 2 * 210 * 160 + 128 + 7056; }
@@ -771,7 +766,7 @@ size_t atari_env_footprint(int n_envs, int n_roms, const atari_config *cfg) {
   if (!cfg || n_envs < 0 || n_roms < 0) return 0;
   size_t n = (size_t)n_envs;
   size_t b = 0;
-  b += (size_t)n_roms * ROM_SLOT + (size_t)n_roms * 4 + 1024 + 512;  // images, info, decode word and byte tables
+  b += (size_t)n_roms * ROM_SLOT + (size_t)n_roms * 4 + 1024 + DEC_BYTES;  // images, info, decode word and byte tables
   b += n * (4 + 4 + 256);                                 // env_rom, env_key, state
   b += (size_t)n_roms * cfg->n_cache * 256;               // cache
   b += n * 2 * (size_t)cfg->log_cap * 4;                  // log
@@ -825,7 +820,7 @@ int atari_env_create(const uint8_t *const *roms, const size_t *rom_sizes, const 
       (rc = dalloc(&E->d_meta, n * 2 * 2 * 4, T)) ||
       (c.form == ATARI_FORM_PLAIN && (rc = dalloc(&E->d_frames, n * 2 * 210 * 160, T))) ||
       (rc = dalloc(&E->d_rew, n * 4, T)) || (rc = dalloc(&E->d_done, n, T)) || (rc = dalloc(&E->d_ctr, n * 12, T)) ||
-      (rc = dalloc(&E->d_act, n, T)) || (rc = dalloc(&E->d_luma, 128, T)) || (rc = dalloc(&E->d_dec_op, 512, T)))
+      (rc = dalloc(&E->d_act, n, T)) || (rc = dalloc(&E->d_luma, 128, T)) || (rc = dalloc(&E->d_dec_op, DEC_BYTES, T)))
     return bail(rc);
   if (c.output_mode == ATARI_OUT_STACK) {
     if ((rc = dalloc(&E->d_ring, n * 4 * 7056, T)) || (rc = dalloc(&E->d_head, n, T))) return bail(rc);
@@ -873,7 +868,7 @@ int atari_env_create(const uint8_t *const *roms, const size_t *rom_sizes, const 
   };
   const std::vector<uint8_t> dec_op = build_dec_op(dec);
   if ((rc = up(E->d_roms, img.data(), img.size())) || (rc = up(E->d_info, info.data(), info.size() * 4)) ||
-      (rc = up(E->d_dec, dec.data(), 1024)) || (rc = up(E->d_dec_op, dec_op.data(), 512)) || (rc = up(E->d_env_rom, env_rom, n * 4)) ||
+      (rc = up(E->d_dec, dec.data(), 1024)) || (rc = up(E->d_dec_op, dec_op.data(), DEC_BYTES)) || (rc = up(E->d_env_rom, env_rom, n * 4)) ||
       (rc = up(E->d_env_key, keys.data(), n * 4)))
     return bail(rc);
   if (luma && (rc = up(E->d_luma, luma, 128))) return bail(rc);
@@ -891,7 +886,8 @@ int atari_env_create(const uint8_t *const *roms, const size_t *rom_sizes, const 
     uint32_t max_banks = 1;
     for (int r = 0; r < n_roms; ++r) max_banks = std::max(max_banks, E->h_banks[r]);
     const int stage = (int)max_banks * 4096;
-    const size_t cache_smem = (size_t)stage + 16 + 512 + RAM_BYTES + 4 * IO_STRIDE + TIA_STRIDE;
+    const size_t cache_smem = (size_t)stage + 16 + DEC_BYTES + ENV_SMEM;
+    cudaFuncSetAttribute(k_cache_run, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cache_smem);
     k_cache_run<<<n_roms, 128, cache_smem>>>(d_work, d_snaps, E->d_roms, E->d_info, E->d_dec_op, stage,
                                            c.startup_frames, c.max_noops);
     int tot = n_roms * c.n_cache;
@@ -1139,31 +1135,7 @@ int autotune(atari_env *E) {
     }
     E->grouping = tg[2] < 0.97f * tg[1] ? 2 : 1;
   }
-  // opcode dispatch on the chosen shape and grouping: the full hot switch, or
-  // the compact one (rare forms through the general decoder); the compact
-  // switch must be 3 % faster to be taken
   E->compact = E->cfg.dispatch == 2;
-  if (!rc && E->cfg.dispatch == 0) {
-    float td[2] = {0, 0};
-    for (int cmp = 0; cmp <= 1 && !rc; ++cmp) {
-      E->compact = cmp != 0;
-      BatchArgs a = batch_args(E, E->d_act, nullptr, nullptr);
-      for (int rep = 0; rep < 2; ++rep) {
-        if (cudaMemcpy(E->d_state, st_bak, n * 256, cudaMemcpyDeviceToDevice) != cudaSuccess ||
-            cudaMemset(E->d_queue, 0, sizeof(int)) != cudaSuccess) {
-          rc = fail(ATARI_ECUDA, "autotune: state restore failed");
-          break;
-        }
-        cudaEventRecord(e0);
-        if (E->grouping == 2) launch_regroup(E, nullptr);
-        launch_interp(E, a, E->grid, nullptr);
-        cudaEventRecord(e1);
-        cudaEventSynchronize(e1);
-        cudaEventElapsedTime(&td[cmp], e0, e1);
-      }
-    }
-    E->compact = td[1] < 0.97f * td[0];
-  }
   if (!rc && E->cfg.output_mode == ATARI_OUT_STACK) {
     if (!(rc = dalloc(&ring_bak, n * 4 * 7056, dummy)) && !(rc = dalloc(&head_bak, n, dummy))) {
       cudaMemcpy(ring_bak, E->d_ring, n * 4 * 7056, cudaMemcpyDeviceToDevice);

@@ -27,7 +27,7 @@ struct BatchArgs {
   const uint8_t *cache;
   const uint8_t *romb;       // [n_roms][ROMB_SLOT] cartridge bytes, banks of 4096
   const uint32_t *info;      // per ROM: scheme | score << 8 | gameover << 16 | banks << 24
-  const uint8_t *dec_op;     // 512 bytes: op per opcode, then mode/cycles/penalty per opcode
+  const uint8_t *dec_op;     // DEC_BYTES: op per opcode, mode/cycles/penalty per opcode, control words
   const uint8_t *actions;
   int32_t *rew_int;
   uint8_t *done_int;
@@ -64,96 +64,99 @@ __device__ __forceinline__ void fast_reset_from_cache(uint8_t *st, const uint8_t
   *reinterpret_cast<uint32_t *>(st + S::EPISODE) = episode;
 }
 
-// Env slot i; o = where its action is read and its reward and done written.
-// Split form: logged-frame setup, frame records and the log count happen on
-// the TIA side, in queue order; the step ends once the TIA side has caught up.
-template <bool SPLIT, bool COMPACT>
-__device__ __forceinline__ void fast_step_env(FastConsoleT<SPLIT, COMPACT> &m, uint8_t *st, int i, int o, const BatchArgs &a,
-                                              uint32_t rom, uint32_t score, uint32_t gameover) {
-  const uint32_t *ew = reinterpret_cast<const uint32_t *>(st + S::EPISODE);
-  uint32_t episode = ew[0], step_no = ew[1], env_key = ew[2], env_status = ew[3];
-  uint32_t last = st[S::LAST_ACTION];
-  uint32_t score_prev = st[S::SCORE_PREV];
-  uint32_t action = a.actions[o];
-  if (action >= 18) { env_status |= ST_BAD_ACTION; action = 0; }
-  int32_t reward = 0;
-  uint32_t log_total = 0;
-  const int F = a.frameskip;
-  for (int f = 1; f <= F; ++f) {
+// Where the TIA side of env slot i leaves its logs and snapshots.
+__device__ __forceinline__ TiaOut tia_out_of(const BatchArgs &a, int i) {
+  return TiaOut{a.log + (size_t)i * 2 * a.log_cap, a.snap + (size_t)i * 128, a.bsnap ? a.bsnap + (size_t)i * 384 : nullptr,
+                a.meta + (size_t)i * 4, (uint32_t)a.log_cap};
+}
+
+// The frames of one env's step: the action of each frame (sticky draws), the
+// logged frames' marks, and the reward.
+template <bool SPLIT>
+struct StepHook {
+  const BatchArgs *a;
+  uint32_t score;
+  uint32_t env_key, step_no, episode, action, last, score_prev;
+  int32_t reward;
+  int f;
+
+  __device__ void start_frame(FastConsoleT<SPLIT> &m) {
     uint32_t act = action;
-    if (a.sticky) {
-      uint32_t u = philox_x0(a.seed, env_key, step_no, (uint32_t)f | PURPOSE_STICKY << 8, episode);
+    if (a->sticky) {
+      const uint32_t u = philox_x0(a->seed, env_key, step_no, (uint32_t)f | PURPOSE_STICKY << 8, episode);
       if (u < 0x40000000u) act = last;
     }
     last = act;
     m.apply_action(act);
-    const int slot = f - (F - 1);
-    const bool logging = slot >= a.first_slot;
-    if constexpr (SPLIT) {
-      if (logging) m.push(EV_BEGIN_LOG | (uint32_t)slot);
-      m.run_frame();
-      if (logging) m.push(EV_END_LOG | (uint32_t)slot);
-    } else {
-      if (logging) {
-        m.snapshot(a.snap + ((size_t)i * 2 + slot) * 64);
-        m.set_log(a.log + ((size_t)i * 2 + slot) * a.log_cap, (uint32_t)a.log_cap,
-                  a.bsnap ? a.bsnap + ((size_t)i * 2 + slot) * 3 * 64 : nullptr);
-      } else {
-        m.set_log(nullptr, 0, nullptr);
-      }
-      const uint32_t lines = m.run_frame();
-      if (logging) {
-        m.finish_bands();
-        uint32_t *mt = a.meta + ((size_t)i * 2 + slot) * 2;
-        const uint32_t nrec = m.log_count();
-        mt[0] = nrec;
-        mt[1] = lines;
-        log_total += nrec;
-      }
-    }
-    const uint32_t s = m.ram[score];
+    const int slot = f - (a->frameskip - 1);
+    if (slot >= a->first_slot) m.push(EV_BEGIN_LOG | (uint32_t)slot);
+  }
+  __device__ bool frame_done(FastConsoleT<SPLIT> &m) {
+    const int slot = f - (a->frameskip - 1);
+    if (slot >= a->first_slot) m.push(EV_END_LOG | (uint32_t)slot);
+    const uint32_t s = m.ram(score);
     reward += (int32_t)(int8_t)(uint8_t)(s - score_prev);
     score_prev = s;
+    if (f == a->frameskip) return false;
+    ++f;
+    start_frame(m);
+    return true;
   }
+};
+
+// Env slot i; o = where its action is read and its reward and done written.
+// Split form: the step ends once the TIA side has caught up.
+template <bool SPLIT>
+__device__ __forceinline__ void fast_step_env(FastConsoleT<SPLIT> &m, uint8_t *st, int i, int o, const BatchArgs &a, uint32_t rom, uint32_t score,
+                                              uint32_t gameover) {
+  const uint32_t *ew = reinterpret_cast<const uint32_t *>(st + S::EPISODE);
+  uint32_t env_status = ew[3];
+  uint32_t action = a.actions[o];
+  if (action >= 18) { env_status |= ST_BAD_ACTION; action = 0; }
+  StepHook<SPLIT> h{&a, score, ew[2], ew[1], ew[0], action, st[S::LAST_ACTION], st[S::SCORE_PREV], 0, 1};
+  h.start_frame(m);
+  m.run(h);
   if constexpr (SPLIT) {
     m.push(EV_STEP_END);
-    m.wait_ack(m.nreq + 1);
+    if (!m.broken && !fc_q_wait_ack(m.io, m.nreq + 1)) m.stall();
+  } else {
+    m.drain();
   }
   env_status |= m.all_status();
   if (m.jam) env_status |= ST_ILLEGAL;
-  const uint32_t done = (m.ram[gameover] != 0 || m.jam) ? 1u : 0u;
-  a.rew_int[i] = reward;
+  const uint32_t done = (m.ram(gameover) != 0 || m.jam) ? 1u : 0u;
+  a.rew_int[i] = h.reward;
   a.done_int[i] = (uint8_t)done;
-  if (a.rew_out) a.rew_out[o] = reward;
+  if (a.rew_out) a.rew_out[o] = h.reward;
   if (a.done_out) a.done_out[o] = (uint8_t)done;
   if (a.counters) {
     a.counters[3 * i] = m.instret;
     a.counters[3 * i + 2] = m.rounds;
-    if constexpr (!SPLIT) a.counters[3 * i + 1] = log_total;
+    if constexpr (!SPLIT) a.counters[3 * i + 1] = m.ts.log_total;
   }
   uint32_t *ewo = reinterpret_cast<uint32_t *>(st + S::EPISODE);
-  ewo[1] = step_no + 1;
+  ewo[1] = h.step_no + 1;
   ewo[3] = env_status;
   if (done) {
-    fast_reset_from_cache(st, a.cache, score, rom, (uint32_t)a.n_cache, a.seed, env_key, episode + 1);
+    fast_reset_from_cache(st, a.cache, score, rom, (uint32_t)a.n_cache, a.seed, h.env_key, h.episode + 1);
   } else {
     m.store(st);
-    st[S::LAST_ACTION] = (uint8_t)last;
-    st[S::SCORE_PREV] = (uint8_t)score_prev;
+    st[S::LAST_ACTION] = (uint8_t)h.last;
+    st[S::SCORE_PREV] = (uint8_t)h.score_prev;
   }
 }
 
 // TIA side of the split form for env slot i: applies the CPU side's events in
 // order until the end of the step.  Every wait is bounded; running out sets
 // ST_STALL and ends the loop.
-__device__ void tia_worker(IoCtx c, const uint32_t *q, int i, const BatchArgs &a) {
+__device__ void tia_worker(IoCtx c, uint32_t q, int i, const BatchArgs &a) {
   if (a.tia_off) return;
-  volatile uint32_t *vw = reinterpret_cast<volatile uint32_t *>(c.w());
-  const volatile uint32_t *vq = reinterpret_cast<const volatile uint32_t *>(q);
-  uint32_t head = 0, ack = 0, lines = 0, log_total = 0;
+  const TiaOut out = tia_out_of(a, i);
+  TiaSide s{0, 0, 0, 0};
   uint64_t idle_since = 0;  // global-timer time the queue was first seen empty (0: not idle)
   for (;;) {
-    if (head == vw[IO_QTAIL]) {
+    const uint32_t ev = vsm32(q + 4 * (s.head & (QLEN - 1)));
+    if ((ev ^ lap_bit(s.head)) & 0x80000000u) {
       const uint64_t now = global_ns();
       if (!idle_since) idle_since = now;
       else if (now - idle_since >= WAIT_NS) {
@@ -164,132 +167,63 @@ __device__ void tia_worker(IoCtx c, const uint32_t *q, int i, const BatchArgs &a
       continue;
     }
     idle_since = 0;
-    __threadfence_block();
-    const uint32_t ev = vq[head & (QLEN - 1)];
-    vw[IO_QHEAD] = ++head;
-    const uint32_t kind = ev >> 30;
-    if (kind == 0) {
-      fc_tia_write(c, (ev >> 8) & 0x3F, ev & 0xFF, (ev >> 14) & 0xFFFF, false);
-    } else if (kind == 1) {
-      lines = ev & 0x3FFF;
-      fc_frame_end(c, (ev >> 14) & 0xFFFF, lines);
-    } else {
-      const uint32_t sub = (ev >> 28) & 3, slot = ev & 1;
-      if (sub == 0) {
-        fc_snapshot(c, a.snap + ((size_t)i * 2 + slot) * 64, 0);
-        fc_set_log(c, a.log + ((size_t)i * 2 + slot) * a.log_cap, (uint32_t)a.log_cap,
-                   a.bsnap ? a.bsnap + ((size_t)i * 2 + slot) * 3 * 64 : nullptr);
-      } else if (sub == 1) {
-        if (c.G(IO_BANDN) < 4) fc_band_snap(c, ~0u);
-        const uint32_t nrec = c.G(IO_LOGN);
-        uint32_t *mt = a.meta + ((size_t)i * 2 + slot) * 2;
-        mt[0] = nrec;
-        mt[1] = lines;
-        log_total += nrec;
-        fc_set_log(c, nullptr, 0, nullptr);
-      } else if (sub == 2) {
-        fc_cx_eval(c, 3u * (ev & 0xFFFFu));
-        __threadfence_block();
-        vw[IO_ACK] = ++ack;
-      } else {
-        if (a.counters) a.counters[3 * i + 1] = log_total;
-        __threadfence_block();
-        vw[IO_ACK] = ++ack;
-        break;
-      }
+    ++s.head;
+    __threadfence_block();  // the entry is read before its place is given back
+    c.V(IO_QHEAD) = s.head;
+    const uint32_t r = tia_event(c, ev, s, out);
+    if (r) {
+      if ((r & TIA_END) && a.counters) a.counters[3 * i + 1] = s.log_total;
+      __threadfence_block();
+      c.V(IO_ACK) = ++s.ack;
+      if (r & TIA_END) break;
     }
   }
 }
 
-template <bool COMPACT>
-__global__ void __launch_bounds__(128) k_interp_batched(BatchArgs a) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  uint8_t *rom8 = smem;                                  // rom_stage bytes, then 16 of padding
-  uint8_t *dec_op = smem + (size_t)a.rom_stage + 16;
-  uint8_t *ram = dec_op + 512;
-  uint32_t *iow = reinterpret_cast<uint32_t *>(ram + RAM_BYTES * a.E);
-  uint8_t *tia = reinterpret_cast<uint8_t *>(iow + IO_STRIDE * a.E);
-  __shared__ int s_group;
-  for (int t = threadIdx.x; t < 512; t += blockDim.x) dec_op[t] = a.dec_op[t];
-  int cur_rom = -1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (;;) {
-    __syncthreads();  // everyone is done with the previous item (ROM words, s_group)
-    if (threadIdx.x == 0) s_group = atomicAdd(a.queue, 1);
-    __syncthreads();
-    const int g = s_group;
-    if (g >= a.n_groups) break;
-    const int rom = a.grp_rom[g];
-    if (rom != cur_rom) {
-      const uint32_t banks = a.info[rom] >> 24;
-      const uint4 *src = reinterpret_cast<const uint4 *>(a.romb + (size_t)rom * ROMB_SLOT);
-      uint4 *dst = reinterpret_cast<uint4 *>(rom8);
-      for (uint32_t q = threadIdx.x; q < banks * 256u; q += blockDim.x) dst[q] = src[q];
-      if (threadIdx.x == 0) dst[banks * 256u] = make_uint4(0, 0, 0, 0);
-      cur_rom = rom;
-      __syncthreads();
-    }
-    const int jj = warp * a.lanes + lane;
-    const bool runs = lane < a.lanes && jj < a.grp_count[g];
-    const uint32_t wmask = __ballot_sync(0xFFFFFFFFu, runs);
-    if (runs) {
-      const int j = jj;
-      {
-        const int p = a.grp_start[g] + j;
-        const int i = a.perm[p];
-        const int o = a.opos ? a.opos[p] : i;
-        uint8_t *st = a.state + (size_t)i * 256;
-        const uint32_t inf = a.info[rom];
-        FastConsoleT<false, COMPACT> m;
-        m.rom8 = rom8;
-        m.dec_op = dec_op;
-        m.ram = ram + RAM_BYTES * j;
-        m.io = IoCtx{tia + TIA_STRIDE * j, iow + IO_STRIDE * j};
-        m.scheme = inf & 0xFF;
-        m.wmask = wmask;
-        m.idle = (uint32_t)a.idle;
-        m.load(st);
-        fast_step_env(m, st, i, o, a, (uint32_t)rom, (inf >> 8) & 0x7F, (inf >> 16) & 0x7F);
-      }
-    }
-  }
+// Shared memory of a block: the cartridge stage (and 16 bytes of padding),
+// the decoder's bytes and control words, then per env RAM, I/O words, TIA
+// file and event queue.
+__device__ __forceinline__ EnvOff env_off(uint32_t rom_stage, uint32_t envs, uint32_t j) {
+  EnvOff o;
+  o.rom = 0;
+  o.dec = rom_stage + 16;
+  const uint32_t ram = o.dec + DEC_BYTES;
+  const uint32_t io = ram + RAM_BYTES * envs, tia = io + 4 * IO_STRIDE * envs, q = tia + TIA_STRIDE * envs;
+  o.ram = ram + RAM_BYTES * j;
+  o.io = io + 4 * IO_STRIDE * j;
+  o.tia = tia + TIA_STRIDE * j;
+  o.q = q + 4 * QSTRIDE * j;
+  return o;
 }
 
-// Split form: blockDim = 2 W warps; warps [0, W) run the CPUs of the work
-// item's envs, warp W + w the TIA side of CPU warp w's envs (lane for lane).
-// Shared memory: cartridge stage, decoder table, per-env RAM, I/O words, TIA
-// file, then the per-env event queues.
-template <bool COMPACT>
-__global__ void __launch_bounds__(256, 2) k_interp_split(BatchArgs a) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  uint8_t *rom8 = smem;
-  uint8_t *dec_op = smem + (size_t)a.rom_stage + 16;
-  uint8_t *ram = dec_op + 512;
-  uint32_t *iow = reinterpret_cast<uint32_t *>(ram + RAM_BYTES * a.E);
-  uint8_t *tia = reinterpret_cast<uint8_t *>(iow + IO_STRIDE * a.E);
-  uint32_t *qs = reinterpret_cast<uint32_t *>(tia + TIA_STRIDE * a.E);
+// blockDim = W warps (single-warp form) or 2 W (split form); warps [0, W) run
+// the CPUs of the work item's envs, in the split form warp W + w the TIA side
+// of CPU warp w's envs (lane for lane).
+template <bool SPLIT>
+__device__ __forceinline__ void interp_block(const BatchArgs &a) {
   __shared__ int s_group;
-  for (int t = threadIdx.x; t < 512; t += blockDim.x) dec_op[t] = a.dec_op[t];
+  for (uint32_t t = threadIdx.x; t < DEC_BYTES / 4; t += blockDim.x)
+    sm32((uint32_t)a.rom_stage + 16 + 4 * t) = reinterpret_cast<const uint32_t *>(a.dec_op)[t];
   int cur_rom = -1;
   const int W = a.E / a.lanes;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool cpu = warp < W;
   const int cw = cpu ? warp : warp - W;
   for (;;) {
-    __syncthreads();
+    __syncthreads();  // everyone is done with the previous item (cartridge, s_group)
     if (threadIdx.x == 0) s_group = atomicAdd(a.queue, 1);
     __syncthreads();
     const int g = s_group;
     if (g >= a.n_groups) break;
     const int rom = a.grp_rom[g];
+    const uint32_t inf = a.info[rom];
     if (rom != cur_rom) {
-      const uint32_t banks = a.info[rom] >> 24;
+      const uint32_t banks = inf >> 24;
       const uint4 *src = reinterpret_cast<const uint4 *>(a.romb + (size_t)rom * ROMB_SLOT);
-      uint4 *dst = reinterpret_cast<uint4 *>(rom8);
+      uint4 *dst = reinterpret_cast<uint4 *>(g_smem);
       for (uint32_t q = threadIdx.x; q < banks * 256u; q += blockDim.x) dst[q] = src[q];
       if (threadIdx.x == 0) dst[banks * 256u] = make_uint4(0, 0, 0, 0);
       cur_rom = rom;
-      __syncthreads();
     }
     const int jj = cw * a.lanes + lane;
     const bool runs = lane < a.lanes && jj < a.grp_count[g];
@@ -298,28 +232,25 @@ __global__ void __launch_bounds__(256, 2) k_interp_split(BatchArgs a) {
     const int i = runs ? a.perm[p] : 0;
     const int o = runs ? (a.opos ? a.opos[p] : i) : 0;
     uint8_t *st = a.state + (size_t)i * 256;
-    const uint32_t inf = a.info[rom];
-    const IoCtx io{tia + TIA_STRIDE * jj, iow + IO_STRIDE * jj};
-    uint32_t *q = qs + QSTRIDE * jj;
-    FastConsoleT<true, COMPACT> m;
+    const EnvOff off = env_off((uint32_t)a.rom_stage, (uint32_t)a.E, (uint32_t)jj);
+    FastConsoleT<SPLIT> m;
     if (cpu && runs) {
-      m.rom8 = rom8;
-      m.dec_op = dec_op;
-      m.ram = ram + RAM_BYTES * jj;
-      m.io = io;
-      m.q = q;
+      m.attach(off);
       m.scheme = inf & 0xFF;
       m.wmask = wmask;
       m.idle = (uint32_t)a.idle;
+      m.to = tia_out_of(a, i);
       m.load(st);
     }
-    __syncthreads();  // the envs' state is in shared memory before the TIA side starts
+    __syncthreads();  // the cartridge and the envs' state are in shared memory
     if (runs) {
-      if (cpu) fast_step_env<true, COMPACT>(m, st, i, o, a, (uint32_t)rom, (inf >> 8) & 0x7F, (inf >> 16) & 0x7F);
-      else tia_worker(io, q, i, a);
+      if (cpu) fast_step_env<SPLIT>(m, st, i, o, a, (uint32_t)rom, (inf >> 8) & 0x7F, (inf >> 16) & 0x7F);
+      else tia_worker(IoCtx{off.tia, off.io}, off.q, i, a);
     }
   }
 }
+__global__ void __launch_bounds__(128) k_interp_batched(const __grid_constant__ BatchArgs a) { interp_block<false>(a); }
+__global__ void __launch_bounds__(256, 2) k_interp_split(const __grid_constant__ BatchArgs a) { interp_block<true>(a); }
 
 // Bank-aware grouping: within each cartridge's run [seg[r], seg[r+1]) of the
 // env list, envs are ordered by the bank their canonical state holds at the

@@ -1,25 +1,26 @@
 // Console for the batched form, laid out for the issue rate of sm_103a.
 //
 // Same machine and canonical state as Console in device_machine.cuh:
-//   - the hot loop is a single switch on the opcode byte; every case has its
-//     addressing mode and cycle count folded in;
-//   - CPU registers (flags split, N and Z kept as the last result byte),
-//     the cycle counter and the bank in registers;
+//   - the hot loop is one branch-free sequence for every common instruction,
+//     steered by control words per opcode (opcode_ctl.h);
+//   - CPU registers, flags, the cycle counter and the bank in registers;
 //   - RAM (bytes), the TIA register file (bytes) and the I/O state
 //     (collision cursor and latches, RIOT timer and ports, inputs, log
 //     cursor, frame base line) in shared memory, one block per env with odd
 //     word strides, so lanes reading the same field never bank-conflict and
-//     every access is a base pointer plus an offset;
+//     every access is a base offset plus a constant or one add;
 //   - the block's cartridge staged in shared memory as bytes (16 KB for an
 //     F6 cartridge); an instruction's bytes are fetched as two aligned words
 //     joined by one funnel shift.
-// Instructions the hot switch does not take (BRK, RTI, JMP (ind), undocumented
-// opcodes, stack or pointer bytes outside RAM, fetches outside the cartridge
-// or next to a bank hotspot) run the general decoder out of line.
+// Instructions the hot loop does not take (TIA and RIOT reads, RIOT, VSYNC
+// and VBLANK writes, stack and pointer instructions, undocumented opcodes,
+// decimal arithmetic, fetches outside the cartridge or next to a bank
+// hotspot) run the general decoder out of line.
 #pragma once
 #include <cstdint>
 
 #include "device_machine.cuh"
+#include "opcode_ctl.h"
 
 namespace atari {
 
@@ -35,10 +36,10 @@ enum IoWord : uint32_t {
   IO_JOY, IO_FIRE, IO_LATCH, IO_LOGLO, IO_LOGHI, IO_LOGN, IO_LOGCAP, IO_STATUS,
   IO_BANDN,      // next quarter-frame band whose start snapshot is due (1..3), 4: none
   IO_BSLO, IO_BSHI,  // where this frame's band snapshots go (3 x 64 bytes)
-  IO_QHEAD, IO_QTAIL, IO_ACK,  // split form: TIA event queue cursors and the TIA side's acknowledgements
+  IO_QHEAD, IO_QTAIL, IO_ACK,  // split form: the TIA side's queue cursor and acknowledgements
   IO_WORDS
 };
-constexpr uint32_t IO_WSYNC = 1u, IO_VSYNC_RISE = 2u;
+constexpr uint32_t IO_WSYNC = 1u;
 
 
 // Per-env blocks of shared memory, env-major, with strides chosen so that a
@@ -50,26 +51,33 @@ constexpr uint32_t IO_WSYNC = 1u, IO_VSYNC_RISE = 2u;
 constexpr uint32_t RAM_BYTES = 132, IO_STRIDE = IO_WORDS, TIA_STRIDE = 44;
 static_assert(IO_STRIDE % 2 == 1 && (TIA_STRIDE / 4) % 2 == 1 && (RAM_BYTES / 4) % 2 == 1 && RAM_BYTES % 4 == 0,
               "odd word strides");
-constexpr uint32_t ENV_SMEM = RAM_BYTES + 4 * IO_STRIDE + TIA_STRIDE;
+constexpr uint32_t QLEN = 32;             // event queue entries per env (a power of two)
+constexpr uint32_t QSTRIDE = QLEN + 1;    // shared-memory words per env queue (odd)
+constexpr uint32_t ENV_SMEM = RAM_BYTES + 4 * IO_STRIDE + TIA_STRIDE + 4 * QSTRIDE;
 // bytes per cartridge in the batched form's device copy (up to eight 4 KB banks, F4)
 constexpr uint32_t ROMB_SLOT = 32768;
 
-// Shared-memory views of one env's TIA file and I/O state.  The pointers
-// reach the out-of-line I/O functions as plain pointers; the assumption lets
-// the compiler address them as shared memory there too.
+// The block's dynamic shared memory; every block of an env is a byte offset
+// into it, so that out-of-line functions address it as shared memory too.
+extern __shared__ __align__(16) uint8_t g_smem[];
+__device__ __forceinline__ uint8_t &sm8(uint32_t off) { return g_smem[off]; }
+__device__ __forceinline__ uint32_t &sm32(uint32_t off) { return *reinterpret_cast<uint32_t *>(g_smem + off); }
+__device__ __forceinline__ volatile uint32_t &vsm32(uint32_t off) {
+  return *reinterpret_cast<volatile uint32_t *>(g_smem + off);
+}
+
+// Views of one env's TIA file and I/O state.
 struct IoCtx {
-  uint8_t *tia;
-  uint32_t *io;
-  __device__ __forceinline__ uint8_t *t() const { __builtin_assume(__isShared(tia)); return tia; }
-  __device__ __forceinline__ uint32_t *w() const { __builtin_assume(__isShared(io)); return io; }
-  __device__ __forceinline__ uint32_t T(uint32_t s) const { return t()[s]; }
-  __device__ __forceinline__ void Tset(uint32_t s, uint32_t v) const { t()[s] = (uint8_t)v; }
-  __device__ __forceinline__ uint32_t G(uint32_t i) const { return w()[i]; }
-  __device__ __forceinline__ void Sset(uint32_t i, uint32_t v) const { w()[i] = v; }
-  __device__ __forceinline__ uint64_t G64(uint32_t i) const { return (uint64_t)w()[i] | (uint64_t)w()[i + 1] << 32; }
+  uint32_t tia, io;
+  __device__ __forceinline__ uint32_t T(uint32_t s) const { return sm8(tia + s); }
+  __device__ __forceinline__ void Tset(uint32_t s, uint32_t v) const { sm8(tia + s) = (uint8_t)v; }
+  __device__ __forceinline__ uint32_t G(uint32_t i) const { return sm32(io + 4 * i); }
+  __device__ __forceinline__ void Sset(uint32_t i, uint32_t v) const { sm32(io + 4 * i) = v; }
+  __device__ __forceinline__ volatile uint32_t &V(uint32_t i) const { return vsm32(io + 4 * i); }
+  __device__ __forceinline__ uint64_t G64(uint32_t i) const { return (uint64_t)G(i) | (uint64_t)G(i + 1) << 32; }
   __device__ __forceinline__ void S64(uint32_t i, uint64_t v) const {
-    w()[i] = (uint32_t)v;
-    w()[i + 1] = (uint32_t)(v >> 32);
+    Sset(i, (uint32_t)v);
+    Sset(i + 1, (uint32_t)(v >> 32));
   }
 };
 
@@ -177,21 +185,6 @@ __device__ __forceinline__ uint32_t fc_riot_read(IoCtx c, uint32_t a, uint64_t n
 __device__ __forceinline__ uint32_t fc_cx_byte(uint32_t cx, uint32_t reg) {
   return (((cx >> (2 * reg + 1)) & 1u) << 7) | (((cx >> (2 * reg)) & 1u) << 6);
 }
-// Read a TIA or RIOT address (13-bit, neither RAM nor cartridge) at cycle t.
-__device__ __noinline__ uint32_t fc_io_read(IoCtx c, uint32_t a, uint32_t t) {
-  if (!(a & 0x80)) {
-    const uint32_t reg = a & 0x0F;
-    if (reg < 8) {
-      fc_cx_eval(c, 3u * t);
-      return fc_cx_byte(c.G(IO_CX), reg);
-    }
-    if (reg == 0x0C) return (c.G(IO_FIRE) || c.G(IO_LATCH)) ? 0x00u : 0x80u;
-    if (reg == 0x0D) return 0x80u;
-    return 0;
-  }
-  return fc_riot_read(c, a, 76ull * c.G64(IO_L0LO) + t);
-}
-
 // 64-byte render snapshot: TIA file (canonical bytes 0x20..0x44), HMOVE bar
 // line, frame base line; word 14 = the number of log records before it.
 __device__ __forceinline__ void fc_snapshot(IoCtx c, uint8_t *o, uint32_t nrec) {
@@ -256,10 +249,6 @@ __device__ __forceinline__ void fc_log(IoCtx c, uint32_t eff, uint32_t reg, uint
   }
 }
 
-// TIA registers whose writes only set a colour or a motion register: logged,
-// no collision or timing effect (COLUP0, COLUP1, COLUPF, COLUBK, HMP0..HMBL).
-constexpr uint64_t FAST_TIA_REGS = (0xFull << 0x06) | (0x1Full << 0x20);
-
 // Write a RIOT address at absolute CPU cycle `now`.
 __device__ __forceinline__ void fc_riot_write(IoCtx c, uint32_t a, uint32_t v, uint64_t now) {
   if (!(a & 4)) {
@@ -272,27 +261,15 @@ __device__ __forceinline__ void fc_riot_write(IoCtx c, uint32_t a, uint32_t v, u
     c.S64(IO_TCWLO, now);
   }
 }
-// The TIA part of a write (register reg at cycle t): collisions up to the
-// write, log record, register update.  cpu_latch: this thread also keeps the
-// fire-button latch (the split form keeps it on the CPU side).
-__device__ __forceinline__ uint32_t fc_tia_write(IoCtx c, uint32_t reg, uint32_t v, uint32_t t, bool cpu_latch) {
+// Apply a TIA write (register reg at cycle t): collisions up to the write,
+// log record, register update.
+__device__ __forceinline__ void fc_tia_write(IoCtx c, uint32_t reg, uint32_t v, uint32_t t) {
   const uint32_t eff = 3u * (t + 1u);
   if ((COLL_REGS >> reg) & 1ull) fc_cx_eval(c, eff);
   if ((LOG_REGS >> reg) & 1ull) fc_log(c, eff, reg, v);
-  uint32_t flags = 0;
   switch (reg) {
-    case 0x00:
-      if (!(c.T(T_VSYNC) & 2) && (v & 2)) flags |= IO_VSYNC_RISE;
-      c.Tset(T_VSYNC, v);
-      break;
-    case 0x01:
-      c.Tset(T_VBLANK, v);
-      if (cpu_latch) {
-        if (!(v & 0x40)) c.Sset(IO_LATCH, 0);
-        else if (c.G(IO_FIRE)) c.Sset(IO_LATCH, 1);
-      }
-      break;
-    case 0x02: flags |= IO_WSYNC; break;
+    case 0x00: c.Tset(T_VSYNC, v); break;
+    case 0x01: c.Tset(T_VBLANK, v); break;
     case 0x04: case 0x05: case 0x06: case 0x07: case 0x08: case 0x09: case 0x0A: case 0x0B: case 0x0C:
     case 0x0D: case 0x0E: case 0x0F:
       c.Tset(reg - 2, v); break;                 // NUSIZ0 .. PF2 are slots 2 .. 13
@@ -334,40 +311,31 @@ __device__ __forceinline__ uint32_t fc_tia_write(IoCtx c, uint32_t reg, uint32_t
       break;
     default: break;  // RSYNC, audio, unused addresses
   }
-  return flags;
-}
-// Write a TIA or RIOT address at cycle t; returns IO_WSYNC / IO_VSYNC_RISE.
-__device__ __noinline__ uint32_t fc_io_write(IoCtx c, uint32_t a, uint32_t v, uint32_t t) {
-  if (a & 0x80) {
-    fc_riot_write(c, a, v, 76ull * c.G64(IO_L0LO) + t);
-    return 0;
-  }
-  return fc_tia_write(c, a & 0x3F, v, t, true);
 }
 
-// End of a frame: collisions up to the current cycle, then rebase to the next frame.
-__device__ __noinline__ void fc_frame_end(IoCtx c, uint32_t kf, uint32_t next_rel) {
-  fc_cx_eval(c, 3u * kf);
-  c.S64(IO_L0LO, c.G64(IO_L0LO) + next_rel);
-  c.Sset(IO_CEVAL, c.G(IO_CEVAL) - 228u * next_rel);
-}
-
-// ---------------------------------------------------------------- split form
-// In the split form a block's warps come in pairs: a CPU warp runs the 6507
-// and RIOT and pushes every TIA write into a per-env queue in shared memory;
-// the paired TIA warp (same lane, same env) applies the writes, logs them and
-// evaluates collisions.  The CPU keeps its own copies of VSYNC, VBLANK, the
-// fire latch and the frame base line; it waits for the TIA side only when it
-// reads a collision register and at the end of the step.  Events (32 bits):
-//   write       0b00 | cycle:16 | register:6 | value:8
-//   frame end   0b01 | cycle of the end:16 | lines to the next frame:14
-//   control     0b10 | kind:2 | argument   (begin/end of a logged frame,
-//               collision sync up to a cycle, end of the step)
-constexpr uint32_t QLEN = 32;             // queue entries per env (a power of two)
-constexpr uint32_t QSTRIDE = QLEN + 1;    // shared-memory words per env queue (odd)
-constexpr uint32_t EV_WRITE = 0u, EV_FRAME_END = 1u << 30, EV_CTRL = 2u << 30;
-constexpr uint32_t EV_BEGIN_LOG = EV_CTRL, EV_END_LOG = EV_CTRL | 1u << 28, EV_SYNC = EV_CTRL | 2u << 28,
-                   EV_STEP_END = EV_CTRL | 3u << 28;
+// ---------------------------------------------------------------- event queue
+// The CPU side pushes every TIA write into a per-env queue in shared memory;
+// the TIA side applies the writes, logs them and evaluates collisions.  In
+// the split form the TIA side is a second warp of the block (same lane, same
+// env); in the single-warp form the warp drains its own queues between
+// batches of instructions.  The CPU keeps its own copies of VSYNC, VBLANK,
+// the fire latch and the frame base line; it waits for the TIA side only when
+// it reads a collision register and at the end of the step.
+// An event is one 32-bit word, written and read whole, so the word itself
+// tells that it is there: bit 31 holds the parity of the queue's lap (1 in
+// the first lap over the zeroed queue), and no fence orders data behind a
+// cursor.  Bits 0-30:
+//   write       0 | cycle:16 | register:6 | value:8
+//   control     1 | kind:2 | argument:
+//     mark      begin / end of a logged frame, end of the step
+//     sync      evaluate collisions up to a cycle and acknowledge
+//     frame end evaluate collisions up to the frame's last cycle
+//     rebase    lines to the next frame's first line (follows the frame end)
+constexpr uint32_t EV_CTRL = 1u << 30, EV_MARK = EV_CTRL, EV_SYNC = EV_CTRL | 1u << 28,
+                   EV_FRAME_END = EV_CTRL | 2u << 28, EV_REBASE = EV_CTRL | 3u << 28;
+constexpr uint32_t EV_BEGIN_LOG = EV_MARK, EV_END_LOG = EV_MARK | 1u << 26, EV_STEP_END = EV_MARK | 2u << 26;
+// Lap parity of queue position k, in bit 31.
+__device__ __forceinline__ uint32_t lap_bit(uint32_t k) { return (~k << 26) & 0x80000000u; }
 // A wait between an env's CPU and TIA warps gives up after WAIT_NS of the
 // GPU's global timer and the env is declared stalled.  The longest legitimate
 // wait is about one frame of the slowest lane of the partner warp (a few
@@ -378,87 +346,137 @@ __device__ __forceinline__ uint64_t global_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-// registers whose writes reach the TIA side (WSYNC, RSYNC, audio and unused
-// addresses change nothing there)
-constexpr uint64_t SPLIT_PUSH_REGS = LOG_REGS | COLL_REGS | 1ull | (1ull << 0x2C);
+
+// Where the TIA side of one env leaves its logs and snapshots.
+struct TiaOut {
+  uint32_t *log;      // two logs of log_cap records
+  uint8_t *snap;      // two 64-byte snapshots
+  uint8_t *bsnap;     // null, or two times three band snapshots
+  uint32_t *meta;     // two times (records, lines)
+  uint32_t log_cap;
+};
+struct TiaSide {
+  uint32_t head, ack, lines, log_total;
+};
+constexpr uint32_t TIA_ACK = 1u, TIA_END = 2u;
+// Apply one event; returns TIA_ACK when the CPU side waits for it, and
+// TIA_END when it ends the step.
+__device__ __forceinline__ uint32_t tia_event(IoCtx c, uint32_t ev, TiaSide &s, const TiaOut &o) {
+  if (!(ev & EV_CTRL)) {
+    fc_tia_write(c, (ev >> 8) & 0x3F, ev & 0xFF, (ev >> 14) & 0xFFFF);
+    return 0;
+  }
+  const uint32_t kind = (ev >> 28) & 3;
+  if (kind == 1) {
+    fc_cx_eval(c, 3u * (ev & 0xFFFFu));
+    return TIA_ACK;
+  }
+  if (kind == 2) {
+    fc_cx_eval(c, 3u * (ev & 0xFFFFu));
+    return 0;
+  }
+  if (kind == 3) {
+    s.lines = ev & 0xFFFFFFFu;
+    c.S64(IO_L0LO, c.G64(IO_L0LO) + s.lines);
+    c.Sset(IO_CEVAL, c.G(IO_CEVAL) - 228u * s.lines);
+    return 0;
+  }
+  const uint32_t sub = (ev >> 26) & 3, slot = ev & 1;
+  if (sub == 0) {
+    fc_snapshot(c, o.snap + slot * 64, 0);
+    fc_set_log(c, o.log + (size_t)slot * o.log_cap, o.log_cap, o.bsnap ? o.bsnap + slot * 3 * 64 : nullptr);
+    return 0;
+  }
+  if (sub == 1) {
+    if (c.G(IO_BANDN) < 4) fc_band_snap(c, ~0u);
+    const uint32_t nrec = c.G(IO_LOGN);
+    o.meta[2 * slot] = nrec;
+    o.meta[2 * slot + 1] = s.lines;
+    s.log_total += nrec;
+    fc_set_log(c, nullptr, 0, nullptr);
+    return 0;
+  }
+  return TIA_ACK | TIA_END;
+}
+// Single-warp form: apply an env's queued events [s.head, tail).
+__device__ __noinline__ void tia_drain(IoCtx c, uint32_t q, TiaSide &s, const TiaOut &o, uint32_t tail) {
+  while (s.head != tail) {
+    const uint32_t ev = sm32(q + 4 * (s.head & (QLEN - 1)));
+    ++s.head;
+    tia_event(c, ev, s, o);
+  }
+}
 
 // ---------------------------------------------------------------- the console
 // Split form, CPU side: bounded waits on the TIA side's cursors in this env's
-// I/O block.  Wait until the queue has room behind `qtail` (returns the last
-// head read: still full means the wait ran out), or until `n` events are
-// acknowledged (false means the wait ran out).
-__device__ __noinline__ uint32_t fc_q_wait_room(uint32_t *iow, uint32_t qtail) {
-  __builtin_assume(__isShared(iow));
-  const volatile uint32_t *h = iow + IO_QHEAD;
-  uint32_t head = *h;
-  if (qtail - head < QLEN) return head;
-  const uint64_t t0 = global_ns();
-  while (qtail - head >= QLEN && global_ns() - t0 < WAIT_NS) {
-    __nanosleep(32);
-    head = *h;
+// I/O block.  Wait until the queue has `room` free entries behind `qtail`
+// (returns the last head read: still less room means the wait ran out), or
+// until `n` events are acknowledged (false means the wait ran out).
+__device__ __noinline__ uint32_t fc_q_wait_room(IoCtx c, uint32_t qtail, uint32_t room) {
+  uint32_t head = c.V(IO_QHEAD);
+  if (qtail - head > QLEN - room) {
+    const uint64_t t0 = global_ns();
+    while (qtail - head > QLEN - room && global_ns() - t0 < WAIT_NS) {
+      __nanosleep(32);
+      head = c.V(IO_QHEAD);
+    }
   }
+  __threadfence_block();  // the TIA side has read the entries that are overwritten next
   return head;
 }
-__device__ __noinline__ bool fc_q_wait_ack(uint32_t *iow, uint32_t n) {
-  __builtin_assume(__isShared(iow));
-  const volatile uint32_t *a = iow + IO_ACK;
-  if ((int32_t)(*a - n) >= 0) return true;
-  const uint64_t t0 = global_ns();
-  while ((int32_t)(*a - n) < 0) {
-    if (global_ns() - t0 >= WAIT_NS) return false;
-    __nanosleep(32);
+__device__ __noinline__ bool fc_q_wait_ack(IoCtx c, uint32_t n) {
+  if ((int32_t)(c.V(IO_ACK) - n) < 0) {
+    const uint64_t t0 = global_ns();
+    while ((int32_t)(c.V(IO_ACK) - n) < 0) {
+      if (global_ns() - t0 >= WAIT_NS) return false;
+      __nanosleep(32);
+    }
   }
+  __threadfence_block();
   return true;
 }
 
-// Split form, CPU side: read a TIA or RIOT address (13-bit, neither RAM nor
-// cartridge) at cycle t, out of line so that the many read sites of the
-// opcode switch stay small.  A collision-latch read first pushes a sync event
-// at queue position qtail (waiting, bounded, for room behind the TIA side's
-// cursor qhead_seen) and waits until the TIA side has acknowledged nreq + 1
-// sync events, i.e. has evaluated collisions up to cycle t.  Returns the
-// value in bits 0-7; bit 8 when the sync event was pushed (the caller counts
-// it, and the queue is then empty), bit 9 when a wait ran out (the caller
-// halts the env).  `broken` (an earlier wait ran out) skips the sync and
-// returns the latches as they stand.
-constexpr uint32_t SIO_PUSHED = 0x100u, SIO_STALL = 0x200u;
-__device__ __noinline__ uint32_t fc_split_io_read(IoCtx c, uint32_t *q, uint32_t qtail, uint32_t qhead_seen,
-                                                  uint32_t nreq, uint32_t broken, uint32_t a, uint32_t t,
-                                                  uint64_t l0) {
-  if (a & 0x80) return fc_riot_read(c, a, 76ull * l0 + t);
-  const uint32_t reg = a & 0x0F;
-  if (reg == 0x0C) return (c.G(IO_FIRE) || c.G(IO_LATCH)) ? 0x00u : 0x80u;
-  if (reg == 0x0D) return 0x80u;
-  if (reg >= 8) return 0;
-  volatile uint32_t *vw = reinterpret_cast<volatile uint32_t *>(c.w());
-  if (broken) return fc_cx_byte(vw[IO_CX], reg);
-  if (qtail - qhead_seen >= QLEN) {
-    qhead_seen = fc_q_wait_room(c.w(), qtail);
-    if (qtail - qhead_seen >= QLEN) return SIO_STALL | fc_cx_byte(vw[IO_CX], reg);
-  }
-  __builtin_assume(__isShared(q));
-  reinterpret_cast<volatile uint32_t *>(q)[qtail & (QLEN - 1)] = EV_SYNC | (t & 0xFFFFu);
-  __threadfence_block();
-  vw[IO_QTAIL] = qtail + 1;
-  if (!fc_q_wait_ack(c.w(), nreq + 1)) return SIO_PUSHED | SIO_STALL | fc_cx_byte(vw[IO_CX], reg);
-  __threadfence_block();
-  return SIO_PUSHED | fc_cx_byte(vw[IO_CX], reg);
+// Byte permutation with the sign-replicating selectors (selector bit 3).
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+  return r;
+}
+// Predicated stores (addresses in the shared window), without a branch.
+__device__ __forceinline__ void sts8_if(bool c, uint32_t a, uint32_t v) {
+  asm volatile("{.reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.u8 [%1], %2;}" ::"r"((uint32_t)c), "r"(a), "r"(v)
+               : "memory");
+}
+__device__ __forceinline__ void sts32_if(bool c, uint32_t a, uint32_t v) {
+  asm volatile("{.reg .pred p; setp.ne.u32 p, %0, 0; @p st.volatile.shared.u32 [%1], %2;}" ::"r"((uint32_t)c), "r"(a),
+               "r"(v)
+               : "memory");
+}
+// Loads of the staged cartridge and the control words, which do not change
+// while a work item runs: free to move past the stores of other lanes.
+__device__ __forceinline__ uint32_t lds_const(uint32_t a) {
+  uint32_t v;
+  asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint4 lds_const4(uint32_t a) {
+  uint4 v;
+  asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
 }
 
-// COMPACT: the hot opcode switch keeps only the common addressing forms
-// (implied, accumulator, immediate, zero page and absolute reads, writes and
-// branches, indexed loads and stores); the indirect forms, BIT, stack
-// pushes and pulls and indexed or absolute read-modify-writes go to the
-// general decoder.  A smaller hot loop for the instruction cache; the
-// results are the same either way.
-template <bool SPLIT, bool COMPACT = false> struct FastConsoleT;
-template <bool SPLIT, bool COMPACT> __device__ __forceinline__ void fc_exec_general(FastConsoleT<SPLIT, COMPACT> *self);
+// Byte offsets of an env's blocks in the block's dynamic shared memory.
+struct EnvOff {
+  uint32_t rom, dec, ram, io, tia, q;
+};
+// Rounds between two looks at the lanes that wait for service.  A look costs
+// about 60 cycles beside rounds of about 270; a lane that waits loses half a
+// batch.
+constexpr uint32_t BATCH = 8;
 
-template <bool SPLIT, bool COMPACT>
+template <bool SPLIT>
 struct FastConsoleT {
-  const uint8_t *rom8;     // staged cartridge bytes (banks of 4096, then 16 bytes of padding)
-  const uint8_t *dec_op;   // general decoder: opcode -> operation | penalty << 7, then mode | cycles << 4
-  uint8_t *ram;            // this env's RAM block (shared memory, 4-byte aligned)
+  EnvOff off;              // this env's blocks of shared memory
   IoCtx io;
   uint32_t A, X, Y, SP, PC, fc, fv, fn, fz, fdi;  // fdi holds the D (0x08) and I (0x04) bits
   uint32_t bank, jam, scheme;
@@ -466,13 +484,14 @@ struct FastConsoleT {
   uint32_t pend;           // I/O flags of the current instruction
   uint32_t vs_kf;          // cycle of a VSYNC rise in this frame, ~0 if none
   uint32_t status, instret, frame_no;
-  uint32_t rounds;         // lockstep issue rounds of this env's warp in the step (the same on every lane)
-  uint32_t wmask;          // lanes of this warp running envs (lockstep issue)
+  uint32_t frame_inst;     // instret at the frame's start
+  uint32_t rounds;         // issue rounds of this env's warp in the step (the same on every lane)
+  uint32_t wmask;          // lanes of this warp running envs
   uint32_t idle;           // retire RIOT-timer wait-loop iterations at once
-  // split form: this env's TIA event queue and the CPU side's copies
-  uint32_t *q;
   uint32_t qtail, qhead_seen, nreq, vsync_c, vblank_c, broken;  // qhead_seen: the TIA side's cursor as last read
   uint64_t l0c;
+  TiaSide ts;              // single-warp form: the TIA side
+  TiaOut to;
 
   __device__ __forceinline__ uint32_t P() const {
     return (fn & 0x80) | fv | 0x20 | fdi | ((fz & 0xFF) ? 0u : 2u) | fc;
@@ -480,6 +499,13 @@ struct FastConsoleT {
   __device__ __forceinline__ void setP(uint32_t p) {
     fn = p & 0x80; fv = p & 0x40; fdi = p & 0x0C; fz = (p & 2) ? 0u : 1u; fc = p & 1;
   }
+
+  __device__ __forceinline__ void attach(const EnvOff &o) {
+    off = o;
+    io = IoCtx{o.tia, o.io};
+  }
+  __device__ __forceinline__ uint8_t &ram(uint32_t i) const { return sm8(off.ram + i); }
+  __device__ __forceinline__ uint32_t rom(uint32_t i) const { return sm8(off.rom + i); }
 
   // ---- canonical state I/O ----
   __device__ void load(const uint8_t *s) {
@@ -496,37 +522,37 @@ struct FastConsoleT {
     jam = (w7 >> 16) & 0xFF;
     io.Sset(IO_LATCH, w7 >> 24);
 #pragma unroll
-    for (int q = 0; q < 10; ++q) {
-      const uint32_t v = w[8 + q];
+    for (int q_ = 0; q_ < 10; ++q_) {
+      const uint32_t v = w[8 + q_];
 #pragma unroll
       for (int b = 0; b < 4; ++b)
-        if (q * 4 + b < 37) io.Tset(q * 4 + b, v >> (8 * b));
+        if (q_ * 4 + b < 37) io.Tset(q_ * 4 + b, v >> (8 * b));
     }
     io.Sset(IO_CX, w[17] >> 16);
     io.Sset(IO_BARLO, w[18]); io.Sset(IO_BARHI, w[19]);
     io.Sset(IO_L0LO, w[20]); io.Sset(IO_L0HI, w[21]);
     frame_no = w[22];
-    const uint64_t L0 = (uint64_t)w[20] | (uint64_t)w[21] << 32;
-    kf = (uint32_t)(k - 76ull * L0);
+    l0c = (uint64_t)w[20] | (uint64_t)w[21] << 32;
+    kf = (uint32_t)(k - 76ull * l0c);
     io.Sset(IO_CEVAL, 3u * kf);
     io.Sset(IO_JOY, 0xFF); io.Sset(IO_FIRE, 0);
     io.Sset(IO_LOGLO, 0); io.Sset(IO_LOGHI, 0); io.Sset(IO_LOGN, 0); io.Sset(IO_LOGCAP, 0);
+    io.Sset(IO_BANDN, 4);
     io.Sset(IO_STATUS, 0);
     const uint4 *r4 = reinterpret_cast<const uint4 *>(s + S::RAM);
-    uint32_t *r32 = reinterpret_cast<uint32_t *>(ram);
+    uint32_t *r32 = &sm32(off.ram);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const uint4 v = r4[q];
-      r32[4 * q] = v.x; r32[4 * q + 1] = v.y; r32[4 * q + 2] = v.z; r32[4 * q + 3] = v.w;
+    for (int q_ = 0; q_ < 8; ++q_) {
+      const uint4 v = r4[q_];
+      r32[4 * q_] = v.x; r32[4 * q_ + 1] = v.y; r32[4 * q_ + 2] = v.z; r32[4 * q_ + 3] = v.w;
     }
-    status = 0; instret = 0; rounds = 0; pend = 0; vs_kf = ~0u;
-    if constexpr (SPLIT) {
-      vsync_c = io.T(T_VSYNC);
-      vblank_c = io.T(T_VBLANK);
-      l0c = L0;
-      qtail = qhead_seen = nreq = broken = 0;
-      io.Sset(IO_QHEAD, 0); io.Sset(IO_QTAIL, 0); io.Sset(IO_ACK, 0);
-    }
+    for (uint32_t e = 0; e < QLEN; ++e) sm32(off.q + 4 * e) = 0;
+    status = 0; instret = 0; frame_inst = 0; rounds = 0; pend = 0; vs_kf = ~0u;
+    vsync_c = io.T(T_VSYNC);
+    vblank_c = io.T(T_VBLANK);
+    qtail = qhead_seen = nreq = broken = 0;
+    io.Sset(IO_QHEAD, 0); io.Sset(IO_QTAIL, 0); io.Sset(IO_ACK, 0);
+    ts = TiaSide{0, 0, 0, 0};
   }
   __device__ void store(uint8_t *s) const {
     uint32_t *w = reinterpret_cast<uint32_t *>(s);
@@ -540,29 +566,23 @@ struct FastConsoleT {
     w[6] = io.G(IO_TV) | io.G(IO_TSH) << 8 | (ports & 0xFFFF) << 16;
     w[7] = (ports >> 16) | jam << 16 | io.G(IO_LATCH) << 24;
 #pragma unroll
-    for (int q = 0; q < 10; ++q) {
+    for (int q_ = 0; q_ < 10; ++q_) {
       uint32_t v = 0;
 #pragma unroll
       for (int b = 0; b < 4; ++b)
-        if (q * 4 + b < 37) v |= io.T(q * 4 + b) << (8 * b);
-      if (q == 9) v = (v & 0xFFFFu) | io.G(IO_CX) << 16;
-      w[8 + q] = v;
+        if (q_ * 4 + b < 37) v |= io.T(q_ * 4 + b) << (8 * b);
+      if (q_ == 9) v = (v & 0xFFFFu) | io.G(IO_CX) << 16;
+      w[8 + q_] = v;
     }
     w[18] = io.G(IO_BARLO); w[19] = io.G(IO_BARHI);
     w[20] = (uint32_t)L0; w[21] = (uint32_t)(L0 >> 32);
     w[22] = frame_no; w[23] = 0;
     uint4 *r4 = reinterpret_cast<uint4 *>(s + S::RAM);
-    const uint32_t *r32 = reinterpret_cast<const uint32_t *>(ram);
+    const uint32_t *r32 = &sm32(off.ram);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) r4[q] = make_uint4(r32[4 * q], r32[4 * q + 1], r32[4 * q + 2], r32[4 * q + 3]);
+    for (int q_ = 0; q_ < 8; ++q_)
+      r4[q_] = make_uint4(r32[4 * q_], r32[4 * q_ + 1], r32[4 * q_ + 2], r32[4 * q_ + 3]);
   }
-  __device__ void snapshot(uint8_t *o) const { fc_snapshot(io, o, 0); }
-  __device__ void set_log(uint32_t *p, uint32_t cap, uint8_t *bands) { fc_set_log(io, p, cap, bands); }
-  // Band starts the frame never reached take its final state.
-  __device__ void finish_bands() {
-    if (io.G(IO_BANDN) < 4) fc_band_snap(io, ~0u);
-  }
-  __device__ uint32_t log_count() const { return io.G(IO_LOGN); }
   __device__ uint32_t all_status() const { return status | io.G(IO_STATUS); }
 
   __device__ void apply_action(uint32_t a) {
@@ -582,145 +602,102 @@ struct FastConsoleT {
                               ((d & 1) ? 0x10u : 0u)));
     const uint32_t fire = (a == 1 || a >= 10) ? 1u : 0u;
     io.Sset(IO_FIRE, fire);
-    const uint32_t vb = SPLIT ? vblank_c : io.T(T_VBLANK);
-    if (fire && (vb & 0x40)) io.Sset(IO_LATCH, 1);
+    if (fire && (vblank_c & 0x40)) io.Sset(IO_LATCH, 1);
   }
 
   // Cartridge bytes i .. i+3 of the stage, byte i lowest (i + 3 may run into
   // the padding after the last bank).
   __device__ __forceinline__ uint32_t fetch4(uint32_t i) const {
-    const uint32_t *r32 = reinterpret_cast<const uint32_t *>(rom8);
-    const uint32_t q = i >> 2;
-    return __funnelshift_r(r32[q], r32[q + 1], (i & 3u) * 8u);
+    const uint32_t a = off.rom + (i & ~3u);
+    return __funnelshift_r(sm32(a), sm32(a + 4), (i & 3u) * 8u);
   }
+  // Last offset in a bank whose instruction bytes are fetched from the stage:
+  // no such fetch touches a hotspot (F8/F6 hotspots start at $FF6, F4's at $FF4).
+  __device__ __forceinline__ uint32_t fetch_limit() const { return scheme == 3 ? 0xFF1u : scheme ? 0xFF3u : 0xFFCu; }
 
   // ---- bus ----
-  __device__ __forceinline__ void hotspot(uint32_t off) {
-    if (scheme == 1) { if (off == 0xFF8 || off == 0xFF9) bank = off - 0xFF8; }
-    else if (scheme == 2) { if (off >= 0xFF6 && off <= 0xFF9) bank = off - 0xFF6; }
-    else if (scheme == 3) { if (off >= 0xFF4 && off <= 0xFFB) bank = off - 0xFF4; }
-  }
-  __device__ __forceinline__ void note_vsync(uint32_t t) {
-    if (vs_kf == ~0u) vs_kf = t;
-  }
-  // ---- split form: the queue to the TIA side ----
-  __device__ __forceinline__ volatile uint32_t *vio(uint32_t i) const {
-    return reinterpret_cast<volatile uint32_t *>(io.w() + i);
+  __device__ __forceinline__ void hotspot(uint32_t at) {
+    if (scheme == 1) { if (at == 0xFF8 || at == 0xFF9) bank = at - 0xFF8; }
+    else if (scheme == 2) { if (at >= 0xFF6 && at <= 0xFF9) bank = at - 0xFF6; }
+    else if (scheme == 3) { if (at >= 0xFF4 && at <= 0xFFB) bank = at - 0xFF4; }
   }
   __device__ __forceinline__ void stall() {
     broken = 1;
     status |= ST_STALL;
     jam = 1;
   }
-  // Append an event (waits, bounded, while the queue is full).  The TIA
-  // side's cursor is reread only when the queue looks full; the waits run out
-  // of line so that each inlined push stays small.
-  __device__ __forceinline__ void push(uint32_t ev) {
+  // Append an event; when the queue is full the split form waits (bounded)
+  // for the TIA side, the single-warp form applies what is queued.
+  __device__ void push(uint32_t ev) {
     if (broken) return;
     if (qtail - qhead_seen >= QLEN) {
-      qhead_seen = fc_q_wait_room(io.w(), qtail);
-      if (qtail - qhead_seen >= QLEN) { stall(); return; }
+      if constexpr (SPLIT) {
+        qhead_seen = fc_q_wait_room(io, qtail, 1);
+        if (qtail - qhead_seen >= QLEN) { stall(); return; }
+      } else {
+        drain();
+      }
     }
-    reinterpret_cast<volatile uint32_t *>(q)[qtail & (QLEN - 1)] = ev;
-    __threadfence_block();
+    vsm32(off.q + 4 * (qtail & (QLEN - 1))) = ev | lap_bit(qtail);
     ++qtail;
-    *vio(IO_QTAIL) = qtail;
   }
-  // Wait (bounded) until the TIA side has acknowledged n events.
-  __device__ __forceinline__ void wait_ack(uint32_t n) {
-    if (broken) return;
-    if (!fc_q_wait_ack(io.w(), n)) { stall(); return; }
-    __threadfence_block();
+  __device__ __forceinline__ void drain() {
+    tia_drain(io, off.q, ts, to, qtail);
+    qhead_seen = ts.head;
   }
-  // TIA write in the split form: WSYNC, the VSYNC rise and the VBLANK latch
-  // effects here, the register itself on the TIA side.
-  __device__ __forceinline__ void tia_out(uint32_t reg, uint32_t v, uint32_t t) {
+  // Collisions up to cycle t are in the latches when this returns.
+  __device__ void sync_collisions(uint32_t t) {
+    if constexpr (SPLIT) {
+      if (broken) return;
+      push(EV_SYNC | (t & 0xFFFFu));
+      ++nreq;
+      if (!broken && !fc_q_wait_ack(io, nreq)) stall();
+      qhead_seen = qtail;  // acknowledged: the queue is empty
+    } else {
+      drain();
+      fc_cx_eval(io, 3u * t);
+    }
+  }
+  // Read / write a TIA or RIOT address (13-bit, neither RAM nor cartridge) at cycle t.
+  __device__ uint32_t io_read(uint32_t a, uint32_t t) {
+    if (a & 0x80) return fc_riot_read(io, a, 76ull * l0c + t);
+    const uint32_t reg = a & 0x0F;
+    if (reg < 8) {
+      sync_collisions(t);
+      return fc_cx_byte(io.V(IO_CX), reg);
+    }
+    if (reg == 0x0C) return (io.G(IO_FIRE) || io.G(IO_LATCH)) ? 0x00u : 0x80u;
+    return reg == 0x0D ? 0x80u : 0u;
+  }
+  // WSYNC, the VSYNC rise and the VBLANK latch effects happen here, the
+  // register itself on the TIA side.
+  __device__ void io_write(uint32_t a, uint32_t v, uint32_t t) {
+    if (a & 0x80) { fc_riot_write(io, a, v, 76ull * l0c + t); return; }
+    const uint32_t reg = a & 0x3F;
     if (reg == 0x02) { pend |= IO_WSYNC; return; }
     if (reg == 0x00) {
-      if (!(vsync_c & 2) && (v & 2)) { pend |= IO_VSYNC_RISE; note_vsync(t); }
+      if (!(vsync_c & 2) && (v & 2) && vs_kf == ~0u) vs_kf = t;
       vsync_c = v;
     } else if (reg == 0x01) {
       vblank_c = v;
       if (!(v & 0x40)) io.Sset(IO_LATCH, 0);
       else if (io.G(IO_FIRE)) io.Sset(IO_LATCH, 1);
     }
-    if ((SPLIT_PUSH_REGS >> reg) & 1ull) push(EV_WRITE | t << 14 | reg << 8 | v);
-  }
-  // Read / write a TIA or RIOT address at cycle t.
-  __device__ __forceinline__ uint32_t io_read(uint32_t a, uint32_t t) {
-    if constexpr (!SPLIT) {
-      return fc_io_read(io, a, t);
-    } else {
-      const uint32_t r = fc_split_io_read(io, q, qtail, qhead_seen, nreq, broken, a, t, l0c);
-      if (r & SIO_PUSHED) { ++qtail; ++nreq; qhead_seen = qtail; }
-      if (r & SIO_STALL) stall();
-      return r & 0xFFu;
-    }
-  }
-  __device__ __forceinline__ void io_write(uint32_t a, uint32_t v, uint32_t t) {
-    if constexpr (!SPLIT) {
-      const uint32_t f = fc_io_write(io, a, v, t);
-      pend |= f;
-      if (f & IO_VSYNC_RISE) note_vsync(t);
-    } else {
-      if (a & 0x80) fc_riot_write(io, a, v, 76ull * l0c + t);
-      else tia_out(a & 0x3F, v, t);
-    }
-  }
-  __device__ __forceinline__ void frame_end_out(uint32_t next_rel) {
-    if constexpr (!SPLIT) {
-      fc_frame_end(io, kf, next_rel);
-    } else {
-      push(EV_FRAME_END | kf << 14 | next_rel);
-      l0c += next_rel;
-    }
-  }
-
-  // zero-page access: RAM for $80-$FF, TIA below
-  __device__ __forceinline__ uint32_t rdz(uint32_t z, uint32_t t) {
-    return (z & 0x80) ? ram[z & 0x7F] : io_read(z, t);
-  }
-  __device__ __forceinline__ void wrz(uint32_t z, uint32_t v, uint32_t t) {
-    if (z & 0x80) ram[z & 0x7F] = v & 0xFF;
-    else io_write(z, v & 0xFF, t);
+    push((t & 0xFFFFu) << 14 | reg << 8 | v);
   }
   __device__ __forceinline__ uint32_t rd(uint32_t addr, uint32_t t) {
     const uint32_t a = addr & 0x1FFF;
-    if ((a & 0x1280) == 0x0080) return ram[a & 0x7F];
+    if ((a & 0x1280) == 0x0080) return ram(a & 0x7F);
     if (a & 0x1000) {
-      const uint32_t off = a & 0xFFF;
-      if (scheme) hotspot(off);
-      return rom8[bank * 4096u + off];
+      if (scheme) hotspot(a & 0xFFF);
+      return rom(bank * 4096u + (a & 0xFFF));
     }
     return io_read(a, t);
   }
   __device__ __forceinline__ void wr(uint32_t addr, uint32_t v, uint32_t t) {
     const uint32_t a = addr & 0x1FFF;
-    if ((a & 0x1280) == 0x0080) { ram[a & 0x7F] = v & 0xFF; return; }
+    if ((a & 0x1280) == 0x0080) { ram(a & 0x7F) = (uint8_t)v; return; }
     if (a & 0x1000) { if (scheme) hotspot(a & 0xFFF); return; }
-    io_write(a, v & 0xFF, t);
-  }
-
-  // Store instructions write through here (one inlined copy): RAM, cartridge
-  // hotspots, WSYNC and the colour / motion registers inline, every other
-  // TIA or RIOT address through the out-of-line writer.
-  __device__ __forceinline__ void bus_store(uint32_t addr, uint32_t v, uint32_t t) {
-    const uint32_t a = addr & 0x1FFF;
-    if ((a & 0x1280) == 0x0080) { ram[a & 0x7F] = v & 0xFF; return; }
-    if (a & 0x1000) { if (scheme) hotspot(a & 0xFFF); return; }
-    if (!(a & 0x80)) {
-      const uint32_t reg = a & 0x3F;
-      if constexpr (SPLIT) {
-        tia_out(reg, v & 0xFF, t);
-        return;
-      }
-      if (reg == 0x02) { pend |= IO_WSYNC; return; }
-      if ((FAST_TIA_REGS >> reg) & 1ull) {
-        fc_log(io, 3u * (t + 1u), reg, v & 0xFF);
-        io.Tset(reg < 0x20 ? reg - 2 : reg - 5, v & 0xFF);
-        return;
-      }
-    }
     io_write(a, v & 0xFF, t);
   }
 
@@ -792,12 +769,12 @@ struct FastConsoleT {
   __device__ __forceinline__ uint32_t idle_forward(uint32_t w, uint32_t pc, uint32_t k0) {
     const uint32_t a = (w >> 8) & 0xFFFF;
     if ((a & 0x1285u) != 0x0284u || (w >> 24) != 0xD0u) return k0;  // INTIM (any mirror), then BNE
-    const uint32_t off = pc & 0xFFF;
-    if (off > 0xFFBu || rom8[bank * 4096u + off + 4] != 0xFBu) return k0;  // BNE offset -5: back to pc
+    const uint32_t at = pc & 0xFFF;
+    // BNE offset -5: back to pc, its bytes below the cartridge's hotspots
+    if (at > (scheme == 3 ? 0xFEFu : scheme ? 0xFF1u : 0xFFBu) || rom(bank * 4096u + at + 4) != 0xFBu) return k0;
     const uint32_t sh = io.G(IO_TSH);
     if (sh < 3) return k0;
-    const uint64_t l0 = SPLIT ? l0c : io.G64(IO_L0LO);
-    const uint64_t n0 = 76ull * l0 + k0 + 3 - (io.G64(IO_TCWLO) + 1);  // the read's cycle, as the timer counts it
+    const uint64_t n0 = 76ull * l0c + k0 + 3 - (io.G64(IO_TCWLO) + 1);  // the read's cycle, as the timer counts it
     const uint64_t zero = (uint64_t)io.G(IO_TV) << sh;                 // first cycle reading 0
     if (n0 >= zero) return k0;
     const uint32_t period = (((pc + 5) ^ pc) & 0xFF00) ? 8u : 7u;
@@ -807,198 +784,15 @@ struct FastConsoleT {
     return (uint32_t)k1;
   }
 
-  // ---- one instruction, hot form ----
-  // Returns false (with nothing changed) for the cases the general decoder
-  // takes.  Each case sets the cycle count n and the next PC; the tail
-  // applies the WSYNC stall.
-  // w = cartridge bytes PC .. PC+3 of the current bank (fetch4).
-  __device__ __forceinline__ bool exec(uint32_t w) {
-    const uint32_t pc = PC;
-    const uint32_t off = pc & 0xFFF;
-    // no hot fetch may touch a hotspot: F8/F6 hotspots start at $FF6, F4's at $FF4
-    if (!(pc & 0x1000) || off > (scheme == 3 ? 0xFF1u : scheme ? 0xFF3u : 0xFFCu)) return false;
-    const uint32_t k0 = kf;
-    const uint32_t b1 = (w >> 8) & 0xFF;
-    const uint32_t a16 = (w >> 8) & 0xFFFF;
-    uint32_t n;
-    uint32_t sa = ~0u, sv = 0, stc = 0;  // pending store: address (~0: none), value, cycle
-    pend = 0;
-#define ZPX_ ((b1 + X) & 0xFF)
-#define ZPY_ ((b1 + Y) & 0xFF)
-#define ABX_ ((a16 + X) & 0xFFFF)
-#define ABY_ ((a16 + Y) & 0xFFFF)
-#define XPG(base, ea) ((((base) ^ (ea)) >> 8) & 1u)
-#define NZ(v) (fn = fz = (v))
-#define COLD_ if constexpr (COMPACT) return false;
-// read instructions: imm, zp, zp,X, abs, abs,X, abs,Y, (zp,X), (zp),Y
-#define RD_OPS(OPI, OPZ, OPZX, OPA, OPAX, OPAY, OPIX, OPIY, BODY)                                          \
-  case OPI: { const uint32_t v = b1; BODY; n = 2; PC = pc + 2; break; }                                      \
-  case OPZ: { const uint32_t v = rdz(b1, k0 + 2); BODY; n = 3; PC = pc + 2; break; }                          \
-  case OPZX: { const uint32_t v = rdz(ZPX_, k0 + 3); BODY; n = 4; PC = pc + 2; break; }                       \
-  case OPA: { const uint32_t ka = (OPA == 0xAD && idle) ? idle_forward(w, pc, k0) : k0;                     \
-              const uint32_t v = rd(a16, ka + 3); BODY; n = 4 + (ka - k0); PC = pc + 3; break; }             \
-  case OPAX: { const uint32_t ea = ABX_; n = 4 + XPG(a16, ea); const uint32_t v = rd(ea, k0 + n - 1); BODY;   \
-               PC = pc + 3; break; }                                                                          \
-  case OPAY: { const uint32_t ea = ABY_; n = 4 + XPG(a16, ea); const uint32_t v = rd(ea, k0 + n - 1); BODY;   \
-               PC = pc + 3; break; }                                                                          \
-  case OPIX: { COLD_ const uint32_t z = ZPX_; if (!(z & 0x80) || z == 0xFF) return false;                   \
-               const uint32_t ea = ram[z & 0x7F] | ram[(z + 1) & 0x7F] << 8;                      \
-               const uint32_t v = rd(ea, k0 + 5); BODY; n = 6; PC = pc + 2; break; }                           \
-  case OPIY: { COLD_ if (!(b1 & 0x80) || b1 == 0xFF) return false;                                           \
-               const uint32_t base = ram[b1 & 0x7F] | ram[(b1 + 1) & 0x7F] << 8;                  \
-               const uint32_t ea = (base + Y) & 0xFFFF; n = 5 + XPG(base, ea);                                \
-               const uint32_t v = rd(ea, k0 + n - 1); BODY; PC = pc + 2; break; }
-// read-modify-write: acc, zp, zp,X, abs, abs,X.  The memory forms take RAM
-// here (where the old-value write is invisible); a TIA, RIOT or cartridge
-// address goes to the general decoder, which models both writes.
-#define RMW_MEM_OPS(OPZ, OPZX, OPA, OPAX, FN)                                                                \
-  case OPZ: { if (!(b1 & 0x80)) return false;                                                                 \
-              ram[b1 & 0x7F] = FN(ram[b1 & 0x7F]); n = 5; PC = pc + 2; break; }                              \
-  case OPZX: { COLD_ const uint32_t z = ZPX_; if (!(z & 0x80)) return false;                                 \
-               ram[z & 0x7F] = FN(ram[z & 0x7F]); n = 6; PC = pc + 2; break; }                                \
-  case OPA: { COLD_ if ((a16 & 0x1280) != 0x0080) return false;                                              \
-              ram[a16 & 0x7F] = FN(ram[a16 & 0x7F]); n = 6; PC = pc + 3; break; }                            \
-  case OPAX: { COLD_ const uint32_t ea = ABX_; if ((ea & 0x1280) != 0x0080) return false;                   \
-               ram[ea & 0x7F] = FN(ram[ea & 0x7F]); n = 7; PC = pc + 3; break; }
-#define RMW_OPS(OPACC, OPZ, OPZX, OPA, OPAX, FN)                                                             \
-  case OPACC: { A = FN(A); n = 2; PC = pc + 1; break; }                                                       \
-  RMW_MEM_OPS(OPZ, OPZX, OPA, OPAX, FN)
-// memory-only read-modify-write (INC, DEC): zp, zp,X, abs, abs,X
-#define RMWM_OPS(OPZ, OPZX, OPA, OPAX, FN) RMW_MEM_OPS(OPZ, OPZX, OPA, OPAX, FN)
-#define BR(OPC, COND)                                                                                          \
-  case OPC: {                                                                                                 \
-    const uint32_t nx = (pc + 2) & 0xFFFF;                                                                    \
-    n = 2; PC = nx;                                                                                           \
-    if (COND) { const uint32_t tg = (nx + (uint32_t)(int32_t)(int8_t)(uint8_t)b1) & 0xFFFF;                   \
-                n += ((nx ^ tg) & 0xFF00) ? 2u : 1u; PC = tg; }                                               \
-    break; }
-#define IMPL(OPC, BODY) case OPC: { BODY; n = 2; PC = pc + 1; break; }
-    switch (w & 0xFF) {
-      RD_OPS(0xA9, 0xA5, 0xB5, 0xAD, 0xBD, 0xB9, 0xA1, 0xB1, { A = v; NZ(A); })            // LDA
-      RD_OPS(0x69, 0x65, 0x75, 0x6D, 0x7D, 0x79, 0x61, 0x71, { adc(v); })                  // ADC
-      RD_OPS(0xE9, 0xE5, 0xF5, 0xED, 0xFD, 0xF9, 0xE1, 0xF1, { sbc(v); })                  // SBC
-      RD_OPS(0x29, 0x25, 0x35, 0x2D, 0x3D, 0x39, 0x21, 0x31, { A &= v; NZ(A); })           // AND
-      RD_OPS(0x09, 0x05, 0x15, 0x0D, 0x1D, 0x19, 0x01, 0x11, { A |= v; NZ(A); })           // ORA
-      RD_OPS(0x49, 0x45, 0x55, 0x4D, 0x5D, 0x59, 0x41, 0x51, { A ^= v; NZ(A); })           // EOR
-      RD_OPS(0xC9, 0xC5, 0xD5, 0xCD, 0xDD, 0xD9, 0xC1, 0xD1, { cmp(A, v); })               // CMP
-      // LDX: imm, zp, zp,Y, abs, abs,Y
-      case 0xA2: X = b1; NZ(X); n = 2; PC = pc + 2; break;
-      case 0xA6: X = rdz(b1, k0 + 2); NZ(X); n = 3; PC = pc + 2; break;
-      case 0xB6: X = rdz(ZPY_, k0 + 3); NZ(X); n = 4; PC = pc + 2; break;
-      case 0xAE: X = rd(a16, k0 + 3); NZ(X); n = 4; PC = pc + 3; break;
-      case 0xBE: { const uint32_t ea = ABY_; n = 4 + XPG(a16, ea); X = rd(ea, k0 + n - 1); NZ(X); PC = pc + 3; break; }
-      // LDY: imm, zp, zp,X, abs, abs,X
-      case 0xA0: Y = b1; NZ(Y); n = 2; PC = pc + 2; break;
-      case 0xA4: Y = rdz(b1, k0 + 2); NZ(Y); n = 3; PC = pc + 2; break;
-      case 0xB4: Y = rdz(ZPX_, k0 + 3); NZ(Y); n = 4; PC = pc + 2; break;
-      case 0xAC: Y = rd(a16, k0 + 3); NZ(Y); n = 4; PC = pc + 3; break;
-      case 0xBC: { const uint32_t ea = ABX_; n = 4 + XPG(a16, ea); Y = rd(ea, k0 + n - 1); NZ(Y); PC = pc + 3; break; }
-      // CPX, CPY: imm, zp, abs
-      case 0xE0: cmp(X, b1); n = 2; PC = pc + 2; break;
-      case 0xE4: cmp(X, rdz(b1, k0 + 2)); n = 3; PC = pc + 2; break;
-      case 0xEC: cmp(X, rd(a16, k0 + 3)); n = 4; PC = pc + 3; break;
-      case 0xC0: cmp(Y, b1); n = 2; PC = pc + 2; break;
-      case 0xC4: cmp(Y, rdz(b1, k0 + 2)); n = 3; PC = pc + 2; break;
-      case 0xCC: cmp(Y, rd(a16, k0 + 3)); n = 4; PC = pc + 3; break;
-      // BIT: zp, abs
-      case 0x24: { COLD_ const uint32_t v = rdz(b1, k0 + 2); fn = v; fv = v & 0x40; fz = A & v; n = 3; PC = pc + 2; break; }
-      case 0x2C: { COLD_ const uint32_t v = rd(a16, k0 + 3); fn = v; fv = v & 0x40; fz = A & v; n = 4; PC = pc + 3; break; }
-      // stores
-      case 0x85: sa = b1; sv = A; stc = k0 + 2; n = 3; PC = pc + 2; break;
-      case 0x95: sa = ZPX_; sv = A; stc = k0 + 3; n = 4; PC = pc + 2; break;
-      case 0x8D: sa = a16; sv = A; stc = k0 + 3; n = 4; PC = pc + 3; break;
-      case 0x9D: sa = ABX_; sv = A; stc = k0 + 4; n = 5; PC = pc + 3; break;
-      case 0x99: sa = ABY_; sv = A; stc = k0 + 4; n = 5; PC = pc + 3; break;
-      case 0x81: { COLD_ const uint32_t z = ZPX_; if (!(z & 0x80) || z == 0xFF) return false;
-                   sa = ram[z & 0x7F] | ram[(z + 1) & 0x7F] << 8; sv = A; stc = k0 + 5; n = 6; PC = pc + 2; break; }
-      case 0x91: { COLD_ if (!(b1 & 0x80) || b1 == 0xFF) return false;
-                   const uint32_t base = ram[b1 & 0x7F] | ram[(b1 + 1) & 0x7F] << 8;
-                   sa = (base + Y) & 0xFFFF; sv = A; stc = k0 + 5; n = 6; PC = pc + 2; break; }
-      case 0x86: sa = b1; sv = X; stc = k0 + 2; n = 3; PC = pc + 2; break;
-      case 0x96: sa = ZPY_; sv = X; stc = k0 + 3; n = 4; PC = pc + 2; break;
-      case 0x8E: sa = a16; sv = X; stc = k0 + 3; n = 4; PC = pc + 3; break;
-      case 0x84: sa = b1; sv = Y; stc = k0 + 2; n = 3; PC = pc + 2; break;
-      case 0x94: sa = ZPX_; sv = Y; stc = k0 + 3; n = 4; PC = pc + 2; break;
-      case 0x8C: sa = a16; sv = Y; stc = k0 + 3; n = 4; PC = pc + 3; break;
-      RMW_OPS(0x0A, 0x06, 0x16, 0x0E, 0x1E, asl)
-      RMW_OPS(0x4A, 0x46, 0x56, 0x4E, 0x5E, lsr)
-      RMW_OPS(0x2A, 0x26, 0x36, 0x2E, 0x3E, rol)
-      RMW_OPS(0x6A, 0x66, 0x76, 0x6E, 0x7E, ror)
-      RMWM_OPS(0xE6, 0xF6, 0xEE, 0xFE, inc)
-      RMWM_OPS(0xC6, 0xD6, 0xCE, 0xDE, dec)
-      BR(0x10, !(fn & 0x80))
-      BR(0x30, (fn & 0x80))
-      BR(0x50, !fv)
-      BR(0x70, fv)
-      BR(0x90, !fc)
-      BR(0xB0, fc)
-      BR(0xD0, (fz & 0xFF))
-      BR(0xF0, !(fz & 0xFF))
-      IMPL(0xE8, { X = (X + 1) & 0xFF; NZ(X); })
-      IMPL(0xC8, { Y = (Y + 1) & 0xFF; NZ(Y); })
-      IMPL(0xCA, { X = (X - 1) & 0xFF; NZ(X); })
-      IMPL(0x88, { Y = (Y - 1) & 0xFF; NZ(Y); })
-      IMPL(0xAA, { X = A; NZ(X); })
-      IMPL(0xA8, { Y = A; NZ(Y); })
-      IMPL(0x8A, { A = X; NZ(A); })
-      IMPL(0x98, { A = Y; NZ(A); })
-      IMPL(0xBA, { X = SP; NZ(X); })
-      IMPL(0x9A, { SP = X; })
-      IMPL(0x18, { fc = 0; })
-      IMPL(0x38, { fc = 1; })
-      IMPL(0x58, { fdi &= ~0x04u; })
-      IMPL(0x78, { fdi |= 0x04u; })
-      IMPL(0xB8, { fv = 0; })
-      IMPL(0xD8, { fdi &= ~0x08u; })
-      IMPL(0xF8, { fdi |= 0x08u; })
-      IMPL(0xEA, {})
-      case 0x48: COLD_ if (!(SP & 0x80)) return false; ram[SP & 0x7F] = A; SP = (SP - 1) & 0xFF; n = 3; PC = pc + 1; break;
-      case 0x08: COLD_ if (!(SP & 0x80)) return false; ram[SP & 0x7F] = P() | 0x10u; SP = (SP - 1) & 0xFF; n = 3; PC = pc + 1; break;
-      case 0x68: { COLD_ const uint32_t s1 = (SP + 1) & 0xFF; if (!(s1 & 0x80)) return false;
-                   SP = s1; A = ram[s1 & 0x7F]; NZ(A); n = 4; PC = pc + 1; break; }
-      case 0x28: { COLD_ const uint32_t s1 = (SP + 1) & 0xFF; if (!(s1 & 0x80)) return false;
-                   SP = s1; setP(ram[s1 & 0x7F]); n = 4; PC = pc + 1; break; }
-      case 0x4C: PC = a16; n = 3; break;
-      case 0x20: { if (SP < 0x81) return false;
-                   const uint32_t ret = (pc + 2) & 0xFFFF;
-                   ram[SP & 0x7F] = ret >> 8; ram[(SP - 1) & 0x7F] = ret & 0xFF;
-                   SP = (SP - 2) & 0xFF; PC = a16; n = 6; break; }
-      case 0x60: { const uint32_t s1 = (SP + 1) & 0xFF, s2 = (SP + 2) & 0xFF;
-                   if (!(s1 & 0x80) || !(s2 & 0x80)) return false;
-                   PC = ((ram[s1 & 0x7F] | ram[s2 & 0x7F] << 8) + 1) & 0xFFFF; SP = s2; n = 6; break; }
-      default: return false;  // BRK, RTI, JMP (ind), undocumented
-    }
-#undef ZPX_
-#undef ZPY_
-#undef ABX_
-#undef ABY_
-#undef XPG
-#undef NZ
-#undef COLD_
-#undef RD_OPS
-#undef RMW_MEM_OPS
-#undef RMW_OPS
-#undef RMWM_OPS
-#undef BR
-#undef IMPL
-    if (sa != ~0u) bus_store(sa, sv, stc);
-    PC &= 0xFFFF;
-    uint32_t k = k0 + n;
-    if (pend & IO_WSYNC) k = ((k + 75u) / 76u) * 76u;
-    kf = k;
-    instret++;
-    return true;
-  }
-
-  // ---- one instruction, general form (every case; run out of line) ----
+  // ---- one instruction, general form (every case) ----
   __device__ void exec_general() {
     const uint32_t k0 = kf;
     pend = 0;
     const uint32_t pc = PC;
     const uint32_t opcode = rd(pc, k0);
-    const uint32_t opb = dec_op[opcode];
+    const uint32_t opb = sm8(off.dec + opcode);
     const uint32_t op = opb & 0x7F;
-    const uint32_t info = dec_op[256 + opcode];
+    const uint32_t info = sm8(off.dec + 256 + opcode);
     const uint32_t mode = info & 0xF;
     uint32_t n = info >> 4;
     if (op == O_JAM) { jam = 1; status |= ST_ILLEGAL; return; }
@@ -1162,68 +956,187 @@ struct FastConsoleT {
     kf = k;
   }
 
-  // One frame.  Lanes of a warp issue in program order of the laggard: each
-  // round the lane with the smallest emulated cycle count leads, and every
-  // lane whose PC equals the leader's executes its instruction with it.  Lanes
-  // that ran a shorter path wait at the join point until the laggard reaches
-  // it, so the warp reconverges on code rather than on time (lanes a few
-  // cycles apart after a page-crossing or a different branch path still run
-  // together), and the executing lanes take one case of the opcode switch.
-  // One warp reduction elects the leader: the minimum of (cycle << 16 | PC)
-  // over the active lanes gives its PC directly (ties in the cycle go to the
-  // smaller PC), and all-ones means no lane is active.  The cycle saturates
-  // below 0xFFFF, so the key always names a lane's actual PC.  The leader
-  // always advances (every instruction takes at least 2 cycles, and a frame
-  // ends after at most 400 lines), so the loop ends.
-  __device__ __forceinline__ uint32_t run_frame() {
-    uint32_t next_rel = 0;
-    vs_kf = ~0u;
-    bool active = !jam;
-    if (jam) next_rel = kf / 76u;
-    for (;;) {
-      // next instruction word, fetched before the election so the two latencies overlap
-      // (bank < banks of the staged cartridge, so the index stays in the stage)
-      const uint32_t w = fetch4(bank * 4096u + (PC & 0xFFFu));
-      const uint32_t key = active ? (min(kf, 0xFFFEu) << 16 | (PC & 0xFFFFu)) : 0xFFFFFFFFu;
-      const uint32_t lead = __reduce_min_sync(wmask, key);
-      if (lead == 0xFFFFFFFFu) break;
-      ++rounds;
-      if (active && PC == (lead & 0xFFFFu)) {
-        if (!exec(w)) fc_exec_general<SPLIT, COMPACT>(this);
-        if (jam | (vs_kf != ~0u) | (kf >= 76u * CAP_LINES)) {
-          if (jam) next_rel = kf / 76u;
-          else if (vs_kf != ~0u) next_rel = vs_kf / 76u;
-          else { status |= ST_FRAME_CAP; next_rel = kf / 76u; }
-          active = false;
-        }
-      }
-    }
-    frame_end_out(next_rel);
+  // Append the end of the current frame and start counting the next.
+  __device__ __forceinline__ void end_frame(uint32_t next_rel) {
+    push(EV_FRAME_END | (kf & 0xFFFFu));
+    push(EV_REBASE | (next_rel & 0xFFFFFFFu));
+    l0c += next_rel;
     kf -= 76u * next_rel;
     frame_no++;
-    return next_rel;
+    vs_kf = ~0u;
+    frame_inst = instret;
   }
+
+  // Run this env (every lane of wmask its own) until hook.frame_done() says
+  // that the step is over.
+  //
+  // The hot loop is one branch-free instruction sequence for every common
+  // instruction, steered by the opcode's control words (opcode_ctl.h): one
+  // adder with masks covers loads, transfers, arithmetic, logic, shifts left,
+  // increments and compares, one sum covers the effective address, the branch
+  // target and the immediate operand, and one load covers RAM and cartridge.
+  // So lanes at different instructions still execute together: each lane
+  // runs its own program at one instruction per round, with no leader, no
+  // reconvergence and a loop that stays in the instruction cache's first
+  // level.  What it does not take (RIOT accesses, collision reads, VSYNC and
+  // VBLANK, stack and pointer instructions, bank hotspots, frame ends) stops
+  // the lane in front of the instruction; every BATCH rounds the lanes that
+  // wait are served together by the general decoder, at once when no lane is
+  // left running, otherwise after at most one more batch, so that lanes a few
+  // rounds apart share one call.
+  template <class Hook> __device__ __forceinline__ void run(Hook &hook);
 };
 
-using FastConsole = FastConsoleT<false, false>;
-
-// Out-of-line general instruction on a copy of the console.  Only the CPU
-// and timing state comes back: the caller's pointers into shared memory are
-// never reloaded from the copy, so they keep their shared address space.
-template <bool SPLIT, bool COMPACT>
-__device__ __noinline__ void fc_exec_general_impl(FastConsoleT<SPLIT, COMPACT> *c) { c->exec_general(); }
-template <bool SPLIT, bool COMPACT>
-__device__ __forceinline__ void fc_exec_general(FastConsoleT<SPLIT, COMPACT> *self) {
-  FastConsoleT<SPLIT, COMPACT> tmp = *self;
-  fc_exec_general_impl<SPLIT, COMPACT>(&tmp);
-  self->A = tmp.A; self->X = tmp.X; self->Y = tmp.Y; self->SP = tmp.SP; self->PC = tmp.PC;
-  self->fc = tmp.fc; self->fv = tmp.fv; self->fn = tmp.fn; self->fz = tmp.fz; self->fdi = tmp.fdi;
-  self->bank = tmp.bank; self->jam = tmp.jam; self->kf = tmp.kf; self->pend = tmp.pend; self->vs_kf = tmp.vs_kf;
-  self->status = tmp.status; self->instret = tmp.instret; self->frame_no = tmp.frame_no;
-  if constexpr (SPLIT) {
-    self->qtail = tmp.qtail; self->qhead_seen = tmp.qhead_seen; self->nreq = tmp.nreq; self->vsync_c = tmp.vsync_c; self->vblank_c = tmp.vblank_c;
-    self->broken = tmp.broken; self->l0c = tmp.l0c;
+// One service of a waiting lane: the frame's end, or the instruction at PC by
+// the general decoder (after a timer wait loop's idle iterations).  Returns
+// false when the step is over.
+template <bool SPLIT, class Hook>
+__device__ __noinline__ bool fc_service(FastConsoleT<SPLIT> *c, Hook *h) {
+  const uint32_t cap = 76u * CAP_LINES;
+  // at least one instruction runs in every frame before the line cap ends it
+  bool ended = c->jam || (c->kf >= cap && c->instret != c->frame_inst);
+  if (!ended) {
+    const uint32_t at = c->PC & 0xFFF;
+    if (c->idle && (c->PC & 0x1000) && at <= c->fetch_limit()) {
+      const uint32_t w = c->fetch4(c->bank * 4096u + at);
+      if ((w & 0xFF) == 0xAD) c->kf = c->idle_forward(w, c->PC, c->kf);
+    }
+    c->exec_general();
+    ended = c->jam || c->vs_kf != ~0u || c->kf >= cap;
   }
+  while (ended) {
+    uint32_t next_rel;
+    if (c->jam) next_rel = c->kf / 76u;
+    else if (c->vs_kf != ~0u) next_rel = c->vs_kf / 76u;
+    else { c->status |= ST_FRAME_CAP; next_rel = c->kf / 76u; }
+    c->end_frame(next_rel);
+    if (!h->frame_done(*c)) return false;
+    ended = c->jam != 0;
+  }
+  return true;
+}
+
+template <bool SPLIT>
+template <class Hook>
+__device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
+  const EnvOff o = off;
+  const uint32_t smb = (uint32_t)__cvta_generic_to_shared(g_smem);
+  const uint32_t cap = 76u * CAP_LINES;
+  const uint32_t ctl = o.dec + 512, romb = smb + o.rom;
+  const uint32_t lim = fetch_limit();
+  // cartridge reads below the first hotspot are plain loads
+  const uint32_t hot = scheme == 3 ? 0xFF4u : scheme == 2 ? 0xFF6u : scheme == 1 ? 0xFF8u : 0x1000u;
+  uint32_t R, Pf, pc, k, inst, qt, bk;
+  uint32_t rec, cb;
+  uint4 c;
+  bool wait = false, active = true;
+  // instruction bytes at p; the control words of opcode op
+  auto bytes_at = [&](uint32_t p) {
+    const uint32_t i = bk + (p & 0xFFFu);
+    const uint32_t a = romb + (i & ~3u);
+    return __funnelshift_r(lds_const(a), lds_const(a + 4), i * 8u);
+  };
+  auto control = [&](uint32_t op) {
+    c = lds_const4(smb + ctl + op * 16u);
+    cb = lds_const(smb + ctl + CTL_B_OFF + op * 4u);
+  };
+  // the console's fields to the loop's registers, and the next instruction
+  auto enter = [&](bool stay) {
+    R = A | X << 8 | Y << 16;
+    Pf = P(); pc = PC; k = kf; inst = instret; qt = qtail; bk = bank * 4096u;
+    rec = bytes_at(pc);
+    wait = stay || ((pc & 0x1FFFu) - 0x1000u) > lim || k >= cap;
+    control(wait ? CTL_HALT : rec & 0xFFu);
+  };
+  enter(jam != 0);
+  uint32_t held = 0, act = wmask;
+  for (;;) {
+#pragma unroll 1
+    for (uint32_t r = 0; r < BATCH; ++r) {
+      // --- next instruction (branches and JMP abs: the sum is the target)
+      const uint32_t pcn = pc + (c.w >> 28);
+      const uint32_t base = prmt(rec, pcn, c.x);
+      const uint32_t sum = base + prmt(R, rec, c.y);
+      const bool tk = ((Pf ^ (c.y >> 24)) & (c.y >> 16) & 0xFFu) != 0;
+      const uint32_t npc = tk ? sum & 0xFFFFu : pcn;
+      const uint32_t nrec = bytes_at(npc);
+      const bool nbad = ((npc & 0x1FFFu) - 0x1000u) > lim;
+      // --- cycles
+      const uint32_t tk1 = tk ? 1u : 0u;
+      const uint32_t n = ((cb >> 8) & 0x7Fu) + tk1 + (((base ^ sum) >> 8) & (((cb >> 15) & 1u) | tk1));
+      const uint32_t kn = k + n;
+      // --- operand
+      const uint32_t ea = sum & (c.x >> 16);
+      const bool is_ram = (ea & 0x1280u) == 0x0080u;
+      const bool is_cart = ea - 0x1000u < hot;
+      const uint32_t tia = ea & 0x10BFu;                  // below $40: a TIA register
+      const uint32_t at = is_ram ? o.ram + (ea & 0x7Fu) : o.rom + bk + (ea & 0xFFFu);
+      const uint32_t ld = sm8(at);
+      const uint32_t y = ((cb & CT_MEM) ? ld : sum) ^ (c.z >> 24);
+      const uint32_t x = prmt(R, y | 0xFF00u, c.z);
+      // --- what the general decoder takes
+      const bool is_ld = (cb & CT_LD) != 0, is_st = (cb & CT_ST) != 0, is_rmw = (cb & CT_RMW) != 0;
+      const bool ok = is_ram | (is_ld & is_cart) | (is_st & (tia - 2u < 0x3Eu));
+      const bool slow = ((cb & CT_SLOW) != 0) | ((is_ld | is_st | is_rmw) & !ok) | ((Pf & (cb >> 24) & 0x08u) != 0);
+      // --- result
+      const uint32_t cin = (Pf & cb & 1u) | ((cb >> 1) & 1u);
+      const uint32_t add = (x & y) * ((cb >> 24) & 3u) + ((x ^ y) & (c.z >> 16)) + cin;
+      const uint32_t rot = (((y + (cin << 8)) * 513u) >> 1) & 0x1FFu;
+      const uint32_t s = (cb & CT_SHR) ? rot : add;
+      // --- flags
+      uint32_t nf = (s & 0x80u) | ((s >> 8) & 1u) | ((((x ^ s) & ~(x ^ y)) & 0x80u) >> 1) | ((s & 0xFFu) ? 0u : 2u);
+      const uint32_t bits = (cb >> 16) & 0xFFu, pm = slow ? 0u : (c.w >> 16) & 0xFFu;
+      nf = (nf & ~bits) | (y & bits);
+      // --- commit
+      const uint32_t sv = (is_rmw ? s : x) & 0xFFu;
+      sts8_if((is_st | is_rmw) & is_ram & !slow, smb + at, sv);
+      const bool out = is_st & (tia - 3u < 0x3Du) & !slow;
+      sts32_if(out, smb + o.q + (qt & (QLEN - 1)) * 4u, ((kn - 1u) << 14 | tia << 8 | sv) ^ lap_bit(qt));
+      qt += out ? 1u : 0u;
+      const uint32_t kw = (is_st & (tia == 2u)) ? (kn + 75u) / 76u * 76u : kn;
+      R = prmt(R, s, slow ? 0x3210u : c.w);
+      Pf = (Pf & ~pm) | (nf & pm);
+      inst += slow ? 0u : (cb >> 28) & 1u;
+      pc = slow ? pc : npc;
+      k = slow ? k : kw;
+      wait = wait | slow | nbad | (k >= cap);
+      rec = nrec;
+      control(wait ? CTL_HALT : nrec & 0xFFu);
+    }
+    // --- service: waiting lanes, and queues without room for another batch
+    rounds += BATCH;
+    const bool full = qt - qhead_seen > QLEN - BATCH;
+    uint32_t m = __ballot_sync(wmask, (wait | full) & active);
+    if (m == 0) continue;
+    m = __ballot_sync(wmask, wait & active);
+    if (m != 0 && (m == act || ++held > 1)) {
+      held = 0;
+      ++rounds;
+      if (active && wait) {
+        A = R & 0xFF; X = (R >> 8) & 0xFF; Y = (R >> 16) & 0xFF;
+        setP(Pf); PC = pc; kf = k; instret = inst; qtail = qt;
+        active = fc_service<SPLIT, Hook>(this, &hook);
+        enter(!active);
+      }
+      act = __ballot_sync(wmask, active);
+      if (act == 0) break;
+    }
+    // room for a batch of events
+    if constexpr (SPLIT) {
+      if (active & (qt - qhead_seen > QLEN - BATCH)) {
+        qhead_seen = fc_q_wait_room(io, qt, BATCH);
+        if (qt - qhead_seen > QLEN - BATCH) { stall(); wait = true; control(CTL_HALT); }
+      }
+    } else {
+      if (__any_sync(wmask, qt - qhead_seen > QLEN - BATCH)) {
+        qtail = qt;
+        drain();
+      }
+    }
+    __syncwarp(wmask);
+  }
+  A = R & 0xFF; X = (R >> 8) & 0xFF; Y = (R >> 16) & 0xFF;
+  setP(Pf); PC = pc; kf = k; instret = inst; qtail = qt;
 }
 
 }  // namespace atari
