@@ -84,7 +84,8 @@ typedef struct {
     int envs_per_block;   /* batched form: envs per interpreter block, <= 128 (0 = autotune) */
     int envs_per_warp;    /* batched form: envs per warp, 1..32 (0 = autotune); fewer than 32 trades
                              SIMT width for more independent instruction streams on small batches */
-    int raster_warps_per_frame; /* batched form: warps rendering one frame, 1..4 (0 = autotune) */
+    int raster_warps_per_frame; /* batched form, 0..4.  Kept for callers: the painting kernels' blocks have one
+                                   shape, and every value runs the same code */
     uint64_t seed;        /* Philox4x32-10 key for start states, resets and sticky draws */
     int tia_warps;        /* batched form: 1 = each warp runs its envs' CPU and TIA; 2 = a TIA warp per
                              CPU warp takes the TIA writes, logging and collisions off the CPU's

@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(128) k_cache_run(uint8_t *work, uint8_t *snaps
   m.scheme = inf & 0xFF;
   m.wmask = 1u;
   m.idle = 1u;
-  m.to = TiaOut{nullptr, nullptr, nullptr, nullptr, 0};
+  m.to = TiaOut{nullptr, nullptr, nullptr, 0};
   m.load(st);
   m.apply_action(0);
   CacheHook h{st, snaps + (size_t)r * (max_noops + 1) * 256, startup, max_noops, 0};
@@ -510,8 +510,8 @@ struct atari_env {
   uint8_t *d_state = nullptr;
   uint8_t *d_cache = nullptr;
   uint32_t *d_log = nullptr;
-  uint8_t *d_snap = nullptr;
-  uint8_t *d_bsnap = nullptr;   // batched stack form: [n][2][3][64] band start snapshots
+  uint8_t *d_snap = nullptr;    // plain form: [n][2][64] render state at the start of frames F-1 and F
+  uint8_t *d_bsnap = nullptr;   // batched form: [n][logged frames][BANDS][BAND_SNAP] band start snapshots
   uint32_t *d_meta = nullptr;
   uint8_t *d_frames = nullptr;
   uint8_t *d_ring = nullptr;
@@ -531,7 +531,8 @@ struct atari_env {
   int grouping = 1;                 // 1 env order, 2 bank-aware
   bool banked = false;              // some cartridge has more than one bank
   int *d_queue = nullptr;
-  int n_groups = 0, lanes = 32, warps = 4, wpf = 4, grid = 0, rom_stage = 4096, max_blocks = 1;
+  int wpf = 4;  // cfg.raster_warps_per_frame, reported by atari_env_launch_shape; the painter's blocks have one shape
+  int n_groups = 0, lanes = 32, warps = 4, grid = 0, rom_stage = 4096, max_blocks = 1;
   bool split = false;   // paired CPU / TIA warps (k_interp_split)
   bool compact = false; // cfg.dispatch == 2, reported by atari_env_launch_shape; no effect on the kernels
   std::vector<int32_t> h_env_rom;
@@ -662,7 +663,6 @@ BatchArgs batch_args(atari_env *E, const uint8_t *d_actions, int32_t *d_rewards,
   a.rew_out = d_rewards;
   a.done_out = d_dones;
   a.log = E->d_log;
-  a.snap = E->d_snap;
   a.bsnap = E->d_bsnap;
   a.meta = E->d_meta;
   a.counters = E->d_ctr;
@@ -693,8 +693,6 @@ void launch_interp(atari_env *E, const BatchArgs &a, int grid, cudaStream_t s) {
   if (E->split) k_interp_split<<<grid, th, interp_smem(E), s>>>(a);
   else k_interp_batched<<<grid, th, interp_smem(E), s>>>(a);
 }
-
-size_t fused_smem() { return 2 * 210 * 160 + 128 + 7056; }
 
 // Bank-aware grouping: the env list of this step, re-sorted by bank within
 // each cartridge from the states as they stand.
@@ -762,6 +760,10 @@ void atari_default_config(atari_config *c) {
 
 const char *atari_last_error(void) { return g_err.c_str(); }
 
+static size_t band_bytes(const atari_config &c) {  // an env's band snapshots, of one frame (palette output) or two
+  return (c.output_mode == ATARI_OUT_STACK ? 2 : 1) * (size_t)BANDS * BAND_SNAP;
+}
+
 size_t atari_env_footprint(int n_envs, int n_roms, const atari_config *cfg) {
   if (!cfg || n_envs < 0 || n_roms < 0) return 0;
   size_t n = (size_t)n_envs;
@@ -770,11 +772,11 @@ size_t atari_env_footprint(int n_envs, int n_roms, const atari_config *cfg) {
   b += n * (4 + 4 + 256);                                 // env_rom, env_key, state
   b += (size_t)n_roms * cfg->n_cache * 256;               // cache
   b += n * 2 * (size_t)cfg->log_cap * 4;                  // log
-  b += n * 2 * 64 + n * 2 * 2 * 4;                        // snapshots, meta
-  if (cfg->form == ATARI_FORM_PLAIN) b += n * 2 * 210 * 160;   // frames (plain form only)
+  b += n * 2 * 2 * 4;                                     // frame records
+  if (cfg->form == ATARI_FORM_PLAIN) b += n * 2 * 210 * 160 + n * 2 * 64;   // frames and snapshots (plain form only)
   else b += (size_t)n_roms * ROMB_SLOT + n * 8 + 64 + (size_t)(n_roms + 1) * 4;  // stage bytes, work items, regrouping
   if (cfg->output_mode == ATARI_OUT_STACK) b += n * 4 * 7056 + n;
-  if (cfg->output_mode == ATARI_OUT_STACK && cfg->form == ATARI_FORM_BATCHED) b += n * 2 * 3 * 64;  // band snapshots
+  if (cfg->form == ATARI_FORM_BATCHED) b += n * band_bytes(*cfg);
   b += n * (4 + 1 + 12 + 1);                              // rewards, dones, counters, action staging
   return b;
 }
@@ -816,19 +818,20 @@ int atari_env_create(const uint8_t *const *roms, const size_t *rom_sizes, const 
       (rc = dalloc(&E->d_dec, 1024, T)) || (rc = dalloc(&E->d_env_rom, n * 4, T)) ||
       (rc = dalloc(&E->d_env_key, n * 4, T)) || (rc = dalloc(&E->d_state, n * 256, T)) ||
       (rc = dalloc(&E->d_cache, (size_t)n_roms * c.n_cache * 256, T)) ||
-      (rc = dalloc(&E->d_log, n * 2 * (size_t)c.log_cap * 4, T)) || (rc = dalloc(&E->d_snap, n * 2 * 64, T)) ||
-      (rc = dalloc(&E->d_meta, n * 2 * 2 * 4, T)) ||
-      (c.form == ATARI_FORM_PLAIN && (rc = dalloc(&E->d_frames, n * 2 * 210 * 160, T))) ||
+      (rc = dalloc(&E->d_log, n * 2 * (size_t)c.log_cap * 4, T)) || (rc = dalloc(&E->d_meta, n * 2 * 2 * 4, T)) ||
+      (c.form == ATARI_FORM_PLAIN &&
+       ((rc = dalloc(&E->d_frames, n * 2 * 210 * 160, T)) || (rc = dalloc(&E->d_snap, n * 2 * 64, T)))) ||
+      (c.form == ATARI_FORM_BATCHED && (rc = dalloc(&E->d_bsnap, n * band_bytes(c), T))) ||
       (rc = dalloc(&E->d_rew, n * 4, T)) || (rc = dalloc(&E->d_done, n, T)) || (rc = dalloc(&E->d_ctr, n * 12, T)) ||
       (rc = dalloc(&E->d_act, n, T)) || (rc = dalloc(&E->d_luma, 128, T)) || (rc = dalloc(&E->d_dec_op, DEC_BYTES, T)))
     return bail(rc);
   if (c.output_mode == ATARI_OUT_STACK) {
     if ((rc = dalloc(&E->d_ring, n * 4 * 7056, T)) || (rc = dalloc(&E->d_head, n, T))) return bail(rc);
-    if (c.form == ATARI_FORM_BATCHED && (rc = dalloc(&E->d_bsnap, n * 2 * 3 * 64, T))) return bail(rc);
   }
   // render inputs start zeroed (a step that failed to write them still renders defined values)
-  if (n && (cudaMemset(E->d_snap, 0, n * 2 * 64) != cudaSuccess || cudaMemset(E->d_meta, 0, n * 2 * 2 * 4) != cudaSuccess ||
-            (E->d_bsnap && cudaMemset(E->d_bsnap, 0, n * 2 * 3 * 64) != cudaSuccess)))
+  if (n && ((E->d_snap && cudaMemset(E->d_snap, 0, n * 2 * 64) != cudaSuccess) ||
+            cudaMemset(E->d_meta, 0, n * 2 * 2 * 4) != cudaSuccess ||
+            (E->d_bsnap && cudaMemset(E->d_bsnap, 0, n * band_bytes(c)) != cudaSuccess)))
     return bail(fail(ATARI_ECUDA, "zeroing render buffers failed"));
 
   // cartridges: 2K images mirrored to 4K, each in a 16 KB slot
@@ -1015,12 +1018,12 @@ int launch_batched(atari_env *E, const uint8_t *d_actions, uint8_t *d_obs, int32
   CUDA_TRY(cudaGetLastError());
   if (c.output_mode == ATARI_OUT_STACK) {
     ProfScope p(E, ATARI_PROF_FUSED, s);
-    k_raster_preprocess<<<E->n, 64 * E->wpf, fused_smem(), s>>>(E->d_log, E->d_snap, E->d_bsnap, E->d_meta, E->d_luma, E->d_ring,
-                                                                E->d_head, E->d_done, d_obs, E->n, c.log_cap, E->wpf, nullptr, nullptr, 0);
+    k_raster_preprocess<<<E->n, PAINT_THREADS, PAINT_SMEM, s>>>(E->d_log, E->d_bsnap, E->d_meta, E->d_luma, E->d_ring,
+                                                                 E->d_head, E->d_done, d_obs, E->n, c.log_cap, nullptr,
+                                                                 nullptr, 0);
   } else if (d_obs) {
     ProfScope p(E, ATARI_PROF_RASTER, s);
-    k_raster<<<(unsigned)((E->n + 3) / 4), 128, 0, s>>>(E->d_log, E->d_snap, E->d_meta, d_obs, (size_t)210 * 160,
-                                                         E->n, 1, c.log_cap);
+    k_raster_palette<<<E->n, PAINT_THREADS, PAINT_SMEM, s>>>(E->d_log, E->d_bsnap, E->d_meta, d_obs, E->n, c.log_cap);
   }
   CUDA_TRY(cudaGetLastError());
   return 0;
@@ -1058,12 +1061,11 @@ int step_batched(atari_env *E, const uint8_t *d_actions, uint8_t *d_obs, int32_t
 
 
 // Time the batched interpreter on a copy of the current state and keep the
-// fastest (envs per warp, warps per block); then the fastest number of warps
-// per frame in the fused replay.  Every configuration computes the same
-// results; only speed differs.  The state, stack ring and heads are restored.
+// fastest (envs per warp, warps per block).  Every configuration computes the
+// same results; only speed differs.  The state is restored.
 int autotune(atari_env *E) {
   const size_t n = (size_t)E->n;
-  uint8_t *st_bak = nullptr, *ring_bak = nullptr, *head_bak = nullptr;
+  uint8_t *st_bak = nullptr;
   size_t dummy = 0;
   if (int rc = dalloc(&st_bak, n * 256, dummy)) return rc;
   CUDA_TRY(cudaMemcpy(st_bak, E->d_state, n * 256, cudaMemcpyDeviceToDevice));
@@ -1136,32 +1138,9 @@ int autotune(atari_env *E) {
     E->grouping = tg[2] < 0.97f * tg[1] ? 2 : 1;
   }
   E->compact = E->cfg.dispatch == 2;
-  if (!rc && E->cfg.output_mode == ATARI_OUT_STACK) {
-    if (!(rc = dalloc(&ring_bak, n * 4 * 7056, dummy)) && !(rc = dalloc(&head_bak, n, dummy))) {
-      cudaMemcpy(ring_bak, E->d_ring, n * 4 * 7056, cudaMemcpyDeviceToDevice);
-      cudaMemcpy(head_bak, E->d_head, n, cudaMemcpyDeviceToDevice);
-      float fb = 1e30f;
-      for (int wpf : {4, 2, 1}) {  // a later (smaller) split must be 3 % faster to be taken
-        float t = 0;
-        for (int rep = 0; rep < 2; ++rep) {
-          cudaEventRecord(e0);
-          k_raster_preprocess<<<E->n, 64 * wpf, fused_smem()>>>(E->d_log, E->d_snap, E->d_bsnap, E->d_meta, E->d_luma, E->d_ring,
-                                                               E->d_head, E->d_done, nullptr, E->n, E->cfg.log_cap, wpf, nullptr, nullptr, 0);
-          cudaEventRecord(e1);
-          cudaEventSynchronize(e1);
-          cudaEventElapsedTime(&t, e0, e1);
-        }
-        if (t < 0.97f * fb) { fb = t; E->wpf = wpf; }
-      }
-      cudaMemcpy(E->d_ring, ring_bak, n * 4 * 7056, cudaMemcpyDeviceToDevice);
-      cudaMemcpy(E->d_head, head_bak, n, cudaMemcpyDeviceToDevice);
-    }
-  }
   CUDA_TRY(cudaMemcpy(E->d_state, st_bak, n * 256, cudaMemcpyDeviceToDevice));
   cudaError_t ce = cudaDeviceSynchronize();
   cudaFree(st_bak);
-  if (ring_bak) cudaFree(ring_bak);
-  if (head_bak) cudaFree(head_bak);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   E->profiling = was_prof;
@@ -1189,11 +1168,12 @@ int setup_batched(atari_env *E, const std::vector<uint8_t> &img, const std::vect
   if (int rc = dalloc(&E->d_queue, 64, T)) return rc;
   CUDA_TRY(cudaMemcpy(E->d_romb, bytes.data(), bytes.size(), cudaMemcpyHostToDevice));
   CUDA_TRY(cudaStreamCreateWithFlags(&E->cap_stream, cudaStreamNonBlocking));
-  CUDA_TRY(cudaFuncSetAttribute(k_raster_preprocess, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_smem()));
+  CUDA_TRY(cudaFuncSetAttribute(k_raster_preprocess, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAINT_SMEM));
+  CUDA_TRY(cudaFuncSetAttribute(k_raster_palette, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAINT_SMEM));
   const atari_config &c = E->cfg;
+  if (c.raster_warps_per_frame > 0) E->wpf = c.raster_warps_per_frame;
   if (c.envs_per_block > 0 && c.envs_per_warp > 0) {
     int L = std::min(32, c.envs_per_warp), W = std::max(1, std::min(4, c.envs_per_block / L));
-    E->wpf = c.raster_warps_per_frame > 0 ? c.raster_warps_per_frame : 4;
     E->grouping = c.grouping ? c.grouping : 1;
     E->compact = c.dispatch == 2;
     return build_groups(E, L, W, c.tia_warps >= 2);
@@ -1256,9 +1236,9 @@ int step_host_overlapped(atari_env *E, uint8_t *obs, int32_t *rewards, uint8_t *
     const int b0 = (int)((int64_t)n * k / chunks), b1 = (int)((int64_t)n * (k + 1) / chunks);
     {
       ProfScope p(E, ATARI_PROF_FUSED, s);
-      k_raster_preprocess<<<b1 - b0, 64 * E->wpf, fused_smem(), s>>>(
-          E->d_log, E->d_snap, E->d_bsnap, E->d_meta, E->d_luma, E->d_ring, E->d_head, E->d_done, E->d_obs_tmp, n,
-          c.log_cap, E->wpf, nullptr, nullptr, b0);
+      k_raster_preprocess<<<b1 - b0, PAINT_THREADS, PAINT_SMEM, s>>>(E->d_log, E->d_bsnap, E->d_meta, E->d_luma,
+                                                                     E->d_ring, E->d_head, E->d_done, E->d_obs_tmp, n,
+                                                                     c.log_cap, nullptr, nullptr, b0);
     }
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaEventRecord(E->copy_ev[k + 1], s));
@@ -1705,9 +1685,9 @@ int serve_tick(atari_env *E, const ServeTick &t, cudaStream_t s) {
   const int grid = std::max(1, std::min(t.n_groups, E->max_blocks));
   launch_interp(E, a, grid, s);
   CUDA_TRY(cudaGetLastError());
-  k_raster_preprocess<<<t.n_active, 64 * E->wpf, fused_smem(), s>>>(E->d_log, E->d_snap, E->d_bsnap, E->d_meta, E->d_luma,
-                                                                   E->d_ring, E->d_head, E->d_done, t.d_obs,
-                                                                   t.n_active, c.log_cap, E->wpf, a.perm, a.opos, 0);
+  k_raster_preprocess<<<t.n_active, PAINT_THREADS, PAINT_SMEM, s>>>(E->d_log, E->d_bsnap, E->d_meta, E->d_luma, E->d_ring,
+                                                                    E->d_head, E->d_done, t.d_obs, t.n_active,
+                                                                    c.log_cap, a.perm, a.opos, 0);
   CUDA_TRY(cudaGetLastError());
   return 0;
 }

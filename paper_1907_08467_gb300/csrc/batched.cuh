@@ -18,6 +18,7 @@
 
 #include "device_machine.cuh"
 #include "fast_console.cuh"
+#include "paint.cuh"
 #include "render.cuh"
 
 namespace atari {
@@ -34,8 +35,7 @@ struct BatchArgs {
   int32_t *rew_out;
   uint8_t *done_out;
   uint32_t *log;
-  uint8_t *snap;
-  uint8_t *bsnap;            // null, or [n][2][3][64] quarter-frame band start snapshots
+  uint8_t *bsnap;            // [n][logged frames][BANDS][BAND_SNAP] band start snapshots
   uint32_t *meta;
   uint32_t *counters;
   const int32_t *grp_rom, *grp_start, *grp_count, *perm;
@@ -66,7 +66,8 @@ __device__ __forceinline__ void fast_reset_from_cache(uint8_t *st, const uint8_t
 
 // Where the TIA side of env slot i leaves its logs and snapshots.
 __device__ __forceinline__ TiaOut tia_out_of(const BatchArgs &a, int i) {
-  return TiaOut{a.log + (size_t)i * 2 * a.log_cap, a.snap + (size_t)i * 128, a.bsnap ? a.bsnap + (size_t)i * 384 : nullptr,
+  const long long frame = (long long)i * (2 - a.first_slot) - a.first_slot;  // frames before this env's frame F-1
+  return TiaOut{a.log + (size_t)i * 2 * a.log_cap, a.bsnap + frame * (long long)(BANDS * BAND_SNAP),
                 a.meta + (size_t)i * 4, (uint32_t)a.log_cap};
 }
 
@@ -309,156 +310,125 @@ __global__ void __launch_bounds__(256) k_group_by_bank(const uint8_t *state, con
   }
 }
 
-// Render rows [r0, r1) of one frame with one warp into a shared-memory frame.
-// R holds the render state after records [0, ri0); records from ri0 on that
-// take effect before the band's first row are applied first.
-__device__ inline void render_rows_warp(RenderRegs &R, const uint32_t *recs, uint32_t n_rec, uint32_t n_lines,
-                                        uint32_t r0, uint32_t r1, uint8_t *frame, uint32_t ri0) {
-  const uint32_t lane = threadIdx.x & 31;
-  uint32_t ri = ri0, base = ri0;
-  uint32_t chunk = base + lane < n_rec ? recs[base + lane] : 0xFFFFFFFFu;
-  // records that take effect before the band's first row: apply only
-  const uint32_t start_clk = 228u * (WINDOW_Y0 + r0);
-  while (ri < n_rec) {
-    if (ri - base >= 32) {
-      base += 32;
-      chunk = base + lane < n_rec ? recs[base + lane] : 0xFFFFFFFFu;
-    }
-    const uint32_t rec = __shfl_sync(0xFFFFFFFFu, chunk, ri - base);
-    const uint32_t c = rec >> 14;
-    if (c >= start_clk) break;
-    R.apply((rec >> 8) & 0x3F, rec & 0xFF, c);
-    ++ri;
-  }
-  for (uint32_t r = r0; r < r1; ++r) {
-    uint8_t *row = frame + r * FRAME_W;
-    const uint32_t line = WINDOW_Y0 + r;
-    if (line >= n_lines) {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) row[lane + 32 * k] = 0;
-      continue;
-    }
-    const uint32_t cl = 228u * line, end = cl + 228u;
-    uint32_t k = 0;
-    while (ri < n_rec) {
-      if (ri - base >= 32) {
-        base += 32;
-        chunk = base + lane < n_rec ? recs[base + lane] : 0xFFFFFFFFu;
-      }
-      const uint32_t rec = __shfl_sync(0xFFFFFFFFu, chunk, ri - base);
-      const uint32_t c = rec >> 14;
-      if (c >= end) break;
-      R.prepare(k < 5 && cl + 68u + lane + 32u * k < c, lane);
-      while (k < 5 && cl + 68u + lane + 32u * k < c) {
-        row[lane + 32 * k] = (uint8_t)R.pixel_k(k);
-        ++k;
-      }
-      R.apply((rec >> 8) & 0x3F, rec & 0xFF, c);
-      ++ri;
-    }
-    R.prepare(k < 5, lane);
-    R.row_from(k, lane, row);
-    R.hmove_bar(lane, line, row);
-  }
+// Shared memory of the painting kernels: the frame, the threads' register
+// files, the tables.
+constexpr int PAINT_THREADS = 128;
+constexpr uint32_t PAINT_FILES = PAINT_FRAME, PAINT_LUT = PAINT_FILES + PAINT_THREADS * FILE_STRIDE;
+constexpr uint32_t PAINT_SMEM = PAINT_LUT + PAINT_TABS;
+static_assert(PAINT_THREADS >= (int)BANDS, "one thread per band");
+__device__ __forceinline__ RowPainter painter() {
+  RowPainter p;
+  p.tabs = PaintTabs{PAINT_LUT + 1024, PAINT_LUT + 1024 + 128, PAINT_LUT};
+  p.file = PAINT_FILES + threadIdx.x * FILE_STRIDE;
+  return p;
+}
+// Frame slot (0: F-1, 1: F) of env i: this thread's band, into the frame in shared memory.
+template <bool MAX>
+__device__ __forceinline__ void paint_frame(RowPainter &p, int i, int slot, int first_slot, const uint32_t *log,
+                                            const uint8_t *bsnap, const uint32_t *meta, int log_cap) {
+  const uint32_t band = threadIdx.x;
+  if (band >= BANDS) return;
+  const uint32_t *mt = meta + (size_t)i * 4 + slot * 2;
+  const uint32_t n_rec = min(mt[0], (uint32_t)log_cap);
+  const size_t f = (size_t)i * (2 - first_slot) + (slot - first_slot);
+  const uint32_t ri = min(p.start(bsnap + (f * BANDS + band) * BAND_SNAP), n_rec);
+  const uint32_t r0 = band * BAND_ROWS, r1 = min(r0 + BAND_ROWS, (uint32_t)FRAME_H);
+  p.paint<MAX>(r0, r1, mt[1], log + ((size_t)i * 2 + slot) * log_cap, ri, n_rec, 0);
 }
 
-// One block per env: warps [0, W) render frame F-1, warps [W, 2W) frame F,
-// each warp a band of rows; then luma max, 84x84 area resampling, stack push.
-__global__ void __launch_bounds__(256, 3) k_raster_preprocess(const uint32_t *log, const uint8_t *snap, const uint8_t *bsnap,
-                                                           const uint32_t *meta,
-                                                           const uint8_t *luma_g, uint8_t *ring, uint8_t *head,
-                                                           const uint8_t *done, uint8_t *obs, int n, int log_cap,
-                                                           int warps_per_frame, const int32_t *perm,
-                                                           const int32_t *opos, int base) {
-  extern __shared__ __align__(16) uint8_t sm[];
-  uint8_t *fa = sm;                        // frame F-1, later the luma maximum
-  uint8_t *fb = sm + FRAME_H * FRAME_W;    // frame F
-  uint8_t *luma = fb + FRAME_H * FRAME_W;
-  uint8_t *plane = luma + 128;
+// One block per env: the rows of frames F-1 and F as luma, their pixelwise
+// maximum, 84x84 area resampling, stack push.  A thread paints its rows of
+// frame F-1 and then frame F's over them, so one frame (36 KB) is kept and
+// five blocks fit an SM.
+__global__ void __launch_bounds__(PAINT_THREADS, 5)
+    k_raster_preprocess(const uint32_t *log, const uint8_t *bsnap, const uint32_t *meta, const uint8_t *luma_g,
+                        uint8_t *ring, uint8_t *head, const uint8_t *done, uint8_t *obs, int n, int log_cap,
+                        const int32_t *perm, const int32_t *opos, int base) {
   // block b (counted from base) serves env slot perm[b] and writes its stack
   // at position opos[b]
   const int blk = base + (int)blockIdx.x;
   if (blk >= n) return;
   const int i = perm ? perm[blk] : blk;
   const int o = opos ? opos[blk] : i;
-  const int warp = threadIdx.x >> 5;
-  for (int t = threadIdx.x; t < 128; t += blockDim.x) luma[t] = luma_g[t];
-  if (warp < 2 * warps_per_frame) {
-    const int slot = warp / warps_per_frame, band = warp % warps_per_frame;
-    const uint32_t r0 = (uint32_t)(FRAME_H * band / warps_per_frame);
-    const uint32_t r1 = (uint32_t)(FRAME_H * (band + 1) / warps_per_frame);
-    const size_t fs = (size_t)i * 2 + slot;
-    const uint32_t *mt = meta + fs * 2;
-    const uint32_t n_rec = mt[0] < (uint32_t)log_cap ? mt[0] : (uint32_t)log_cap;
-    // a band starting at a quarter of the frame starts from the interpreter's
-    // snapshot there; the first band from the frame's start
-    const uint32_t q = (uint32_t)(band * 4 / warps_per_frame);
-    RenderRegs R;
-    uint32_t ri0 = 0;
-    if (bsnap && q > 0 && (band * 4) % warps_per_frame == 0) {
-      const uint8_t *bs = bsnap + (fs * 3 + q - 1) * 64;
-      R.load(bs);
-      ri0 = reinterpret_cast<const uint32_t *>(bs)[14];
-      ri0 = ri0 < n_rec ? ri0 : n_rec;
-    } else {
-      R.load(snap + fs * 64);
-    }
-    render_rows_warp(R, log + fs * log_cap, n_rec, mt[1], r0, r1, slot ? fb : fa, ri0);
-  }
+  RowPainter p = painter();
+  paint_tables(p.tabs, luma_g);
   __syncthreads();
-  {
-    uint32_t *a4 = reinterpret_cast<uint32_t *>(fa);
-    const uint32_t *b4 = reinterpret_cast<const uint32_t *>(fb);
-    for (int q = threadIdx.x; q < FRAME_H * FRAME_W / 4; q += blockDim.x) {
-      uint32_t x = a4[q], y = b4[q], r = 0;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        uint32_t la = luma[((x >> (8 * k)) & 0xFF) >> 1], lb = luma[((y >> (8 * k)) & 0xFF) >> 1];
-        r |= (la > lb ? la : lb) << (8 * k);
-      }
-      a4[q] = r;
-    }
-  }
-  __syncthreads();
-  for (int o = threadIdx.x; o < 84 * 84; o += blockDim.x) {
-    uint32_t oi = o / 84, oj = o % 84;
-    uint32_t y0 = (5u * oi) >> 1;
-    uint32_t wy0 = (oi & 1) ? 42u : 84u, wy1 = 84u, wy2 = (oi & 1) ? 84u : 42u;
-    uint32_t x0, wx0, wx1, wx2;
-    col_weights(oj, x0, wx0, wx1, wx2);
-    const uint8_t *r0 = fa + y0 * FRAME_W + x0;
-    const uint8_t *r1 = r0 + FRAME_W;
-    const uint8_t *r2 = r1 + FRAME_W;
-    uint32_t rs0 = wx0 * r0[0] + wx1 * r0[1] + (wx2 ? wx2 * r0[2] : 0u);
-    uint32_t rs1 = wx0 * r1[0] + wx1 * r1[1] + (wx2 ? wx2 * r1[2] : 0u);
-    uint32_t rs2 = wx0 * r2[0] + wx1 * r2[1] + (wx2 ? wx2 * r2[2] : 0u);
-    plane[o] = (uint8_t)((wy0 * rs0 + wy1 * rs1 + wy2 * rs2 + 16800u) / 33600u);
-  }
-  __syncthreads();
+  paint_frame<false>(p, i, 0, 0, log, bsnap, meta, log_cap);
+  paint_frame<true>(p, i, 1, 0, log, bsnap, meta, log_cap);
   const uint32_t h = head[i];
+  const bool finished = done[i] != 0;
   uint8_t *rg = ring + (size_t)i * 4 * 7056;
-  const uint32_t *pl32 = reinterpret_cast<const uint32_t *>(plane);
-  if (obs) {
-    uint8_t *ob = obs + (size_t)o * 4 * 7056;
+  uint8_t *ob = obs ? obs + (size_t)o * 4 * 7056 : nullptr;
+  // the three kept planes, oldest first, to the stack
+  if (ob) {
     for (int s = 0; s < 3; ++s) {
       const uint4 *src = reinterpret_cast<const uint4 *>(rg + ((h + 1 + s) & 3) * 7056);
       uint4 *dst = reinterpret_cast<uint4 *>(ob + s * 7056);
-      for (int q = threadIdx.x; q < 7056 / 16; q += blockDim.x) dst[q] = src[q];
+      for (int q = threadIdx.x; q < 7056 / 16; q += PAINT_THREADS) dst[q] = src[q];
     }
-    const uint4 *p16 = reinterpret_cast<const uint4 *>(plane);
-    uint4 *dst = reinterpret_cast<uint4 *>(ob + 3 * 7056);
-    for (int q = threadIdx.x; q < 7056 / 16; q += blockDim.x) dst[q] = p16[q];
   }
-  __syncthreads();
-  if (done[i]) {
+  __syncthreads();  // the frame is painted and the kept planes are read
+  // Resampling.  Output row i covers source rows [2.5 i, 2.5 i + 2.5), output
+  // column j columns [160 j / 84, 160 (j + 1) / 84).  In units of 1/21 column
+  // and 1/2 row the weights are whole numbers of at most 21 and 2, and the
+  // area's weight is 40 x 5 = 200: out = (sum + 100) / 200, the same value as
+  // with 1/84 units and 33600.  A thread takes four columns and every sixth
+  // pair of output rows (five source rows): a column's three pixels are one
+  // byte dot product per source row.
+  const uint32_t m = threadIdx.x % 21u, k0 = threadIdx.x / 21u;
+  if (k0 < 6u) {
+    uint32_t wt[4], sh[4], at[4];
+#pragma unroll
+    for (uint32_t c = 0; c < 4; ++c) {
+      uint32_t x0, w0, w1, w2;
+      col_weights(4u * m + c, x0, w0, w1, w2);
+      wt[c] = (w0 >> 2) | (w1 >> 2) << 8 | (w2 >> 2) << 16;
+      at[c] = x0 & ~3u;
+      sh[c] = 8u * (x0 & 3u);
+    }
+    uint32_t *out0 = reinterpret_cast<uint32_t *>(rg + h * 7056);
+    uint32_t *out1 = ob ? reinterpret_cast<uint32_t *>(ob + 3 * 7056) : nullptr;
+    for (uint32_t k = k0; k < 42u; k += 6u) {
+      uint32_t even = 0, odd = 0;
+#pragma unroll
+      for (uint32_t c = 0; c < 4; ++c) {
+        uint32_t px[5];
+#pragma unroll
+        for (uint32_t r = 0; r < 5; ++r) {
+          const uint32_t a = row_off(5u * k + r) + at[c];
+          px[r] = __funnelshift_r(sm32(a), sm32(a + 4), sh[c]);
+        }
+        const uint32_t mid = __dp4a(px[2], wt[c], 100u), w2 = wt[c] * 2u;
+        even |= __dp4a(px[0], w2, __dp4a(px[1], w2, mid)) / 200u << (8u * c);
+        odd |= __dp4a(px[4], w2, __dp4a(px[3], w2, mid)) / 200u << (8u * c);
+      }
+      const uint32_t q = 42u * k + m;  // word of output row 2 k
+      if (out1) { out1[q] = even; out1[q + 21] = odd; }
+      if (!finished) { out0[q] = even; out0[q + 21] = odd; }
+    }
+  }
+  if (finished) {
     uint4 *z = reinterpret_cast<uint4 *>(rg);
-    for (int q = threadIdx.x; q < 4 * 7056 / 16; q += blockDim.x) z[q] = make_uint4(0, 0, 0, 0);
+    for (int q = threadIdx.x; q < 4 * 7056 / 16; q += PAINT_THREADS) z[q] = make_uint4(0, 0, 0, 0);
     if (threadIdx.x == 0) head[i] = 0;
-  } else {
-    uint32_t *dst = reinterpret_cast<uint32_t *>(rg + h * 7056);
-    for (int q = threadIdx.x; q < 7056 / 4; q += blockDim.x) dst[q] = pl32[q];
-    if (threadIdx.x == 0) head[i] = (uint8_t)((h + 1) & 3);
+  } else if (threadIdx.x == 0) {
+    head[i] = (uint8_t)((h + 1) & 3);
   }
+}
+
+// Palette output: one block per env, frame F to the observation.
+__global__ void __launch_bounds__(PAINT_THREADS, 5)
+    k_raster_palette(const uint32_t *log, const uint8_t *bsnap, const uint32_t *meta, uint8_t *obs, int n, int log_cap) {
+  const int i = (int)blockIdx.x;
+  if (i >= n) return;
+  RowPainter p = painter();
+  paint_tables(p.tabs, nullptr);
+  __syncthreads();
+  paint_frame<false>(p, i, 1, 1, log, bsnap, meta, log_cap);
+  __syncthreads();
+  uint32_t *dst = reinterpret_cast<uint32_t *>(obs + (size_t)i * (FRAME_H * FRAME_W));
+  for (uint32_t q = threadIdx.x; q < FRAME_H * FRAME_W / 4; q += PAINT_THREADS)
+    dst[q] = sm32(row_off(q / 40u) + 4u * (q % 40u));
 }
 
 }  // namespace atari

@@ -34,8 +34,8 @@ enum TiaSlot : uint32_t {
 enum IoWord : uint32_t {
   IO_CEVAL = 0, IO_CX, IO_L0LO, IO_L0HI, IO_BARLO, IO_BARHI, IO_TCWLO, IO_TCWHI, IO_TV, IO_TSH, IO_PORTS,
   IO_JOY, IO_FIRE, IO_LATCH, IO_LOGLO, IO_LOGHI, IO_LOGN, IO_LOGCAP, IO_STATUS,
-  IO_BANDN,      // next quarter-frame band whose start snapshot is due (1..3), 4: none
-  IO_BSLO, IO_BSHI,  // where this frame's band snapshots go (3 x 64 bytes)
+  IO_BANDN,      // next band whose start snapshot is due, BANDS: none
+  IO_BSLO, IO_BSHI,  // where this frame's band snapshots go
   IO_QHEAD, IO_QTAIL, IO_ACK,  // split form: the TIA side's queue cursor and acknowledgements
   IO_WORDS
 };
@@ -185,52 +185,47 @@ __device__ __forceinline__ uint32_t fc_riot_read(IoCtx c, uint32_t a, uint64_t n
 __device__ __forceinline__ uint32_t fc_cx_byte(uint32_t cx, uint32_t reg) {
   return (((cx >> (2 * reg + 1)) & 1u) << 7) | (((cx >> (2 * reg)) & 1u) << 6);
 }
-// 64-byte render snapshot: TIA file (canonical bytes 0x20..0x44), HMOVE bar
-// line, frame base line; word 14 = the number of log records before it.
-__device__ __forceinline__ void fc_snapshot(IoCtx c, uint8_t *o, uint32_t nrec) {
-  uint32_t v[16];
-#pragma unroll
-  for (int q = 0; q < 10; ++q) {
-    uint32_t x = 0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-      if (q * 4 + b < 37) x |= c.T(q * 4 + b) << (8 * b);
-    v[q] = x;
-  }
-  v[9] &= 0xFFu;
-  v[10] = c.G(IO_BARLO); v[11] = c.G(IO_BARHI);
-  v[12] = c.G(IO_L0LO); v[13] = c.G(IO_L0HI);
-  v[14] = nrec; v[15] = 0;
-  uint4 *d = reinterpret_cast<uint4 *>(o);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) d[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-}
-
-// First color clock of quarter-frame band q (rows 210 q / 4 of the window).
-__device__ __forceinline__ uint32_t fc_band_clk(uint32_t q) { return 228u * (WINDOW_Y0 + (FRAME_H * q) / 4u); }
+// Bands: groups of BAND_ROWS rows of the 210-row window.  While a frame is
+// logged, the render state at the start of every band is kept (48 bytes), so
+// that the painter's threads start their bands there instead of replaying the
+// frame from its first record.
+constexpr uint32_t BAND_ROWS = 2, BANDS = (FRAME_H + BAND_ROWS - 1) / BAND_ROWS, BAND_SNAP = 48;
+// First color clock of band q.
+__device__ __forceinline__ uint32_t fc_band_clk(uint32_t q) { return 228u * (WINDOW_Y0 + BAND_ROWS * q); }
 
 // Snapshot the render state at the start of every band due by clock eff: the
-// state after all records of earlier clocks, so the rasteriser's warps start
-// their bands there instead of replaying the frame from its first record.
+// state after all records of earlier clocks.  Words 0..8: the TIA file's first
+// 36 bytes; word 9: its last byte and, in the high half, the frame-relative
+// line of the HMOVE bar or 0xFFFF; word 10: the log records before it.
 __device__ __noinline__ void fc_band_snap(IoCtx c, uint32_t eff) {
   uint32_t bn = c.G(IO_BANDN);
   uint8_t *base = reinterpret_cast<uint8_t *>((uint64_t)c.G(IO_BSLO) | (uint64_t)c.G(IO_BSHI) << 32);
+  const uint64_t bar = c.G64(IO_BARLO), l0 = c.G64(IO_L0LO);
+  const uint32_t rel = bar != NO_LINE && bar >= l0 && bar - l0 < 1024 ? (uint32_t)(bar - l0) : 0xFFFFu;
   const uint32_t nrec = c.G(IO_LOGN);
-  while (bn < 4 && eff >= fc_band_clk(bn)) {
-    fc_snapshot(c, base + (bn - 1) * 64, nrec);
+  uint32_t v[10];
+#pragma unroll
+  for (int q = 0; q < 10; ++q) v[q] = sm32(c.tia + 4 * q);
+  v[9] = (v[9] & 0xFFu) | rel << 16;
+  uint4 *d = reinterpret_cast<uint4 *>(base) + 3 * bn;
+  while (bn < BANDS && eff >= fc_band_clk(bn)) {
+    d[0] = make_uint4(v[0], v[1], v[2], v[3]);
+    d[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    d[2] = make_uint4(v[8], v[9], nrec, 0);
+    d += 3;
     ++bn;
   }
   c.Sset(IO_BANDN, bn);
 }
 
-// Log the frame's TIA writes to p (cap records; p null: no log); bands:
-// where the three quarter-frame start snapshots go, or null for none.
+// Log the frame's TIA writes to p (cap records; p null: no log) and the band
+// starts to bands.
 __device__ __forceinline__ void fc_set_log(IoCtx c, uint32_t *p, uint32_t cap, uint8_t *bands) {
   c.Sset(IO_LOGLO, (uint32_t)(uint64_t)p);
   c.Sset(IO_LOGHI, (uint32_t)((uint64_t)p >> 32));
   c.Sset(IO_LOGN, 0);
   c.Sset(IO_LOGCAP, cap);
-  c.Sset(IO_BANDN, bands ? 1u : 4u);
+  c.Sset(IO_BANDN, bands ? 0u : BANDS);
   c.Sset(IO_BSLO, (uint32_t)(uint64_t)bands);
   c.Sset(IO_BSHI, (uint32_t)((uint64_t)bands >> 32));
 }
@@ -240,7 +235,7 @@ __device__ __forceinline__ void fc_set_log(IoCtx c, uint32_t *p, uint32_t cap, u
 __device__ __forceinline__ void fc_log(IoCtx c, uint32_t eff, uint32_t reg, uint32_t v) {
   const uint32_t lo = c.G(IO_LOGLO), hi = c.G(IO_LOGHI);
   if (lo | hi) {
-    if (c.G(IO_BANDN) < 4 && eff >= fc_band_clk(c.G(IO_BANDN))) fc_band_snap(c, eff);
+    if (c.G(IO_BANDN) < BANDS && eff >= fc_band_clk(c.G(IO_BANDN))) fc_band_snap(c, eff);
     uint32_t *lp = reinterpret_cast<uint32_t *>((uint64_t)lo | (uint64_t)hi << 32);
     const uint32_t nrec = c.G(IO_LOGN);
     if (nrec < c.G(IO_LOGCAP)) lp[nrec] = eff << 14 | reg << 8 | v;
@@ -350,8 +345,7 @@ __device__ __forceinline__ uint64_t global_ns() {
 // Where the TIA side of one env leaves its logs and snapshots.
 struct TiaOut {
   uint32_t *log;      // two logs of log_cap records
-  uint8_t *snap;      // two 64-byte snapshots
-  uint8_t *bsnap;     // null, or two times three band snapshots
+  uint8_t *bsnap;     // the band snapshots of frames F-1 and F (frame F-1's place is not used when it is not logged)
   uint32_t *meta;     // two times (records, lines)
   uint32_t log_cap;
 };
@@ -383,12 +377,11 @@ __device__ __forceinline__ uint32_t tia_event(IoCtx c, uint32_t ev, TiaSide &s, 
   }
   const uint32_t sub = (ev >> 26) & 3, slot = ev & 1;
   if (sub == 0) {
-    fc_snapshot(c, o.snap + slot * 64, 0);
-    fc_set_log(c, o.log + (size_t)slot * o.log_cap, o.log_cap, o.bsnap ? o.bsnap + slot * 3 * 64 : nullptr);
+    fc_set_log(c, o.log + (size_t)slot * o.log_cap, o.log_cap, o.bsnap + (size_t)slot * BANDS * BAND_SNAP);
     return 0;
   }
   if (sub == 1) {
-    if (c.G(IO_BANDN) < 4) fc_band_snap(c, ~0u);
+    if (c.G(IO_BANDN) < BANDS) fc_band_snap(c, ~0u);  // band starts that the frame never reached take its last state
     const uint32_t nrec = c.G(IO_LOGN);
     o.meta[2 * slot] = nrec;
     o.meta[2 * slot + 1] = s.lines;
@@ -537,7 +530,7 @@ struct FastConsoleT {
     io.Sset(IO_CEVAL, 3u * kf);
     io.Sset(IO_JOY, 0xFF); io.Sset(IO_FIRE, 0);
     io.Sset(IO_LOGLO, 0); io.Sset(IO_LOGHI, 0); io.Sset(IO_LOGN, 0); io.Sset(IO_LOGCAP, 0);
-    io.Sset(IO_BANDN, 4);
+    io.Sset(IO_BANDN, BANDS);
     io.Sset(IO_STATUS, 0);
     const uint4 *r4 = reinterpret_cast<const uint4 *>(s + S::RAM);
     uint32_t *r32 = &sm32(off.ram);
