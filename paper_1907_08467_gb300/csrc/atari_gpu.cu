@@ -213,15 +213,11 @@ struct CacheHook {
 };
 __global__ void __launch_bounds__(128) k_cache_run(uint8_t *work, uint8_t *snaps, const uint8_t *roms,
                                                     const uint32_t *info, const uint8_t *dec_op_g, int rom_stage,
-                                                    int startup, int max_noops) {
+                                                    int startup, int max_noops, int unit) {
   const int r = blockIdx.x;
   const uint32_t inf = info[r];
-  const uint32_t banks = inf >> 24;
-  const uint4 *src = reinterpret_cast<const uint4 *>(roms + (size_t)r * ROM_SLOT);
-  uint4 *dst = reinterpret_cast<uint4 *>(g_smem);
-  for (uint32_t q = threadIdx.x; q < banks * 256u; q += blockDim.x) dst[q] = src[q];
-  if (threadIdx.x == 0) dst[banks * 256u] = make_uint4(0, 0, 0, 0);
-  for (uint32_t t = threadIdx.x; t < DEC_BYTES; t += blockDim.x) sm8(rom_stage + 16 + t) = dec_op_g[t];
+  stage_cartridge(roms + (size_t)r * ROM_SLOT, inf >> 24, inf & 0xFF);
+  for (uint32_t t = threadIdx.x; t < DEC_BYTES; t += blockDim.x) sm8(OFF_DEC + t) = dec_op_g[t];
   __syncthreads();
   if (threadIdx.x != 0) return;
   uint8_t *st = work + (size_t)r * 256;
@@ -231,6 +227,7 @@ __global__ void __launch_bounds__(128) k_cache_run(uint8_t *work, uint8_t *snaps
   m.scheme = inf & 0xFF;
   m.wmask = 1u;
   m.idle = 1u;
+  m.unit = (uint32_t)unit;
   m.to = TiaOut{nullptr, nullptr, nullptr, 0};
   m.load(st);
   m.apply_action(0);
@@ -587,8 +584,9 @@ int validate(const atari_config &c) {
 
 namespace {
 
+constexpr size_t MAX_SMEM = 227 * 1024 - 64;  // a block's dynamic shared memory, beside a few static bytes
 size_t interp_smem(const atari_env *E) {
-  return (size_t)E->rom_stage + 16 + DEC_BYTES + (size_t)E->lanes * E->warps * ENV_SMEM;
+  return shared_part((uint32_t)E->rom_stage) + (size_t)E->lanes * E->warps * ENV_SMEM;
 }
 
 // Envs grouped by cartridge into work items of E envs (ascending env index
@@ -684,6 +682,7 @@ BatchArgs batch_args(atari_env *E, const uint8_t *d_actions, int32_t *d_rewards,
   a.seed = c.seed;
   a.tia_off = c.tia_warps == 3 ? 1 : 0;
   a.idle = c.idle_skip;
+  a.unit = 1;
   return a;
 }
 
@@ -889,10 +888,10 @@ int atari_env_create(const uint8_t *const *roms, const size_t *rom_sizes, const 
     uint32_t max_banks = 1;
     for (int r = 0; r < n_roms; ++r) max_banks = std::max(max_banks, E->h_banks[r]);
     const int stage = (int)max_banks * 4096;
-    const size_t cache_smem = (size_t)stage + 16 + DEC_BYTES + ENV_SMEM;
+    const size_t cache_smem = shared_part((uint32_t)stage) + ENV_SMEM;
     cudaFuncSetAttribute(k_cache_run, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cache_smem);
     k_cache_run<<<n_roms, 128, cache_smem>>>(d_work, d_snaps, E->d_roms, E->d_info, E->d_dec_op, stage,
-                                           c.startup_frames, c.max_noops);
+                                           c.startup_frames, c.max_noops, 1);
     int tot = n_roms * c.n_cache;
     k_cache_pick<<<(tot + 127) / 128, 128>>>(E->d_cache, d_snaps, n_roms, c.n_cache, c.max_noops, c.seed);
     if (n_envs > 0)
@@ -1076,14 +1075,15 @@ int autotune(atari_env *E) {
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  // (envs per warp, CPU warps per block, paired TIA warps)
-  const int cand[][3] = {{32, 4, 0}, {32, 2, 0}, {32, 1, 0}, {16, 4, 0}, {16, 2, 0}, {16, 1, 0}, {8, 4, 0},
-                         {8, 2, 0},  {8, 1, 0},  {4, 4, 0},  {4, 2, 0},  {4, 1, 0},  {2, 4, 0},  {2, 2, 0},
-                         {1, 4, 0},  {32, 4, 1}, {32, 2, 1}, {32, 1, 1}, {16, 4, 1}, {16, 2, 1}, {16, 1, 1},
-                         {8, 4, 1},  {8, 2, 1},  {8, 1, 1}};
+  // (envs per warp, CPU warps per block, paired TIA warps).  A round costs about
+  // 210 cycles with one CPU warp on an SM, 240 with one a scheduler and 370 with
+  // two a scheduler (the integer pipe is then full), so small batches spread
+  // over the SMs and large ones fill them; a block of eight CPU warps stages
+  // its cartridge once for all of them.
+  const int cand[][3] = {{32, 1, 1}, {32, 2, 1}, {32, 4, 1}, {32, 8, 1}, {16, 1, 1}, {8, 1, 1}, {32, 1, 0},
+                         {32, 4, 0}, {16, 1, 0}, {4, 1, 0}};
   // shapes within 3 % of the fastest count as equal; the first of them in
-  // candidate order (the widest warps) is taken, so the choice is stable
-  // from run to run
+  // candidate order is taken, so the choice is stable from run to run
   std::vector<std::pair<float, int>> timed;
   bool was_prof = E->profiling;
   E->profiling = false;
@@ -1091,6 +1091,7 @@ int autotune(atari_env *E) {
     const auto &c = cand[ci];
     if ((size_t)c[0] * c[1] > 4 * n && c[0] * c[1] > 32) continue;  // far more slots than envs
     if ((E->cfg.tia_warps == 1 && c[2]) || (E->cfg.tia_warps >= 2 && !c[2])) continue;
+    if (shared_part((uint32_t)E->rom_stage) + (size_t)c[0] * c[1] * ENV_SMEM > MAX_SMEM) continue;
     if (int rc = build_groups(E, c[0], c[1], c[2] != 0)) { cudaFree(st_bak); return rc; }
     BatchArgs a = batch_args(E, E->d_act, nullptr, nullptr);
     float t = 0;

@@ -41,10 +41,11 @@ struct BatchArgs {
   const int32_t *grp_rom, *grp_start, *grp_count, *perm;
   const int32_t *opos;       // null, or the packed action/output position of each work-list entry
   int *queue;
-  int n_groups, lanes, E, rom_stage;  // rom_stage: bytes staged per block (largest cartridge)
+  int n_groups, lanes, E, rom_stage;  // rom_stage: bytes of the largest cartridge
   int frameskip, sticky, n_cache, log_cap, first_slot;
   int tia_off;               // split form test mode: the TIA side takes no events
   int idle;                  // retire RIOT-timer wait-loop iterations at once
+  int unit;                  // 1
   uint64_t seed;
 };
 
@@ -150,18 +151,21 @@ __device__ __forceinline__ void fast_step_env(FastConsoleT<SPLIT> &m, uint8_t *s
 // TIA side of the split form for env slot i: applies the CPU side's events in
 // order until the end of the step.  Every wait is bounded; running out sets
 // ST_STALL and ends the loop.
-__device__ void tia_worker(IoCtx c, uint32_t q, int i, const BatchArgs &a) {
+__device__ void tia_worker(IoCtx c, uint32_t q, const uint8_t *st, int i, const BatchArgs &a) {
   if (a.tia_off) return;
   const TiaOut out = tia_out_of(a, i);
-  TiaSide s{0, 0, 0, 0};
+  const uint64_t l0 = *reinterpret_cast<const uint64_t *>(st + S::FRAME_LINE);
+  const uint64_t cycles = *reinterpret_cast<const uint64_t *>(st + S::CYCLES);
+  TiaSide s = tia_start(c, l0, (uint32_t)(cycles - 76ull * l0));
   uint64_t idle_since = 0;  // global-timer time the queue was first seen empty (0: not idle)
   for (;;) {
     const uint32_t ev = vsm32(q + 4 * (s.head & (QLEN - 1)));
-    if ((ev ^ lap_bit(s.head)) & 0x80000000u) {
+    if ((ev ^ lap_bit(s.head)) & EV_LAP) {
       const uint64_t now = global_ns();
       if (!idle_since) idle_since = now;
       else if (now - idle_since >= WAIT_NS) {
-        c.Sset(IO_STATUS, c.G(IO_STATUS) | ST_STALL);
+        s.status |= ST_STALL;
+        c.Sset(IO_STATUS, s.status);
         break;
       }
       __nanosleep(128);  // an idle TIA lane polls gently: the CPU warps share the SM's memory pipe
@@ -173,7 +177,11 @@ __device__ void tia_worker(IoCtx c, uint32_t q, int i, const BatchArgs &a) {
     c.V(IO_QHEAD) = s.head;
     const uint32_t r = tia_event(c, ev, s, out);
     if (r) {
-      if ((r & TIA_END) && a.counters) a.counters[3 * i + 1] = s.log_total;
+      c.Sset(IO_CX, s.cx);
+      if (r & TIA_END) {
+        c.Sset(IO_STATUS, s.status);
+        if (a.counters) a.counters[3 * i + 1] = s.log_total;
+      }
       __threadfence_block();
       c.V(IO_ACK) = ++s.ack;
       if (r & TIA_END) break;
@@ -181,14 +189,13 @@ __device__ void tia_worker(IoCtx c, uint32_t q, int i, const BatchArgs &a) {
   }
 }
 
-// Shared memory of a block: the cartridge stage (and 16 bytes of padding),
-// the decoder's bytes and control words, then per env RAM, I/O words, TIA
-// file and event queue.
+// Shared memory of a block: the tables, the cartridge stage, then per env
+// RAM, I/O words, TIA file and event queue.
+__host__ __device__ inline uint32_t shared_part(uint32_t rom_stage) { return OFF_ROM + 4 * rom_stage; }
 __device__ __forceinline__ EnvOff env_off(uint32_t rom_stage, uint32_t envs, uint32_t j) {
   EnvOff o;
-  o.rom = 0;
-  o.dec = rom_stage + 16;
-  const uint32_t ram = o.dec + DEC_BYTES;
+  o.rom = OFF_ROM;
+  const uint32_t ram = shared_part(rom_stage);
   const uint32_t io = ram + RAM_BYTES * envs, tia = io + 4 * IO_STRIDE * envs, q = tia + TIA_STRIDE * envs;
   o.ram = ram + RAM_BYTES * j;
   o.io = io + 4 * IO_STRIDE * j;
@@ -196,7 +203,14 @@ __device__ __forceinline__ EnvOff env_off(uint32_t rom_stage, uint32_t envs, uin
   o.q = q + 4 * QSTRIDE * j;
   return o;
 }
-
+// Stage a cartridge (banks of 4096 bytes at src, 4-byte aligned) and its
+// region table with the whole block.
+__device__ __forceinline__ void stage_cartridge(const uint8_t *src, uint32_t banks, uint32_t scheme) {
+  const uint32_t limit = scheme_fetch_limit(scheme);
+  for (uint32_t g = threadIdx.x; g < banks * 1024u; g += blockDim.x)
+    reinterpret_cast<uint4 *>(g_smem + OFF_ROM)[g] = stage_words(src + (g >> 10) * 4096u, 4u * (g & 1023u), limit);
+  for (uint32_t p = threadIdx.x; p < REGION_BYTES; p += blockDim.x) sm8(OFF_REG + p) = (uint8_t)region_byte(p, scheme);
+}
 // blockDim = W warps (single-warp form) or 2 W (split form); warps [0, W) run
 // the CPUs of the work item's envs, in the split form warp W + w the TIA side
 // of CPU warp w's envs (lane for lane).
@@ -204,7 +218,7 @@ template <bool SPLIT>
 __device__ __forceinline__ void interp_block(const BatchArgs &a) {
   __shared__ int s_group;
   for (uint32_t t = threadIdx.x; t < DEC_BYTES / 4; t += blockDim.x)
-    sm32((uint32_t)a.rom_stage + 16 + 4 * t) = reinterpret_cast<const uint32_t *>(a.dec_op)[t];
+    sm32(OFF_DEC + 4 * t) = reinterpret_cast<const uint32_t *>(a.dec_op)[t];
   int cur_rom = -1;
   const int W = a.E / a.lanes;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -219,11 +233,7 @@ __device__ __forceinline__ void interp_block(const BatchArgs &a) {
     const int rom = a.grp_rom[g];
     const uint32_t inf = a.info[rom];
     if (rom != cur_rom) {
-      const uint32_t banks = inf >> 24;
-      const uint4 *src = reinterpret_cast<const uint4 *>(a.romb + (size_t)rom * ROMB_SLOT);
-      uint4 *dst = reinterpret_cast<uint4 *>(g_smem);
-      for (uint32_t q = threadIdx.x; q < banks * 256u; q += blockDim.x) dst[q] = src[q];
-      if (threadIdx.x == 0) dst[banks * 256u] = make_uint4(0, 0, 0, 0);
+      stage_cartridge(a.romb + (size_t)rom * ROMB_SLOT, inf >> 24, inf & 0xFF);
       cur_rom = rom;
     }
     const int jj = cw * a.lanes + lane;
@@ -240,18 +250,19 @@ __device__ __forceinline__ void interp_block(const BatchArgs &a) {
       m.scheme = inf & 0xFF;
       m.wmask = wmask;
       m.idle = (uint32_t)a.idle;
+      m.unit = (uint32_t)a.unit;
       m.to = tia_out_of(a, i);
       m.load(st);
     }
     __syncthreads();  // the cartridge and the envs' state are in shared memory
     if (runs) {
       if (cpu) fast_step_env<SPLIT>(m, st, i, o, a, (uint32_t)rom, (inf >> 8) & 0x7F, (inf >> 16) & 0x7F);
-      else tia_worker(IoCtx{off.tia, off.io}, off.q, i, a);
+      else tia_worker(IoCtx{off.tia, off.io}, off.q, st, i, a);
     }
   }
 }
-__global__ void __launch_bounds__(128) k_interp_batched(const __grid_constant__ BatchArgs a) { interp_block<false>(a); }
-__global__ void __launch_bounds__(256, 2) k_interp_split(const __grid_constant__ BatchArgs a) { interp_block<true>(a); }
+__global__ void __launch_bounds__(256, 2) k_interp_batched(const __grid_constant__ BatchArgs a) { interp_block<false>(a); }
+__global__ void __launch_bounds__(512, 1) k_interp_split(const __grid_constant__ BatchArgs a) { interp_block<true>(a); }
 
 // Bank-aware grouping: within each cartridge's run [seg[r], seg[r+1]) of the
 // env list, envs are ordered by the bank their canonical state holds at the

@@ -5,13 +5,12 @@
 //     steered by control words per opcode (opcode_ctl.h);
 //   - CPU registers, flags, the cycle counter and the bank in registers;
 //   - RAM (bytes), the TIA register file (bytes) and the I/O state
-//     (collision cursor and latches, RIOT timer and ports, inputs, log
-//     cursor, frame base line) in shared memory, one block per env with odd
+//     (collision latches, RIOT timer and ports, inputs) in shared memory, one block per env with odd
 //     word strides, so lanes reading the same field never bank-conflict and
 //     every access is a base offset plus a constant or one add;
-//   - the block's cartridge staged in shared memory as bytes (16 KB for an
-//     F6 cartridge); an instruction's bytes are fetched as two aligned words
-//     joined by one funnel shift.
+//   - the block's cartridge staged in shared memory as one word per byte (64 KB
+//     for an F6 cartridge), the byte and the two after it: an instruction is
+//     one load, and a data byte the first byte of its word.
 // Instructions the hot loop does not take (TIA and RIOT reads, RIOT, VSYNC
 // and VBLANK writes, stack and pointer instructions, undocumented opcodes,
 // decimal arithmetic, fetches outside the cartridge or next to a bank
@@ -32,11 +31,9 @@ enum TiaSlot : uint32_t {
 };
 // I/O state words (shared memory, interleaved by env)
 enum IoWord : uint32_t {
-  IO_CEVAL = 0, IO_CX, IO_L0LO, IO_L0HI, IO_BARLO, IO_BARHI, IO_TCWLO, IO_TCWHI, IO_TV, IO_TSH, IO_PORTS,
-  IO_JOY, IO_FIRE, IO_LATCH, IO_LOGLO, IO_LOGHI, IO_LOGN, IO_LOGCAP, IO_STATUS,
-  IO_BANDN,      // next band whose start snapshot is due, BANDS: none
-  IO_BSLO, IO_BSHI,  // where this frame's band snapshots go
-  IO_QHEAD, IO_QTAIL, IO_ACK,  // split form: the TIA side's queue cursor and acknowledgements
+  IO_CX = 0, IO_BARLO, IO_BARHI, IO_TCWLO, IO_TCWHI, IO_TV, IO_TSH, IO_PORTS, IO_JOY, IO_FIRE, IO_LATCH, IO_STATUS,
+  IO_QHEAD, IO_ACK,  // split form: the TIA side's queue cursor and acknowledgements
+  IO_PAD,            // an odd stride
   IO_WORDS
 };
 constexpr uint32_t IO_WSYNC = 1u;
@@ -81,70 +78,111 @@ struct IoCtx {
   }
 };
 
-// ---------------------------------------------------------------- collisions (cold)
-__device__ __noinline__ uint32_t fc_collide_cols(IoCtx c, uint32_t live, uint32_t lo, uint32_t hi) {
-  M160 r{range_word(0, lo, hi), range_word(1, lo, hi), range_word(2, lo, hi), range_word(3, lo, hi),
-         range_word(4, lo, hi)};
-  M160 z{0, 0, 0, 0, 0};
-  const uint32_t nus0 = c.T(T_NUSIZ0), nus1 = c.T(T_NUSIZ1), ctrl = c.T(T_CTRLPF);
-  M160 p0 = (live & 1) ? player_mask((c.T(T_VDELP0) & 1) ? c.T(T_GRP0_O) : c.T(T_GRP0_N), c.T(T_REFP0), nus0,
-                                     c.T(T_P0))
-                       : z;
-  M160 p1 = (live & 2) ? player_mask((c.T(T_VDELP1) & 1) ? c.T(T_GRP1_O) : c.T(T_GRP1_N), c.T(T_REFP1), nus1,
-                                     c.T(T_P1))
-                       : z;
-  M160 m0 = (live & 4) ? missile_mask(nus0, c.T(T_M0)) : z;
-  M160 m1 = (live & 8) ? missile_mask(nus1, c.T(T_M1)) : z;
-  M160 b = (live & 16) ? ball_mask(ctrl, c.T(T_BL)) : z;
-  M160 f = (live & 32) ? pf_mask(c.T(T_PF0), c.T(T_PF1), c.T(T_PF2), ctrl) : z;
-  uint32_t x = 0;
-  x |= (uint32_t)meet(m0, p1, r) << 1 | (uint32_t)meet(m0, p0, r) << 0;
-  x |= (uint32_t)meet(m1, p0, r) << 3 | (uint32_t)meet(m1, p1, r) << 2;
-  x |= (uint32_t)meet(p0, f, r) << 5 | (uint32_t)meet(p0, b, r) << 4;
-  x |= (uint32_t)meet(p1, f, r) << 7 | (uint32_t)meet(p1, b, r) << 6;
-  x |= (uint32_t)meet(m0, f, r) << 9 | (uint32_t)meet(m0, b, r) << 8;
-  x |= (uint32_t)meet(m1, f, r) << 11 | (uint32_t)meet(m1, b, r) << 10;
-  x |= (uint32_t)meet(b, f, r) << 13;
-  x |= (uint32_t)meet(p0, p1, r) << 15 | (uint32_t)meet(m0, m1, r) << 14;
-  return x;
+// ---------------------------------------------------------------- collisions
+// Where the TIA side of one env leaves its logs and snapshots.
+struct TiaOut {
+  uint32_t *log;      // two logs of log_cap records
+  uint8_t *bsnap;     // the band snapshots of frames F-1 and F (frame F-1's place is not used when it is not logged)
+  uint32_t *meta;     // two times (records, lines)
+  uint32_t log_cap;
+};
+// The TIA side's cursors, in registers while events are applied.
+struct TiaSide {
+  uint32_t head, ack, lines, log_total;
+  uint32_t ceval;     // collisions are accounted for every color clock before it (frame-relative)
+  uint32_t cx;        // collision latches
+  uint32_t bar;       // frame-relative line of the HMOVE bar, ~0: none in this frame or later
+  uint64_t l0;        // first line of the frame
+  uint32_t *log;      // next record of the logged frame, null: not logged
+  uint32_t nrec;      // records so far
+  uint8_t *bands;     // the frame's band snapshots
+  uint32_t band, band_clk;  // next band whose start snapshot is due, and its first color clock
+  uint32_t status;
+};
+constexpr uint32_t NO_BAR = ~0u;
+
+// The n lowest bits of a word (all of them from 32 on).
+__device__ __forceinline__ uint32_t low_bits(uint32_t n) {
+  uint32_t m;
+  asm("bmsk.clamp.b32 %0, 0, %1;" : "=r"(m) : "r"(n));
+  return m;
+}
+// Bits below n of word w of a 160-bit mask.
+__device__ __forceinline__ uint32_t below(uint32_t n, int w) {
+  const int k = (int)n - 32 * w;
+  return low_bits((uint32_t)(k < 0 ? 0 : k));
 }
 
-__device__ __forceinline__ uint32_t fc_live(IoCtx c) {
-  const uint32_t g0 = (c.T(T_VDELP0) & 1) ? c.T(T_GRP0_O) : c.T(T_GRP0_N);
-  const uint32_t g1 = (c.T(T_VDELP1) & 1) ? c.T(T_GRP1_O) : c.T(T_GRP1_N);
-  const uint32_t eb = (c.T(T_VDELBL) & 1) ? c.T(T_ENABL_O) : c.T(T_ENABL_N);
-  return (g0 ? 1u : 0u) | (g1 ? 2u : 0u) | (((c.T(T_ENAM0) & 2) && !(c.T(T_RESMP0) & 2)) ? 4u : 0u) |
-         (((c.T(T_ENAM1) & 2) && !(c.T(T_RESMP1) & 2)) ? 8u : 0u) | ((eb & 2) ? 16u : 0u) |
-         (((c.T(T_PF0) & 0xF0) | c.T(T_PF1) | c.T(T_PF2)) ? 32u : 0u);
+// Latch bits of each object (P0, P1, M0, M1, BL, PF): a pair's bit is in both its objects' sets.
+constexpr uint32_t CXP_P0 = 0x8039u, CXP_P1 = 0x80C6u, CXP_M0 = 0x4303u, CXP_M1 = 0x4C0Cu, CXP_BL = 0x2550u,
+                   CXP_PF = 0x2AA0u, CXP_ALL = 0xEFFFu;
+
+// Collisions from (line la, clock xa) to (line lb, clock xb) under the current
+// registers: the latch bits that are not in `cx` yet.  The registers do not
+// change in between, so the visible columns of all the lines it covers count
+// together: one evaluation whatever the number of lines.
+__device__ __noinline__ uint32_t fc_collide(IoCtx c, uint32_t la, uint32_t xa, uint32_t lb, uint32_t xb, uint32_t bar,
+                                            uint32_t cx) {
+  const uint32_t w0 = sm32(c.tia), w2 = sm32(c.tia + 8), w3 = sm32(c.tia + 12), w4 = sm32(c.tia + 16),
+                 w5 = sm32(c.tia + 20), w6 = sm32(c.tia + 24), w8 = sm32(c.tia + 32);
+  // the registers as bytes of the file's words (TiaSlot order)
+  const uint32_t g0 = (w5 & 0x10000u) ? w4 >> 24 : (w4 >> 16) & 0xFFu;         // VDELP0: GRP0 old or new
+  const uint32_t g1 = (w5 & 0x1000000u) ? (w5 >> 8) & 0xFFu : w5 & 0xFFu;      // VDELP1
+  const uint32_t bl = (w6 & 1u) ? w4 >> 8 : w4;                                // VDELBL
+  uint32_t off = g0 ? 0u : CXP_P0;
+  off |= g1 ? 0u : CXP_P1;
+  off |= (w3 & 0x20000u) && !(w6 & 0x200u) ? 0u : CXP_M0;                      // ENAM0, RESMP0
+  off |= (w3 & 0x2000000u) && !(w6 & 0x20000u) ? 0u : CXP_M1;
+  off |= (bl & 2u) ? 0u : CXP_BL;
+  off |= ((w2 & 0xF0000000u) | (w3 & 0xFFFFu)) ? 0u : CXP_PF;
+  const uint32_t need = CXP_ALL & ~off & ~cx;
+  if (need == 0) return 0;
+  // visible columns: [a, 160) of line la, whole lines, [b0, b) of line lb; one line: [a, b)
+  const bool one = la == lb;
+  uint32_t a = xa > 68u ? xa - 68u : 0u;
+  if (la == bar && a < 8u) a = 8u;
+  const uint32_t b = xb > 68u ? xb - 68u : 0u;
+  const uint32_t mid = lb > la + 1u && !one ? ~0u : 0u;
+  M160 r;
+  uint32_t *rw = &r.w0;
+  const uint32_t bar8 = lb == bar ? ~0xFFu : ~0u;                              // line lb under the bar
+  const uint32_t mid8 = la + 1u == bar && lb == la + 2u ? ~0xFFu : ~0u;        // the only whole line under it
+#pragma unroll
+  for (int w = 0; w < 5; ++w) {
+    const uint32_t ge = ~below(a, w);
+    uint32_t lt = below(b, w), md = mid;
+    if (w == 0) { md &= mid8; lt &= one ? ~0u : bar8; }
+    rw[w] = one ? ge & lt : ge | md | lt;
+  }
+  const M160 z{0, 0, 0, 0, 0};
+  auto clip = [&](M160 m) { return M160{m.w0 & r.w0, m.w1 & r.w1, m.w2 & r.w2, m.w3 & r.w3, m.w4 & r.w4}; };
+  const uint32_t nus0 = w0 >> 16, nus1 = w0 >> 24, ctrl = w2;
+  const M160 p0 = (need & CXP_P0) ? clip(player_mask(g0, w2 >> 8, nus0, w8 & 0xFFu)) : z;
+  const M160 p1 = (need & CXP_P1) ? clip(player_mask(g1, w2 >> 16, nus1, (w8 >> 8) & 0xFFu)) : z;
+  const M160 m0 = (need & CXP_M0) ? clip(missile_mask(nus0, (w8 >> 16) & 0xFFu)) : z;
+  const M160 m1 = (need & CXP_M1) ? clip(missile_mask(nus1, w8 >> 24)) : z;
+  const M160 bm = (need & CXP_BL) ? clip(ball_mask(ctrl, sm8(c.tia + T_BL))) : z;
+  const M160 f = (need & CXP_PF) ? pf_mask(w2 >> 24, w3 & 0xFFu, (w3 >> 8) & 0xFFu, ctrl) : z;
+  auto pair = [](const M160 &u, const M160 &v, uint32_t bit) {
+    return ((u.w0 & v.w0) | (u.w1 & v.w1) | (u.w2 & v.w2) | (u.w3 & v.w3) | (u.w4 & v.w4)) ? 1u << bit : 0u;
+  };
+  uint32_t x = pair(m0, p0, 0) | pair(m0, p1, 1) | pair(m1, p1, 2) | pair(m1, p0, 3) | pair(p0, p1, 15) |
+               pair(m0, m1, 14);
+  x |= pair(p0, bm, 4) | pair(p1, bm, 6) | pair(m0, bm, 8) | pair(m1, bm, 10);
+  x |= pair(p0, f, 5) | pair(p1, f, 7) | pair(m0, f, 9) | pair(m1, f, 11) | pair(bm, f, 13);
+  return x & need;
 }
 
-// Account collisions for every color clock in [ceval, upto) (frame-relative).
-__device__ __forceinline__ void fc_cx_eval(IoCtx c, uint32_t upto) {
-  const uint32_t from = c.G(IO_CEVAL);
+// Account collisions for every color clock before `upto` (frame-relative).
+__device__ __forceinline__ void fc_cx_eval(IoCtx c, TiaSide &s, uint32_t upto) {
+  const uint32_t from = s.ceval;
   if (upto <= from) return;
-  c.Sset(IO_CEVAL, upto);
+  s.ceval = upto;
   if (c.T(T_VBLANK) & 2) return;
   const uint32_t la = from / 228u, xa = from - la * 228u;
   const uint32_t lb = upto / 228u, xb = upto - lb * 228u;
   if (la == lb && xb <= 68) return;  // the span lies in one line's horizontal blank
-  const uint32_t live = fc_live(c);
-  if (__popc(live) < 2) return;
-  const uint64_t L0 = c.G64(IO_L0LO), bar = c.G64(IO_BARLO);
-  uint32_t x = 0;
-  auto seg = [&](uint32_t line, uint32_t x0, uint32_t x1) {
-    if (x1 <= 68) return;
-    uint32_t lo = x0 > 68 ? x0 - 68 : 0, hi = x1 - 68;
-    if (L0 + line == bar && lo < 8) lo = 8;
-    if (lo < hi) x |= fc_collide_cols(c, live, lo, hi);
-  };
-  if (la == lb) {
-    seg(la, xa, xb);
-  } else {
-    seg(la, xa, 228);
-    if (lb > la + 1) seg(la + 1, 0, 228);
-    if (xb) seg(lb, 0, xb);
-  }
-  c.Sset(IO_CX, c.G(IO_CX) | x);
+  s.cx |= fc_collide(c, la, xa, lb, xb, s.bar, s.cx);
 }
 
 // ---------------------------------------------------------------- I/O (cold)
@@ -197,51 +235,35 @@ __device__ __forceinline__ uint32_t fc_band_clk(uint32_t q) { return 228u * (WIN
 // state after all records of earlier clocks.  Words 0..8: the TIA file's first
 // 36 bytes; word 9: its last byte and, in the high half, the frame-relative
 // line of the HMOVE bar or 0xFFFF; word 10: the log records before it.
-__device__ __noinline__ void fc_band_snap(IoCtx c, uint32_t eff) {
-  uint32_t bn = c.G(IO_BANDN);
-  uint8_t *base = reinterpret_cast<uint8_t *>((uint64_t)c.G(IO_BSLO) | (uint64_t)c.G(IO_BSHI) << 32);
-  const uint64_t bar = c.G64(IO_BARLO), l0 = c.G64(IO_L0LO);
-  const uint32_t rel = bar != NO_LINE && bar >= l0 && bar - l0 < 1024 ? (uint32_t)(bar - l0) : 0xFFFFu;
-  const uint32_t nrec = c.G(IO_LOGN);
+__device__ __noinline__ uint32_t fc_band_snap(IoCtx c, uint8_t *bands, uint32_t band, uint32_t bar, uint32_t nrec,
+                                              uint32_t eff) {
   uint32_t v[10];
 #pragma unroll
   for (int q = 0; q < 10; ++q) v[q] = sm32(c.tia + 4 * q);
-  v[9] = (v[9] & 0xFFu) | rel << 16;
-  uint4 *d = reinterpret_cast<uint4 *>(base) + 3 * bn;
-  while (bn < BANDS && eff >= fc_band_clk(bn)) {
+  v[9] = (v[9] & 0xFFu) | (bar < 1024u ? bar : 0xFFFFu) << 16;
+  uint4 *d = reinterpret_cast<uint4 *>(bands) + 3 * band;
+  while (band < BANDS && eff >= fc_band_clk(band)) {
     d[0] = make_uint4(v[0], v[1], v[2], v[3]);
     d[1] = make_uint4(v[4], v[5], v[6], v[7]);
     d[2] = make_uint4(v[8], v[9], nrec, 0);
     d += 3;
-    ++bn;
+    ++band;
   }
-  c.Sset(IO_BANDN, bn);
+  return band;
 }
-
-// Log the frame's TIA writes to p (cap records; p null: no log) and the band
-// starts to bands.
-__device__ __forceinline__ void fc_set_log(IoCtx c, uint32_t *p, uint32_t cap, uint8_t *bands) {
-  c.Sset(IO_LOGLO, (uint32_t)(uint64_t)p);
-  c.Sset(IO_LOGHI, (uint32_t)((uint64_t)p >> 32));
-  c.Sset(IO_LOGN, 0);
-  c.Sset(IO_LOGCAP, cap);
-  c.Sset(IO_BANDN, bands ? 0u : BANDS);
-  c.Sset(IO_BSLO, (uint32_t)(uint64_t)bands);
-  c.Sset(IO_BSHI, (uint32_t)((uint64_t)bands >> 32));
+__device__ __forceinline__ void fc_bands_due(IoCtx c, TiaSide &s, uint32_t eff) {
+  s.band = fc_band_snap(c, s.bands, s.band, s.bar, s.nrec, eff);
+  s.band_clk = s.band < BANDS ? fc_band_clk(s.band) : ~0u;
 }
 
 // Append one TIA write record (effect clock, register, value) to the log of
 // a rendered frame.
-__device__ __forceinline__ void fc_log(IoCtx c, uint32_t eff, uint32_t reg, uint32_t v) {
-  const uint32_t lo = c.G(IO_LOGLO), hi = c.G(IO_LOGHI);
-  if (lo | hi) {
-    if (c.G(IO_BANDN) < BANDS && eff >= fc_band_clk(c.G(IO_BANDN))) fc_band_snap(c, eff);
-    uint32_t *lp = reinterpret_cast<uint32_t *>((uint64_t)lo | (uint64_t)hi << 32);
-    const uint32_t nrec = c.G(IO_LOGN);
-    if (nrec < c.G(IO_LOGCAP)) lp[nrec] = eff << 14 | reg << 8 | v;
-    else c.Sset(IO_STATUS, c.G(IO_STATUS) | ST_LOG_OVERFLOW);
-    c.Sset(IO_LOGN, nrec + 1);
-  }
+__device__ __forceinline__ void fc_log(IoCtx c, TiaSide &s, uint32_t cap, uint32_t eff, uint32_t reg, uint32_t v) {
+  if (!s.log) return;
+  if (eff >= s.band_clk) fc_bands_due(c, s, eff);
+  if (s.nrec < cap) s.log[s.nrec] = eff << 14 | reg << 8 | v;
+  else s.status |= ST_LOG_OVERFLOW;
+  ++s.nrec;
 }
 
 // Write a RIOT address at absolute CPU cycle `now`.
@@ -258,10 +280,10 @@ __device__ __forceinline__ void fc_riot_write(IoCtx c, uint32_t a, uint32_t v, u
 }
 // Apply a TIA write (register reg at cycle t): collisions up to the write,
 // log record, register update.
-__device__ __forceinline__ void fc_tia_write(IoCtx c, uint32_t reg, uint32_t v, uint32_t t) {
+__device__ __forceinline__ void fc_tia_write(IoCtx c, TiaSide &s, uint32_t cap, uint32_t reg, uint32_t v, uint32_t t) {
   const uint32_t eff = 3u * (t + 1u);
-  if ((COLL_REGS >> reg) & 1ull) fc_cx_eval(c, eff);
-  if ((LOG_REGS >> reg) & 1ull) fc_log(c, eff, reg, v);
+  if ((COLL_REGS >> reg) & 1ull) fc_cx_eval(c, s, eff);
+  if ((LOG_REGS >> reg) & 1ull) fc_log(c, s, cap, eff, reg, v);
   switch (reg) {
     case 0x00: c.Tset(T_VSYNC, v); break;
     case 0x01: c.Tset(T_VBLANK, v); break;
@@ -295,14 +317,17 @@ __device__ __forceinline__ void fc_tia_write(IoCtx c, uint32_t reg, uint32_t v, 
     }
     case 0x2A:
       for (uint32_t o = 0; o < 5; ++o) c.Tset(T_P0 + o, fc_hm_move(c.T(T_P0 + o), c.T(T_HMP0 + o)));
-      if (eff % 228u < 68u) c.S64(IO_BARLO, c.G64(IO_L0LO) + eff / 228u);
+      if (eff % 228u < 68u) {
+        s.bar = eff / 228u;
+        c.S64(IO_BARLO, s.l0 + s.bar);
+      }
       break;
     case 0x2B:
       for (uint32_t o = 0; o < 5; ++o) c.Tset(T_HMP0 + o, 0);
       break;
     case 0x2C:
-      if (eff > c.G(IO_CEVAL)) c.Sset(IO_CEVAL, eff);
-      c.Sset(IO_CX, 0);
+      if (eff > s.ceval) s.ceval = eff;
+      s.cx = 0;
       break;
     default: break;  // RSYNC, audio, unused addresses
   }
@@ -317,20 +342,22 @@ __device__ __forceinline__ void fc_tia_write(IoCtx c, uint32_t reg, uint32_t v, 
 // the fire latch and the frame base line; it waits for the TIA side only when
 // it reads a collision register and at the end of the step.
 // An event is one 32-bit word, written and read whole, so the word itself
-// tells that it is there: bit 31 holds the parity of the queue's lap (1 in
+// tells that it is there: bit 15 holds the parity of the queue's lap (1 in
 // the first lap over the zeroed queue), and no fence orders data behind a
-// cursor.  Bits 0-30:
-//   write       0 | cycle:16 | register:6 | value:8
-//   control     1 | kind:2 | argument:
-//     mark      begin / end of a logged frame, end of the step
-//     sync      evaluate collisions up to a cycle and acknowledge
+// cursor.  Bits 16-31 are a CPU cycle of the frame:
+//   write       bit 14 = 0 | register << 8 | value; the cycle after the write's
+//   control     bit 14 = 1 | kind << 8 | argument:
+//     begin / end of a logged frame (argument: 0 frame F-1, 1 frame F), end of the step
+//     sync      evaluate collisions up to the cycle and acknowledge
 //     frame end evaluate collisions up to the frame's last cycle
-//     rebase    lines to the next frame's first line (follows the frame end)
-constexpr uint32_t EV_CTRL = 1u << 30, EV_MARK = EV_CTRL, EV_SYNC = EV_CTRL | 1u << 28,
-                   EV_FRAME_END = EV_CTRL | 2u << 28, EV_REBASE = EV_CTRL | 3u << 28;
-constexpr uint32_t EV_BEGIN_LOG = EV_MARK, EV_END_LOG = EV_MARK | 1u << 26, EV_STEP_END = EV_MARK | 2u << 26;
-// Lap parity of queue position k, in bit 31.
-__device__ __forceinline__ uint32_t lap_bit(uint32_t k) { return (~k << 26) & 0x80000000u; }
+//     rebase    lines towards the next frame's first line (follow the frame
+//               end; bits 16-31 and, above them, the argument)
+constexpr uint32_t EV_CTRL = 1u << 14, EV_BEGIN_LOG = EV_CTRL, EV_END_LOG = EV_CTRL | 1u << 8,
+                   EV_STEP_END = EV_CTRL | 2u << 8, EV_SYNC = EV_CTRL | 3u << 8, EV_FRAME_END = EV_CTRL | 4u << 8,
+                   EV_REBASE = EV_CTRL | 5u << 8;
+// Lap parity of queue position k.
+constexpr uint32_t EV_LAP = 1u << 15;
+__device__ __forceinline__ uint32_t lap_bit(uint32_t k) { return (~k << 10) & EV_LAP; }
 // A wait between an env's CPU and TIA warps gives up after WAIT_NS of the
 // GPU's global timer and the env is declared stalled.  The longest legitimate
 // wait is about one frame of the slowest lane of the partner warp (a few
@@ -342,62 +369,68 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
-// Where the TIA side of one env leaves its logs and snapshots.
-struct TiaOut {
-  uint32_t *log;      // two logs of log_cap records
-  uint8_t *bsnap;     // the band snapshots of frames F-1 and F (frame F-1's place is not used when it is not logged)
-  uint32_t *meta;     // two times (records, lines)
-  uint32_t log_cap;
-};
-struct TiaSide {
-  uint32_t head, ack, lines, log_total;
-};
 constexpr uint32_t TIA_ACK = 1u, TIA_END = 2u;
 // Apply one event; returns TIA_ACK when the CPU side waits for it, and
 // TIA_END when it ends the step.
 __device__ __forceinline__ uint32_t tia_event(IoCtx c, uint32_t ev, TiaSide &s, const TiaOut &o) {
   if (!(ev & EV_CTRL)) {
-    fc_tia_write(c, (ev >> 8) & 0x3F, ev & 0xFF, (ev >> 14) & 0xFFFF);
+    fc_tia_write(c, s, o.log_cap, (ev >> 8) & 0x3F, ev & 0xFF, ((ev >> 16) - 1u) & 0xFFFFu);
     return 0;
   }
-  const uint32_t kind = (ev >> 28) & 3;
-  if (kind == 1) {
-    fc_cx_eval(c, 3u * (ev & 0xFFFFu));
-    return TIA_ACK;
+  const uint32_t kind = (ev >> 8) & 0x3F, slot = ev & 1, cycle = ev >> 16;
+  switch (kind) {
+    case 3: fc_cx_eval(c, s, 3u * cycle); return TIA_ACK;
+    case 4:
+      fc_cx_eval(c, s, 3u * cycle);
+      s.lines = 0;
+      return 0;
+    case 5: {
+      const uint32_t n = cycle | (ev & 0xFFu) << 16;
+      s.lines += n;
+      s.l0 += n;
+      s.ceval -= 228u * n;
+      s.bar = s.bar != NO_BAR && s.bar >= n ? s.bar - n : NO_BAR;
+      return 0;
+    }
+    case 0:
+      s.log = o.log + (size_t)slot * o.log_cap;
+      s.nrec = 0;
+      s.bands = o.bsnap + (size_t)slot * BANDS * BAND_SNAP;
+      s.band = 0;
+      s.band_clk = fc_band_clk(0);
+      return 0;
+    case 1:
+      if (s.band < BANDS) fc_bands_due(c, s, ~0u);  // band starts that the frame never reached take its last state
+      o.meta[2 * slot] = s.nrec;
+      o.meta[2 * slot + 1] = s.lines;
+      s.log_total += s.nrec;
+      s.log = nullptr;
+      return 0;
+    default: return TIA_ACK | TIA_END;
   }
-  if (kind == 2) {
-    fc_cx_eval(c, 3u * (ev & 0xFFFFu));
-    return 0;
-  }
-  if (kind == 3) {
-    s.lines = ev & 0xFFFFFFFu;
-    c.S64(IO_L0LO, c.G64(IO_L0LO) + s.lines);
-    c.Sset(IO_CEVAL, c.G(IO_CEVAL) - 228u * s.lines);
-    return 0;
-  }
-  const uint32_t sub = (ev >> 26) & 3, slot = ev & 1;
-  if (sub == 0) {
-    fc_set_log(c, o.log + (size_t)slot * o.log_cap, o.log_cap, o.bsnap + (size_t)slot * BANDS * BAND_SNAP);
-    return 0;
-  }
-  if (sub == 1) {
-    if (c.G(IO_BANDN) < BANDS) fc_band_snap(c, ~0u);  // band starts that the frame never reached take its last state
-    const uint32_t nrec = c.G(IO_LOGN);
-    o.meta[2 * slot] = nrec;
-    o.meta[2 * slot + 1] = s.lines;
-    s.log_total += nrec;
-    fc_set_log(c, nullptr, 0, nullptr);
-    return 0;
-  }
-  return TIA_ACK | TIA_END;
+}
+// The TIA side at the start of a step: the latches, the HMOVE bar and the
+// frame's first line l0 as loaded, collisions accounted up to CPU cycle kf.
+__device__ __forceinline__ TiaSide tia_start(IoCtx c, uint64_t l0, uint32_t kf) {
+  const uint64_t bar = c.G64(IO_BARLO);
+  TiaSide s{};
+  s.ceval = 3u * kf;
+  s.cx = c.G(IO_CX);
+  s.bar = bar != NO_LINE && bar >= l0 && bar - l0 < (1u << 30) ? (uint32_t)(bar - l0) : NO_BAR;
+  s.l0 = l0;
+  return s;
 }
 // Single-warp form: apply an env's queued events [s.head, tail).
-__device__ __noinline__ void tia_drain(IoCtx c, uint32_t q, TiaSide &s, const TiaOut &o, uint32_t tail) {
+__device__ __noinline__ void tia_drain(IoCtx c, uint32_t q, TiaSide &side, const TiaOut &out, uint32_t tail) {
+  TiaSide s = side;
+  const TiaOut o = out;
   while (s.head != tail) {
     const uint32_t ev = sm32(q + 4 * (s.head & (QLEN - 1)));
     ++s.head;
     tia_event(c, ev, s, o);
   }
+  c.Sset(IO_CX, s.cx);
+  side = s;
 }
 
 // ---------------------------------------------------------------- the console
@@ -435,21 +468,25 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
   asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
   return r;
 }
-// Predicated stores (addresses in the shared window), without a branch.
-__device__ __forceinline__ void sts8_if(bool c, uint32_t a, uint32_t v) {
-  asm volatile("{.reg .pred p; setp.ne.u32 p, %0, 0; @p st.shared.u8 [%1], %2;}" ::"r"((uint32_t)c), "r"(a), "r"(v)
-               : "memory");
-}
-__device__ __forceinline__ void sts32_if(bool c, uint32_t a, uint32_t v) {
-  asm volatile("{.reg .pred p; setp.ne.u32 p, %0, 0; @p st.volatile.shared.u32 [%1], %2;}" ::"r"((uint32_t)c), "r"(a),
-               "r"(v)
-               : "memory");
+// a * b + c on the FMA pipe.  The interpreter's loop is bound by the integer
+// ALU (two cycles a warp instruction), and adds, shifts left and address
+// arithmetic would all go there; with a multiplier that is not a known
+// constant they run beside it.
+__device__ __forceinline__ uint32_t mad(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t r;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
 }
 // Loads of the staged cartridge and the control words, which do not change
 // while a work item runs: free to move past the stores of other lanes.
 __device__ __forceinline__ uint32_t lds_const(uint32_t a) {
   uint32_t v;
   asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds8_const(uint32_t a) {
+  uint32_t v;
+  asm("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
   return v;
 }
 __device__ __forceinline__ uint4 lds_const4(uint32_t a) {
@@ -460,8 +497,30 @@ __device__ __forceinline__ uint4 lds_const4(uint32_t a) {
 
 // Byte offsets of an env's blocks in the block's dynamic shared memory.
 struct EnvOff {
-  uint32_t rom, dec, ram, io, tia, q;
+  uint32_t rom, ram, io, tia, q;
 };
+// The block's tables come first, at fixed offsets: region table, general
+// decoder's bytes, control words.  The cartridge follows, then the envs.
+constexpr uint32_t OFF_REG = 0, OFF_DEC = OFF_REG + REGION_BYTES, OFF_CTL = OFF_DEC + 512, OFF_ROM = OFF_DEC + DEC_BYTES;
+__device__ __forceinline__ uint32_t scheme_fetch_limit(uint32_t scheme) {
+  return scheme == 3 ? 0xFF1u : scheme ? 0xFF3u : 0xFFCu;
+}
+// The cartridge is staged as one word per byte: the byte and the two after it
+// (an instruction in one load), and in the top byte 0x80 where no instruction
+// is fetched from the stage.  Words i .. i+3 of a bank of 4096 bytes at src
+// (4-byte aligned), i a multiple of 4.
+constexpr uint32_t REC_BAD = 0x80000000u;
+__device__ __forceinline__ uint4 stage_words(const uint8_t *src, uint32_t i, uint32_t limit) {
+  const uint32_t *b = reinterpret_cast<const uint32_t *>(src + i);
+  const uint32_t lo = b[0], hi = i + 4u < 4096u ? b[1] : 0u, m = 0xFFFFFFu;
+  uint4 r = make_uint4(lo & m, __funnelshift_r(lo, hi, 8) & m, __funnelshift_r(lo, hi, 16) & m,
+                       __funnelshift_r(lo, hi, 24) & m);
+  r.x |= i > limit ? REC_BAD : 0u;
+  r.y |= i + 1u > limit ? REC_BAD : 0u;
+  r.z |= i + 2u > limit ? REC_BAD : 0u;
+  r.w |= i + 3u > limit ? REC_BAD : 0u;
+  return r;
+}
 // Rounds between two looks at the lanes that wait for service.  A look costs
 // about 60 cycles beside rounds of about 270; a lane that waits loses half a
 // batch.
@@ -481,6 +540,7 @@ struct FastConsoleT {
   uint32_t rounds;         // issue rounds of this env's warp in the step (the same on every lane)
   uint32_t wmask;          // lanes of this warp running envs
   uint32_t idle;           // retire RIOT-timer wait-loop iterations at once
+  uint32_t unit;           // 1, as a value that the compiler does not know (see mad)
   uint32_t qtail, qhead_seen, nreq, vsync_c, vblank_c, broken;  // qhead_seen: the TIA side's cursor as last read
   uint64_t l0c;
   TiaSide ts;              // single-warp form: the TIA side
@@ -498,7 +558,7 @@ struct FastConsoleT {
     io = IoCtx{o.tia, o.io};
   }
   __device__ __forceinline__ uint8_t &ram(uint32_t i) const { return sm8(off.ram + i); }
-  __device__ __forceinline__ uint32_t rom(uint32_t i) const { return sm8(off.rom + i); }
+  __device__ __forceinline__ uint32_t rom(uint32_t i) const { return sm8(off.rom + 4 * i); }
 
   // ---- canonical state I/O ----
   __device__ void load(const uint8_t *s) {
@@ -523,14 +583,10 @@ struct FastConsoleT {
     }
     io.Sset(IO_CX, w[17] >> 16);
     io.Sset(IO_BARLO, w[18]); io.Sset(IO_BARHI, w[19]);
-    io.Sset(IO_L0LO, w[20]); io.Sset(IO_L0HI, w[21]);
     frame_no = w[22];
     l0c = (uint64_t)w[20] | (uint64_t)w[21] << 32;
     kf = (uint32_t)(k - 76ull * l0c);
-    io.Sset(IO_CEVAL, 3u * kf);
     io.Sset(IO_JOY, 0xFF); io.Sset(IO_FIRE, 0);
-    io.Sset(IO_LOGLO, 0); io.Sset(IO_LOGHI, 0); io.Sset(IO_LOGN, 0); io.Sset(IO_LOGCAP, 0);
-    io.Sset(IO_BANDN, BANDS);
     io.Sset(IO_STATUS, 0);
     const uint4 *r4 = reinterpret_cast<const uint4 *>(s + S::RAM);
     uint32_t *r32 = &sm32(off.ram);
@@ -544,12 +600,12 @@ struct FastConsoleT {
     vsync_c = io.T(T_VSYNC);
     vblank_c = io.T(T_VBLANK);
     qtail = qhead_seen = nreq = broken = 0;
-    io.Sset(IO_QHEAD, 0); io.Sset(IO_QTAIL, 0); io.Sset(IO_ACK, 0);
-    ts = TiaSide{0, 0, 0, 0};
+    io.Sset(IO_QHEAD, 0); io.Sset(IO_ACK, 0);
+    if constexpr (!SPLIT) ts = tia_start(io, l0c, kf);
   }
   __device__ void store(uint8_t *s) const {
     uint32_t *w = reinterpret_cast<uint32_t *>(s);
-    const uint64_t L0 = io.G64(IO_L0LO);
+    const uint64_t L0 = l0c;
     w[0] = A | X << 8 | Y << 16 | SP << 24;
     w[1] = P() | bank << 8 | PC << 16;
     const uint64_t k = 76ull * L0 + kf;
@@ -576,7 +632,7 @@ struct FastConsoleT {
     for (int q_ = 0; q_ < 8; ++q_)
       r4[q_] = make_uint4(r32[4 * q_], r32[4 * q_ + 1], r32[4 * q_ + 2], r32[4 * q_ + 3]);
   }
-  __device__ uint32_t all_status() const { return status | io.G(IO_STATUS); }
+  __device__ uint32_t all_status() const { return status | io.G(IO_STATUS) | (SPLIT ? 0u : ts.status); }
 
   __device__ void apply_action(uint32_t a) {
     uint32_t d;
@@ -598,15 +654,9 @@ struct FastConsoleT {
     if (fire && (vblank_c & 0x40)) io.Sset(IO_LATCH, 1);
   }
 
-  // Cartridge bytes i .. i+3 of the stage, byte i lowest (i + 3 may run into
-  // the padding after the last bank).
-  __device__ __forceinline__ uint32_t fetch4(uint32_t i) const {
-    const uint32_t a = off.rom + (i & ~3u);
-    return __funnelshift_r(sm32(a), sm32(a + 4), (i & 3u) * 8u);
-  }
   // Last offset in a bank whose instruction bytes are fetched from the stage:
   // no such fetch touches a hotspot (F8/F6 hotspots start at $FF6, F4's at $FF4).
-  __device__ __forceinline__ uint32_t fetch_limit() const { return scheme == 3 ? 0xFF1u : scheme ? 0xFF3u : 0xFFCu; }
+  __device__ __forceinline__ uint32_t fetch_limit() const { return scheme_fetch_limit(scheme); }
 
   // ---- bus ----
   __device__ __forceinline__ void hotspot(uint32_t at) {
@@ -642,13 +692,14 @@ struct FastConsoleT {
   __device__ void sync_collisions(uint32_t t) {
     if constexpr (SPLIT) {
       if (broken) return;
-      push(EV_SYNC | (t & 0xFFFFu));
+      push(EV_SYNC | t << 16);
       ++nreq;
       if (!broken && !fc_q_wait_ack(io, nreq)) stall();
       qhead_seen = qtail;  // acknowledged: the queue is empty
     } else {
       drain();
-      fc_cx_eval(io, 3u * t);
+      fc_cx_eval(io, ts, 3u * t);
+      io.Sset(IO_CX, ts.cx);
     }
   }
   // Read / write a TIA or RIOT address (13-bit, neither RAM nor cartridge) at cycle t.
@@ -676,7 +727,7 @@ struct FastConsoleT {
       if (!(v & 0x40)) io.Sset(IO_LATCH, 0);
       else if (io.G(IO_FIRE)) io.Sset(IO_LATCH, 1);
     }
-    push((t & 0xFFFFu) << 14 | reg << 8 | v);
+    push((t + 1u) << 16 | reg << 8 | v);
   }
   __device__ __forceinline__ uint32_t rd(uint32_t addr, uint32_t t) {
     const uint32_t a = addr & 0x1FFF;
@@ -759,9 +810,9 @@ struct FastConsoleT {
   // the issue rounds execute.  Anything else (no such loop, a faster
   // timer, the timer already at 0 or past it, a frame that would reach the
   // line cap) returns k0 unchanged.
-  __device__ __forceinline__ uint32_t idle_forward(uint32_t w, uint32_t pc, uint32_t k0) {
+  __device__ __forceinline__ uint32_t idle_forward(uint32_t w, uint32_t next_op, uint32_t pc, uint32_t k0) {
     const uint32_t a = (w >> 8) & 0xFFFF;
-    if ((a & 0x1285u) != 0x0284u || (w >> 24) != 0xD0u) return k0;  // INTIM (any mirror), then BNE
+    if ((a & 0x1285u) != 0x0284u || next_op != 0xD0u) return k0;  // INTIM (any mirror), then BNE
     const uint32_t at = pc & 0xFFF;
     // BNE offset -5: back to pc, its bytes below the cartridge's hotspots
     if (at > (scheme == 3 ? 0xFEFu : scheme ? 0xFF1u : 0xFFBu) || rom(bank * 4096u + at + 4) != 0xFBu) return k0;
@@ -783,9 +834,9 @@ struct FastConsoleT {
     pend = 0;
     const uint32_t pc = PC;
     const uint32_t opcode = rd(pc, k0);
-    const uint32_t opb = sm8(off.dec + opcode);
+    const uint32_t opb = sm8(OFF_DEC + opcode);
     const uint32_t op = opb & 0x7F;
-    const uint32_t info = sm8(off.dec + 256 + opcode);
+    const uint32_t info = sm8(OFF_DEC + 256 + opcode);
     const uint32_t mode = info & 0xF;
     uint32_t n = info >> 4;
     if (op == O_JAM) { jam = 1; status |= ST_ILLEGAL; return; }
@@ -951,8 +1002,12 @@ struct FastConsoleT {
 
   // Append the end of the current frame and start counting the next.
   __device__ __forceinline__ void end_frame(uint32_t next_rel) {
-    push(EV_FRAME_END | (kf & 0xFFFFu));
-    push(EV_REBASE | (next_rel & 0xFFFFFFFu));
+    push(EV_FRAME_END | kf << 16);
+    for (uint32_t left = next_rel; left;) {  // one event, but for loaded states far past the line cap
+      const uint32_t n = left < 0xFFFFFFu ? left : 0xFFFFFFu;
+      push(EV_REBASE | n << 16 | n >> 16);
+      left -= n;
+    }
     l0c += next_rel;
     kf -= 76u * next_rel;
     frame_no++;
@@ -991,11 +1046,17 @@ __device__ __noinline__ bool fc_service(FastConsoleT<SPLIT> *c, Hook *h) {
   if (!ended) {
     const uint32_t at = c->PC & 0xFFF;
     if (c->idle && (c->PC & 0x1000) && at <= c->fetch_limit()) {
-      const uint32_t w = c->fetch4(c->bank * 4096u + at);
-      if ((w & 0xFF) == 0xAD) c->kf = c->idle_forward(w, c->PC, c->kf);
+      const uint32_t i = c->bank * 4096u + at;
+      if (c->rom(i) == 0xAD && at + 4u < 4096u)
+        c->kf = c->idle_forward(sm32(c->off.rom + 4 * i) & 0xFFFFFFu, c->rom(i + 3), c->PC, c->kf);
     }
-    c->exec_general();
-    ended = c->jam || c->vs_kf != ~0u || c->kf >= cap;
+    // decimal mode is the general decoder's: its instructions run on here
+    for (int n = 0; n < 16; ++n) {
+      if (n) ++c->rounds;  // the first one is counted with the whole warp's round
+      c->exec_general();
+      ended = c->jam || c->vs_kf != ~0u || c->kf >= cap;
+      if (ended || !(c->fdi & 0x08)) break;
+    }
   }
   while (ended) {
     uint32_t next_rel;
@@ -1013,33 +1074,48 @@ template <bool SPLIT>
 template <class Hook>
 __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
   const EnvOff o = off;
-  const uint32_t smb = (uint32_t)__cvta_generic_to_shared(g_smem);
+  uint32_t smb;  // the shared window's address, taken here: no load of the stage moves above the block's barrier
+  asm volatile("mov.u32 %0, %1;" : "=r"(smb) : "r"((uint32_t)__cvta_generic_to_shared(g_smem)) : "memory");
   const uint32_t cap = 76u * CAP_LINES;
-  const uint32_t ctl = o.dec + 512, romb = smb + o.rom;
-  const uint32_t lim = fetch_limit();
-  // cartridge reads below the first hotspot are plain loads
-  const uint32_t hot = scheme == 3 ? 0xFF4u : scheme == 2 ? 0xFF6u : scheme == 1 ? 0xFF8u : 0x1000u;
-  uint32_t R, Pf, pc, k, inst, qt, bk;
-  uint32_t rec, cb;
-  uint4 c;
+  const uint32_t ctl = smb + OFF_CTL, reg = smb + OFF_REG;
+  const uint32_t k1 = unit, k4 = unit * 4u, k256 = unit * 256u;
+  // R: A, X, Y and FF as bytes.  G: flags (FL_*; V apart, in bit 7 of vv; D
+  // and I do not change here).  pk: PC, and the frame's CPU cycle in the high
+  // half.  nl: the first line start at or after that cycle, in the high half,
+  // over FFFF.  qi: queue position, and the instructions retired since the
+  // last service in the high half.  bk: the bank's words.
+  uint32_t R, G, vv, pk, nl, qi, bk;
+  uint32_t rec;
+  uint4 c, d, e, f;  // control words 0-3, 4-7, 8-11, 12-15
   bool wait = false, active = true;
-  // instruction bytes at p; the control words of opcode op
-  auto bytes_at = [&](uint32_t p) {
-    const uint32_t i = bk + (p & 0xFFFu);
-    const uint32_t a = romb + (i & ~3u);
-    return __funnelshift_r(lds_const(a), lds_const(a + 4), i * 8u);
-  };
-  auto control = [&](uint32_t op) {
-    c = lds_const4(smb + ctl + op * 16u);
-    cb = lds_const(smb + ctl + CTL_B_OFF + op * 4u);
+  auto word_at = [&](uint32_t p) { return lds_const(mad(p & 0xFFFu, k4, smb + bk)); };
+  auto control = [&] {
+    const uint32_t a = mad(rec & 0xFFu, unit * CTL_STRIDE, ctl);
+    c = lds_const4(a);
+    d = lds_const4(a + 16);
+    e = lds_const4(a + 32);
+    f = lds_const4(a + 48);
   };
   // the console's fields to the loop's registers, and the next instruction
   auto enter = [&](bool stay) {
-    R = A | X << 8 | Y << 16;
-    Pf = P(); pc = PC; k = kf; inst = instret; qt = qtail; bk = bank * 4096u;
-    rec = bytes_at(pc);
-    wait = stay || ((pc & 0x1FFFu) - 0x1000u) > lim || k >= cap;
-    control(wait ? CTL_HALT : rec & 0xFFu);
+    R = A | X << 8 | Y << 16 | 0xFF000000u;
+    G = ((fz & 0xFFu) ? 1u : 0u) | fc << 8 | (fn & 0x80u) << 16;
+    vv = fv << 1;
+    pk = (PC & 0xFFFFu) | min(kf, 0xFFFFu) << 16;
+    nl = ((min(kf, 0xFFFFu) + 75u) / 76u * 76u) << 16 | 0xFFFFu;
+    qi = qtail & 0xFFu;
+    bk = o.rom + bank * 16384u;
+    rec = word_at(pk);
+    wait = stay | ((pk & 0x1000u) == 0) | (rec >= REC_BAD) | (kf >= cap) | ((fdi & 0x08u) != 0);
+    control();
+  };
+  auto leave = [&] {
+    A = R & 0xFF; X = (R >> 8) & 0xFF; Y = (R >> 16) & 0xFF;
+    fz = G & FL_Z; fc = (G >> 8) & 1u; fn = (G >> 16) & 0x80u; fv = (vv >> 1) & 0x40u;
+    PC = pk & 0xFFFFu;
+    if ((pk >> 16) != 0xFFFFu) kf = pk >> 16;  // a loaded cycle count past 16 bits stays as it was
+    qtail += (qi & 0xFFFFu) - (qtail & 0xFFu);
+    instret += qi >> 16;
   };
   enter(jam != 0);
   uint32_t held = 0, act = wmask;
@@ -1047,58 +1123,53 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
 #pragma unroll 1
     for (uint32_t r = 0; r < BATCH; ++r) {
       // --- next instruction (branches and JMP abs: the sum is the target)
-      const uint32_t pcn = pc + (c.w >> 28);
-      const uint32_t base = prmt(rec, pcn, c.x);
-      const uint32_t sum = base + prmt(R, rec, c.y);
-      const bool tk = ((Pf ^ (c.y >> 24)) & (c.y >> 16) & 0xFFu) != 0;
-      const uint32_t npc = tk ? sum & 0xFFFFu : pcn;
-      const uint32_t nrec = bytes_at(npc);
-      const bool nbad = ((npc & 0x1FFFu) - 0x1000u) > lim;
-      // --- cycles
-      const uint32_t tk1 = tk ? 1u : 0u;
-      const uint32_t n = ((cb >> 8) & 0x7Fu) + tk1 + (((base ^ sum) >> 8) & (((cb >> 15) & 1u) | tk1));
-      const uint32_t kn = k + n;
+      const uint32_t pn = mad(pk, k1, d.z);
+      const uint32_t base = prmt(rec, pn, c.x);
+      const uint32_t sum = mad(base, k1, prmt(R, rec, c.y));
+      const bool tk = ((G & d.w) != 0) ^ ((int)e.w < 0);
+      const uint32_t nrec = word_at(tk ? sum : pn);
+      // a cycle for a taken branch, another one at a page crossing
+      uint32_t pnext = mad((base ^ sum) & (tk ? 0x100u : f.z), k256, pn);
+      if (tk) pnext = prmt(pnext, sum, 0x3254) + 0x10000u;
       // --- operand
-      const uint32_t ea = sum & (c.x >> 16);
-      const bool is_ram = (ea & 0x1280u) == 0x0080u;
-      const bool is_cart = ea - 0x1000u < hot;
-      const uint32_t tia = ea & 0x10BFu;                  // below $40: a TIA register
-      const uint32_t at = is_ram ? o.ram + (ea & 0x7Fu) : o.rom + bk + (ea & 0xFFFu);
+      const uint32_t ea = sum & d.y;
+      const uint32_t rg = lds8_const(reg + (ea >> 5));
+      const uint32_t at = (ea & 0x1280u) == 0x0080u ? mad(ea & 0x7Fu, k1, o.ram) : mad(ea & 0xFFFu, k4, bk);
       const uint32_t ld = sm8(at);
-      const uint32_t y = ((cb & CT_MEM) ? ld : sum) ^ (c.z >> 24);
-      const uint32_t x = prmt(R, y | 0xFF00u, c.z);
-      // --- what the general decoder takes
-      const bool is_ld = (cb & CT_LD) != 0, is_st = (cb & CT_ST) != 0, is_rmw = (cb & CT_RMW) != 0;
-      const bool ok = is_ram | (is_ld & is_cart) | (is_st & (tia - 2u < 0x3Eu));
-      const bool slow = ((cb & CT_SLOW) != 0) | ((is_ld | is_st | is_rmw) & !ok) | ((Pf & (cb >> 24) & 0x08u) != 0);
+      const uint32_t y = prmt(ld, sum, d.x) ^ e.y;
+      const uint32_t x = prmt(R, y, c.z);
       // --- result
-      const uint32_t cin = (Pf & cb & 1u) | ((cb >> 1) & 1u);
-      const uint32_t add = (x & y) * ((cb >> 24) & 3u) + ((x ^ y) & (c.z >> 16)) + cin;
-      const uint32_t rot = (((y + (cin << 8)) * 513u) >> 1) & 0x1FFu;
-      const uint32_t s = (cb & CT_SHR) ? rot : add;
-      // --- flags
-      uint32_t nf = (s & 0x80u) | ((s >> 8) & 1u) | ((((x ^ s) & ~(x ^ y)) & 0x80u) >> 1) | ((s & 0xFFu) ? 0u : 2u);
-      const uint32_t bits = (cb >> 16) & 0xFFu, pm = slow ? 0u : (c.w >> 16) & 0xFFu;
-      nf = (nf & ~bits) | (y & bits);
+      const uint32_t one = f.w >> 16;
+      const uint32_t raw = mad(x & y, e.z, mad(x ^ y, f.y, mad(prmt(G, 0, e.w), k1, one)));
+      const uint32_t s = __funnelshift_r(raw, 0, f.w);
+      // --- what the general decoder takes: no region fits, VSYNC, VBLANK
+      const uint32_t m = ea & 0x3Fu;                      // of the TIA: the register
+      const uint32_t put = rg & f.x;
+      const bool tia = (put & RG_WTIA) != 0;
+      const bool skip = wait | ((put & RG_ALL) == 0) | (tia & (m < 2u));
       // --- commit
-      const uint32_t sv = (is_rmw ? s : x) & 0xFFu;
-      sts8_if((is_st | is_rmw) & is_ram & !slow, smb + at, sv);
-      const bool out = is_st & (tia - 3u < 0x3Du) & !slow;
-      sts32_if(out, smb + o.q + (qt & (QLEN - 1)) * 4u, ((kn - 1u) << 14 | tia << 8 | sv) ^ lap_bit(qt));
-      qt += out ? 1u : 0u;
-      const uint32_t kw = (is_st & (tia == 2u)) ? (kn + 75u) / 76u * 76u : kn;
-      R = prmt(R, s, slow ? 0x3210u : c.w);
-      Pf = (Pf & ~pm) | (nf & pm);
-      inst += slow ? 0u : (cb >> 28) & 1u;
-      pc = slow ? pc : npc;
-      k = slow ? k : kw;
-      wait = wait | slow | nbad | (k >= cap);
+      const bool out = tia & (m > 2u) & !wait, ws = tia & (m == 2u);
+      if (((put & RG_WRAM) != 0) & !wait) sm8(at) = (uint8_t)s;
+      // events past another lap's bit: the lap's complement is bit 15 of -qi * 1024 - 1024
+      const uint32_t ev = mad(m, k256, s) | (mad(qi, unit * 0xFFFFFC00u, 0xFFFFFC00u) & EV_LAP);
+      if (out) vsm32(mad(qi & (QLEN - 1), k4, o.q)) = prmt(ev, pnext, 0x7610);
+      if (pnext > nl) nl += 76u << 16;                    // one step: no instruction is longer than a line
+      if (ws) pnext = prmt(pnext, nl, 0x7610);            // WSYNC: on to the next line's first cycle
+      if (!skip) R = prmt(R, s, c.w);
+      if (!skip) G = (G & ~e.x) | ((s * FL_COPY) & e.x);
+      if ((!skip) & ((int)d.x < 0)) vv = (x ^ s) & ~(x ^ y);
+      if (!skip) pk = pnext;
+      if (!skip) qi += 0x10000u;
+      if (out) ++qi;
+      // bit 31: no instruction word there, the PC outside the cartridge, the line cap
+      const uint32_t stop = nrec | mad(pnext, unit * 0xFFF80000u, 0xFFF80000u) | mad(pnext, 0u - unit, (cap << 16) - 1u);
+      wait = skip | ((int)stop < 0);
       rec = nrec;
-      control(wait ? CTL_HALT : nrec & 0xFFu);
+      control();
     }
     // --- service: waiting lanes, and queues without room for another batch
     rounds += BATCH;
-    const bool full = qt - qhead_seen > QLEN - BATCH;
+    const bool full = ((qi - qhead_seen) & 0xFFu) > QLEN - BATCH;
     uint32_t m = __ballot_sync(wmask, (wait | full) & active);
     if (m == 0) continue;
     m = __ballot_sync(wmask, wait & active);
@@ -1106,8 +1177,7 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
       held = 0;
       ++rounds;
       if (active && wait) {
-        A = R & 0xFF; X = (R >> 8) & 0xFF; Y = (R >> 16) & 0xFF;
-        setP(Pf); PC = pc; kf = k; instret = inst; qtail = qt;
+        leave();
         active = fc_service<SPLIT, Hook>(this, &hook);
         enter(!active);
       }
@@ -1116,20 +1186,21 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
     }
     // room for a batch of events
     if constexpr (SPLIT) {
-      if (active & (qt - qhead_seen > QLEN - BATCH)) {
+      if (active & (((qi - qhead_seen) & 0xFFu) > QLEN - BATCH)) {
+        const uint32_t qt = qtail + (qi & 0xFFFFu) - (qtail & 0xFFu);
         qhead_seen = fc_q_wait_room(io, qt, BATCH);
-        if (qt - qhead_seen > QLEN - BATCH) { stall(); wait = true; control(CTL_HALT); }
+        if (qt - qhead_seen > QLEN - BATCH) { stall(); wait = true; }
       }
     } else {
-      if (__any_sync(wmask, qt - qhead_seen > QLEN - BATCH)) {
-        qtail = qt;
-        drain();
+      if (__any_sync(wmask, ((qi - qhead_seen) & 0xFFu) > QLEN - BATCH)) {
+        const uint32_t qt = qtail + (qi & 0xFFFFu) - (qtail & 0xFFu);
+        tia_drain(io, off.q, ts, to, qt);
+        qhead_seen = qt;
       }
     }
     __syncwarp(wmask);
   }
-  A = R & 0xFF; X = (R >> 8) & 0xFF; Y = (R >> 16) & 0xFF;
-  setP(Pf); PC = pc; kf = k; instret = inst; qtail = qt;
+  leave();
 }
 
 }  // namespace atari

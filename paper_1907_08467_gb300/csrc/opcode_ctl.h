@@ -1,13 +1,16 @@
-// Control words of the batched interpreter: one set per opcode, built on the
-// host from the decode table and copied to shared memory by every block.
+// Control words and tables of the batched interpreter, built on the host from
+// the decode table and copied to shared memory by every block.
 //
 // The interpreter runs every common instruction through one branch-free
-// sequence (fast_console.cuh); these words tell it which operand bytes, index,
-// registers, adder inputs and flags the opcode uses.  On sm_103a a switch on
-// the opcode costs about 30 cycles for each level of its compare tree (one
-// warp, warp-uniform value: 49 cycles for 2 cases, 178 for 36, 241 for 150),
-// and a jump table 100 cycles while its handlers fit the instruction cache's
-// first level and 280-450 when they do not, so data beats code here.
+// sequence (fast_console.cuh); an opcode's control words tell it which operand
+// bytes, index, registers, adder inputs and flags the instruction uses.  On
+// sm_103a a switch on the opcode costs about 30 cycles for each level of its
+// compare tree (one warp, warp-uniform value: 49 cycles for 2 cases, 178 for
+// 36, 241 for 150), and a jump table 100 cycles while its handlers fit the
+// instruction cache's first level and 280-450 when they do not, so data beats
+// code here.  The sequence is bound by the integer pipe (two cycles a warp
+// instruction), so the words come in the form in which they are used, with as
+// little unpacking as possible: 64 bytes an opcode, four 16-byte loads.
 #pragma once
 #include <cstdint>
 #include <cstring>
@@ -16,110 +19,137 @@
 
 namespace atari {
 
-// words 0..3 (one 16-byte load per round):
-//   0  byte selector of the address base from (instruction bytes, next PC)
-//      | address mask << 16
-//   1  byte selector of the index from (A X Y 0, instruction bytes)
-//      | branch flag mask << 16 | branch flag invert << 24
-//   2  byte selector of the adder's x from (A X Y 0, operand FF) | xor mask << 16 | operand invert << 24
-//   3  byte selector of the written registers from (A X Y 0, result)
-//      | flag write mask << 16 | length << 28
-// word 4: the bits below, cycles << 8, page-cross penalty << 15, flags taken
-//   from the operand (BIT) << 16, carries of (x & y) << 24, decimal check << 27
-constexpr uint32_t CT_CIN = 1u, CT_ONE = 2u, CT_MEM = 4u, CT_LD = 8u, CT_ST = 16u, CT_RMW = 32u, CT_SHR = 64u,
-                   CT_SLOW = 128u, CT_COUNT = 1u << 28;
-constexpr uint32_t CTL_HALT = 256;             // entry that changes nothing: a lane waiting for service
-constexpr uint32_t CTL_N = 257;
-constexpr uint32_t CTL_B_OFF = 16 * CTL_N;     // word 4 of every entry follows the 16-byte entries
-constexpr uint32_t CTL_BYTES = (CTL_B_OFF + 4 * CTL_N + 15) / 16 * 16;
+// Regions of the 13-bit bus: RAM, cartridge below its first hotspots, TIA; RAM
+// and TIA again for the writes that a control word asks for.
+constexpr uint32_t RG_RAM = 1u, RG_CART = 2u, RG_TIA = 4u, RG_ALL = 7u, RG_WRAM = 8u, RG_WTIA = 16u;
+
+// Word by word (byte selectors are those of a 32-bit byte permute and use the
+// low half):
+//   0  selector of the address base from (instruction bytes, next PC)
+//   1  selector of the index from (A X Y FF, instruction bytes)
+//   2  selector of the adder's x from (A X Y FF, operand)
+//   3  selector of the written registers from (A X Y FF, result)
+//   4  selector of the operand from (memory byte, sum of base and index) | V is written << 31
+//   5  address mask
+//   6  length | cycles << 16
+//   7  branch: flag bits of which any takes it
+//   8  flag bits that are written
+//   9  operand invert
+//  10  multiplier of (x & y): 0 eor, 1 and / or, 2 add, 513 shift right
+//  11  selector of the carry-in from the flags (their byte 1 is the carry) | the branch is taken when no flag
+//      bit is set << 31
+//  12  regions that the access may fall in (none: the general decoder's instruction), RG_WRAM: the result is
+//      stored there, RG_WTIA: it is written there
+//  13  multiplier of (x ^ y): 0 and, 1 otherwise
+//  14  page-cross penalty << 8
+//  15  right shift of the sum | carry-in 1 << 16
+constexpr uint32_t CTL_WORDS = 16, CTL_STRIDE = 4 * CTL_WORDS, CTL_N = 256;
+constexpr uint32_t CTL_BYTES = CTL_STRIDE * CTL_N;
 constexpr uint32_t DEC_BYTES = 512 + CTL_BYTES;  // general decoder's bytes, then the control words
+constexpr uint32_t REGION_BYTES = 256;           // region table of the cartridge, indexed by address >> 5
+
+// Flags as the interpreter holds them: the 9-bit result that set them, twice.
+// Bits 0-7 are zero when Z is set, bit 8 is C, bit 23 is N (BIT and PLP can set
+// N and Z both, so N has its own copy); the other bits are not looked at.
+constexpr uint32_t FL_NZ = 0xFFu | 0xFFu << 16, FL_C = 0x100u | 0x100u << 16, FL_Z = 0xFFu, FL_N = 0x80u << 16;
+constexpr uint32_t FL_COPY = 0x10001u;         // result -> both copies
+
+// Region byte of addresses at << 5 ..  scheme != 0: the last 128 bytes hold
+// bank hotspots and are left to the general decoder.
+__host__ __device__ inline uint32_t region_byte(uint32_t at, uint32_t scheme) {
+  const uint32_t page = at >> 2;
+  if (page >= 32u) return page == 63u && scheme ? 0u : RG_CART;
+  if ((page & 5u) == 1u) return RG_RAM | RG_WRAM;
+  return (page & 1u) ? 0u : RG_TIA | RG_WTIA;
+}
 
 // dec: per opcode, operation | mode << 8 | cycles << 12 | page-cross penalty << 16 (0: halts the CPU).
 inline void build_ctl(const uint32_t *dec, uint8_t *out) {
   memset(out, 0, CTL_BYTES);
   for (uint32_t o = 0; o < CTL_N; ++o) {
-    const uint32_t op = o < 256 ? dec[o] & 0xFF : (uint32_t)O_NOP, mode = o < 256 ? (dec[o] >> 8) & 0xF : (uint32_t)IMP;
-    uint32_t cyc = o < 256 ? (dec[o] >> 12) & 0xF : 0u;
-    const uint32_t pen = o < 256 ? (dec[o] >> 16) & 1 : 0u;
-    uint32_t len = o == CTL_HALT ? 0u : mode <= ACC ? 1u : mode >= ABS && mode <= IND ? 3u : 2u;
-    uint32_t selB = 0x6666, selI = 0x3333, selX = 0x3333, selD = 0x3210, em = 0x1FFF;
-    uint32_t bm = 0, binv = 0, m2 = 0xFF, inv = 0, pm = 0, cb = o == CTL_HALT ? 0u : CT_COUNT, k = 2;
+    const uint32_t op = dec[o] & 0xFF, mode = (dec[o] >> 8) & 0xF;
+    uint32_t cyc = (dec[o] >> 12) & 0xF;
+    const uint32_t pen = (dec[o] >> 16) & 1;
+    const uint32_t len = mode <= ACC ? 1u : mode >= ABS && mode <= IND ? 3u : 2u;
+    // zero bytes: byte 3 of the instruction bytes, byte 1 of the operand
+    uint32_t selB = 0x3333, selI = 0x7777, selX = 0x5555, selD = 0x3210, selV = 0x7654, em = 0;
+    uint32_t bm = 0, m2 = 1, inv = 0, gm = 0, k = 2, selC = 0x4444, one = 0, binv = 0, vset = 0, regions = RG_ALL, wr = 0;
     bool mem = true, slow = op == O_JAM;
     switch (mode) {
-      case IMM: selB = 0x6661; mem = false; break;
-      case ZP: selB = 0x6661; em = 0xFF; break;
-      case ZPX: selB = 0x6661; selI = 0x3331; em = 0xFF; break;
-      case ZPY: selB = 0x6661; selI = 0x3332; em = 0xFF; break;
-      case ABS: selB = 0x6621; break;
-      case ABX: selB = 0x6621; selI = 0x3331; break;
-      case ABY: selB = 0x6621; selI = 0x3332; break;
-      case ACC: selI = 0x3330; mem = false; break;  // the operand is the sum of base and index: A
-      case REL: selB = 0x6654; selI = 0xDDD5; mem = false; break;
+      case IMM: selB = 0x3331; mem = false; break;
+      case ZP: selB = 0x3331; em = 0xFF; break;
+      case ZPX: selB = 0x3331; selI = 0x7771; em = 0xFF; break;
+      case ZPY: selB = 0x3331; selI = 0x7772; em = 0xFF; break;
+      case ABS: selB = 0x3321; em = 0x1FFF; break;
+      case ABX: selB = 0x3321; selI = 0x7771; em = 0x1FFF; break;
+      case ABY: selB = 0x3321; selI = 0x7772; em = 0x1FFF; break;
+      case ACC: selI = 0x7770; mem = false; break;  // the operand is the sum of base and index: A
+      case REL: selB = 0x3354; selI = 0xDDD5; mem = false; break;
       case IMP: mem = false; break;
       default: slow = true; break;                  // pointers through RAM: the general decoder
     }
-    const uint32_t NZ = 0x82, NZC = 0x83, A_ = 0x3330, X_ = 0x3331, Y_ = 0x3332, V_ = 0x3334, FF = 0x3335;
+    const uint32_t NZ = FL_NZ, NZC = FL_NZ | FL_C, C1 = 0x4441, A_ = 0x5550, X_ = 0x5551, Y_ = 0x5552, V_ = 0x5554, FF = 0x5553;
     const uint32_t dA = 0x3214, dX = 0x3240, dY = 0x3410;
     bool ld = false, st = false, rmw = false;
     switch (op) {
-      case O_LDA: selD = dA; pm = NZ; ld = mem; break;
-      case O_LDX: selD = dX; pm = NZ; ld = mem; break;
-      case O_LDY: selD = dY; pm = NZ; ld = mem; break;
-      case O_ADC: selX = A_; selD = dA; pm = 0xC3; cb |= CT_CIN | 1u << 27; ld = mem; break;
-      case O_SBC: selX = A_; selD = dA; pm = 0xC3; inv = 0xFF; cb |= CT_CIN | 1u << 27; ld = mem; break;
-      case O_AND: selX = A_; selD = dA; pm = NZ; k = 1; m2 = 0; ld = mem; break;
-      case O_ORA: selX = A_; selD = dA; pm = NZ; k = 1; ld = mem; break;
-      case O_EOR: selX = A_; selD = dA; pm = NZ; k = 0; ld = mem; break;
-      case O_BIT: selX = A_; pm = 0xC2; k = 1; m2 = 0; cb |= 0xC0u << 16; ld = mem; break;
-      case O_CMP: selX = A_; pm = NZC; inv = 0xFF; cb |= CT_ONE; ld = mem; break;
-      case O_CPX: selX = X_; pm = NZC; inv = 0xFF; cb |= CT_ONE; ld = mem; break;
-      case O_CPY: selX = Y_; pm = NZC; inv = 0xFF; cb |= CT_ONE; ld = mem; break;
+      case O_LDA: selD = dA; gm = NZ; ld = mem; break;
+      case O_LDX: selD = dX; gm = NZ; ld = mem; break;
+      case O_LDY: selD = dY; gm = NZ; ld = mem; break;
+      case O_ADC: selX = A_; selD = dA; gm = NZC; vset = 1; selC = C1; ld = mem; break;
+      case O_SBC: selX = A_; selD = dA; gm = NZC; vset = 1; selC = C1; inv = 0xFF; ld = mem; break;
+      case O_AND: selX = A_; selD = dA; gm = NZ; k = 1; m2 = 0; ld = mem; break;
+      case O_ORA: selX = A_; selD = dA; gm = NZ; k = 1; ld = mem; break;
+      case O_EOR: selX = A_; selD = dA; gm = NZ; k = 0; ld = mem; break;
+      case O_CMP: selX = A_; gm = NZC; inv = 0xFF; one = 1; ld = mem; break;
+      case O_CPX: selX = X_; gm = NZC; inv = 0xFF; one = 1; ld = mem; break;
+      case O_CPY: selX = Y_; gm = NZC; inv = 0xFF; one = 1; ld = mem; break;
       case O_STA: selX = A_; st = true; break;
       case O_STX: selX = X_; st = true; break;
       case O_STY: selX = Y_; st = true; break;
-      case O_ASL: selX = V_; pm = NZC; rmw = mem; break;
-      case O_ROL: selX = V_; pm = NZC; cb |= CT_CIN; rmw = mem; break;
-      case O_LSR: pm = NZC; cb |= CT_SHR; rmw = mem; break;
-      case O_ROR: pm = NZC; cb |= CT_SHR | CT_CIN; rmw = mem; break;
-      case O_INC: pm = NZ; cb |= CT_ONE; rmw = true; break;
-      case O_DEC: selX = FF; pm = NZ; rmw = true; break;
-      case O_INX: selX = X_; selD = dX; pm = NZ; cb |= CT_ONE; break;
-      case O_INY: selX = Y_; selD = dY; pm = NZ; cb |= CT_ONE; break;
-      case O_DEX: selX = X_; selD = dX; pm = NZ; inv = 0xFF; break;
-      case O_DEY: selX = Y_; selD = dY; pm = NZ; inv = 0xFF; break;
-      case O_TAX: selX = A_; selD = dX; pm = NZ; break;
-      case O_TAY: selX = A_; selD = dY; pm = NZ; break;
-      case O_TXA: selX = X_; selD = dA; pm = NZ; break;
-      case O_TYA: selX = Y_; selD = dA; pm = NZ; break;
-      case O_CLC: pm = 0x01; break;
-      case O_SEC: pm = 0x01; inv = 0xFF; cb |= CT_ONE; break;  // 0 + FF + 1 carries
-      case O_CLI: pm = 0x04; break;
-      case O_CLV: pm = 0x40; break;
-      case O_CLD: pm = 0x08; break;
-      case O_BCC: bm = binv = 0x01; break;
-      case O_BCS: bm = 0x01; break;
-      case O_BNE: bm = binv = 0x02; break;
-      case O_BEQ: bm = 0x02; break;
-      case O_BVC: bm = binv = 0x40; break;
-      case O_BVS: bm = 0x40; break;
-      case O_BPL: bm = binv = 0x80; break;
-      case O_BMI: bm = 0x80; break;
-      // a branch always taken (P bit 5 is always set): base = the operand, the taken branch's cycle counted
-      case O_JMP: if (mode == ABS) { bm = 0x20; cyc = 2; } else slow = true; break;
+      case O_ASL: selX = V_; gm = NZC; rmw = mem; break;
+      case O_ROL: selX = V_; gm = NZC; selC = C1; rmw = mem; break;
+      // y * 513 >> 1 holds y >> 1 in bits 0-6 and y's bit 0 in bit 8; the carry comes in at 256 >> 1
+      case O_LSR: selX = V_; gm = NZC; k = 513; rmw = mem; break;
+      case O_ROR: selX = V_; gm = NZC; k = 513; selC = 0x4414; rmw = mem; break;
+      case O_INC: gm = NZ; one = 1; rmw = true; break;
+      case O_DEC: selX = FF; gm = NZ; rmw = true; break;
+      case O_INX: selX = X_; selD = dX; gm = NZ; one = 1; break;
+      case O_INY: selX = Y_; selD = dY; gm = NZ; one = 1; break;
+      case O_DEX: selX = X_; selD = dX; gm = NZ; inv = 0xFF; break;
+      case O_DEY: selX = Y_; selD = dY; gm = NZ; inv = 0xFF; break;
+      case O_TAX: selX = A_; selD = dX; gm = NZ; break;
+      case O_TAY: selX = A_; selD = dY; gm = NZ; break;
+      case O_TXA: selX = X_; selD = dA; gm = NZ; break;
+      case O_TYA: selX = Y_; selD = dA; gm = NZ; break;
+      case O_CLC: gm = FL_C; break;
+      case O_SEC: gm = FL_C; inv = 0xFF; one = 1; break;  // 0 + FF + 1 carries
+      case O_BCS: bm = 0x100; break;
+      case O_BCC: bm = 0x100; binv = 1; break;
+      case O_BNE: bm = FL_Z; break;
+      case O_BEQ: bm = FL_Z; binv = 1; break;
+      case O_BMI: bm = FL_N; break;
+      case O_BPL: bm = FL_N; binv = 1; break;
+      // a branch always taken: base = the operand, the taken branch's cycle counted
+      case O_JMP: if (mode == ABS) { binv = 1; cyc = 2; } else slow = true; break;
       case O_NOP: if (mode != IMP && mode != IMM) slow = true; break;  // its operand read may switch a bank
-      default: slow = true; break;  // stack operations, SEI, SED, undocumented opcodes
+      default: slow = true; break;  // stack operations, BIT, BVC, BVS, other flag operations, undocumented opcodes
     }
-    if (op == O_JMP) mem = false;
+    if (op == O_JMP) em = 0;
     if (mode == ACC) selD = dA;
-    if (slow && o != CTL_HALT) {  // nothing happens here: the lane waits for the general decoder
-      selD = 0x3210; pm = bm = binv = 0; ld = st = rmw = false;
-      cb |= CT_SLOW;
+    if (slow) {  // nothing happens here: the lane waits for the general decoder
+      selD = 0x3210; gm = bm = binv = vset = regions = 0; ld = st = rmw = false;
+    } else if (ld) {
+      regions = RG_RAM | RG_CART; selV = 0x3210;
+    } else if (st) {
+      regions = RG_RAM | RG_TIA; wr = RG_WRAM | RG_WTIA; selV = 0x1111;  // operand 0: the result is x
+    } else if (rmw) {
+      regions = RG_RAM; wr = RG_WRAM; selV = 0x3210;
+    } else {
+      em = 0;  // no access: address 0, which every region list but an empty one takes
     }
-    cb |= (ld ? CT_MEM | CT_LD : 0u) | (st ? CT_ST : 0u) | (rmw ? CT_MEM | CT_RMW : 0u) | cyc << 8 | pen << 15 | k << 24;
-    const uint32_t w[4] = {selB | em << 16, selI | bm << 16 | binv << 24, selX | m2 << 16 | inv << 24,
-                           selD | pm << 16 | len << 28};
-    memcpy(out + 16 * o, w, 16);
-    memcpy(out + CTL_B_OFF + 4 * o, &cb, 4);
+    const uint32_t w[CTL_WORDS] = {selB, selI, selX, selD, selV | vset << 31, em, len | cyc << 16, bm,
+                                   gm, inv, k, selC | binv << 31, regions | wr, m2, pen << 8, (k == 513 ? 1u : 0u) | one << 16};
+    memcpy(out + CTL_STRIDE * o, w, CTL_STRIDE);
   }
 }
 

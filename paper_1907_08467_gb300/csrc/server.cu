@@ -339,8 +339,11 @@ int atari_server_create(const uint8_t *const *roms, const size_t *rom_sizes, con
 
   atari_config ec = *cfg;
   if (ec.envs_per_warp <= 0 || ec.envs_per_block <= 0) {
+    // ticks of a few hundred to some 20,000 envs in sessions of one cartridge each: work items of 64 envs spread a
+    // small tick over the SMs, and two blocks of paired CPU and TIA warps share an SM in a large one
     ec.envs_per_warp = 32;
-    ec.envs_per_block = 128;
+    ec.envs_per_block = 64;
+    if (ec.tia_warps == 0) ec.tia_warps = 2;
   }
   std::vector<int32_t> env_rom((size_t)slots, 0);
   std::vector<uint32_t> env_key((size_t)slots);
