@@ -904,6 +904,10 @@ int atari_env_create(const uint8_t *const *roms, const size_t *rom_sizes, const 
   cudaFree(d_work);
   cudaFree(d_snaps);
   if (rc) return bail(rc);
+  if (c.output_mode == ATARI_OUT_STACK) {
+    const cudaError_t e = cudaFuncSetAttribute(k_policy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)POLICY_SMEM);
+    if (e != cudaSuccess) return bail(fail(ATARI_ECUDA, std::string("policy kernel: ") + cudaGetErrorString(e)));
+  }
   if (c.form == ATARI_FORM_BATCHED) {
     if ((rc = setup_batched(E, img, dec))) return bail(rc);
   }
@@ -1353,7 +1357,7 @@ int atari_env_policy(atari_env *E, const uint8_t *d_obs, const uint16_t *d_weigh
   cudaStream_t s = (cudaStream_t)stream;
   {
     ProfScope p(E, ATARI_PROF_POLICY, s);
-    k_policy<<<(E->n + POLICY_TPB - 1) / POLICY_TPB, POLICY_TPB, 0, s>>>(d_obs, d_weights, E->d_state, d_actions,
+    k_policy<<<(E->n + POLICY_ENVS - 1) / POLICY_ENVS, POLICY_TPB, POLICY_SMEM, s>>>(d_obs, d_weights, E->d_state, d_actions,
                                                                       d_logits, nullptr, E->n, E->cfg.seed);
   }
   CUDA_TRY(cudaGetLastError());
@@ -1376,7 +1380,7 @@ int atari_env_rollout_ex(atari_env *E, const uint16_t *d_weights, int n_steps, u
     const int slot = (int)(((long long)ring_start + t) % ring_depth);
     {
       ProfScope p(E, ATARI_PROF_POLICY, s);
-      k_policy<<<(E->n + POLICY_TPB - 1) / POLICY_TPB, POLICY_TPB, 0, s>>>(
+      k_policy<<<(E->n + POLICY_ENVS - 1) / POLICY_ENVS, POLICY_TPB, POLICY_SMEM, s>>>(
           d_obs, d_weights, E->d_state, d_actions, nullptr, d_ring_mu ? d_ring_mu + (size_t)slot * E->n : nullptr,
           E->n, E->cfg.seed);
     }

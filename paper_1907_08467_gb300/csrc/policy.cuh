@@ -40,78 +40,162 @@ __device__ __forceinline__ float exp_cw(float x) {
   return __fmul_rn(p, __int_as_float((k + 127) << 23));
 }
 
-constexpr int POLICY_TPB = 64;     // envs (threads) per block
-constexpr int POLICY_DEPTH = 9;    // partial-sum stack entries: the tree over 512 slots has 9 levels
+// A block serves 128 envs with eight warps: warp p takes the chunk slots
+// i = p mod 8, a subtree of the halving tree (its levels h = 256 .. 8), and
+// every lane four envs, so that a weight read from shared memory (a 16-byte
+// load occupies the load path for four cycles of the SM, in which it could
+// issue 16 warp-wide multiply-adds) serves four envs' sums.  With one env a
+// lane the loads took four times the multiply-adds' time.  Two neighbouring
+// sums share one packed fp32x2 multiply-add.
+//
+// A subtree's 64 slots are visited in bit-reversed order, in which the two
+// slots the tree adds at every level are neighbours, so the tree is the one a
+// binary counter builds from left to right: the first of two leaves waits in
+// registers, and the pair's sum is pushed on a stack (two levels in shared
+// memory, the deeper, rarely touched ones in local memory) and added to the
+// entries below it as the carry of the pair number ripples.  The eight
+// subtree sums meet in the levels h = 4, 2, 1.  They are the same additions of
+// the same operands as the halving tree, hence the same bits.
+//
+// 16384 envs: 8.3 G multiply-adds are 0.21 ms at 152 SMs x 128 lanes x 2.07 GHz.
+// Measured 0.45 ms, 1.77 before (128 of the SMs hold a block, and the byte
+// conversions share the FMA pipe); a block takes the same time whatever the
+// number of envs it holds.
+constexpr int POLICY_PARTS = 8, POLICY_E = 4, POLICY_ENVS = 32 * POLICY_E, POLICY_TPB = 32 * POLICY_PARTS;
+constexpr int POLICY_V = POLICY_E * POLICY_A;             // sums a thread keeps
+constexpr int POLICY_WROW = 20;                           // floats per staged row of W (16-byte rows)
+constexpr int POLICY_WBUF = 64 * POLICY_WROW;             // floats per staged chunk
+constexpr int POLICY_LEVELS = 6;                          // stack entries of a subtree (its 32 pairs)
+constexpr size_t POLICY_SMEM = 4 * ((size_t)POLICY_PARTS * POLICY_WBUF + (size_t)2 * POLICY_V * POLICY_TPB);
 
-// One thread per env.  The tree's leaves (the 512 chunk slots, 441 chunks
-// and zero padding) are visited in bit-reversed slot order k -> c = rev9(k).
-// In that order the two slots the tree adds at every level (i and i + h)
-// are neighbours, so the tree is the one a binary counter builds from left
-// to right.  Each chunk partial is pushed on a stack and added to the entries
-// below it as the carry of k ripples (leaf k merges trailing_ones(k) times):
-// the same additions of the same operands as the halving tree, hence the same
-// bits.  The block stages chunk c of W, widened to fp32 (exact), in shared
-// memory once for all its envs; every env's 84x84x4 stack is read once.
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 // mu_out (may be null) receives the behaviour probability of the sampled
 // action, its weight over the total (fp32 division), for a V-trace buffer.
-__global__ void __launch_bounds__(POLICY_TPB) k_policy(const uint8_t *obs, const uint16_t *W, const uint8_t *state,
-                                                      uint8_t *actions, float *logits_out, float *mu_out, int n,
-                                                      uint64_t seed) {
-  __shared__ float wsm[64 * POLICY_A];
-  __shared__ float stk[POLICY_DEPTH * POLICY_A][POLICY_TPB];
-  const int t = threadIdx.x;
-  const int i = blockIdx.x * POLICY_TPB + t;
-  const bool live = i < n;
-  const uint8_t *xs = obs + (size_t)(live ? i : 0) * POLICY_K;  // idle threads read env 0 and discard it
+__global__ void __launch_bounds__(POLICY_TPB, 1) k_policy(const uint8_t *obs, const uint16_t *W, const uint8_t *state,
+                                                         uint8_t *actions, float *logits_out, float *mu_out, int n,
+                                                         uint64_t seed) {
+  extern __shared__ __align__(16) uint8_t g_smem[];
+  float *wsm = reinterpret_cast<float *>(g_smem) + (threadIdx.x >> 5) * POLICY_WBUF;
+  uint64_t *stk = reinterpret_cast<uint64_t *>(reinterpret_cast<float *>(g_smem) + POLICY_PARTS * POLICY_WBUF);
+  constexpr int H = POLICY_V / 2;  // packed sums
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+  const int env0 = blockIdx.x * POLICY_ENVS + lane;  // and + 32, + 64, + 96
+  const uint8_t *xs[POLICY_E];
+#pragma unroll
+  for (int e = 0; e < POLICY_E; ++e)  // idle lanes read env 0 and discard it
+    xs[e] = obs + (size_t)(env0 + 32 * e < n ? env0 + 32 * e : 0) * POLICY_K;
+  const bool words = (reinterpret_cast<uintptr_t>(W) & 3u) == 0;  // W in 4-byte loads
+  uint64_t acc[H], first[H], deep[POLICY_LEVELS - 2][H];
   int sp = 0;
 #pragma unroll 1
-  for (uint32_t k = 0; k < 512; ++k) {
-    const uint32_t c = __brev(k) >> 23;
-    float acc[POLICY_A];
+  for (uint32_t k = 0; k < 64; ++k) {
+    const uint32_t c = (__brev(k) >> 26) * POLICY_PARTS + part;
 #pragma unroll
-    for (int j = 0; j < POLICY_A; ++j) acc[j] = 0.0f;
-    if (c < (uint32_t)POLICY_CHUNKS) {  // the same for every thread of the block
-      __syncthreads();                  // the previous chunk's readers are done
+    for (int q = 0; q < H; ++q) acc[q] = 0;
+    if (c < (uint32_t)POLICY_CHUNKS) {  // the same for every lane of the warp
       const uint16_t *wc = W + (size_t)c * 64 * POLICY_A;
-      for (int q = t; q < 64 * POLICY_A; q += POLICY_TPB) wsm[q] = __uint_as_float((uint32_t)wc[q] << 16);
-      __syncthreads();
-      const uint4 *x4 = reinterpret_cast<const uint4 *>(xs + (size_t)c * 64);
+      __syncwarp();  // the previous chunk's readers are done
+#pragma unroll
+      for (int t = 0; t < POLICY_A; ++t) {
+        const int q = 2 * (t * 32 + lane);  // pairs do not straddle rows: POLICY_A is even
+        const uint32_t w2 = words ? *reinterpret_cast<const uint32_t *>(wc + q) : wc[q] | (uint32_t)wc[q + 1] << 16;
+        *reinterpret_cast<float2 *>(wsm + q / POLICY_A * POLICY_WROW + q % POLICY_A) =
+            make_float2(__uint_as_float(w2 << 16), __uint_as_float(w2 & 0xFFFF0000u));
+      }
+      __syncwarp();
 #pragma unroll 1
       for (int q4 = 0; q4 < 4; ++q4) {
-        const uint4 xv4 = x4[q4];
-        const uint32_t xw[4] = {xv4.x, xv4.y, xv4.z, xv4.w};
+        uint4 xv[POLICY_E];
+#pragma unroll
+        for (int e = 0; e < POLICY_E; ++e) xv[e] = reinterpret_cast<const uint4 *>(xs[e] + (size_t)c * 64)[q4];
 #pragma unroll
         for (int b = 0; b < 16; ++b) {
-          const float xv = (float)((xw[b >> 2] >> (8 * (b & 3))) & 0xFF);
-          const float *wr = wsm + (q4 * 16 + b) * POLICY_A;
+          const float *wr = wsm + (q4 * 16 + b) * POLICY_WROW;
+          uint64_t w[POLICY_A / 2];
 #pragma unroll
-          for (int j = 0; j < POLICY_A; ++j) acc[j] = __fmaf_rn(xv, wr[j], acc[j]);
+          for (int j = 0; j < POLICY_A / 4; ++j) {
+            const ulonglong2 v = reinterpret_cast<const ulonglong2 *>(wr)[j];
+            w[2 * j] = v.x;
+            w[2 * j + 1] = v.y;
+          }
+          w[POLICY_A / 2 - 1] = reinterpret_cast<const uint64_t *>(wr)[POLICY_A / 2 - 1];
+#pragma unroll
+          for (int e = 0; e < POLICY_E; ++e) {
+            const uint32_t xw = (b >> 2) == 0 ? xv[e].x : (b >> 2) == 1 ? xv[e].y : (b >> 2) == 2 ? xv[e].z : xv[e].w;
+            // 2^23 + byte as fp32 bits, less 2^23: the byte, exactly
+            const float x = __fsub_rn(__uint_as_float(__byte_perm(xw, 0x4B000000u, 0x7440u | (b & 3))), 8388608.0f);
+            uint64_t x2;
+            asm("mov.b64 %0, {%1, %1};" : "=l"(x2) : "f"(x));
+#pragma unroll
+            for (int j = 0; j < POLICY_A / 2; ++j) acc[e * (POLICY_A / 2) + j] = fma2(x2, w[j], acc[e * (POLICY_A / 2) + j]);
+          }
         }
       }
     }
-#pragma unroll 1
-    for (uint32_t m = __ffs(~k) - 1; m > 0; --m) {
-      --sp;
+    if ((k & 1u) == 0) {
 #pragma unroll
-      for (int j = 0; j < POLICY_A; ++j) acc[j] = __fadd_rn(stk[sp * POLICY_A + j][t], acc[j]);
+      for (int q = 0; q < H; ++q) first[q] = acc[q];
+      continue;
     }
 #pragma unroll
-    for (int j = 0; j < POLICY_A; ++j) stk[sp * POLICY_A + j][t] = acc[j];
+    for (int q = 0; q < H; ++q) acc[q] = add2(first[q], acc[q]);
+#pragma unroll 1
+    for (uint32_t m = __ffs(~(k >> 1)) - 1; m > 0; --m) {
+      --sp;
+      if (sp < 2) {
+#pragma unroll
+        for (int q = 0; q < H; ++q) acc[q] = add2(stk[(size_t)(sp * H + q) * POLICY_TPB + threadIdx.x], acc[q]);
+      } else {
+#pragma unroll
+        for (int q = 0; q < H; ++q) acc[q] = add2(deep[sp - 2][q], acc[q]);
+      }
+    }
+    if (sp < 2) {
+#pragma unroll
+      for (int q = 0; q < H; ++q) stk[(size_t)(sp * H + q) * POLICY_TPB + threadIdx.x] = acc[q];
+    } else {
+#pragma unroll
+      for (int q = 0; q < H; ++q) deep[sp - 2][q] = acc[q];
+    }
     ++sp;
   }
-  if (live) {
+  // entry 0 of every thread's stack is its subtree's sum
+  __syncthreads();
+  const int t = threadIdx.x;
+  const int i = blockIdx.x * POLICY_ENVS + t;
+  if (t < POLICY_ENVS && i < n) {
     float l[POLICY_A];
-    float m = stk[0][t];
+    const int e = t >> 5;
 #pragma unroll
-    for (int j = 0; j < POLICY_A; ++j) {
-      l[j] = stk[j][t];
-      m = l[j] > m ? l[j] : m;
+    for (int jj = 0; jj < POLICY_A / 2; ++jj) {
+      uint64_t v[POLICY_PARTS];
+#pragma unroll
+      for (int p = 0; p < POLICY_PARTS; ++p) v[p] = stk[(size_t)(e * (POLICY_A / 2) + jj) * POLICY_TPB + p * 32 + lane];
+#pragma unroll
+      for (int h = POLICY_PARTS / 2; h > 0; h >>= 1)
+#pragma unroll
+        for (int p = 0; p < h; ++p) v[p] = add2(v[p], v[p + h]);
+      l[2 * jj] = __uint_as_float((uint32_t)v[0]);
+      l[2 * jj + 1] = __uint_as_float((uint32_t)(v[0] >> 32));
     }
-    float e[POLICY_A], tot = 0.0f;
+    float m = l[0];
+#pragma unroll
+    for (int j = 0; j < POLICY_A; ++j) m = l[j] > m ? l[j] : m;
+    float ex[POLICY_A], tot = 0.0f;
 #pragma unroll
     for (int j = 0; j < POLICY_A; ++j) {
-      e[j] = exp_cw(__fsub_rn(l[j], m));
-      tot = __fadd_rn(tot, e[j]);
+      ex[j] = exp_cw(__fsub_rn(l[j], m));
+      tot = __fadd_rn(tot, ex[j]);
     }
     const uint8_t *st = state + (size_t)i * 256;
     const uint32_t *ew = reinterpret_cast<const uint32_t *>(st + S::EPISODE);
@@ -121,16 +205,16 @@ __global__ void __launch_bounds__(POLICY_TPB) k_policy(const uint8_t *obs, const
     int act = -1, last = 0;
 #pragma unroll
     for (int j = 0; j < POLICY_A; ++j) {
-      c = __fadd_rn(c, e[j]);
-      if (e[j] > 0.0f) last = j;
+      c = __fadd_rn(c, ex[j]);
+      if (ex[j] > 0.0f) last = j;
       if (act < 0 && c > thr) act = j;
     }
     const int a = act < 0 ? last : act;
     actions[i] = (uint8_t)a;
     if (mu_out) {
-      float ea = e[0];
+      float ea = ex[0];
 #pragma unroll
-      for (int j = 1; j < POLICY_A; ++j) ea = j == a ? e[j] : ea;
+      for (int j = 1; j < POLICY_A; ++j) ea = j == a ? ex[j] : ea;
       mu_out[i] = __fdiv_rn(ea, tot);
     }
     if (logits_out) {
