@@ -1417,7 +1417,7 @@ int atari_nstep_returns(const float *d_rewards, const uint8_t *d_dones, int ring
   if (int rc = check_rollout_args(d_rewards, d_dones, ring_depth, ring_start, d_values, T, n, gamma)) return rc;
   if (n == 0) return 0;
   if (!d_returns) return fail(ATARI_EINVAL, "NULL buffer");
-  k_nstep_returns<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(d_rewards, d_dones, ring_depth,
+  k_nstep_returns<<<(n + TARGET_TPB - 1) / TARGET_TPB, TARGET_TPB, 0, (cudaStream_t)stream>>>(d_rewards, d_dones, ring_depth,
                                                                      ring_start % ring_depth, d_values, T, n, gamma,
                                                                      d_returns);
   CUDA_TRY(cudaGetLastError());
@@ -1432,7 +1432,7 @@ int atari_vtrace(const float *d_rewards, const uint8_t *d_dones, const float *d_
   if (!(c_bar >= 0.0f && rho_bar >= c_bar)) return fail(ATARI_EINVAL, "need rho_bar >= c_bar >= 0");
   if (n == 0) return 0;
   if (!d_mu || !d_pi || !d_vs || !d_pg_adv) return fail(ATARI_EINVAL, "NULL buffer");
-  k_vtrace<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(d_rewards, d_dones, d_mu, ring_depth,
+  k_vtrace<<<(n + TARGET_TPB - 1) / TARGET_TPB, TARGET_TPB, 0, (cudaStream_t)stream>>>(d_rewards, d_dones, d_mu, ring_depth,
                                                               ring_start % ring_depth, d_values, d_pi, T, n, gamma,
                                                               rho_bar, c_bar, d_vs, d_pg_adv);
   CUDA_TRY(cudaGetLastError());
