@@ -12,7 +12,8 @@
 // lanes applied every record to 32 copies of the registers, 182,482
 // warp-instructions per env-step on the banked workload, at two thirds of the
 // issue slots.  Painting, maximum and resampling of 32768 envs went from 7.1
-// to 2.4 ms with it, of 4096 sprite envs from 0.85 to 0.27 ms.
+// to 2.4 ms with it, of 4096 sprite envs from 0.85 to 0.27 ms.  Keeping each
+// object's mask and rebuilding only what a write staled: 2.17 and 0.24 ms.
 #pragma once
 #include <cstdint>
 
@@ -27,26 +28,39 @@ constexpr uint32_t ROW_WORDS = 42;            // 40 words of pixels; with the sk
 __device__ __forceinline__ uint32_t row_off(uint32_t r) { return 4u * (ROW_WORDS * r + 2u * (r / BAND_ROWS)); }
 constexpr uint32_t PAINT_FRAME = 4 * (ROW_WORDS * FRAME_H + 2 * BANDS);  // bytes of a frame in shared memory
 
-// What a register write does to the picture: slot of the register file, and
-// 0x40 = the classes may change, 0x80 = the colours may change, 0xC0 = needs
-// its own case.
+// Objects whose masks a register write can change.
+constexpr uint32_t OB_A = 1u, OB_B = 2u, OB_BL = 4u, OB_PF = 8u, OB_ALL = 15u;  // player and missile 0, 1, ball, playfield
+// What a register write does to the picture: its slot of the register file,
+// 0x40 = it only sets that slot, 0x80 = the colours may change too, 0xC0 = it
+// needs its own case; the objects it may change << 8.
 __device__ __forceinline__ uint32_t paint_reg(uint32_t reg) {
-  if (reg < 0x10) {
-    if (reg == 0x01 || (reg >= 0x06 && reg <= 0x09)) return 0x80u | (reg == 1 ? (uint32_t)T_VBLANK : reg - 2);
-    return 0x40u | (reg - 2);                     // NUSIZ0 .. PF2 (0x02, 0x03 and VSYNC are never logged)
+  switch (reg) {
+    case 0x01: return 0x80u | T_VBLANK;
+    case 0x04: return 0x40u | T_NUSIZ0 | OB_A << 8;
+    case 0x05: return 0x40u | T_NUSIZ1 | OB_B << 8;
+    case 0x06: case 0x07: case 0x08: case 0x09: return 0x80u | (reg - 2);
+    case 0x0A: return 0x40u | T_CTRLPF | (OB_BL | OB_PF) << 8;
+    case 0x0B: return 0x40u | T_REFP0 | OB_A << 8;
+    case 0x0C: return 0x40u | T_REFP1 | OB_B << 8;
+    case 0x0D: case 0x0E: case 0x0F: return 0x40u | (reg - 2) | OB_PF << 8;
+    case 0x1D: return 0x40u | T_ENAM0 | OB_A << 8;
+    case 0x1E: return 0x40u | T_ENAM1 | OB_B << 8;
+    case 0x10: case 0x12: case 0x25: case 0x28: return 0xC0u | OB_A << 8;
+    case 0x11: case 0x13: case 0x26: case 0x29: return 0xC0u | OB_B << 8;
+    case 0x14: case 0x1F: case 0x27: return 0xC0u | OB_BL << 8;
+    case 0x1B: case 0x1C: return 0xC0u;  // the graphics shown depend on the vertical delays
+    case 0x2A: return 0xC0u | (OB_A | OB_B | OB_BL) << 8;
+    default: return reg >= 0x20 && reg <= 0x24 ? 0x40u | (T_HMP0 + reg - 0x20) : 0xC0u;
   }
-  if (reg == 0x1D || reg == 0x1E) return 0x40u | (T_ENAM0 + reg - 0x1D);
-  if (reg >= 0x20 && reg <= 0x24) return T_HMP0 + reg - 0x20;
-  return 0xC0u;
 }
 
 // Offsets into shared memory of what the threads of a block share.
 struct PaintTabs {
   uint32_t luma;    // 128 bytes: colour index -> output byte
-  uint32_t regs;    // 64 bytes: paint_reg()
+  uint32_t regs;    // 64 half words: paint_reg()
   uint32_t spread;  // 256 words: bit i -> bit 4 i
 };
-constexpr uint32_t PAINT_TABS = 128 + 64 + 1024;
+constexpr uint32_t PAINT_TABS = 128 + 128 + 1024;
 __device__ __forceinline__ uint32_t spread_nibbles(uint32_t b) {
   uint32_t x = (b | b << 12) & 0x000F000Fu;
   x = (x | x << 6) & 0x03030303u;
@@ -64,9 +78,9 @@ struct RowPainter {
   PaintTabs tabs;
   uint32_t file;       // offset of this thread's register file
   uint32_t bar;        // frame-relative line of the HMOVE bar, or 0xFFFF
-  uint32_t f0[5], f1[5];  // class planes of a whole row under the current registers
+  uint32_t a[5], b[5], l[5], f[5];  // masks: player and missile 0, player and missile 1, ball, playfield
   uint32_t c0[5], c1[5];  // class planes of the row being painted
-  bool fresh;          // f0, f1 are up to date
+  uint32_t stale;      // OB_*: the masks that the registers have left behind
 
   __device__ __forceinline__ uint32_t F(uint32_t s) const { return sm8(file + s); }
   __device__ __forceinline__ void Fset(uint32_t s, uint32_t v) const { sm8(file + s) = (uint8_t)v; }
@@ -76,51 +90,52 @@ struct RowPainter {
     const M160 r = rot160(u, pos);
     m[0] |= r.w0; m[1] |= r.w1; m[2] |= r.w2; m[3] |= r.w3; m[4] |= r.w4;
   }
-  // Class planes from the registers.  Normal priority: player 0 and missile 0
-  // (class 1), then player 1 and missile 1 (class 2), then playfield and ball
-  // (class 3), then background (class 0); in score mode the playfield takes
-  // class 1 left of column 80 and 2 right of it, and the ball shows where
-  // there is no playfield.  Playfield priority (CTRLPF bit 2): playfield and
-  // ball first, score mode off.
+  // Rebuild the stale masks.  A write stales one object as a rule, and the
+  // rows of a warp's threads, two apart, stale the same one at the same time.
   __device__ __forceinline__ void refresh() {
-    uint32_t a[5] = {0, 0, 0, 0, 0}, b[5] = {0, 0, 0, 0, 0}, l[5] = {0, 0, 0, 0, 0};
     const uint32_t ctrl = F(T_CTRLPF);
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
+      if (!(stale & (p ? OB_B : OB_A))) continue;
       uint32_t *m = p ? b : a;
+#pragma unroll
+      for (int w = 0; w < 5; ++w) m[w] = 0;
       const uint32_t nus = F(T_NUSIZ0 + p);
       const uint32_t g = p ? ((F(T_VDELP1) & 1) ? F(T_GRP1_O) : F(T_GRP1_N)) : ((F(T_VDELP0) & 1) ? F(T_GRP0_O) : F(T_GRP0_N));
       if (g) place(m, player_base(g, F(T_REFP0 + p), nus), F(T_P0 + p));
       if ((F(T_ENAM0 + p) & 2) && !(F(T_RESMP0 + p) & 2)) place(m, missile_base(nus), F(T_M0 + p));
     }
-    if (((F(T_VDELBL) & 1) ? F(T_ENABL_O) : F(T_ENABL_N)) & 2) place(l, ball_base(ctrl), F(T_BL));
-    const M160 pf = pf_mask(F(T_PF0), F(T_PF1), F(T_PF2), ctrl);
-    const uint32_t f[5] = {pf.w0, pf.w1, pf.w2, pf.w3, pf.w4};
-    const bool pfp = (ctrl & 4) != 0;
+    if (stale & OB_BL) {
+#pragma unroll
+      for (int w = 0; w < 5; ++w) l[w] = 0;
+      if (((F(T_VDELBL) & 1) ? F(T_ENABL_O) : F(T_ENABL_N)) & 2) place(l, ball_base(ctrl), F(T_BL));
+    }
+    if (stale & OB_PF) {
+      const M160 pf = pf_mask(F(T_PF0), F(T_PF1), F(T_PF2), ctrl);
+      f[0] = pf.w0; f[1] = pf.w1; f[2] = pf.w2; f[3] = pf.w3; f[4] = pf.w4;
+    }
+    stale = 0;
+  }
+  // Columns [x0, x1) of the row take the current registers' classes.  Normal
+  // priority: player 0 and missile 0 (class 1), then player 1 and missile 1
+  // (class 2), then playfield and ball (class 3), then background (class 0);
+  // in score mode the playfield takes class 1 left of column 80 and 2 right of
+  // it, and the ball shows where there is no playfield.  Playfield priority
+  // (CTRLPF bit 2): playfield and ball first, score mode off.
+  __device__ __forceinline__ void take(uint32_t x0, uint32_t x1) {
+    if (stale) refresh();
+    const uint32_t ctrl = F(T_CTRLPF);
+    const uint32_t front = (ctrl & 4) ? ~0u : 0u;
     const uint32_t score = (ctrl & 6) == 2 ? ~0u : 0u;
 #pragma unroll
     for (int w = 0; w < 5; ++w) {
+      const uint32_t m = below(x1, w) & ~below(x0, w);
       const uint32_t right = score & (w < 2 ? 0u : w == 2 ? 0xFFFF0000u : ~0u), left = score & ~right;
-      const uint32_t ab = a[w] | b[w], both = l[w] & ~(f[w] & score);
-      const uint32_t lo = (f[w] & ~right) | both, hi = (f[w] & ~left) | both, all = f[w] | l[w];
-      f0[w] = a[w] | (pfp ? all : lo & ~ab);
-      f1[w] = (b[w] & ~a[w]) | (pfp ? all : hi & ~ab);
-    }
-    fresh = true;
-  }
-  // Columns [x0, x1) of the row take the current registers' classes.
-  __device__ __forceinline__ void take(uint32_t x0, uint32_t x1) {
-    if (!fresh) refresh();
-    if (x0 == 0 && x1 == 160) {
-#pragma unroll
-      for (int w = 0; w < 5; ++w) { c0[w] = f0[w]; c1[w] = f1[w]; }
-      return;
-    }
-#pragma unroll
-    for (int w = 0; w < 5; ++w) {
-      const uint32_t m = range_word(w, x0, x1);
-      c0[w] = (c0[w] & ~m) | (f0[w] & m);
-      c1[w] = (c1[w] & ~m) | (f1[w] & m);
+      const uint32_t ab = (a[w] | b[w]) & ~front, both = l[w] & ~(f[w] & score);
+      const uint32_t lo = (f[w] & ~right) | both, hi = (f[w] & ~left) | both;
+      const uint32_t n0 = a[w] | (lo & ~ab), n1 = (b[w] & ~a[w]) | (hi & ~ab);
+      c0[w] = (c0[w] & ~m) | (n0 & m);
+      c1[w] = (c1[w] & ~m) | (n1 & m);
     }
   }
   // The four class colours as output bytes.
@@ -185,7 +200,7 @@ struct RowPainter {
 #pragma unroll
     for (int q = 0; q < 10; ++q) sm32(file + 4u * q) = w[q];
     bar = c.y >> 16;
-    fresh = false;
+    stale = OB_ALL;
     return c.z;
   }
 
@@ -215,40 +230,44 @@ struct RowPainter {
         while ((rec >> 14) < cl + 228u) {
           const uint32_t clk = rec >> 14, reg = (rec >> 8) & 0x3Fu, v = rec & 0xFFu;
           const uint32_t x = clk > cl + 68u ? clk - cl - 68u : 0u;
-          const uint32_t info = sm8(tabs.regs + reg);
+          const uint32_t word = *reinterpret_cast<const uint16_t *>(&sm8(tabs.regs + 2u * reg));
+          const uint32_t info = word & 0xFFu;
           uint32_t slot = info & 0x3Fu, val = v;
-          bool planes = false;
+          uint32_t hit = word >> 8;  // the objects that change
           if (info < 0xC0u) {
             const bool change = F(slot) != v;
             if (change & ((info & 0x80u) != 0) & (x > xe)) { stop = x; break; }
-            planes = change & ((info & 0x40u) != 0);
-            if (planes & (x > xs)) { stop = x; colour = false; break; }
+            if (!change) hit = 0;
           } else {
-            uint32_t from = T_VSYNC, to = T_VSYNC;  // a delayed copy that the write makes
+            uint32_t from, to;  // the delayed copy that the write makes
             switch (reg) {
               // GRP0 sets P0's new graphic and copies P1's new graphic to its old one (shown when the vertical
               // delay is on); GRP1 likewise, and the ball's enable to its delayed copy
               case 0x1B:
                 slot = T_GRP0_N; from = T_GRP1_N; to = T_GRP1_O;
-                planes = (!(F(T_VDELP0) & 1) && v != F(slot)) || ((F(T_VDELP1) & 1) && F(from) != F(to));
+                hit = (!(F(T_VDELP0) & 1) && v != F(slot) ? OB_A : 0u) | ((F(T_VDELP1) & 1) && F(from) != F(to) ? OB_B : 0u);
                 break;
               case 0x1C:
                 slot = T_GRP1_N; from = T_GRP0_N; to = T_GRP0_O;
-                planes = (!(F(T_VDELP1) & 1) && v != F(slot)) || ((F(T_VDELP0) & 1) && F(from) != F(to)) ||
-                         ((F(T_VDELBL) & 1) && ((F(T_ENABL_O) ^ F(T_ENABL_N)) & 2));
+                hit = (!(F(T_VDELP1) & 1) && v != F(slot) ? OB_B : 0u) | ((F(T_VDELP0) & 1) && F(from) != F(to) ? OB_A : 0u) |
+                      ((F(T_VDELBL) & 1) && ((F(T_ENABL_O) ^ F(T_ENABL_N)) & 2) ? OB_BL : 0u);
                 break;
-              case 0x1F: slot = T_ENABL_N; planes = !(F(T_VDELBL) & 1) && ((F(slot) ^ v) & 2); break;
+              case 0x1F: slot = T_ENABL_N; hit = !(F(T_VDELBL) & 1) && ((F(slot) ^ v) & 2) ? hit : 0u; break;
               case 0x10: case 0x11: case 0x12: case 0x13: case 0x14:
                 slot = T_P0 + reg - 0x10;
                 val = reg < 0x12 ? fc_res_pos(clk, 5, 3) : fc_res_pos(clk, 4, 2);
-                planes = F(slot) != val;
+                hit = F(slot) != val ? hit : 0u;
                 break;
-              case 0x25: case 0x26: case 0x27: slot = T_VDELP0 + reg - 0x25; planes = ((F(slot) ^ v) & 1) != 0; break;
-              case 0x28: case 0x29: slot = T_RESMP0 + reg - 0x28; planes = true; break;
-              default: slot = T_VSYNC; planes = reg == 0x2A; break;  // HMOVE, HMCLR
+              case 0x25: case 0x26: case 0x27: slot = T_VDELP0 + reg - 0x25; hit = ((F(slot) ^ v) & 1) ? hit : 0u; break;
+              case 0x28: case 0x29: slot = T_RESMP0 + reg - 0x28; break;
+              default: slot = T_VSYNC; break;  // HMOVE, HMCLR
             }
-            if (planes & (x > xs)) { stop = x; colour = false; break; }
-            Fset(to, F(from));
+          }
+          if ((hit != 0) & (x > xs)) { stop = x; colour = false; break; }
+          if (info >= 0xC0u) {
+            if (reg == 0x1B || reg == 0x1C) {  // the delayed copies
+              Fset(reg == 0x1B ? T_GRP1_O : T_GRP0_O, F(reg == 0x1B ? T_GRP1_N : T_GRP0_N));
+            }
             if (reg == 0x1C) Fset(T_ENABL_O, F(T_ENABL_N));
             if (reg >= 0x28) {
               if (reg == 0x2A) {
@@ -262,7 +281,7 @@ struct RowPainter {
               }
             }
           }
-          if (planes) fresh = false;
+          stale |= hit;
           Fset(slot, val);
           ++ri;
           rec = ahead;
@@ -282,7 +301,7 @@ struct RowPainter {
 // The threads' register-effect and spread tables, and the colour table.
 __device__ __forceinline__ void paint_tables(const PaintTabs &t, const uint8_t *luma) {
   for (uint32_t i = threadIdx.x; i < 128; i += blockDim.x) sm8(t.luma + i) = luma ? luma[i] : (uint8_t)(2 * i);
-  for (uint32_t i = threadIdx.x; i < 64; i += blockDim.x) sm8(t.regs + i) = (uint8_t)paint_reg(i);
+  for (uint32_t i = threadIdx.x; i < 64; i += blockDim.x) *reinterpret_cast<uint16_t *>(&sm8(t.regs + 2 * i)) = (uint16_t)paint_reg(i);
   for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) sm32(t.spread + 4 * i) = spread_nibbles(i);
 }
 
