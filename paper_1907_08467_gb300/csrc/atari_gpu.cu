@@ -1021,7 +1021,7 @@ int launch_batched(atari_env *E, const uint8_t *d_actions, uint8_t *d_obs, int32
   CUDA_TRY(cudaGetLastError());
   if (c.output_mode == ATARI_OUT_STACK) {
     ProfScope p(E, ATARI_PROF_FUSED, s);
-    k_raster_preprocess<<<E->n, PAINT_THREADS, PAINT_SMEM, s>>>(E->d_log, E->d_bsnap, E->d_meta, E->d_luma, E->d_ring,
+    k_raster_preprocess<<<E->n, PAINT_THREADS + 32, PAINT_SMEM, s>>>(E->d_log, E->d_bsnap, E->d_meta, E->d_luma, E->d_ring,
                                                                  E->d_head, E->d_done, d_obs, E->n, c.log_cap, nullptr,
                                                                  nullptr, 0);
   } else if (d_obs) {
@@ -1241,7 +1241,7 @@ int step_host_overlapped(atari_env *E, uint8_t *obs, int32_t *rewards, uint8_t *
     const int b0 = (int)((int64_t)n * k / chunks), b1 = (int)((int64_t)n * (k + 1) / chunks);
     {
       ProfScope p(E, ATARI_PROF_FUSED, s);
-      k_raster_preprocess<<<b1 - b0, PAINT_THREADS, PAINT_SMEM, s>>>(E->d_log, E->d_bsnap, E->d_meta, E->d_luma,
+      k_raster_preprocess<<<b1 - b0, PAINT_THREADS + 32, PAINT_SMEM, s>>>(E->d_log, E->d_bsnap, E->d_meta, E->d_luma,
                                                                      E->d_ring, E->d_head, E->d_done, E->d_obs_tmp, n,
                                                                      c.log_cap, nullptr, nullptr, b0);
     }
@@ -1690,7 +1690,7 @@ int serve_tick(atari_env *E, const ServeTick &t, cudaStream_t s) {
   const int grid = std::max(1, std::min(t.n_groups, E->max_blocks));
   launch_interp(E, a, grid, s);
   CUDA_TRY(cudaGetLastError());
-  k_raster_preprocess<<<t.n_active, PAINT_THREADS, PAINT_SMEM, s>>>(E->d_log, E->d_bsnap, E->d_meta, E->d_luma, E->d_ring,
+  k_raster_preprocess<<<t.n_active, PAINT_THREADS + 32, PAINT_SMEM, s>>>(E->d_log, E->d_bsnap, E->d_meta, E->d_luma, E->d_ring,
                                                                     E->d_head, E->d_done, t.d_obs, t.n_active,
                                                                     c.log_cap, a.perm, a.opos, 0);
   CUDA_TRY(cudaGetLastError());

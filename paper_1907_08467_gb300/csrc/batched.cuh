@@ -322,36 +322,44 @@ __global__ void __launch_bounds__(256) k_group_by_bank(const uint8_t *state, con
 }
 
 // Shared memory of the painting kernels: the frame, the threads' register
-// files, the tables.
-constexpr int PAINT_THREADS = 128;
+// files, the tables.  A warp paints 30 bands, 60 rows, which are 24 output rows
+// of the resampling, so that warps need not wait for one another.
+constexpr int PAINT_BANDS = 30, PAINT_WARPS = 4, PAINT_THREADS = 32 * PAINT_WARPS;
 constexpr uint32_t PAINT_FILES = PAINT_FRAME, PAINT_LUT = PAINT_FILES + PAINT_THREADS * FILE_STRIDE;
 constexpr uint32_t PAINT_SMEM = PAINT_LUT + PAINT_TABS;
-static_assert(PAINT_THREADS >= (int)BANDS, "one thread per band");
+static_assert(PAINT_BANDS * PAINT_WARPS >= (int)BANDS && PAINT_BANDS * BAND_ROWS % 5 == 0, "warps cover the frame in fives of rows");
 __device__ __forceinline__ RowPainter painter() {
   RowPainter p;
-  p.tabs = PaintTabs{PAINT_LUT + 1024, PAINT_LUT + 1024 + 128, PAINT_LUT};
-  p.file = PAINT_FILES + threadIdx.x * FILE_STRIDE;
+  p.tabs = PaintTabs{PAINT_LUT + 1024, PAINT_LUT + 1152, PAINT_LUT, PAINT_LUT + 1280};
+  p.file = PAINT_FILES + (threadIdx.x & (PAINT_THREADS - 1)) * FILE_STRIDE;
   return p;
 }
-// Frame slot (0: F-1, 1: F) of env i: this thread's band, into the frame in shared memory.
-template <bool MAX>
-__device__ __forceinline__ void paint_frame(RowPainter &p, int i, int slot, int first_slot, const uint32_t *log,
-                                            const uint8_t *bsnap, const uint32_t *meta, int log_cap) {
-  const uint32_t band = threadIdx.x;
-  if (band >= BANDS) return;
-  const uint32_t *mt = meta + (size_t)i * 4 + slot * 2;
-  const uint32_t n_rec = min(mt[0], (uint32_t)log_cap);
-  const size_t f = (size_t)i * (2 - first_slot) + (slot - first_slot);
-  const uint32_t ri = min(p.start(bsnap + (f * BANDS + band) * BAND_SNAP), n_rec);
+// Frames first_slot .. 1 (0: F-1, 1: F) of env i, one over the other: this
+// thread's band, into the frame in shared memory.
+__device__ __forceinline__ void paint_frames(RowPainter &p, int i, int first_slot, const uint32_t *log,
+                                             const uint8_t *bsnap, const uint32_t *meta, int log_cap) {
+  const uint32_t lane = threadIdx.x & 31, band = (threadIdx.x >> 5) * PAINT_BANDS + lane;
+  if (lane >= PAINT_BANDS || band >= BANDS) return;
   const uint32_t r0 = band * BAND_ROWS, r1 = min(r0 + BAND_ROWS, (uint32_t)FRAME_H);
-  p.paint<MAX>(r0, r1, mt[1], log + ((size_t)i * 2 + slot) * log_cap, ri, n_rec, 0);
+  const uint8_t *snap = bsnap + ((size_t)i * (2 - first_slot) * BANDS + band) * BAND_SNAP;
+  if (first_slot == 0) asm volatile("prefetch.global.L1 [%0];" ::"l"(snap + BANDS * BAND_SNAP));
+#pragma unroll 1
+  for (int slot = first_slot; slot < 2; ++slot) {
+    const uint32_t *mt = meta + (size_t)i * 4 + slot * 2;
+    const uint32_t *recs = log + ((size_t)i * 2 + slot) * log_cap;
+    const uint32_t n_rec = min(mt[0], (uint32_t)log_cap);
+    const uint32_t ri = min(p.start(snap), n_rec);
+    p.paint(slot != first_slot, r0, r1, mt[1], recs, ri, n_rec, 0);
+    snap += BANDS * BAND_SNAP;
+  }
 }
 
 // One block per env: the rows of frames F-1 and F as luma, their pixelwise
-// maximum, 84x84 area resampling, stack push.  A thread paints its rows of
-// frame F-1 and then frame F's over them, so one frame (36 KB) is kept and
-// five blocks fit an SM.
-__global__ void __launch_bounds__(PAINT_THREADS, 5)
+// maximum, 84x84 area resampling, stack push.  Four warps paint; a thread
+// paints its rows of frame F-1 and then frame F's over them, so one frame
+// (36 KB) is kept and five blocks fit an SM, and a warp resamples its own
+// rows.  The fifth warp copies the kept planes meanwhile.
+__global__ void __launch_bounds__(PAINT_THREADS + 32, 5)
     k_raster_preprocess(const uint32_t *log, const uint8_t *bsnap, const uint32_t *meta, const uint8_t *luma_g,
                         uint8_t *ring, uint8_t *head, const uint8_t *done, uint8_t *obs, int n, int log_cap,
                         const int32_t *perm, const int32_t *opos, int base) {
@@ -363,67 +371,67 @@ __global__ void __launch_bounds__(PAINT_THREADS, 5)
   const int o = opos ? opos[blk] : i;
   RowPainter p = painter();
   paint_tables(p.tabs, luma_g);
-  __syncthreads();
-  paint_frame<false>(p, i, 0, 0, log, bsnap, meta, log_cap);
-  paint_frame<true>(p, i, 1, 0, log, bsnap, meta, log_cap);
-  const uint32_t h = head[i];
-  const bool finished = done[i] != 0;
-  uint8_t *rg = ring + (size_t)i * 4 * 7056;
-  uint8_t *ob = obs ? obs + (size_t)o * 4 * 7056 : nullptr;
-  // the three kept planes, oldest first, to the stack
-  if (ob) {
-    for (int s = 0; s < 3; ++s) {
-      const uint4 *src = reinterpret_cast<const uint4 *>(rg + ((h + 1 + s) & 3) * 7056);
-      uint4 *dst = reinterpret_cast<uint4 *>(ob + s * 7056);
-      for (int q = threadIdx.x; q < 7056 / 16; q += PAINT_THREADS) dst[q] = src[q];
-    }
-  }
-  __syncthreads();  // the frame is painted and the kept planes are read
   // Resampling.  Output row i covers source rows [2.5 i, 2.5 i + 2.5), output
   // column j columns [160 j / 84, 160 (j + 1) / 84).  In units of 1/21 column
   // and 1/2 row the weights are whole numbers of at most 21 and 2, and the
   // area's weight is 40 x 5 = 200: out = (sum + 100) / 200, the same value as
-  // with 1/84 units and 33600.  A thread takes four columns and every sixth
-  // pair of output rows (five source rows): a column's three pixels are one
-  // byte dot product per source row.
-  const uint32_t m = threadIdx.x % 21u, k0 = threadIdx.x / 21u;
-  if (k0 < 6u) {
-    uint32_t wt[4], sh[4], at[4];
+  // with 1/84 units and 33600.
+  for (uint32_t c = threadIdx.x; c < 84u; c += blockDim.x) {
+    uint32_t x0, w0, w1, w2;
+    col_weights(c, x0, w0, w1, w2);
+    *reinterpret_cast<uint2 *>(&sm32(p.tabs.cols + 8u * c)) = make_uint2(x0, (w0 >> 2) | (w1 >> 2) << 8 | (w2 >> 2) << 16);
+  }
+  const uint32_t h = head[i];
+  const bool finished = done[i] != 0;
+  __syncthreads();  // the tables are built and the head is read
+  uint8_t *rg = ring + (size_t)i * 4 * 7056;
+  uint8_t *ob = obs ? obs + (size_t)o * 4 * 7056 : nullptr;
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp == PAINT_WARPS) {
+    // the three kept planes, oldest first, to the stack; a finished env's ring is cleared
+    if (ob) {
+      for (int s = 0; s < 3; ++s) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(rg + ((h + 1 + s) & 3) * 7056);
+        uint4 *dst = reinterpret_cast<uint4 *>(ob + s * 7056);
+#pragma unroll 7
+        for (uint32_t q = lane; q < 7056 / 16; q += 32) dst[q] = src[q];
+      }
+    }
+    __syncwarp();
+    if (finished) {
+      uint4 *z = reinterpret_cast<uint4 *>(rg);
+      for (uint32_t q = lane; q < 4 * 7056 / 16; q += 32) z[q] = make_uint4(0, 0, 0, 0);
+    }
+    if (lane == 0) head[i] = finished ? 0 : (uint8_t)((h + 1) & 3);
+    return;
+  }
+  paint_frames(p, i, 0, log, bsnap, meta, log_cap);
+  __syncwarp();
+  // A lane takes four columns of a pair of output rows (five source rows): a
+  // column's three pixels are one byte dot product per source row.
+  const uint32_t pairs = PAINT_BANDS * BAND_ROWS / 5, k0 = warp * pairs, nk = min(pairs, 42u - k0);
+  uint32_t *out0 = finished ? nullptr : reinterpret_cast<uint32_t *>(rg + h * 7056);
+  uint32_t *out1 = ob ? reinterpret_cast<uint32_t *>(ob + 3 * 7056) : nullptr;
+  for (uint32_t u = lane; u < 21u * nk; u += 32u) {
+    const uint32_t k = k0 + u / 21u, m = u % 21u;
+    uint32_t even = 0, odd = 0;
 #pragma unroll
     for (uint32_t c = 0; c < 4; ++c) {
-      uint32_t x0, w0, w1, w2;
-      col_weights(4u * m + c, x0, w0, w1, w2);
-      wt[c] = (w0 >> 2) | (w1 >> 2) << 8 | (w2 >> 2) << 16;
-      at[c] = x0 & ~3u;
-      sh[c] = 8u * (x0 & 3u);
-    }
-    uint32_t *out0 = reinterpret_cast<uint32_t *>(rg + h * 7056);
-    uint32_t *out1 = ob ? reinterpret_cast<uint32_t *>(ob + 3 * 7056) : nullptr;
-    for (uint32_t k = k0; k < 42u; k += 6u) {
-      uint32_t even = 0, odd = 0;
+      const uint2 col = *reinterpret_cast<const uint2 *>(&sm32(p.tabs.cols + 8u * (4u * m + c)));
+      const uint32_t at = col.x & ~3u, sh = col.x * 8u;  // the funnel shift takes it modulo 32
+      uint32_t px[5];
 #pragma unroll
-      for (uint32_t c = 0; c < 4; ++c) {
-        uint32_t px[5];
-#pragma unroll
-        for (uint32_t r = 0; r < 5; ++r) {
-          const uint32_t a = row_off(5u * k + r) + at[c];
-          px[r] = __funnelshift_r(sm32(a), sm32(a + 4), sh[c]);
-        }
-        const uint32_t mid = __dp4a(px[2], wt[c], 100u), w2 = wt[c] * 2u;
-        even |= __dp4a(px[0], w2, __dp4a(px[1], w2, mid)) / 200u << (8u * c);
-        odd |= __dp4a(px[4], w2, __dp4a(px[3], w2, mid)) / 200u << (8u * c);
+      for (uint32_t r = 0; r < 5; ++r) {
+        const uint32_t a = row_off(5u * k + r) + at;
+        px[r] = __funnelshift_r(sm32(a), sm32(a + 4), sh);
       }
-      const uint32_t q = 42u * k + m;  // word of output row 2 k
-      if (out1) { out1[q] = even; out1[q + 21] = odd; }
-      if (!finished) { out0[q] = even; out0[q + 21] = odd; }
+      const uint32_t mid = __dp4a(px[2], col.y, 100u), w2 = col.y * 2u;
+      even |= __dp4a(px[0], w2, __dp4a(px[1], w2, mid)) / 200u << (8u * c);
+      odd |= __dp4a(px[4], w2, __dp4a(px[3], w2, mid)) / 200u << (8u * c);
     }
-  }
-  if (finished) {
-    uint4 *z = reinterpret_cast<uint4 *>(rg);
-    for (int q = threadIdx.x; q < 4 * 7056 / 16; q += PAINT_THREADS) z[q] = make_uint4(0, 0, 0, 0);
-    if (threadIdx.x == 0) head[i] = 0;
-  } else if (threadIdx.x == 0) {
-    head[i] = (uint8_t)((h + 1) & 3);
+    const uint32_t q = 42u * k + m;  // word of output row 2 k
+    if (out1) { out1[q] = even; out1[q + 21] = odd; }
+    if (out0) { out0[q] = even; out0[q + 21] = odd; }
   }
 }
 
@@ -435,11 +443,12 @@ __global__ void __launch_bounds__(PAINT_THREADS, 5)
   RowPainter p = painter();
   paint_tables(p.tabs, nullptr);
   __syncthreads();
-  paint_frame<false>(p, i, 1, 1, log, bsnap, meta, log_cap);
-  __syncthreads();
+  paint_frames(p, i, 1, log, bsnap, meta, log_cap);
+  __syncwarp();
   uint32_t *dst = reinterpret_cast<uint32_t *>(obs + (size_t)i * (FRAME_H * FRAME_W));
-  for (uint32_t q = threadIdx.x; q < FRAME_H * FRAME_W / 4; q += PAINT_THREADS)
-    dst[q] = sm32(row_off(q / 40u) + 4u * (q % 40u));
+  const uint32_t rows = PAINT_BANDS * BAND_ROWS, q0 = (threadIdx.x >> 5) * rows * 40u;
+  const uint32_t q1 = min(q0 + rows * 40u, (uint32_t)(FRAME_H * FRAME_W / 4));
+  for (uint32_t q = q0 + (threadIdx.x & 31); q < q1; q += 32) dst[q] = sm32(row_off(q / 40u) + 4u * (q % 40u));
 }
 
 }  // namespace atari

@@ -14,6 +14,8 @@
 // issue slots.  Painting, maximum and resampling of 32768 envs went from 7.1
 // to 2.4 ms with it, of 4096 sprite envs from 0.85 to 0.27 ms.  Keeping each
 // object's mask and rebuilding only what a write staled: 2.17 and 0.24 ms.
+// Warps that resample their own rows, a fifth warp for the kept planes and one
+// copy of the code for both frames: 1.97 and 0.22 ms.
 #pragma once
 #include <cstdint>
 
@@ -59,8 +61,9 @@ struct PaintTabs {
   uint32_t luma;    // 128 bytes: colour index -> output byte
   uint32_t regs;    // 64 half words: paint_reg()
   uint32_t spread;  // 256 words: bit i -> bit 4 i
+  uint32_t cols;    // 84 pairs: source byte of an output column, its three weights in units of 1/21 column
 };
-constexpr uint32_t PAINT_TABS = 128 + 128 + 1024;
+constexpr uint32_t PAINT_TABS = 1024 + 128 + 128 + 672;
 __device__ __forceinline__ uint32_t spread_nibbles(uint32_t b) {
   uint32_t x = (b | b << 12) & 0x000F000Fu;
   x = (x | x << 6) & 0x03030303u;
@@ -152,10 +155,11 @@ struct RowPainter {
     return make_uint2(__byte_perm(pal, 0, sel), __byte_perm(pal, 0, sel >> 16));
   }
   // Write columns [x0, x1) of the row at byte offset `row`, x0 = 0 or where
-  // the last write of the row ended: stored, or (MAX) as the maximum with
-  // what is there.  barred: the HMOVE bar blanks columns 0..7.
-  template <bool MAX>
-  __device__ __forceinline__ void emit(uint32_t x0, uint32_t x1, uint32_t row, bool barred) {
+  // the last write of the row ended, as the maximum with what is there (over:
+  // a frame painted over another one) or with nothing.  barred: the HMOVE bar
+  // blanks columns 0..7.  Columns of a group that are left out are 0 until
+  // the next write of the row.
+  __device__ __forceinline__ void emit(bool over, uint32_t x0, uint32_t x1, uint32_t row, bool barred) {
     const uint32_t pal = palette();
     const uint32_t pal0 = barred ? sm8(tabs.luma) * 0x01010101u : pal;
     if (x0 == 0 && x1 == 160) {
@@ -164,7 +168,7 @@ struct RowPainter {
         uint2 p = pixels8(g == 0 ? pal0 : pal, (c0[g >> 2] >> (8 * (g & 3))) & 0xFFu,
                           (c1[g >> 2] >> (8 * (g & 3))) & 0xFFu, 0);
         uint2 *d = reinterpret_cast<uint2 *>(&sm32(row + 8u * g));
-        if (MAX) {
+        if (over) {
           const uint2 q = *d;
           p = make_uint2(max_u8x4(q.x, p.x), max_u8x4(q.y, p.y));
         }
@@ -179,16 +183,11 @@ struct RowPainter {
       const uint32_t p1 = w == 0 ? c1[0] : w == 1 ? c1[1] : w == 2 ? c1[2] : w == 3 ? c1[3] : c1[4];
       // columns of the group outside [x0, x1)
       const uint32_t off = (x0 > xa ? (1u << (x0 - xa)) - 1u : 0u) | (x1 < xa + 8u ? 0xFFu << (x1 - xa) & 0xFFu : 0u);
-      uint2 p = pixels8(g == 0 ? pal0 : pal, (p0 >> sh) & 0xFFu, (p1 >> sh) & 0xFFu, off | 0x100u);
+      const uint2 p = pixels8(g == 0 ? pal0 : pal, (p0 >> sh) & 0xFFu, (p1 >> sh) & 0xFFu, off | 0x100u);
       uint2 *d = reinterpret_cast<uint2 *>(&sm32(row + 8u * g));
-      if (MAX) {
-        const uint2 q = *d;
-        p = make_uint2(max_u8x4(q.x, p.x), max_u8x4(q.y, p.y));
-      } else if (x0 > xa) {
-        const uint2 q = *d;
-        p = make_uint2(q.x | p.x, q.y | p.y);
-      }
-      *d = p;
+      uint2 q = make_uint2(0, 0);
+      if (over | (x0 > xa)) q = *d;
+      *d = make_uint2(max_u8x4(q.x, p.x), max_u8x4(q.y, p.y));
     }
   }
 
@@ -205,9 +204,9 @@ struct RowPainter {
   }
 
   // Paint rows [r0, r1) of a frame of n_lines lines from its records
-  // [ri, n_rec) (clock << 14 | register << 8 | value).
-  template <bool MAX>
-  __device__ __forceinline__ void paint(uint32_t r0, uint32_t r1, uint32_t n_lines, const uint32_t *recs, uint32_t ri,
+  // [ri, n_rec) (clock << 14 | register << 8 | value); over: as the maximum
+  // with what is in the frame.
+  __device__ __forceinline__ void paint(bool over, uint32_t r0, uint32_t r1, uint32_t n_lines, const uint32_t *recs, uint32_t ri,
                                         uint32_t n_rec, uint32_t frame) {
     // the record at ri and the next one; ~0: a clock beyond every line
     uint32_t rec = ri < n_rec ? recs[ri] : ~0u, ahead = ri + 1 < n_rec ? recs[ri + 1] : ~0u;
@@ -218,7 +217,7 @@ struct RowPainter {
         const uint32_t black = sm8(tabs.luma) * 0x01010101u;
         for (uint32_t q = 0; q < 40; ++q) {
           uint32_t &d = sm32(row + 4u * q);
-          d = MAX ? max_u8x4(d, black) : black;
+          d = over ? max_u8x4(d, black) : black;
         }
         continue;
       }
@@ -289,7 +288,7 @@ struct RowPainter {
         }
         if (stop > xs) { take(xs, stop); xs = stop; }
         if (colour) {
-          emit<MAX>(xe, stop, row, line == bar);
+          emit(over, xe, stop, row, line == bar);
           xe = stop;
           if (stop == 160u) break;
         }
