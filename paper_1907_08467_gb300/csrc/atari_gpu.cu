@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(128) k_cache_run(uint8_t *work, uint8_t *snaps
                                                     int startup, int max_noops, int unit) {
   const int r = blockIdx.x;
   const uint32_t inf = info[r];
-  stage_cartridge(roms + (size_t)r * ROM_SLOT, inf >> 24, inf & 0xFF);
+  stage_cartridge(roms + (size_t)r * ROM_SLOT, inf >> 24, inf & 0xFF, 1);
   for (uint32_t t = threadIdx.x; t < DEC_BYTES; t += blockDim.x) sm8(OFF_DEC + t) = dec_op_g[t];
   __syncthreads();
   if (threadIdx.x != 0) return;
@@ -586,7 +586,7 @@ namespace {
 
 constexpr size_t MAX_SMEM = 227 * 1024 - 64;  // a block's dynamic shared memory, beside a few static bytes
 size_t interp_smem(const atari_env *E) {
-  return shared_part((uint32_t)E->rom_stage) + (size_t)E->lanes * E->warps * ENV_SMEM;
+  return block_smem((uint32_t)E->rom_stage, (uint32_t)(E->lanes * E->warps));
 }
 
 // Envs grouped by cartridge into work items of E envs (ascending env index
@@ -888,7 +888,7 @@ int atari_env_create(const uint8_t *const *roms, const size_t *rom_sizes, const 
     uint32_t max_banks = 1;
     for (int r = 0; r < n_roms; ++r) max_banks = std::max(max_banks, E->h_banks[r]);
     const int stage = (int)max_banks * 4096;
-    const size_t cache_smem = shared_part((uint32_t)stage) + ENV_SMEM;
+    const size_t cache_smem = block_smem((uint32_t)stage, 1);
     cudaFuncSetAttribute(k_cache_run, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cache_smem);
     k_cache_run<<<n_roms, 128, cache_smem>>>(d_work, d_snaps, E->d_roms, E->d_info, E->d_dec_op, stage,
                                            c.startup_frames, c.max_noops, 1);
@@ -1080,7 +1080,7 @@ int autotune(atari_env *E) {
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   // (envs per warp, CPU warps per block, paired TIA warps).  A round costs about
-  // 210 cycles with one CPU warp on an SM, 240 with one a scheduler and 370 with
+  // 157 cycles with one CPU warp on an SM, 185 with one a scheduler and 284 with
   // two a scheduler (the integer pipe is then full), so small batches spread
   // over the SMs and large ones fill them; a block of eight CPU warps stages
   // its cartridge once for all of them.
@@ -1095,7 +1095,7 @@ int autotune(atari_env *E) {
     const auto &c = cand[ci];
     if ((size_t)c[0] * c[1] > 4 * n && c[0] * c[1] > 32) continue;  // far more slots than envs
     if ((E->cfg.tia_warps == 1 && c[2]) || (E->cfg.tia_warps >= 2 && !c[2])) continue;
-    if (shared_part((uint32_t)E->rom_stage) + (size_t)c[0] * c[1] * ENV_SMEM > MAX_SMEM) continue;
+    if (block_smem((uint32_t)E->rom_stage, (uint32_t)(c[0] * c[1])) > MAX_SMEM) continue;
     if (int rc = build_groups(E, c[0], c[1], c[2] != 0)) { cudaFree(st_bak); return rc; }
     BatchArgs a = batch_args(E, E->d_act, nullptr, nullptr);
     float t = 0;

@@ -189,27 +189,29 @@ __device__ void tia_worker(IoCtx c, uint32_t q, const uint8_t *st, int i, const 
   }
 }
 
-// Shared memory of a block: the tables, the cartridge stage, then per env
-// RAM, I/O words, TIA file and event queue.
-__host__ __device__ inline uint32_t shared_part(uint32_t rom_stage) { return OFF_ROM + 4 * rom_stage; }
+// Shared memory of a block: the tables, the envs' RAM, the cartridge stage, then
+// per env I/O words, TIA file and event queue.
 __device__ __forceinline__ EnvOff env_off(uint32_t rom_stage, uint32_t envs, uint32_t j) {
   EnvOff o;
-  o.rom = OFF_ROM;
-  const uint32_t ram = shared_part(rom_stage);
-  const uint32_t io = ram + RAM_BYTES * envs, tia = io + 4 * IO_STRIDE * envs, q = tia + TIA_STRIDE * envs;
-  o.ram = ram + RAM_BYTES * j;
+  o.rom = OFF_RAM + ram_part(envs);
+  const uint32_t io = o.rom + 4 * rom_stage, tia = io + 4 * IO_STRIDE * envs, q = tia + TIA_STRIDE * envs;
+  o.ram = OFF_RAM + j / 4 * RAM_GROUP + j % 4;
   o.io = io + 4 * IO_STRIDE * j;
   o.tia = tia + TIA_STRIDE * j;
   o.q = q + 4 * QSTRIDE * j;
   return o;
 }
-// Stage a cartridge (banks of 4096 bytes at src, 4-byte aligned) and its
-// region table with the whole block.
-__device__ __forceinline__ void stage_cartridge(const uint8_t *src, uint32_t banks, uint32_t scheme) {
+// Stage a cartridge (banks of 4096 bytes at src, 4-byte aligned) for a block of
+// envs and its region table with the whole block.
+__device__ __forceinline__ void stage_cartridge(const uint8_t *src, uint32_t banks, uint32_t scheme, uint32_t envs) {
   const uint32_t limit = scheme_fetch_limit(scheme);
   for (uint32_t g = threadIdx.x; g < banks * 1024u; g += blockDim.x)
-    reinterpret_cast<uint4 *>(g_smem + OFF_ROM)[g] = stage_words(src + (g >> 10) * 4096u, 4u * (g & 1023u), limit);
-  for (uint32_t p = threadIdx.x; p < REGION_BYTES; p += blockDim.x) sm8(OFF_REG + p) = (uint8_t)region_byte(p, scheme);
+    reinterpret_cast<uint4 *>(g_smem + OFF_RAM + ram_part(envs))[g] = stage_words(src + (g >> 10) * 4096u, 4u * (g & 1023u), limit);
+  for (uint32_t p = threadIdx.x; p < REGION_BYTES / 4; p += blockDim.x) {
+    uint32_t w = 0;
+    for (uint32_t b = 0; b < 4; ++b) w |= region_byte(4 * p + b, scheme) << (8 * b);
+    sm32(OFF_REG + 4 * p) = w;
+  }
 }
 // blockDim = W warps (single-warp form) or 2 W (split form); warps [0, W) run
 // the CPUs of the work item's envs, in the split form warp W + w the TIA side
@@ -233,7 +235,7 @@ __device__ __forceinline__ void interp_block(const BatchArgs &a) {
     const int rom = a.grp_rom[g];
     const uint32_t inf = a.info[rom];
     if (rom != cur_rom) {
-      stage_cartridge(a.romb + (size_t)rom * ROMB_SLOT, inf >> 24, inf & 0xFF);
+      stage_cartridge(a.romb + (size_t)rom * ROMB_SLOT, inf >> 24, inf & 0xFF, (uint32_t)a.E);
       cur_rom = rom;
     }
     const int jj = cw * a.lanes + lane;

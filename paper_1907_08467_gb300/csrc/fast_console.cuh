@@ -5,9 +5,11 @@
 //     steered by control words per opcode (opcode_ctl.h);
 //   - CPU registers, flags, the cycle counter and the bank in registers;
 //   - RAM (bytes), the TIA register file (bytes) and the I/O state
-//     (collision latches, RIOT timer and ports, inputs) in shared memory, one block per env with odd
+//     (collision latches, RIOT timer and ports, inputs) in shared memory with odd
 //     word strides, so lanes reading the same field never bank-conflict and
 //     every access is a base offset plus a constant or one add;
+//   - a byte of RAM every four bytes, four envs interleaved, so that RAM and
+//     cartridge addresses scale alike;
 //   - the block's cartridge staged in shared memory as one word per byte (64 KB
 //     for an F6 cartridge), the byte and the two after it: an instruction is
 //     one load, and a data byte the first byte of its word.
@@ -39,18 +41,17 @@ enum IoWord : uint32_t {
 constexpr uint32_t IO_WSYNC = 1u;
 
 
-// Per-env blocks of shared memory, env-major, with strides chosen so that a
-// warp's lanes touching the same field hit 32 different banks: RAM 128 bytes
-// padded to 132 (33 words), I/O state IO_WORDS words, TIA file 44 bytes (11
-// words).  Every access is the lane's base plus a constant or one add.  Bytes
-// rather than one word per RAM byte keep a 64-env work item small enough for
-// four blocks per SM.
-constexpr uint32_t RAM_BYTES = 132, IO_STRIDE = IO_WORDS, TIA_STRIDE = 44;
-static_assert(IO_STRIDE % 2 == 1 && (TIA_STRIDE / 4) % 2 == 1 && (RAM_BYTES / 4) % 2 == 1 && RAM_BYTES % 4 == 0,
+// Blocks of shared memory per env, with strides chosen so that a warp's lanes
+// touching the same field hit 32 different banks: I/O state IO_WORDS words, TIA
+// file 44 bytes (11 words); RAM in groups of four envs of RAM_GROUP bytes, a
+// word holding one byte of each.  Every access is the lane's base plus a
+// constant or one add.
+constexpr uint32_t RAM_GROUP = 516, IO_STRIDE = IO_WORDS, TIA_STRIDE = 44;
+static_assert(IO_STRIDE % 2 == 1 && (TIA_STRIDE / 4) % 2 == 1 && (RAM_GROUP / 4) % 2 == 1 && RAM_GROUP % 4 == 0,
               "odd word strides");
 constexpr uint32_t QLEN = 32;             // event queue entries per env (a power of two)
 constexpr uint32_t QSTRIDE = QLEN + 1;    // shared-memory words per env queue (odd)
-constexpr uint32_t ENV_SMEM = RAM_BYTES + 4 * IO_STRIDE + TIA_STRIDE + 4 * QSTRIDE;
+constexpr uint32_t ENV_SMEM = 4 * IO_STRIDE + TIA_STRIDE + 4 * QSTRIDE;  // beside the RAM
 // bytes per cartridge in the batched form's device copy (up to eight 4 KB banks, F4)
 constexpr uint32_t ROMB_SLOT = 32768;
 
@@ -357,7 +358,7 @@ constexpr uint32_t EV_CTRL = 1u << 14, EV_BEGIN_LOG = EV_CTRL, EV_END_LOG = EV_C
                    EV_REBASE = EV_CTRL | 5u << 8;
 // Lap parity of queue position k.
 constexpr uint32_t EV_LAP = 1u << 15;
-__device__ __forceinline__ uint32_t lap_bit(uint32_t k) { return (~k << 10) & EV_LAP; }
+__device__ __forceinline__ uint32_t lap_bit(uint32_t k) { return (~k * (EV_LAP / QLEN)) & EV_LAP; }
 // A wait between an env's CPU and TIA warps gives up after WAIT_NS of the
 // GPU's global timer and the env is declared stalled.  The longest legitimate
 // wait is about one frame of the slowest lane of the partner warp (a few
@@ -484,15 +485,20 @@ __device__ __forceinline__ uint32_t lds_const(uint32_t a) {
   asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
   return v;
 }
-__device__ __forceinline__ uint32_t lds8_const(uint32_t a) {
-  uint32_t v;
-  asm("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
+template <uint32_t OFF>
 __device__ __forceinline__ uint4 lds_const4(uint32_t a) {
   uint4 v;
-  asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4 + %5];"
+      : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+      : "r"(a), "n"(OFF));
   return v;
+}
+// Any function of three words, bit by bit: bit 4 a + 2 b + c of LUT.
+template <uint32_t LUT>
+__device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t r;
+  asm("lop3.b32 %0, %1, %2, %3, %4;" : "=r"(r) : "r"(a), "r"(b), "r"(c), "n"(LUT));
+  return r;
 }
 
 // Byte offsets of an env's blocks in the block's dynamic shared memory.
@@ -500,30 +506,47 @@ struct EnvOff {
   uint32_t rom, ram, io, tia, q;
 };
 // The block's tables come first, at fixed offsets: region table, general
-// decoder's bytes, control words.  The cartridge follows, then the envs.
-constexpr uint32_t OFF_REG = 0, OFF_DEC = OFF_REG + REGION_BYTES, OFF_CTL = OFF_DEC + 512, OFF_ROM = OFF_DEC + DEC_BYTES;
+// decoder's bytes, control words.  The envs' RAM follows, then the cartridge,
+// then the envs' other blocks.  The hot loop loads from RAM's base + 4 *
+// (address - 0x80) for every address below the cartridge's and looks at the
+// value only when the address is RAM's; the cartridge (16 KB at least) behind
+// the RAM and the tables before it keep those loads inside the block's memory.
+constexpr uint32_t OFF_REG = 0, OFF_DEC = OFF_REG + REGION_BYTES, OFF_CTL = OFF_DEC + 512, OFF_RAM = OFF_DEC + DEC_BYTES;
+static_assert(OFF_RAM % 16 == 0 && OFF_RAM >= 0x4000u, "aligned; rom - 0x4000 and ram - 0x200 stay offsets");
+__host__ __device__ inline uint32_t ram_part(uint32_t envs) { return ((envs + 3) / 4 * RAM_GROUP + 15) / 16 * 16; }
+// Dynamic shared memory of a block of envs with rom_stage cartridge bytes.
+__host__ __device__ inline uint32_t block_smem(uint32_t rom_stage, uint32_t envs) {
+  return OFF_RAM + ram_part(envs) + 4 * rom_stage + envs * ENV_SMEM;
+}
 __device__ __forceinline__ uint32_t scheme_fetch_limit(uint32_t scheme) {
   return scheme == 3 ? 0xFF1u : scheme ? 0xFF3u : 0xFFCu;
 }
 // The cartridge is staged as one word per byte: the byte and the two after it
 // (an instruction in one load), and in the top byte 0x80 where no instruction
-// is fetched from the stage.  Words i .. i+3 of a bank of 4096 bytes at src
-// (4-byte aligned), i a multiple of 4.
+// is fetched from the stage: past limit, and a branch whose target lies past
+// the bank's end (the hot loop's sums would carry into the cycle count there).
+// Words i .. i+3 of a bank of 4096 bytes at src (4-byte aligned), i a multiple
+// of 4.
 constexpr uint32_t REC_BAD = 0x80000000u;
+__device__ __forceinline__ uint32_t stage_bad(uint32_t w, uint32_t i, uint32_t limit) {
+  const uint32_t off = (w >> 8) & 0xFFu;
+  return i > limit || ((w & 0x1Fu) == 0x10u && off < 0x80u && i + 2u + off > 0xFFFu) ? REC_BAD : 0u;
+}
 __device__ __forceinline__ uint4 stage_words(const uint8_t *src, uint32_t i, uint32_t limit) {
   const uint32_t *b = reinterpret_cast<const uint32_t *>(src + i);
   const uint32_t lo = b[0], hi = i + 4u < 4096u ? b[1] : 0u, m = 0xFFFFFFu;
   uint4 r = make_uint4(lo & m, __funnelshift_r(lo, hi, 8) & m, __funnelshift_r(lo, hi, 16) & m,
                        __funnelshift_r(lo, hi, 24) & m);
-  r.x |= i > limit ? REC_BAD : 0u;
-  r.y |= i + 1u > limit ? REC_BAD : 0u;
-  r.z |= i + 2u > limit ? REC_BAD : 0u;
-  r.w |= i + 3u > limit ? REC_BAD : 0u;
+  r.x |= stage_bad(r.x, i, limit);
+  r.y |= stage_bad(r.y, i + 1u, limit);
+  r.z |= stage_bad(r.z, i + 2u, limit);
+  r.w |= stage_bad(r.w, i + 3u, limit);
   return r;
 }
-// Rounds between two looks at the lanes that wait for service.  A look costs
-// about 60 cycles beside rounds of about 270; a lane that waits loses half a
-// batch.
+// Rounds between two looks at the lanes that wait for service, unrolled, so
+// that a round's last instructions overlap the next one's loads (157 cycles a
+// round, 173 as a loop).  A look costs about 60 cycles; a lane that waits loses
+// half a batch, and 16 rounds measure the same as 8.
 constexpr uint32_t BATCH = 8;
 
 template <bool SPLIT>
@@ -557,7 +580,7 @@ struct FastConsoleT {
     off = o;
     io = IoCtx{o.tia, o.io};
   }
-  __device__ __forceinline__ uint8_t &ram(uint32_t i) const { return sm8(off.ram + i); }
+  __device__ __forceinline__ uint8_t &ram(uint32_t i) const { return sm8(off.ram + 4 * i); }
   __device__ __forceinline__ uint32_t rom(uint32_t i) const { return sm8(off.rom + 4 * i); }
 
   // ---- canonical state I/O ----
@@ -588,12 +611,11 @@ struct FastConsoleT {
     kf = (uint32_t)(k - 76ull * l0c);
     io.Sset(IO_JOY, 0xFF); io.Sset(IO_FIRE, 0);
     io.Sset(IO_STATUS, 0);
-    const uint4 *r4 = reinterpret_cast<const uint4 *>(s + S::RAM);
-    uint32_t *r32 = &sm32(off.ram);
-#pragma unroll
-    for (int q_ = 0; q_ < 8; ++q_) {
-      const uint4 v = r4[q_];
-      r32[4 * q_] = v.x; r32[4 * q_ + 1] = v.y; r32[4 * q_ + 2] = v.z; r32[4 * q_ + 3] = v.w;
+    const uint32_t *r32 = reinterpret_cast<const uint32_t *>(s + S::RAM);
+#pragma unroll 8
+    for (uint32_t q_ = 0; q_ < 32; ++q_) {
+      const uint32_t v = r32[q_];
+      for (uint32_t b = 0; b < 4; ++b) ram(4 * q_ + b) = (uint8_t)(v >> (8 * b));
     }
     for (uint32_t e = 0; e < QLEN; ++e) sm32(off.q + 4 * e) = 0;
     status = 0; instret = 0; frame_inst = 0; rounds = 0; pend = 0; vs_kf = ~0u;
@@ -626,11 +648,10 @@ struct FastConsoleT {
     w[18] = io.G(IO_BARLO); w[19] = io.G(IO_BARHI);
     w[20] = (uint32_t)L0; w[21] = (uint32_t)(L0 >> 32);
     w[22] = frame_no; w[23] = 0;
-    uint4 *r4 = reinterpret_cast<uint4 *>(s + S::RAM);
-    const uint32_t *r32 = &sm32(off.ram);
-#pragma unroll
-    for (int q_ = 0; q_ < 8; ++q_)
-      r4[q_] = make_uint4(r32[4 * q_], r32[4 * q_ + 1], r32[4 * q_ + 2], r32[4 * q_ + 3]);
+    uint32_t *r32 = reinterpret_cast<uint32_t *>(s + S::RAM);
+#pragma unroll 8
+    for (uint32_t q_ = 0; q_ < 32; ++q_)
+      r32[q_] = ram(4 * q_) | ram(4 * q_ + 1) << 8 | ram(4 * q_ + 2) << 16 | (uint32_t)ram(4 * q_ + 3) << 24;
   }
   __device__ uint32_t all_status() const { return status | io.G(IO_STATUS) | (SPLIT ? 0u : ts.status); }
 
@@ -1024,9 +1045,16 @@ struct FastConsoleT {
   // increments and compares, one sum covers the effective address, the branch
   // target and the immediate operand, and one load covers RAM and cartridge.
   // So lanes at different instructions still execute together: each lane
-  // runs its own program at one instruction per round, with no leader, no
-  // reconvergence and a loop that stays in the instruction cache's first
-  // level.  What it does not take (RIOT accesses, collision reads, VSYNC and
+  // runs its own program at one instruction per round, with no leader and no
+  // reconvergence.  A lone warp is bound by the round's chain of dependent
+  // loads (instruction word, control words, operand), which is why the next
+  // instruction's words are loaded before this one's result is computed; eight
+  // warps on an SM are bound by the integer pipe, two cycles an instruction,
+  // which is why sums, shifts left and counters are multiply-adds.  One round:
+  // 157 cycles with one warp on an SM, 284 with eight (208 and 365 with the
+  // control words loaded at the round's end, V in a register of its own, the
+  // branch's condition in three operations, RAM addressed apart from the
+  // cartridge and regions of 32 bytes).  What it does not take (RIOT accesses, collision reads, VSYNC and
   // VBLANK, stack and pointer instructions, bank hotspots, frame ends) stops
   // the lane in front of the instruction; every BATCH rounds the lanes that
   // wait are served together by the general decoder, at once when no lane is
@@ -1077,41 +1105,42 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
   uint32_t smb;  // the shared window's address, taken here: no load of the stage moves above the block's barrier
   asm volatile("mov.u32 %0, %1;" : "=r"(smb) : "r"((uint32_t)__cvta_generic_to_shared(g_smem)) : "memory");
   const uint32_t cap = 76u * CAP_LINES;
-  const uint32_t ctl = smb + OFF_CTL, reg = smb + OFF_REG;
+  const uint32_t ctl = smb + OFF_CTL, ramb = o.ram - 0x200u;
   const uint32_t k1 = unit, k4 = unit * 4u, k256 = unit * 256u;
-  // R: A, X, Y and FF as bytes.  G: flags (FL_*; V apart, in bit 7 of vv; D
-  // and I do not change here).  pk: PC, and the frame's CPU cycle in the high
-  // half.  nl: the first line start at or after that cycle, in the high half,
-  // over FFFF.  qi: queue position, and the instructions retired since the
-  // last service in the high half.  bk: the bank's words.
-  uint32_t R, G, vv, pk, nl, qi, bk;
+  // R: A, X, Y and FF as bytes.  G: flags (FL_*; D and I do not change here).
+  // pk: PC, and the frame's CPU cycle in the high half.  nl: the first line
+  // start at or after that cycle, in the high half, over FFFF.  qi: queue
+  // position, and the instructions retired since the last service in the high
+  // half.  bk, bf: the bank's words, for data at 4 * (bus address) and for the
+  // fetch.  run: all ones, or 0 while the lane waits.
+  uint32_t R, G, pk, nl, qi, bk, bf, run;
   uint32_t rec;
   uint4 c, d, e, f;  // control words 0-3, 4-7, 8-11, 12-15
-  bool wait = false, active = true;
-  auto word_at = [&](uint32_t p) { return lds_const(mad(p & 0xFFFu, k4, smb + bk)); };
-  auto control = [&] {
-    const uint32_t a = mad(rec & 0xFFu, unit * CTL_STRIDE, ctl);
-    c = lds_const4(a);
-    d = lds_const4(a + 16);
-    e = lds_const4(a + 32);
-    f = lds_const4(a + 48);
+  bool active = true;
+  auto word_at = [&](uint32_t p) { return lds_const(mad(p & 0xFFFu, k4, bf)); };
+  auto control = [&](uint32_t w, uint4 &c_, uint4 &d_, uint4 &e_, uint4 &f_) {
+    const uint32_t a = mad(w & 0xFFu, unit * 16u, ctl);
+    c_ = lds_const4<0>(a);
+    d_ = lds_const4<CTL_TABLE>(a);
+    e_ = lds_const4<2 * CTL_TABLE>(a);
+    f_ = lds_const4<3 * CTL_TABLE>(a);
   };
   // the console's fields to the loop's registers, and the next instruction
   auto enter = [&](bool stay) {
     R = A | X << 8 | Y << 16 | 0xFF000000u;
-    G = ((fz & 0xFFu) ? 1u : 0u) | fc << 8 | (fn & 0x80u) << 16;
-    vv = fv << 1;
+    G = ((fz & 0xFFu) ? 1u : 0u) | fc << 8 | (fn & 0x80u) << 16 | fv << 25;
     pk = (PC & 0xFFFFu) | min(kf, 0xFFFFu) << 16;
     nl = ((min(kf, 0xFFFFu) + 75u) / 76u * 76u) << 16 | 0xFFFFu;
     qi = qtail & 0xFFu;
-    bk = o.rom + bank * 16384u;
+    bk = o.rom + bank * 16384u - 0x4000u;
+    bf = smb + o.rom + bank * 16384u;
     rec = word_at(pk);
-    wait = stay | ((pk & 0x1000u) == 0) | (rec >= REC_BAD) | (kf >= cap) | ((fdi & 0x08u) != 0);
-    control();
+    run = stay | ((pk & 0x1000u) == 0) | (rec >= REC_BAD) | (kf >= cap) | ((fdi & 0x08u) != 0) ? 0u : ~0u;
+    control(rec, c, d, e, f);
   };
   auto leave = [&] {
     A = R & 0xFF; X = (R >> 8) & 0xFF; Y = (R >> 16) & 0xFF;
-    fz = G & FL_Z; fc = (G >> 8) & 1u; fn = (G >> 16) & 0x80u; fv = (vv >> 1) & 0x40u;
+    fz = G & FL_Z; fc = (G >> 8) & 1u; fn = (G >> 16) & 0x80u; fv = (G >> 25) & 0x40u;
     PC = pk & 0xFFFFu;
     if ((pk >> 16) != 0xFFFFu) kf = pk >> 16;  // a loaded cycle count past 16 bits stays as it was
     qtail += (qi & 0xFFFFu) - (qtail & 0xFFu);
@@ -1120,63 +1149,60 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
   enter(jam != 0);
   uint32_t held = 0, act = wmask;
   for (;;) {
-#pragma unroll 1
+#pragma unroll
     for (uint32_t r = 0; r < BATCH; ++r) {
-      // --- next instruction (branches and JMP abs: the sum is the target)
+      // --- next instruction (branches and JMP abs: the sum is the target and the cycle)
       const uint32_t pn = mad(pk, k1, d.z);
       const uint32_t base = prmt(rec, pn, c.x);
       const uint32_t sum = mad(base, k1, prmt(R, rec, c.y));
-      const bool tk = ((G & d.w) != 0) ^ ((int)e.w < 0);
-      const uint32_t nrec = word_at(tk ? sum : pn);
+      const bool tk = mad(G & d.w, k1, f.w) > e.w;
+      const uint32_t nx = tk ? sum : pn;
+      const uint32_t nrec = word_at(nx);
       // a cycle for a taken branch, another one at a page crossing
-      uint32_t pnext = mad((base ^ sum) & (tk ? 0x100u : f.z), k256, pn);
-      if (tk) pnext = prmt(pnext, sum, 0x3254) + 0x10000u;
+      uint32_t pnext = mad((base ^ sum) & (tk ? 0x100u : f.z), k256, nx);
+      if (tk) pnext = mad(k256, 256u, pnext);
       // --- operand
       const uint32_t ea = sum & d.y;
-      const uint32_t rg = lds8_const(reg + (ea >> 5));
-      const uint32_t at = (ea & 0x1280u) == 0x0080u ? mad(ea & 0x7Fu, k1, o.ram) : mad(ea & 0xFFFu, k4, bk);
-      const uint32_t ld = sm8(at);
-      const uint32_t y = prmt(ld, sum, d.x) ^ e.y;
+      const uint32_t put = sm8(OFF_REG + ea) & f.x & run;
+      const uint32_t at = mad(ea, k4, ea >= 0x1000u ? bk : ramb);
+      const uint32_t y = prmt(sm8(at), sum, d.x);
       const uint32_t x = prmt(R, y, c.z);
-      // --- result
-      const uint32_t one = f.w >> 16;
-      const uint32_t raw = mad(x & y, e.z, mad(x ^ y, f.y, mad(prmt(G, 0, e.w), k1, one)));
+      uint4 cn, dn, en, fn;  // the next instruction's control words, on their way while this one is computed
+      control(nrec, cn, dn, en, fn);
+      // --- result, of x and y ^ e.y
+      const uint32_t xo = lop3<0x96>(x, y, e.y);
+      const uint32_t raw = mad(lop3<0x60>(x, y, e.y), e.z, mad(xo, f.y, prmt(G, k1, e.w)));
       const uint32_t s = __funnelshift_r(raw, 0, f.w);
-      // --- what the general decoder takes: no region fits, VSYNC, VBLANK
-      const uint32_t m = ea & 0x3Fu;                      // of the TIA: the register
-      const uint32_t put = rg & f.x;
-      const bool tia = (put & RG_WTIA) != 0;
-      const bool skip = wait | ((put & RG_ALL) == 0) | (tia & (m < 2u));
-      // --- commit
-      const bool out = tia & (m > 2u) & !wait, ws = tia & (m == 2u);
-      if (((put & RG_WRAM) != 0) & !wait) sm8(at) = (uint8_t)s;
+      // --- commit; nothing in put: the lane waits, or waits from here on for the general decoder
+      const bool out = (put & RG_OUT) != 0;
+      if (put & RG_WRAM) sm8(at) = (uint8_t)s;
       // events past another lap's bit: the lap's complement is bit 15 of -qi * 1024 - 1024
-      const uint32_t ev = mad(m, k256, s) | (mad(qi, unit * 0xFFFFFC00u, 0xFFFFFC00u) & EV_LAP);
+      const uint32_t ev = mad(ea, k256, s) | (mad(qi, unit * (0u - EV_LAP / QLEN), 0u - EV_LAP / QLEN) & EV_LAP);
       if (out) vsm32(mad(qi & (QLEN - 1), k4, o.q)) = prmt(ev, pnext, 0x7610);
-      if (pnext > nl) nl += 76u << 16;                    // one step: no instruction is longer than a line
-      if (ws) pnext = prmt(pnext, nl, 0x7610);            // WSYNC: on to the next line's first cycle
-      if (!skip) R = prmt(R, s, c.w);
-      if (!skip) G = (G & ~e.x) | ((s * FL_COPY) & e.x);
-      if ((!skip) & ((int)d.x < 0)) vv = (x ^ s) & ~(x ^ y);
-      if (!skip) pk = pnext;
-      if (!skip) qi += 0x10000u;
-      if (out) ++qi;
+      if (pnext > nl) nl = mad(k256, 76u << 8, nl);       // one step: no instruction is longer than a line
+      if (put & RG_WSYNC) pnext = prmt(pnext, nl, 0x7610);  // on to the next line's first cycle
+      const bool done = put != 0;  // in single statements: a block of them would become a branch
+      const uint32_t gn = (G & ~e.x) | (prmt(s, lop3<0x14>(x, s, xo), FL_SEL) & e.x);  // V: (x ^ s) & ~(x ^ y)
+      if (done) R = prmt(R, s, c.w);
+      if (done) G = gn;
+      if (done) pk = pnext;
+      if (done) qi = mad(k256, 256u, qi);
+      if (out) qi = mad(k1, k1, qi);
       // bit 31: no instruction word there, the PC outside the cartridge, the line cap
       const uint32_t stop = nrec | mad(pnext, unit * 0xFFF80000u, 0xFFF80000u) | mad(pnext, 0u - unit, (cap << 16) - 1u);
-      wait = skip | ((int)stop < 0);
-      rec = nrec;
-      control();
+      run = !done | ((int)stop < 0) ? 0u : ~0u;
+      rec = nrec; c = cn; d = dn; e = en; f = fn;
     }
     // --- service: waiting lanes, and queues without room for another batch
     rounds += BATCH;
     const bool full = ((qi - qhead_seen) & 0xFFu) > QLEN - BATCH;
-    uint32_t m = __ballot_sync(wmask, (wait | full) & active);
+    uint32_t m = __ballot_sync(wmask, ((run == 0) | full) & active);
     if (m == 0) continue;
-    m = __ballot_sync(wmask, wait & active);
+    m = __ballot_sync(wmask, (run == 0) & active);
     if (m != 0 && (m == act || ++held > 1)) {
       held = 0;
       ++rounds;
-      if (active && wait) {
+      if (active && run == 0) {
         leave();
         active = fc_service<SPLIT, Hook>(this, &hook);
         enter(!active);
@@ -1189,7 +1215,7 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
       if (active & (((qi - qhead_seen) & 0xFFu) > QLEN - BATCH)) {
         const uint32_t qt = qtail + (qi & 0xFFFFu) - (qtail & 0xFFu);
         qhead_seen = fc_q_wait_room(io, qt, BATCH);
-        if (qt - qhead_seen > QLEN - BATCH) { stall(); wait = true; }
+        if (qt - qhead_seen > QLEN - BATCH) { stall(); run = 0; }
       }
     } else {
       if (__any_sync(wmask, ((qi - qhead_seen) & 0xFFu) > QLEN - BATCH)) {

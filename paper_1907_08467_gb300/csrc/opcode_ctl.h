@@ -10,7 +10,9 @@
 // instruction cache's first level and 280-450 when they do not, so data beats
 // code here.  The sequence is bound by the integer pipe (two cycles a warp
 // instruction), so the words come in the form in which they are used, with as
-// little unpacking as possible: 64 bytes an opcode, four 16-byte loads.
+// little unpacking as possible: 64 bytes an opcode, four 16-byte loads, each
+// from a table of its own (lanes at different opcodes then fall into eight
+// bank groups, not two).
 #pragma once
 #include <cstdint>
 #include <cstring>
@@ -19,9 +21,14 @@
 
 namespace atari {
 
-// Regions of the 13-bit bus: RAM, cartridge below its first hotspots, TIA; RAM
-// and TIA again for the writes that a control word asks for.
-constexpr uint32_t RG_RAM = 1u, RG_CART = 2u, RG_TIA = 4u, RG_ALL = 7u, RG_WRAM = 8u, RG_WTIA = 16u;
+// What an access may fall on, a byte per address of the 13-bit bus: RAM (its
+// zero-page addresses), RAM again for a result that is stored, the cartridge
+// but for its hotspots, TIA registers whose writes are only passed on, WSYNC,
+// and address 0 for an instruction without an access.  Every other address
+// (mirrors too) is the general decoder's.  A byte for each address costs 8 KB
+// a block and saves the shift, the mirror masks and four compares a round that
+// a table of 32-byte granules needs.
+constexpr uint32_t RG_RAM = 1u, RG_WRAM = 2u, RG_CART = 4u, RG_OUT = 8u, RG_WSYNC = 16u, RG_NONE = 32u;
 
 // Word by word (byte selectors are those of a 32-bit byte permute and use the
 // low half):
@@ -29,38 +36,36 @@ constexpr uint32_t RG_RAM = 1u, RG_CART = 2u, RG_TIA = 4u, RG_ALL = 7u, RG_WRAM 
 //   1  selector of the index from (A X Y FF, instruction bytes)
 //   2  selector of the adder's x from (A X Y FF, operand)
 //   3  selector of the written registers from (A X Y FF, result)
-//   4  selector of the operand from (memory byte, sum of base and index) | V is written << 31
+//   4  selector of the operand from (memory byte, sum of base and index)
 //   5  address mask
 //   6  length | cycles << 16
 //   7  branch: flag bits of which any takes it
 //   8  flag bits that are written
 //   9  operand invert
 //  10  multiplier of (x & y): 0 eor, 1 and / or, 2 add, 513 shift right
-//  11  selector of the carry-in from the flags (their byte 1 is the carry) | the branch is taken when no flag
-//      bit is set << 31
-//  12  regions that the access may fall in (none: the general decoder's instruction), RG_WRAM: the result is
-//      stored there, RG_WTIA: it is written there
+//  11  selector of the carry-in from (flags, 1) (the flags' byte 1 is the carry, byte 5 a zero); a branch's
+//      threshold
+//  12  what the access may fall on (nothing: the general decoder's instruction)
 //  13  multiplier of (x ^ y): 0 and, 1 otherwise
 //  14  page-cross penalty << 8
-//  15  right shift of the sum | carry-in 1 << 16
-constexpr uint32_t CTL_WORDS = 16, CTL_STRIDE = 4 * CTL_WORDS, CTL_N = 256;
-constexpr uint32_t CTL_BYTES = CTL_STRIDE * CTL_N;
+//  15  right shift of the sum (its low 5 bits); a branch is taken when word 15 + (flags & word 7) > word 11, unsigned
+// Words 4 i .. 4 i + 3 of opcode o are at CTL_TABLE i + 16 o.
+constexpr uint32_t CTL_WORDS = 16, CTL_N = 256, CTL_TABLE = 16 * CTL_N;
+constexpr uint32_t CTL_BYTES = 4 * CTL_WORDS * CTL_N;
 constexpr uint32_t DEC_BYTES = 512 + CTL_BYTES;  // general decoder's bytes, then the control words
-constexpr uint32_t REGION_BYTES = 256;           // region table of the cartridge, indexed by address >> 5
+constexpr uint32_t REGION_BYTES = 8192;          // what each address of the bus is
 
-// Flags as the interpreter holds them: the 9-bit result that set them, twice.
-// Bits 0-7 are zero when Z is set, bit 8 is C, bit 23 is N (BIT and PLP can set
-// N and Z both, so N has its own copy); the other bits are not looked at.
-constexpr uint32_t FL_NZ = 0xFFu | 0xFFu << 16, FL_C = 0x100u | 0x100u << 16, FL_Z = 0xFFu, FL_N = 0x80u << 16;
-constexpr uint32_t FL_COPY = 0x10001u;         // result -> both copies
+// Flags as the interpreter holds them: the 9-bit result that set them (bits 0-7
+// zero when Z is set, bit 8 C), its low byte again (bit 23 is N: BIT and PLP can
+// set N and Z both, so N has its own copy), and a byte whose bit 7 is V.  The
+// bits that no FL_ names are not looked at; byte 1 holds C alone.
+constexpr uint32_t FL_NZ = 0xFFu | 0xFFu << 16, FL_C = 0x100u, FL_Z = 0xFFu, FL_N = 0x80u << 16, FL_V = 0x80u << 24;
+constexpr uint32_t FL_SEL = 0x4010u;           // selector of the flags from (result, overflow byte)
 
-// Region byte of addresses at << 5 ..  scheme != 0: the last 128 bytes hold
-// bank hotspots and are left to the general decoder.
 __host__ __device__ inline uint32_t region_byte(uint32_t at, uint32_t scheme) {
-  const uint32_t page = at >> 2;
-  if (page >= 32u) return page == 63u && scheme ? 0u : RG_CART;
-  if ((page & 5u) == 1u) return RG_RAM | RG_WRAM;
-  return (page & 1u) ? 0u : RG_TIA | RG_WTIA;
+  if (at >= 0x1000u) return scheme && at >= 0x1FF4u && at <= 0x1FFBu ? 0u : RG_CART;
+  if (at >= 0x80u) return at < 0x100u ? RG_RAM | RG_WRAM : 0u;
+  return at == 0u ? RG_NONE : at == 2u ? RG_WSYNC : at > 2u && at < 0x40u ? RG_OUT : 0u;
 }
 
 // dec: per opcode, operation | mode << 8 | cycles << 12 | page-cross penalty << 16 (0: halts the CPU).
@@ -73,7 +78,7 @@ inline void build_ctl(const uint32_t *dec, uint8_t *out) {
     const uint32_t len = mode <= ACC ? 1u : mode >= ABS && mode <= IND ? 3u : 2u;
     // zero bytes: byte 3 of the instruction bytes, byte 1 of the operand
     uint32_t selB = 0x3333, selI = 0x7777, selX = 0x5555, selD = 0x3210, selV = 0x7654, em = 0;
-    uint32_t bm = 0, m2 = 1, inv = 0, gm = 0, k = 2, selC = 0x4444, one = 0, binv = 0, vset = 0, regions = RG_ALL, wr = 0;
+    uint32_t bm = 0, m2 = 1, inv = 0, gm = 0, k = 2, selC = 0x5555, one = 0, a = 0, regions = RG_NONE;
     bool mem = true, slow = op == O_JAM;
     switch (mode) {
       case IMM: selB = 0x3331; mem = false; break;
@@ -84,19 +89,20 @@ inline void build_ctl(const uint32_t *dec, uint8_t *out) {
       case ABX: selB = 0x3321; selI = 0x7771; em = 0x1FFF; break;
       case ABY: selB = 0x3321; selI = 0x7772; em = 0x1FFF; break;
       case ACC: selI = 0x7770; mem = false; break;  // the operand is the sum of base and index: A
-      case REL: selB = 0x3354; selI = 0xDDD5; mem = false; break;
+      // base and sum keep the cycle in their high halves: the sum is the next PC and cycle
+      case REL: selB = 0x7654; selI = 0xDDD5; mem = false; break;
       case IMP: mem = false; break;
       default: slow = true; break;                  // pointers through RAM: the general decoder
     }
-    const uint32_t NZ = FL_NZ, NZC = FL_NZ | FL_C, C1 = 0x4441, A_ = 0x5550, X_ = 0x5551, Y_ = 0x5552, V_ = 0x5554, FF = 0x5553;
+    const uint32_t NZ = FL_NZ, NZC = FL_NZ | FL_C, C1 = 0x5551, A_ = 0x5550, X_ = 0x5551, Y_ = 0x5552, V_ = 0x5554, FF = 0x5553;
     const uint32_t dA = 0x3214, dX = 0x3240, dY = 0x3410;
     bool ld = false, st = false, rmw = false;
     switch (op) {
       case O_LDA: selD = dA; gm = NZ; ld = mem; break;
       case O_LDX: selD = dX; gm = NZ; ld = mem; break;
       case O_LDY: selD = dY; gm = NZ; ld = mem; break;
-      case O_ADC: selX = A_; selD = dA; gm = NZC; vset = 1; selC = C1; ld = mem; break;
-      case O_SBC: selX = A_; selD = dA; gm = NZC; vset = 1; selC = C1; inv = 0xFF; ld = mem; break;
+      case O_ADC: selX = A_; selD = dA; gm = NZC | FL_V; selC = C1; ld = mem; break;
+      case O_SBC: selX = A_; selD = dA; gm = NZC | FL_V; selC = C1; inv = 0xFF; ld = mem; break;
       case O_AND: selX = A_; selD = dA; gm = NZ; k = 1; m2 = 0; ld = mem; break;
       case O_ORA: selX = A_; selD = dA; gm = NZ; k = 1; ld = mem; break;
       case O_EOR: selX = A_; selD = dA; gm = NZ; k = 0; ld = mem; break;
@@ -110,7 +116,7 @@ inline void build_ctl(const uint32_t *dec, uint8_t *out) {
       case O_ROL: selX = V_; gm = NZC; selC = C1; rmw = mem; break;
       // y * 513 >> 1 holds y >> 1 in bits 0-6 and y's bit 0 in bit 8; the carry comes in at 256 >> 1
       case O_LSR: selX = V_; gm = NZC; k = 513; rmw = mem; break;
-      case O_ROR: selX = V_; gm = NZC; k = 513; selC = 0x4414; rmw = mem; break;
+      case O_ROR: selX = V_; gm = NZC; k = 513; selC = 0x5515; rmw = mem; break;
       case O_INC: gm = NZ; one = 1; rmw = true; break;
       case O_DEC: selX = FF; gm = NZ; rmw = true; break;
       case O_INX: selX = X_; selD = dX; gm = NZ; one = 1; break;
@@ -123,33 +129,40 @@ inline void build_ctl(const uint32_t *dec, uint8_t *out) {
       case O_TYA: selX = Y_; selD = dA; gm = NZ; break;
       case O_CLC: gm = FL_C; break;
       case O_SEC: gm = FL_C; inv = 0xFF; one = 1; break;  // 0 + FF + 1 carries
-      case O_BCS: bm = 0x100; break;
-      case O_BCC: bm = 0x100; binv = 1; break;
+      case O_CLV: gm = FL_V; break;
+      // taken when a flag bit is set: 0 + bits > 0; when none is: bits - 1 > FFFF0000
+      case O_BCS: bm = FL_C; break;
+      case O_BCC: bm = FL_C; a = ~0u; break;
       case O_BNE: bm = FL_Z; break;
-      case O_BEQ: bm = FL_Z; binv = 1; break;
+      case O_BEQ: bm = FL_Z; a = ~0u; break;
       case O_BMI: bm = FL_N; break;
-      case O_BPL: bm = FL_N; binv = 1; break;
-      // a branch always taken: base = the operand, the taken branch's cycle counted
-      case O_JMP: if (mode == ABS) { binv = 1; cyc = 2; } else slow = true; break;
+      case O_BPL: bm = FL_N; a = ~0u; break;
+      case O_BVS: bm = FL_V; break;
+      case O_BVC: bm = FL_V; a = ~0u; break;
+      // a branch always taken: base = the operand over the cycle, the taken branch's cycle counted
+      case O_JMP: if (mode == ABS) { a = ~0u; cyc = 2; selB = 0x7621; } else slow = true; break;
       case O_NOP: if (mode != IMP && mode != IMM) slow = true; break;  // its operand read may switch a bank
-      default: slow = true; break;  // stack operations, BIT, BVC, BVS, other flag operations, undocumented opcodes
+      default: slow = true; break;  // stack operations, BIT, other flag operations, undocumented opcodes
     }
     if (op == O_JMP) em = 0;
     if (mode == ACC) selD = dA;
     if (slow) {  // nothing happens here: the lane waits for the general decoder
-      selD = 0x3210; gm = bm = binv = vset = regions = 0; ld = st = rmw = false;
+      selD = 0x3210; gm = bm = a = regions = 0; ld = st = rmw = false;
     } else if (ld) {
       regions = RG_RAM | RG_CART; selV = 0x3210;
     } else if (st) {
-      regions = RG_RAM | RG_TIA; wr = RG_WRAM | RG_WTIA; selV = 0x1111;  // operand 0: the result is x
+      regions = RG_RAM | RG_WRAM | RG_OUT | RG_WSYNC; selV = 0x1111;  // operand 0: the result is x
     } else if (rmw) {
-      regions = RG_RAM; wr = RG_WRAM; selV = 0x3210;
+      regions = RG_RAM | RG_WRAM; selV = 0x3210;
     } else {
-      em = 0;  // no access: address 0, which every region list but an empty one takes
+      em = 0;  // no access: address 0
     }
-    const uint32_t w[CTL_WORDS] = {selB, selI, selX, selD, selV | vset << 31, em, len | cyc << 16, bm,
-                                   gm, inv, k, selC | binv << 31, regions | wr, m2, pen << 8, (k == 513 ? 1u : 0u) | one << 16};
-    memcpy(out + CTL_STRIDE * o, w, CTL_STRIDE);
+    if (one) selC = 0x5554;
+    if (k == 513) a = 1;                               // the shift; no branch: 1 + 0 is below any selector
+    const uint32_t thr = bm || a == ~0u ? a & 0xFFFF0000u : selC;
+    const uint32_t w[CTL_WORDS] = {selB, selI, selX, selD, selV, em, len | cyc << 16, bm,
+                                   gm, inv, k, thr, regions, m2, pen << 8, a};
+    for (uint32_t i = 0; i < 4; ++i) memcpy(out + CTL_TABLE * i + 16 * o, w + 4 * i, 16);
   }
 }
 
