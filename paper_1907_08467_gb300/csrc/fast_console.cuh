@@ -279,11 +279,28 @@ __device__ __forceinline__ void fc_riot_write(IoCtx c, uint32_t a, uint32_t v, u
     c.S64(IO_TCWLO, now);
   }
 }
+// Whether a write can change the collisions after it: whether it changes its
+// register, or a delayed copy that it makes.  RESxx, HMOVE and CXCLR count as
+// changes.
+__device__ __forceinline__ bool fc_coll_change(IoCtx c, uint32_t reg, uint32_t v) {
+  if (reg == 0x2A || reg == 0x2C || (reg >= 0x10 && reg < 0x15)) return true;
+  const uint32_t slot = reg < 0x10 ? (reg == 1 ? (uint32_t)T_VBLANK : reg - 2)
+                                   : reg >= 0x25 ? T_VDELP0 + reg - 0x25
+                                                 : reg >= 0x1D ? (reg == 0x1F ? (uint32_t)T_ENABL_N : T_ENAM0 + reg - 0x1D)
+                                                               : reg == 0x1B ? (uint32_t)T_GRP0_N : (uint32_t)T_GRP1_N;
+  bool change = c.T(slot) != v;
+  if (reg == 0x1B) change |= c.T(T_GRP1_O) != c.T(T_GRP1_N);
+  if (reg == 0x1C) change |= (c.T(T_GRP0_O) != c.T(T_GRP0_N)) | (c.T(T_ENABL_O) != c.T(T_ENABL_N));
+  return change;
+}
 // Apply a TIA write (register reg at cycle t): collisions up to the write,
-// log record, register update.
+// log record, register update.  A kernel writes most registers on every line
+// with the value that they have; such a write leaves the span that the next
+// evaluation covers open, so the TIA warp evaluates a few spans a frame, not
+// several a line.
 __device__ __forceinline__ void fc_tia_write(IoCtx c, TiaSide &s, uint32_t cap, uint32_t reg, uint32_t v, uint32_t t) {
   const uint32_t eff = 3u * (t + 1u);
-  if ((COLL_REGS >> reg) & 1ull) fc_cx_eval(c, s, eff);
+  if (((COLL_REGS >> reg) & 1ull) && fc_coll_change(c, reg, v)) fc_cx_eval(c, s, eff);
   if ((LOG_REGS >> reg) & 1ull) fc_log(c, s, cap, eff, reg, v);
   switch (reg) {
     case 0x00: c.Tset(T_VSYNC, v); break;
