@@ -12,8 +12,9 @@
 // One thread per env walks its T steps from the last back to the first, so
 // every load and store of a step is one coalesced row of the time-major
 // arrays.  A walk is bound by the latency of its loads (a learner's batch is a
-// few warps an SM), so the steps go in groups of TARGET_STEPS whose loads are
-// all issued before the first is used, and blocks are small to spread the
+// few warps an SM), so the steps go in groups of TARGET_STEPS (the last one of
+// what is left, so a five-step return is one group) whose loads are all issued
+// before the first is used, and blocks are small to spread the
 // envs over the SMs (V-trace over 60 x 32768: 67 -> 22 us a call).  fp32
 // throughout, each operation rounded once (no contraction into
 // fused multiply-adds), in this order per step t (g = gamma, or 0 after a
@@ -30,7 +31,7 @@ namespace atari {
 
 constexpr int TARGET_STEPS = 8, TARGET_TPB = 64;
 
-// Steps t = first .. first - N + 1 of env i's walk.
+// Steps t = first .. first - N + 1 of env i's walk, those below 0 left out.
 template <int N>
 __device__ __forceinline__ float nstep_group(const float *rew, const uint8_t *done, int depth, int start, int first,
                                              int n, int i, float gamma, float R, float *ret) {
@@ -38,6 +39,7 @@ __device__ __forceinline__ float nstep_group(const float *rew, const uint8_t *do
   uint8_t d[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) {
+    if (k > first) continue;
     int slot = start + first - k;  // start < depth and t < T <= depth
     slot -= slot >= depth ? depth : 0;
     const size_t s = (size_t)slot * n + i;
@@ -46,6 +48,7 @@ __device__ __forceinline__ float nstep_group(const float *rew, const uint8_t *do
   }
 #pragma unroll
   for (int k = 0; k < N; ++k) {
+    if (k > first) continue;
     R = __fadd_rn(r[k], __fmul_rn(d[k] ? 0.0f : gamma, R));
     ret[(size_t)(first - k) * n + i] = R;
   }
@@ -58,10 +61,8 @@ __global__ void __launch_bounds__(TARGET_TPB) k_nstep_returns(const float *rew,
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   float R = values[(size_t)T * n + i];
-  int t = T - 1;
-  for (; t >= TARGET_STEPS - 1; t -= TARGET_STEPS)
+  for (int t = T - 1; t >= 0; t -= TARGET_STEPS)
     R = nstep_group<TARGET_STEPS>(rew, done, depth, start, t, n, i, gamma, R, ret);
-  for (; t >= 0; --t) R = nstep_group<1>(rew, done, depth, start, t, n, i, gamma, R, ret);
 }
 
 struct VtraceArgs {
@@ -81,6 +82,7 @@ __device__ __forceinline__ void vtrace_group(const VtraceArgs &a, int first, int
   uint8_t d[N];
 #pragma unroll
   for (int k = 0; k < N; ++k) {
+    if (k > first) continue;
     int slot = a.start + first - k;
     slot -= slot >= a.depth ? a.depth : 0;
     const size_t s = (size_t)slot * a.n + i, o = (size_t)(first - k) * a.n + i;
@@ -92,6 +94,7 @@ __device__ __forceinline__ void vtrace_group(const VtraceArgs &a, int first, int
   }
 #pragma unroll
   for (int k = 0; k < N; ++k) {
+    if (k > first) continue;
     const size_t o = (size_t)(first - k) * a.n + i;
     const float g = d[k] ? 0.0f : a.gamma;
     const float ratio = __fdiv_rn(p[k], m[k]);
@@ -114,9 +117,7 @@ __global__ void __launch_bounds__(TARGET_TPB) k_vtrace(const float *rew, const u
   const VtraceArgs a{rew, done, mu, values, pi, vs, adv, depth, start, n, gamma, rho_bar, c_bar};
   float v_next = values[(size_t)T * n + i];  // v_T = V(s_T)
   float V_next = v_next;
-  int t = T - 1;
-  for (; t >= TARGET_STEPS - 1; t -= TARGET_STEPS) vtrace_group<TARGET_STEPS>(a, t, i, v_next, V_next);
-  for (; t >= 0; --t) vtrace_group<1>(a, t, i, v_next, V_next);
+  for (int t = T - 1; t >= 0; t -= TARGET_STEPS) vtrace_group<TARGET_STEPS>(a, t, i, v_next, V_next);
 }
 
 }  // namespace atari
