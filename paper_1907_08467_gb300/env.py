@@ -52,6 +52,8 @@ PROF_NAMES = ["interpreter", "rasteriser", "preprocess", "fused_raster_preproces
 def load_library(path: str | None = None):
     """Build (if stale) and load libatari_gpu.so; declare every exported symbol."""
     global _lib
+    if _lib is not None and path is None:  # set once, after every symbol is declared: no lock on the calls' way
+        return _lib
     with _lock:
         if _lib is not None and path is None:
             return _lib
@@ -127,13 +129,13 @@ def footprint(n_envs: int, n_roms: int, **cfg) -> int:
 def _ptr(t):
     if t is None:
         return None
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()  # the declared argument types make it a pointer
 
 
 def _stream(stream):
     import torch
     s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    return s.cuda_stream
 
 
 class AtariEnv:
