@@ -279,50 +279,49 @@ __device__ __forceinline__ void fc_riot_write(IoCtx c, uint32_t a, uint32_t v, u
     c.S64(IO_TCWLO, now);
   }
 }
-// Whether a write can change the collisions after it: whether it changes its
-// register, or a delayed copy that it makes.  RESxx, HMOVE and CXCLR count as
-// changes.
-__device__ __forceinline__ bool fc_coll_change(IoCtx c, uint32_t reg, uint32_t v) {
-  if (reg == 0x2A || reg == 0x2C || (reg >= 0x10 && reg < 0x15)) return true;
-  const uint32_t slot = reg < 0x10 ? (reg == 1 ? (uint32_t)T_VBLANK : reg - 2)
-                                   : reg >= 0x25 ? T_VDELP0 + reg - 0x25
-                                                 : reg >= 0x1D ? (reg == 0x1F ? (uint32_t)T_ENABL_N : T_ENAM0 + reg - 0x1D)
-                                                               : reg == 0x1B ? (uint32_t)T_GRP0_N : (uint32_t)T_GRP1_N;
-  bool change = c.T(slot) != v;
-  if (reg == 0x1B) change |= c.T(T_GRP1_O) != c.T(T_GRP1_N);
-  if (reg == 0x1C) change |= (c.T(T_GRP0_O) != c.T(T_GRP0_N)) | (c.T(T_ENABL_O) != c.T(T_ENABL_N));
-  return change;
-}
+// Registers whose write only sets a slot of the file: all but the strobes, the
+// graphics with their delayed copies and RESMPx.
+constexpr uint64_t SET_REGS = 0xFFF0ull | (7ull << 0x1D) | (0x1Full << 0x20) | (7ull << 0x25);
 // Apply a TIA write (register reg at cycle t): collisions up to the write,
 // log record, register update.  A kernel writes most registers on every line
 // with the value that they have; such a write leaves the span that the next
-// evaluation covers open, so the TIA warp evaluates a few spans a frame, not
-// several a line.
+// evaluation covers open (the registers are the same on both sides of it), so
+// the TIA warp evaluates a few spans a frame, not several a line.  Writes that
+// only set a slot, nearly all of them, do not come to the switch: a level of
+// its compare tree costs 30 cycles, and the TIA warp has to keep up with
+// rounds of about 160.
 __device__ __forceinline__ void fc_tia_write(IoCtx c, TiaSide &s, uint32_t cap, uint32_t reg, uint32_t v, uint32_t t) {
   const uint32_t eff = 3u * (t + 1u);
-  if (((COLL_REGS >> reg) & 1ull) && fc_coll_change(c, reg, v)) fc_cx_eval(c, s, eff);
+  const bool set = ((SET_REGS >> reg) & 1ull) != 0;
+  // NUSIZ0 .. PF2 are slots 2 .. 13, HMP0 .. HMBL 27 .. 31, ENAM0 .. ENABL 14 .. 16, VDELP0 .. VDELBL 22 .. 24
+  const uint32_t slot = reg - (reg < 0x10u ? 2u : reg - 0x20u < 5u ? 5u : 15u);
+  bool change = true;
+  if (set) change = c.T(slot) != v;
+  else if (reg == 0x1B) change = (c.T(T_GRP0_N) != v) | (c.T(T_GRP1_O) != c.T(T_GRP1_N));
+  else if (reg == 0x1C)
+    change = (c.T(T_GRP1_N) != v) | (c.T(T_GRP0_O) != c.T(T_GRP0_N)) | (c.T(T_ENABL_O) != c.T(T_ENABL_N));
+  if (change & (((COLL_REGS >> reg) & 1ull) != 0)) fc_cx_eval(c, s, eff);
   if ((LOG_REGS >> reg) & 1ull) fc_log(c, s, cap, eff, reg, v);
+  if (set) {
+    c.Tset(slot, v);
+    return;
+  }
+  if (reg == 0x1B) {
+    c.Tset(T_GRP1_O, c.T(T_GRP1_N));
+    c.Tset(T_GRP0_N, v);
+    return;
+  }
+  if (reg == 0x1C) {
+    c.Tset(T_GRP0_O, c.T(T_GRP0_N));
+    c.Tset(T_ENABL_O, c.T(T_ENABL_N));
+    c.Tset(T_GRP1_N, v);
+    return;
+  }
   switch (reg) {
     case 0x00: c.Tset(T_VSYNC, v); break;
     case 0x01: c.Tset(T_VBLANK, v); break;
-    case 0x04: case 0x05: case 0x06: case 0x07: case 0x08: case 0x09: case 0x0A: case 0x0B: case 0x0C:
-    case 0x0D: case 0x0E: case 0x0F:
-      c.Tset(reg - 2, v); break;                 // NUSIZ0 .. PF2 are slots 2 .. 13
-    case 0x10: c.Tset(T_P0, fc_res_pos(eff, 5, 3)); break;
-    case 0x11: c.Tset(T_P1, fc_res_pos(eff, 5, 3)); break;
-    case 0x12: c.Tset(T_M0, fc_res_pos(eff, 4, 2)); break;
-    case 0x13: c.Tset(T_M1, fc_res_pos(eff, 4, 2)); break;
-    case 0x14: c.Tset(T_BL, fc_res_pos(eff, 4, 2)); break;
-    case 0x1B: c.Tset(T_GRP1_O, c.T(T_GRP1_N)); c.Tset(T_GRP0_N, v); break;
-    case 0x1C:
-      c.Tset(T_GRP0_O, c.T(T_GRP0_N)); c.Tset(T_ENABL_O, c.T(T_ENABL_N)); c.Tset(T_GRP1_N, v); break;
-    case 0x1D: c.Tset(T_ENAM0, v); break;
-    case 0x1E: c.Tset(T_ENAM1, v); break;
-    case 0x1F: c.Tset(T_ENABL_N, v); break;
-    case 0x20: case 0x21: case 0x22: case 0x23: case 0x24: c.Tset(T_HMP0 + (reg - 0x20), v); break;
-    case 0x25: c.Tset(T_VDELP0, v); break;
-    case 0x26: c.Tset(T_VDELP1, v); break;
-    case 0x27: c.Tset(T_VDELBL, v); break;
+    case 0x10: case 0x11: c.Tset(T_P0 + reg - 0x10, fc_res_pos(eff, 5, 3)); break;
+    case 0x12: case 0x13: case 0x14: c.Tset(T_P0 + reg - 0x10, fc_res_pos(eff, 4, 2)); break;
     case 0x28: case 0x29: {
       const uint32_t i = reg - 0x28;
       if ((c.T(T_RESMP0 + i) & 2) && !(v & 2)) {
