@@ -347,7 +347,7 @@ __device__ void step_env(Console<Mem> &m, uint8_t *st, int i, const StepArgs &a,
   if (a.counters) {
     a.counters[3 * i] = m.instret;
     a.counters[3 * i + 1] = log_total;
-    a.counters[3 * i + 2] = 0;  // one thread per env: no lockstep issue rounds
+    a.counters[3 * i + 2] = 0;  // one thread per env: no issue rounds
   }
   Console<Mem>::st32(st + S::STATUS, env_status);
   Console<Mem>::st32(st + S::STEP, step_no + 1);
@@ -360,13 +360,19 @@ __device__ void step_env(Console<Mem> &m, uint8_t *st, int i, const StepArgs &a,
   }
 }
 
-// Plain form: one thread per env, state, RAM and ROM in global memory.
-__global__ void __launch_bounds__(128) k_interp_plain(StepArgs a) {
+// Plain form: one thread per env, state, RAM and ROM in global memory; `lanes`
+// threads of a warp run envs.  Lanes at different opcodes take the decoder's
+// branches one after another, so a warp of one env is fastest while all envs
+// fit as warps of their own (ms a step at 1, 2, 4, 8, 32 lanes: 22, 30, 38, 52,
+// 79 for 1024 sprite envs, 46, 60, 74, 80, 84 for 4096); past that the issue
+// slots are full and full warps win (281, 277, 239, 199, 165 for 32768 banked
+// envs).
+__global__ void __launch_bounds__(64) k_interp_plain(StepArgs a, int lanes) {
   __shared__ uint32_t dec[256];
   for (int t = threadIdx.x; t < 256; t += blockDim.x) dec[t] = a.dec[t];
   __syncthreads();
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.n) return;
+  const int lane = threadIdx.x & 31, i = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + lane;
+  if (lane >= lanes || i >= a.n) return;
   uint8_t *st = a.state + (size_t)i * 256;
   uint32_t rom = st[S::ROM] | (uint32_t)st[S::ROM + 1] << 8;
   RomInfo ri = rom_info(a.info, rom);
@@ -976,7 +982,10 @@ int step_plain(atari_env *E, const uint8_t *d_actions, uint8_t *d_obs, int32_t *
   a.seed = c.seed;
   {
     ProfScope p(E, ATARI_PROF_INTERP, s);
-    k_interp_plain<<<(E->n + 127) / 128, 128, 0, s>>>(a);
+    int sms = 0;
+    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, E->device));
+    const int lanes = E->n <= 32 * sms ? 1 : 32, per_block = 2 * lanes;  // blocks of two warps
+    k_interp_plain<<<(E->n + per_block - 1) / per_block, 64, 0, s>>>(a, lanes);
   }
   CUDA_TRY(cudaGetLastError());
   long long warps = (long long)E->n * 2;
