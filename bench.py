@@ -94,7 +94,7 @@ def parse(argv=None):
     p.add_argument("--grouping", type=int, default=0, choices=[0, 1, 2])
     p.add_argument("--dispatch", type=int, default=0, choices=[0, 1, 2])
     p.add_argument("--divergence", action="store_true",
-                   help="divergence study: frames/s and lockstep lane efficiency per window of steps from one shared "
+                   help="divergence study: frames/s and lane efficiency per window of steps from one shared "
                         "start state per cartridge, beside a run from the usual random start states and the oracle "
                         "on the host from the same shared start")
     p.add_argument("--window", type=int, default=10)
@@ -537,7 +537,7 @@ def divergence_run(args, w, rank):
     """Paper Section 4, Fig. 3 and its CPU counterpart in the appendix: start
     every env of a cartridge from the same state (its first cached start
     state) and follow frames/s and the fraction of lanes executing per
-    lockstep issue round window by window as random actions drive the envs
+    issue round window by window as random actions drive the envs
     apart; the same for a run from the usual random start states, and the
     oracle's frames/s on the host from the same shared start (a bounded env
     sample)."""
@@ -767,7 +767,7 @@ def main(argv=None):
     roof = interp_roofline(prof, instr, kern, shape[0], shape_dict(shape)["dispatch"], args.config, w.n_envs,
                            w.frameskip)
     if roof and lane_rounds:
-        # fraction of a warp's lanes executing per lockstep issue round
+        # instructions per lane and issue round: the fraction of a warp's lanes that make progress in a round
         roof["lockstep_lane_efficiency"] = instr / lane_rounds
     roof2 = fused_roofline(prof, logrec, args.config, w.n_envs)
     kernels = {k: {"ms_per_launch": v[0] / max(1, v[1]), "launches": v[1]} for k, v in prof.items()}

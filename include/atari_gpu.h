@@ -3,7 +3,7 @@
  *
  * The library steps thousands of independent consoles (MOS 6507 CPU, TIA
  * video/collision chip, RIOT 6532 RAM/timer/ports, 2-32 KB cartridges with
- * F8, F6 and F4 bank switching) in lockstep on one GPU.  It is the data-parallel
+ * F8, F6 and F4 bank switching) step by step on one GPU.  It is the data-parallel
  * emulation path of "Accelerating Reinforcement Learning through GPU Atari
  * Emulation" (CuLE), Section 3: a CPU-interpreter kernel that logs TIA
  * register writes to a per-env buffer in device memory, a TIA kernel that
@@ -296,11 +296,11 @@ ATARI_API int atari_env_get_cache(atari_env *env, void *d_dst, atari_stream stre
 /* Counters of the last step: 6502 instructions executed (sum over envs; the
  * iterations of a RIOT-timer wait loop that the batched form retires at once,
  * see idle_skip, are not counted), TIA
- * log records written, and lockstep issue rounds summed over the envs (each
+ * log records written, and issue rounds summed over the envs (each
  * env counts the rounds its warp issued, so instructions / lane_rounds is
  * the fraction of a warp's lanes that execute per round: the emulated-
  * instruction SIMT efficiency the paper's divergence discussion in Section 4
- * is about; 0 in the plain form, which has no lockstep issue).  Host
+ * is about; 0 in the plain form, which counts no rounds).  Host
  * pointers, any may be NULL; synchronises `stream`. */
 ATARI_API int atari_env_counters(atari_env *env, uint64_t *instructions, uint64_t *log_records,
                                  uint64_t *lane_rounds, atari_stream stream);

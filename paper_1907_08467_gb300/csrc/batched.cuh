@@ -10,7 +10,7 @@
 //
 // Fused replay + preprocessing (the paper's TIA kernel with the rows of a
 // frame spread over several warps, followed by the agent's preprocessing):
-// one block per env renders frames F-1 and F into shared memory, takes the
+// one block per env paints frame F over frame F-1 in shared memory, as the
 // pixelwise maximum of their lumas, resamples to 84x84 and pushes the plane
 // into the env's stack; frames never reach HBM.
 #pragma once

@@ -256,7 +256,7 @@ class AtariEnv:
         return out
 
     def counters(self, stream=None):
-        """(6502 instructions executed, TIA writes logged, lockstep issue rounds
+        """(6502 instructions executed, TIA writes logged, issue rounds
         summed over envs) of the last step; timer-wait iterations retired at
         once are not counted as executed."""
         a, b, c = C.c_uint64(), C.c_uint64(), C.c_uint64()
