@@ -50,22 +50,20 @@ SM_COUNT, SMSP_PER_SM, SM_MAX_MHZ = 152, 4, 2070.0
 # never captured reports achieved = null.
 INTERP_CAPTURES = {
     # (kernel, envs per warp, opcode dispatch, config): (warp-inst per executed 6502 instruction, DRAM bytes per env-step)
-    ("k_interp_split", 32, 1, 3): (2234457806 / 433965025, (13179648 + 114831104) / 32768),
-    ("k_interp_split", 32, 2, 3): (2213124575 / 433965025, (13961216 + 124522240) / 32768),
-    ("k_interp_split", 32, 1, 2): (445471194 / 94159103, (1266688 + 88064) / 4096),
-    ("k_interp_split", 32, 2, 2): (442946243 / 94159103, (1260288 + 104192) / 4096),
+    ("k_interp_split", 32, 1, 3): (1412574931 / 433986434, (31363840 + 456011776) / 32768),
+    ("k_interp_split", 32, 1, 2): (272340736 / 94164973, (1458432 + 9803264) / 4096),
 }
 # Algorithmic bytes of the fused rasterise + preprocess kernel per env-step,
-# besides 4 bytes per logged TIA write: snapshots and record counts of the two
-# rendered frames (2 x 64 + 2 x 8), the three older stack planes read from the
+# besides 4 bytes per logged TIA write: band snapshots and record counts of the
+# two rendered frames (2 x 105 x 48 + 2 x 8), the three older stack planes read from the
 # ring, the 84x84x4 stack written out, the new plane written to the ring and
 # the ring head.
-FUSED_FIXED_BYTES_PER_ENV_STEP = 2 * 64 + 2 * 8 + 3 * 7056 + 4 * 7056 + 7056 + 1
+FUSED_FIXED_BYTES_PER_ENV_STEP = 2 * 105 * 48 + 2 * 8 + 3 * 7056 + 4 * 7056 + 7056 + 1
 # Warp instructions per env-step of the fused kernel (it is bound by issue,
 # not HBM), from the same captures: smsp__inst_executed.sum / env-steps.
-FUSED_WARP_INST_PER_ENV_STEP = {3: 5979554498 / 32768, 2: 711969603 / 4096}
+FUSED_WARP_INST_PER_ENV_STEP = {3: 1220170065 / 32768, 2: 129733917 / 4096}
 # DRAM bytes per env-step of the fused kernel, from an ncu capture per config.
-FUSED_DRAM_BYTES_PER_ENV_STEP = {3: (863958016 + 1106787000) / 32768, 2: (109476096 + 94397696) / 4096}
+FUSED_DRAM_BYTES_PER_ENV_STEP = {3: (1175249408 + 1110222848) / 32768, 2: (148432640 + 97480704) / 4096}
 
 
 def parse(argv=None):
