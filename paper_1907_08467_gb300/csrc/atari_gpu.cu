@@ -591,6 +591,17 @@ int validate(const atari_config &c) {
 namespace {
 
 constexpr size_t MAX_SMEM = 227 * 1024 - 64;  // a block's dynamic shared memory, beside a few static bytes
+// A kernel's limit on dynamic shared memory belongs to the kernel on the
+// device, not to an env: it is only ever set to the most that any env can ask
+// for, so that no env's launches depend on which envs or servers were made
+// before or after it.  Occupancy follows a launch's own size, not the limit.
+int raise_smem_limits() {
+  constexpr cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  CUDA_TRY(cudaFuncSetAttribute(k_cache_run, at, (int)MAX_SMEM));
+  CUDA_TRY(cudaFuncSetAttribute(k_interp_split, at, (int)MAX_SMEM));
+  CUDA_TRY(cudaFuncSetAttribute(k_interp_batched, at, (int)MAX_SMEM));
+  return 0;
+}
 size_t interp_smem(const atari_env *E) {
   return block_smem((uint32_t)E->rom_stage, (uint32_t)(E->lanes * E->warps));
 }
@@ -638,10 +649,8 @@ int build_groups(atari_env *E, int lanes, int warps, bool split) {
   const size_t smem = interp_smem(E);
   int per_sm = 0;
   if (split) {
-    CUDA_TRY(cudaFuncSetAttribute(k_interp_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp_split, 2 * warps * 32, smem));
   } else {
-    CUDA_TRY(cudaFuncSetAttribute(k_interp_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp_batched, warps * 32, smem));
   }
   int sms = 0;
@@ -881,6 +890,7 @@ int atari_env_create(const uint8_t *const *roms, const size_t *rom_sizes, const 
     return bail(rc);
   if (luma && (rc = up(E->d_luma, luma, 128))) return bail(rc);
 
+  if ((rc = raise_smem_limits())) return bail(rc);
   // start-state cache (Section 3): run each ROM from power-on on the device
   uint8_t *d_work = nullptr, *d_snaps = nullptr;
   size_t scratch = 0;
@@ -895,7 +905,6 @@ int atari_env_create(const uint8_t *const *roms, const size_t *rom_sizes, const 
     for (int r = 0; r < n_roms; ++r) max_banks = std::max(max_banks, E->h_banks[r]);
     const int stage = (int)max_banks * 4096;
     const size_t cache_smem = block_smem((uint32_t)stage, 1);
-    cudaFuncSetAttribute(k_cache_run, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cache_smem);
     k_cache_run<<<n_roms, 128, cache_smem>>>(d_work, d_snaps, E->d_roms, E->d_info, E->d_dec_op, stage,
                                            c.startup_frames, c.max_noops, 1);
     int tot = n_roms * c.n_cache;
