@@ -94,6 +94,7 @@ struct TiaSide {
   uint32_t cx;        // collision latches
   uint32_t bar;       // frame-relative line of the HMOVE bar, ~0: none in this frame or later
   uint64_t l0;        // first line of the frame
+  uint32_t hi;        // bits 16-31 of the cycles that the events carry
   uint32_t *log;      // next record of the logged frame, null: not logged
   uint32_t nrec;      // records so far
   uint8_t *bands;     // the frame's band snapshots
@@ -364,6 +365,8 @@ __device__ __forceinline__ void fc_tia_write(IoCtx c, TiaSide &s, uint32_t cap, 
 // cursor.  Bits 16-31 are a CPU cycle of the frame:
 //   write       bit 14 = 0 | register << 8 | value; the cycle after the write's
 //   control     bit 14 = 1 | kind << 8 | argument:
+//     high      bits 16-31 are those bits of the cycles of all events up to the frame's end (0 at its start;
+//               not 0 only where a state was loaded far past the line cap, for the one instruction that it runs)
 //     begin / end of a logged frame (argument: 0 frame F-1, 1 frame F), end of the step
 //     sync      evaluate collisions up to the cycle and acknowledge
 //     frame end evaluate collisions up to the frame's last cycle
@@ -371,7 +374,7 @@ __device__ __forceinline__ void fc_tia_write(IoCtx c, TiaSide &s, uint32_t cap, 
 //               end; bits 16-31 and, above them, the argument)
 constexpr uint32_t EV_CTRL = 1u << 14, EV_BEGIN_LOG = EV_CTRL, EV_END_LOG = EV_CTRL | 1u << 8,
                    EV_STEP_END = EV_CTRL | 2u << 8, EV_SYNC = EV_CTRL | 3u << 8, EV_FRAME_END = EV_CTRL | 4u << 8,
-                   EV_REBASE = EV_CTRL | 5u << 8;
+                   EV_REBASE = EV_CTRL | 5u << 8, EV_HIGH = EV_CTRL | 6u << 8;
 // Lap parity of queue position k.
 constexpr uint32_t EV_LAP = 1u << 15;
 __device__ __forceinline__ uint32_t lap_bit(uint32_t k) { return (~k * (EV_LAP / QLEN)) & EV_LAP; }
@@ -391,14 +394,15 @@ constexpr uint32_t TIA_ACK = 1u, TIA_END = 2u;
 // TIA_END when it ends the step.
 __device__ __forceinline__ uint32_t tia_event(IoCtx c, uint32_t ev, TiaSide &s, const TiaOut &o) {
   if (!(ev & EV_CTRL)) {
-    fc_tia_write(c, s, o.log_cap, (ev >> 8) & 0x3F, ev & 0xFF, ((ev >> 16) - 1u) & 0xFFFFu);
+    fc_tia_write(c, s, o.log_cap, (ev >> 8) & 0x3F, ev & 0xFF, (ev >> 16 | s.hi) - 1u);
     return 0;
   }
   const uint32_t kind = (ev >> 8) & 0x3F, slot = ev & 1, cycle = ev >> 16;
   switch (kind) {
-    case 3: fc_cx_eval(c, s, 3u * cycle); return TIA_ACK;
+    case 3: fc_cx_eval(c, s, 3u * (cycle | s.hi)); return TIA_ACK;
     case 4:
-      fc_cx_eval(c, s, 3u * cycle);
+      fc_cx_eval(c, s, 3u * (cycle | s.hi));
+      s.hi = 0;
       s.lines = 0;
       return 0;
     case 5: {
@@ -423,6 +427,7 @@ __device__ __forceinline__ uint32_t tia_event(IoCtx c, uint32_t ev, TiaSide &s, 
       s.log_total += s.nrec;
       s.log = nullptr;
       return 0;
+    case 6: s.hi = ev & 0xFFFF0000u; return 0;
     default: return TIA_ACK | TIA_END;
   }
 }
@@ -581,6 +586,7 @@ struct FastConsoleT {
   uint32_t idle;           // retire RIOT-timer wait-loop iterations at once
   uint32_t unit;           // 1, as a value that the compiler does not know (see mad)
   uint32_t qtail, qhead_seen, nreq, vsync_c, vblank_c, broken;  // qhead_seen: the TIA side's cursor as last read
+  uint32_t ev_hi;          // bits 16-31 of the cycles of the events as the TIA side has them
   uint64_t l0c;
   TiaSide ts;              // single-warp form: the TIA side
   TiaOut to;
@@ -637,7 +643,7 @@ struct FastConsoleT {
     status = 0; instret = 0; frame_inst = 0; rounds = 0; pend = 0; vs_kf = ~0u;
     vsync_c = io.T(T_VSYNC);
     vblank_c = io.T(T_VBLANK);
-    qtail = qhead_seen = nreq = broken = 0;
+    qtail = qhead_seen = nreq = broken = ev_hi = 0;
     io.Sset(IO_QHEAD, 0); io.Sset(IO_ACK, 0);
     if constexpr (!SPLIT) ts = tia_start(io, l0c, kf);
   }
@@ -721,6 +727,16 @@ struct FastConsoleT {
     vsm32(off.q + 4 * (qtail & (QLEN - 1))) = ev | lap_bit(qtail);
     ++qtail;
   }
+  // An event at a cycle of the frame, its upper half sent ahead where it
+  // differs from the last event's.  The hot loop's events need none: its
+  // cycles are below the line cap.
+  __device__ __forceinline__ void push_at(uint32_t ev, uint32_t cycle) {
+    if (cycle >> 16 != ev_hi) {
+      ev_hi = cycle >> 16;
+      push(EV_HIGH | ev_hi << 16);
+    }
+    push(ev | cycle << 16);
+  }
   __device__ __forceinline__ void drain() {
     tia_drain(io, off.q, ts, to, qtail);
     qhead_seen = ts.head;
@@ -729,7 +745,7 @@ struct FastConsoleT {
   __device__ void sync_collisions(uint32_t t) {
     if constexpr (SPLIT) {
       if (broken) return;
-      push(EV_SYNC | t << 16);
+      push_at(EV_SYNC, t);
       ++nreq;
       if (!broken && !fc_q_wait_ack(io, nreq)) stall();
       qhead_seen = qtail;  // acknowledged: the queue is empty
@@ -764,7 +780,7 @@ struct FastConsoleT {
       if (!(v & 0x40)) io.Sset(IO_LATCH, 0);
       else if (io.G(IO_FIRE)) io.Sset(IO_LATCH, 1);
     }
-    push((t + 1u) << 16 | reg << 8 | v);
+    push_at(reg << 8 | v, t + 1u);
   }
   __device__ __forceinline__ uint32_t rd(uint32_t addr, uint32_t t) {
     const uint32_t a = addr & 0x1FFF;
@@ -1039,7 +1055,8 @@ struct FastConsoleT {
 
   // Append the end of the current frame and start counting the next.
   __device__ __forceinline__ void end_frame(uint32_t next_rel) {
-    push(EV_FRAME_END | kf << 16);
+    push_at(EV_FRAME_END, kf);
+    ev_hi = 0;
     for (uint32_t left = next_rel; left;) {  // one event, but for loaded states far past the line cap
       const uint32_t n = left < 0xFFFFFFu ? left : 0xFFFFFFu;
       push(EV_REBASE | n << 16 | n >> 16);
