@@ -324,11 +324,11 @@ ATARI_API int atari_env_profile(atari_env *env, int enable);
 ATARI_API int atari_env_profile_read(atari_env *env, double *ms, uint64_t *launches);
 
 /* Launch shape in use (batched form: the autotuned or configured values;
- * plain form: 32 envs per warp, 128 per block, 1 warp per frame, and the
- * grid of the interpreter launch).  tia_warps: 2 when paired TIA warps run
- * the envs' TIA side, else 1.  grouping: 1 env order, 2 bank-aware (see
- * atari_config; the plain form reports 1), plus 4 when the compact opcode
- * switch is in use.  Host pointers; any may be NULL.
+ * plain form: 1 or 32 envs per warp, two warps per block, 1 warp per frame)
+ * and the grid of the interpreter launch.  tia_warps: 2 when paired TIA warps
+ * run the envs' TIA side, else 1.  grouping: 1 env order, 2 bank-aware (see
+ * atari_config; the plain form reports 1), plus 4 when the configuration has
+ * dispatch 2 (which changes nothing else).  Host pointers; any may be NULL.
  * The paper runs one emulator per thread with no grouping (Section 3); the
  * shape is this library's own tuning and changes speed only, never results. */
 ATARI_API int atari_env_launch_shape(atari_env *env, int *envs_per_warp, int *envs_per_block,

@@ -502,6 +502,7 @@ constexpr int HOST_CHUNKS = 8;
 
 struct atari_env {
   int device = 0;
+  int sms = 0;  // the device's multiprocessors
   int n = 0, n_roms = 0;
   atari_config cfg{};
   size_t bytes = 0;
@@ -653,9 +654,7 @@ int build_groups(atari_env *E, int lanes, int warps, bool split) {
   } else {
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_interp_batched, warps * 32, smem));
   }
-  int sms = 0;
-  CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, E->device));
-  E->max_blocks = std::max(1, per_sm) * sms;
+  E->max_blocks = std::max(1, per_sm) * E->sms;
   E->grid = std::max(1, std::min(ng, E->max_blocks));
   for (auto &g : E->graphs) cudaGraphExecDestroy(g.exec);
   E->graphs.clear();
@@ -891,6 +890,10 @@ int atari_env_create(const uint8_t *const *roms, const size_t *rom_sizes, const 
   if (luma && (rc = up(E->d_luma, luma, 128))) return bail(rc);
 
   if ((rc = raise_smem_limits())) return bail(rc);
+  {
+    const cudaError_t e = cudaDeviceGetAttribute(&E->sms, cudaDevAttrMultiProcessorCount, E->device);
+    if (e != cudaSuccess) return bail(fail(ATARI_ECUDA, std::string("device attribute: ") + cudaGetErrorString(e)));
+  }
   // start-state cache (Section 3): run each ROM from power-on on the device
   uint8_t *d_work = nullptr, *d_snaps = nullptr;
   size_t scratch = 0;
@@ -964,6 +967,10 @@ int atari_env_reset(atari_env *E, const uint8_t *d_mask, atari_stream stream) {
 
 namespace {
 
+// Envs a warp and blocks (of two warps) of the plain interpreter's launches.
+int plain_lanes(const atari_env *E) { return E->n <= 32 * E->sms ? 1 : 32; }
+int plain_grid(const atari_env *E) { return (E->n + 2 * plain_lanes(E) - 1) / (2 * plain_lanes(E)); }
+
 int step_plain(atari_env *E, const uint8_t *d_actions, uint8_t *d_obs, int32_t *d_rewards, uint8_t *d_dones,
                cudaStream_t s) {
   const atari_config &c = E->cfg;
@@ -991,10 +998,7 @@ int step_plain(atari_env *E, const uint8_t *d_actions, uint8_t *d_obs, int32_t *
   a.seed = c.seed;
   {
     ProfScope p(E, ATARI_PROF_INTERP, s);
-    int sms = 0;
-    CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, E->device));
-    const int lanes = E->n <= 32 * sms ? 1 : 32, per_block = 2 * lanes;  // blocks of two warps
-    k_interp_plain<<<(E->n + per_block - 1) / per_block, 64, 0, s>>>(a, lanes);
+    k_interp_plain<<<plain_grid(E), 64, 0, s>>>(a, plain_lanes(E));
   }
   CUDA_TRY(cudaGetLastError());
   long long warps = (long long)E->n * 2;
@@ -1486,10 +1490,10 @@ int atari_env_launch_shape(atari_env *E, int *envs_per_warp, int *envs_per_block
   g_err.clear();
   if (!E) return fail(ATARI_EINVAL, "env is NULL");
   const bool b = E->cfg.form == ATARI_FORM_BATCHED;
-  if (envs_per_warp) *envs_per_warp = b ? E->lanes : 32;
-  if (envs_per_block) *envs_per_block = b ? E->lanes * E->warps : 128;
+  if (envs_per_warp) *envs_per_warp = b ? E->lanes : plain_lanes(E);
+  if (envs_per_block) *envs_per_block = b ? E->lanes * E->warps : 2 * plain_lanes(E);
   if (raster_warps_per_frame) *raster_warps_per_frame = b ? E->wpf : 1;
-  if (grid) *grid = b ? E->grid : (E->n + 127) / 128;
+  if (grid) *grid = b ? E->grid : plain_grid(E);
   if (tia_warps) *tia_warps = (b && E->split) ? 2 : 1;
   if (grouping) *grouping = b ? (E->grouping | (E->compact ? 4 : 0)) : 1;
   return 0;

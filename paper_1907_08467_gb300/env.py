@@ -301,8 +301,8 @@ class AtariEnv:
 
     def launch_shape(self):
         """(envs per warp, envs per block, warps per frame, interpreter grid,
-        tia_warps: 2 with paired TIA warps, else 1, grouping: 1 env order, 2 bank-aware, + 4 with the
-        compact opcode switch)."""
+        tia_warps: 2 with paired TIA warps, else 1, grouping: 1 env order, 2 bank-aware, + 4 when
+        dispatch is 2)."""
         v = [C.c_int() for _ in range(6)]
         _check(self.lib.atari_env_launch_shape(self.h, *[C.byref(x) for x in v]))
         return tuple(x.value for x in v)
