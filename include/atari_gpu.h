@@ -81,7 +81,9 @@ typedef struct {
     int output_mode;      /* ATARI_OUT_* */
     int form;             /* ATARI_FORM_* */
     int log_cap;          /* TIA-write log entries per rendered frame (>= 256; default 4096) */
-    int envs_per_block;   /* batched form: envs per interpreter block, <= 128 (0 = autotune) */
+    int envs_per_block;   /* batched form: envs per interpreter block, <= 256 (0 = autotune): up to eight warps,
+                             fewer where the largest cartridge leaves no shared memory for them
+                             (atari_env_launch_shape tells) */
     int envs_per_warp;    /* batched form: envs per warp, 1..32 (0 = autotune); fewer than 32 trades
                              SIMT width for more independent instruction streams on small batches */
     int raster_warps_per_frame; /* batched form, 0..4.  Kept for callers: the painting kernels' blocks have one

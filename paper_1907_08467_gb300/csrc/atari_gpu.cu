@@ -578,10 +578,10 @@ int validate(const atari_config &c) {
   if (c.form != ATARI_FORM_PLAIN && c.form != ATARI_FORM_BATCHED) return fail(ATARI_EINVAL, "bad form");
   if (c.log_cap < 256 || c.log_cap > (1 << 20)) return fail(ATARI_EINVAL, "log_cap must be in 256..2^20");
   if (c.sticky != 0 && c.sticky != 1) return fail(ATARI_EINVAL, "sticky must be 0 or 1");
-  if (c.envs_per_block < 0 || c.envs_per_block > 128 || c.envs_per_warp < 0 || c.envs_per_warp > 32 ||
+  if (c.envs_per_block < 0 || c.envs_per_block > 256 || c.envs_per_warp < 0 || c.envs_per_warp > 32 ||
       c.raster_warps_per_frame < 0 || c.raster_warps_per_frame > 4 || c.tia_warps < 0 || c.tia_warps > 3 ||
       c.grouping < 0 || c.grouping > 2 || c.dispatch < 0 || c.dispatch > 2 || c.idle_skip < 0 || c.idle_skip > 1)
-    return fail(ATARI_EINVAL, "envs_per_block must be 0..128, envs_per_warp 0..32, raster_warps_per_frame 0..4, "
+    return fail(ATARI_EINVAL, "envs_per_block must be 0..256, envs_per_warp 0..32, raster_warps_per_frame 0..4, "
                               "tia_warps 0..3, grouping 0..2, dispatch 0..2, idle_skip 0..1");
   return 0;
 }
@@ -1200,7 +1200,9 @@ int setup_batched(atari_env *E, const std::vector<uint8_t> &img, const std::vect
   const atari_config &c = E->cfg;
   if (c.raster_warps_per_frame > 0) E->wpf = c.raster_warps_per_frame;
   if (c.envs_per_block > 0 && c.envs_per_warp > 0) {
-    int L = std::min(32, c.envs_per_warp), W = std::max(1, std::min(4, c.envs_per_block / L));
+    // at most eight warps, as many as the largest cartridge leaves shared memory for
+    int L = std::min(32, c.envs_per_warp), W = std::max(1, std::min(8, c.envs_per_block / L));
+    while (W > 1 && block_smem((uint32_t)E->rom_stage, (uint32_t)(L * W)) > MAX_SMEM) --W;
     E->grouping = c.grouping ? c.grouping : 1;
     E->compact = c.dispatch == 2;
     return build_groups(E, L, W, c.tia_warps >= 2);
