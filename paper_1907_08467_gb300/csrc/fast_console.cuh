@@ -1234,12 +1234,13 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
     m = __ballot_sync(wmask, (run == 0) & active);
     if (m != 0 && (m == act || ++held > 1)) {
       held = 0;
-      ++rounds;
+      const uint32_t r0 = ++rounds;
       if (active && run == 0) {
         leave();
         active = fc_service<SPLIT, Hook>(this, &hook);
         enter(!active);
       }
+      rounds = r0 + __reduce_max_sync(wmask, rounds - r0);  // a lane's further decoder passes hold up the others
       act = __ballot_sync(wmask, active);
       if (act == 0) break;
     }
