@@ -135,7 +135,8 @@ std::vector<uint32_t> build_decode_table() {
 }
 
 // The batched console's decode bytes: per opcode, operation | page-cross
-// penalty << 7, then mode | cycles << 4, then the control words.
+// penalty << 7, then mode | cycles << 4, then the quick kinds and the control
+// words.
 std::vector<uint8_t> build_dec_op(const std::vector<uint32_t> &dec) {
   std::vector<uint8_t> d(DEC_BYTES, 0);
   for (int o = 0; o < 256; ++o) {
@@ -143,7 +144,7 @@ std::vector<uint8_t> build_dec_op(const std::vector<uint32_t> &dec) {
     d[o] = (uint8_t)((t & 0x7F) | ((t >> 16) & 1u) << 7);
     d[256 + o] = (uint8_t)(((t >> 8) & 0xFu) | ((t >> 12) & 0xFu) << 4);
   }
-  build_ctl(dec.data(), d.data() + 512);
+  build_ctl(dec.data(), d.data());
   return d;
 }
 

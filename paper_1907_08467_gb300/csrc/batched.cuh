@@ -263,7 +263,7 @@ __device__ __forceinline__ void interp_block(const BatchArgs &a) {
     }
   }
 }
-__global__ void __launch_bounds__(256, 2) k_interp_batched(const __grid_constant__ BatchArgs a) { interp_block<false>(a); }
+__global__ void __launch_bounds__(256, 1) k_interp_batched(const __grid_constant__ BatchArgs a) { interp_block<false>(a); }
 __global__ void __launch_bounds__(512, 1) k_interp_split(const __grid_constant__ BatchArgs a) { interp_block<true>(a); }
 
 // Bank-aware grouping: within each cartridge's run [seg[r], seg[r+1]) of the

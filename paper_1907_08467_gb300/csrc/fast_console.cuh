@@ -13,10 +13,12 @@
 //   - the block's cartridge staged in shared memory as one word per byte (64 KB
 //     for an F6 cartridge), the byte and the two after it: an instruction is
 //     one load, and a data byte the first byte of its word.
-// Instructions the hot loop does not take (TIA and RIOT reads, RIOT, VSYNC
-// and VBLANK writes, stack and pointer instructions, undocumented opcodes,
-// decimal arithmetic, fetches outside the cartridge or next to a bank
-// hotspot) run the general decoder out of line.
+// Instructions the hot loop does not take are served beside it, out of line:
+// accesses through pointers, stack instructions, BIT, TIA and RIOT reads, RIOT
+// and VBLANK writes, hotspots, decimal arithmetic and undocumented opcodes with
+// the console in registers (fc_quick), what is left (frame ends, interrupts,
+// JMP through a pointer, fetches outside the cartridge or next to a hotspot) by
+// the general decoder.
 #pragma once
 #include <cstdint>
 
@@ -532,13 +534,16 @@ struct EnvOff {
 // (address - 0x80) for every address below the cartridge's and looks at the
 // value only when the address is RAM's; the cartridge (16 KB at least) behind
 // the RAM and the tables before it keep those loads inside the block's memory.
-constexpr uint32_t OFF_REG = 0, OFF_DEC = OFF_REG + REGION_BYTES, OFF_CTL = OFF_DEC + 512, OFF_RAM = OFF_DEC + DEC_BYTES;
+constexpr uint32_t OFF_REG = 0, OFF_DEC = OFF_REG + REGION_BYTES, OFF_CTL = OFF_DEC + DEC_CTL, 
+                   OFF_RAM = OFF_DEC + DEC_BYTES;
 static_assert(OFF_RAM % 16 == 0 && OFF_RAM >= 0x4000u, "aligned; rom - 0x4000 and ram - 0x200 stay offsets");
 __host__ __device__ inline uint32_t ram_part(uint32_t envs) { return ((envs + 3) / 4 * RAM_GROUP + 15) / 16 * 16; }
 // Dynamic shared memory of a block of envs with rom_stage cartridge bytes.
 __host__ __device__ inline uint32_t block_smem(uint32_t rom_stage, uint32_t envs) {
   return OFF_RAM + ram_part(envs) + 4 * rom_stage + envs * ENV_SMEM;
 }
+// Last offset in a bank whose instruction bytes are fetched from the stage: no
+// such fetch touches a hotspot (F8/F6 hotspots start at $FF6, F4's at $FF4).
 __device__ __forceinline__ uint32_t scheme_fetch_limit(uint32_t scheme) {
   return scheme == 3 ? 0xFF1u : scheme ? 0xFF3u : 0xFFCu;
 }
@@ -546,9 +551,19 @@ __device__ __forceinline__ uint32_t scheme_fetch_limit(uint32_t scheme) {
 // (an instruction in one load), and in the top byte 0x80 where no instruction
 // is fetched from the stage: past limit, and a branch whose target lies past
 // the bank's end (the hot loop's sums would carry into the cycle count there).
+// The operand of a zero-page or absolute access to RAM or the TIA is the
+// address of the first mirror, which is the same to reads and writes and the
+// one that the hot loop knows; data reads see a word's first byte only.
 // Words i .. i+3 of a bank of 4096 bytes at src (4-byte aligned), i a multiple
 // of 4.
 constexpr uint32_t REC_BAD = 0x80000000u;
+__host__ __device__ inline uint32_t stage_operand(uint32_t w) {
+  const uint32_t op = w & 0xFFu, form = op & 0x1Cu, a = (w >> 8) & 0x1FFFu;
+  if (form == 0x04u) return a & 0x80u ? w : w & ~0x4000u;                  // zero page
+  if (form != 0x0Cu || op == 0x4Cu || op == 0x6Cu) return w;               // absolute, but for the jumps
+  if ((a & 0x1280u) == 0x0080u) return op | (0x80u | (a & 0x7Fu)) << 8;    // RAM
+  return (a & 0x1080u) == 0 ? op | (a & 0x3Fu) << 8 : w;                   // TIA
+}
 __device__ __forceinline__ uint32_t stage_bad(uint32_t w, uint32_t i, uint32_t limit) {
   const uint32_t off = (w >> 8) & 0xFFu;
   return i > limit || ((w & 0x1Fu) == 0x10u && off < 0x80u && i + 2u + off > 0xFFFu) ? REC_BAD : 0u;
@@ -556,8 +571,8 @@ __device__ __forceinline__ uint32_t stage_bad(uint32_t w, uint32_t i, uint32_t l
 __device__ __forceinline__ uint4 stage_words(const uint8_t *src, uint32_t i, uint32_t limit) {
   const uint32_t *b = reinterpret_cast<const uint32_t *>(src + i);
   const uint32_t lo = b[0], hi = i + 4u < 4096u ? b[1] : 0u, m = 0xFFFFFFu;
-  uint4 r = make_uint4(lo & m, __funnelshift_r(lo, hi, 8) & m, __funnelshift_r(lo, hi, 16) & m,
-                       __funnelshift_r(lo, hi, 24) & m);
+  uint4 r = make_uint4(stage_operand(lo & m), stage_operand(__funnelshift_r(lo, hi, 8) & m),
+                       stage_operand(__funnelshift_r(lo, hi, 16) & m), stage_operand(__funnelshift_r(lo, hi, 24) & m));
   r.x |= stage_bad(r.x, i, limit);
   r.y |= stage_bad(r.y, i + 1u, limit);
   r.z |= stage_bad(r.z, i + 2u, limit);
@@ -566,9 +581,18 @@ __device__ __forceinline__ uint4 stage_words(const uint8_t *src, uint32_t i, uin
 }
 // Rounds between two looks at the lanes that wait for service, unrolled, so
 // that a round's last instructions overlap the next one's loads (157 cycles a
-// round, 173 as a loop).  A look costs about 60 cycles; a lane that waits loses
-// half a batch, and 16 rounds measure the same as 8.
-constexpr uint32_t BATCH = 8;
+// round, 173 as a loop).  Lanes that wait are served when every lane waits, or
+// when the looks since the first of them add up to more than HOLD rounds: the
+// lanes of a warp run much the same code, and served together they stay in step,
+// which the TIA warp, whose lanes' events then take the same branches, needs
+// more than the wait costs (served at every look, 4096 sprite envs took 2.5 ms a
+// step instead of 1.8).  Of 4 .. 8 rounds a look, 7 is the fastest (sprite 1.70
+// ms, 6: 1.79, 8: 1.74).  When the whole warp waited and was served, a batch of
+// BRIEF rounds follows instead: code full of such instructions has them a few
+// rounds apart (six accesses through pointers a line: 2.6 ms a step, 3.6 without
+// the brief batches; 2 rounds 4.9, 4: 2.9).
+constexpr uint32_t BATCH = 7, HOLD = 16, BRIEF = 3;
+template <uint32_t N> struct Rounds { static constexpr uint32_t value = N; };
 
 template <bool SPLIT>
 struct FastConsoleT {
@@ -697,10 +721,6 @@ struct FastConsoleT {
     if (fire && (vblank_c & 0x40)) io.Sset(IO_LATCH, 1);
   }
 
-  // Last offset in a bank whose instruction bytes are fetched from the stage:
-  // no such fetch touches a hotspot (F8/F6 hotspots start at $FF6, F4's at $FF4).
-  __device__ __forceinline__ uint32_t fetch_limit() const { return scheme_fetch_limit(scheme); }
-
   // ---- bus ----
   __device__ __forceinline__ void hotspot(uint32_t at) {
     if (scheme == 1) { if (at == 0xFF8 || at == 0xFF9) bank = at - 0xFF8; }
@@ -766,6 +786,11 @@ struct FastConsoleT {
     if (reg == 0x0C) return (io.G(IO_FIRE) || io.G(IO_LATCH)) ? 0x00u : 0x80u;
     return reg == 0x0D ? 0x80u : 0u;
   }
+  __device__ __forceinline__ void vblank_write(uint32_t v) {
+    vblank_c = v;
+    if (!(v & 0x40)) io.Sset(IO_LATCH, 0);
+    else if (io.G(IO_FIRE)) io.Sset(IO_LATCH, 1);
+  }
   // WSYNC, the VSYNC rise and the VBLANK latch effects happen here, the
   // register itself on the TIA side.
   __device__ void io_write(uint32_t a, uint32_t v, uint32_t t) {
@@ -776,9 +801,7 @@ struct FastConsoleT {
       if (!(vsync_c & 2) && (v & 2) && vs_kf == ~0u) vs_kf = t;
       vsync_c = v;
     } else if (reg == 0x01) {
-      vblank_c = v;
-      if (!(v & 0x40)) io.Sset(IO_LATCH, 0);
-      else if (io.G(IO_FIRE)) io.Sset(IO_LATCH, 1);
+      vblank_write(v);
     }
     push_at(reg << 8 | v, t + 1u);
   }
@@ -1087,37 +1110,23 @@ struct FastConsoleT {
   // 157 cycles with one warp on an SM, 284 with eight (208 and 365 with the
   // control words loaded at the round's end, V in a register of its own, the
   // branch's condition in three operations, RAM addressed apart from the
-  // cartridge and regions of 32 bytes).  What it does not take (RIOT accesses, collision reads, VSYNC and
-  // VBLANK, stack and pointer instructions, bank hotspots, frame ends) stops
-  // the lane in front of the instruction; every BATCH rounds the lanes that
-  // wait are served together by the general decoder, at once when no lane is
-  // left running, otherwise after at most one more batch, so that lanes a few
-  // rounds apart share one call.
+  // cartridge and regions of 32 bytes).  What it does not take (fc_quick, and the
+  // general decoder for the rest) stops the lane in front of the instruction;
+  // after every BATCH rounds the lanes that wait are looked at, and served
+  // together.
   template <class Hook> __device__ __forceinline__ void run(Hook &hook);
 };
 
 // One service of a waiting lane: the frame's end, or the instruction at PC by
-// the general decoder (after a timer wait loop's idle iterations).  Returns
-// false when the step is over.
+// the general decoder.  Returns false when the step is over.
 template <bool SPLIT, class Hook>
 __device__ __noinline__ bool fc_service(FastConsoleT<SPLIT> *c, Hook *h) {
   const uint32_t cap = 76u * CAP_LINES;
   // at least one instruction runs in every frame before the line cap ends it
   bool ended = c->jam || (c->kf >= cap && c->instret != c->frame_inst);
   if (!ended) {
-    const uint32_t at = c->PC & 0xFFF;
-    if (c->idle && (c->PC & 0x1000) && at <= c->fetch_limit()) {
-      const uint32_t i = c->bank * 4096u + at;
-      if (c->rom(i) == 0xAD && at + 4u < 4096u)
-        c->kf = c->idle_forward(sm32(c->off.rom + 4 * i) & 0xFFFFFFu, c->rom(i + 3), c->PC, c->kf);
-    }
-    // decimal mode is the general decoder's: its instructions run on here
-    for (int n = 0; n < 16; ++n) {
-      if (n) ++c->rounds;  // the first one is counted with the whole warp's round
-      c->exec_general();
-      ended = c->jam || c->vs_kf != ~0u || c->kf >= cap;
-      if (ended || !(c->fdi & 0x08)) break;
-    }
+    c->exec_general();
+    ended = c->jam || c->vs_kf != ~0u || c->kf >= cap;
   }
   while (ended) {
     uint32_t next_rel;
@@ -1129,6 +1138,247 @@ __device__ __noinline__ bool fc_service(FastConsoleT<SPLIT> *c, Hook *h) {
     ended = c->jam != 0;
   }
   return true;
+}
+
+// Serve a waiting lane's instruction (word rec, kind QK_*) beside the loop: the
+// console stays where it is, R, G and pk come and go in registers, and what can
+// be put in a form that the loop takes (the pointer in the place of an absolute
+// address, a value as an immediate operand) runs in the next round.  A call takes
+// 400 to 900 cycles, the general decoder's, which has the whole console in local
+// memory, 2,700 to 4,500; a program with six accesses through pointers a line
+// steps 512 envs in 2.6 ms, 9.8 with the general decoder for each of them.
+// The result's w: QS_NO (nothing is changed: the general decoder has to),
+// QS_DONE (x, y, z: R, G, pk after the instruction) or QS_RUN (x, z: the
+// instruction's word, and its length and cycles, as the loop is to run it with
+// the control words of entry w >> 8; y: G).  QS_SYNC: the event queue's position
+// is the console's, not qi's.
+constexpr uint32_t QS_NO = 0, QS_DONE = 1, QS_RUN = 2, QS_SYNC = 4;
+template <bool SPLIT>
+__device__ __noinline__ uint4 fc_quick(FastConsoleT<SPLIT> *m, uint32_t R, uint32_t G, uint32_t pk, uint32_t rec,
+                                       uint32_t kind, uint32_t qi) {
+  const uint4 no = make_uint4(0, 0, 0, QS_NO);
+  const uint32_t ramb = m->off.ram - 0x200u, fdi = m->fdi;
+  const IoCtx io = m->io;
+  if (m->jam) return no;
+  auto ctl = [&](uint32_t entry, uint32_t t) {
+    return *reinterpret_cast<const uint4 *>(&sm32(OFF_CTL + CTL_TABLE * t + 16u * entry));
+  };
+  const uint32_t opcode = rec & 0xFFu;
+  const uint4 c = ctl(opcode, 0), d = ctl(opcode, 1), f = ctl(opcode, 3);
+  uint32_t pn = pk + d.z;
+  uint32_t base = prmt(rec, pn, c.x), sum = base + prmt(R, rec, c.y), ea = sum & d.y;
+  const uint32_t live = fdi & 0x08u ? RG_DECIMAL : ~0u;
+  auto ram = [&](uint32_t a) -> uint8_t & { return sm8(ramb + 4u * (0x80u | (a & 0x7Fu))); };  // mirrored or not
+  auto is_ram = [](uint32_t a) { return (a & 0x1280u) == 0x0080u; };
+  // the queue's position, from the loop's to the console's
+  uint32_t sync = 0;
+  auto queue = [&] {
+    if (!sync) m->qtail += (qi & 0xFFFFu) - (m->qtail & 0xFFu);
+    sync = QS_SYNC;
+  };
+  // the value at address a, read at cycle t
+  auto value = [&](uint32_t a, uint32_t t) -> uint32_t {
+    if (is_ram(a)) return ram(a);
+    if (a & 0x1000u) {
+      m->hotspot(a & 0xFFFu);
+      return m->rom(m->bank * 4096u + (a & 0xFFFu));
+    }
+    if (a & 0x80u) return fc_riot_read(io, a, 76ull * m->l0c + t);
+    const uint32_t reg = a & 0xFu;
+    if (reg < 8u) {
+      queue();
+      m->sync_collisions(t);
+      return fc_cx_byte(io.V(IO_CX), reg);
+    }
+    return reg == 0xCu ? (io.G(IO_FIRE) || io.G(IO_LATCH) ? 0u : 0x80u) : reg == 0xDu ? 0x80u : 0u;
+  };
+  auto nz = [&](uint32_t v) { G = (G & ~FL_NZ) | v | (v & 0x80u) << 16; };
+  auto run = [&](uint32_t entry, uint32_t word, uint32_t len) {
+    return make_uint4(word, G, len, sync | QS_RUN | entry << 8);
+  };
+  auto done = [&] { return make_uint4(R, G, pn, sync | QS_DONE); };
+  // the operation of opcode o (not a store) on v
+  auto operate = [&](uint32_t o, uint32_t v) -> uint4 {
+    if (((o & 0xE3u) == 0x61u || (o & 0xE3u) == 0xE1u) && (fdi & 0x08u)) {  // decimal ADC, SBC
+      m->A = R & 0xFFu;
+      m->fc = (G >> 8) & 1u;
+      if (o & 0x80u) m->sbc(v); else m->adc(v);
+      R = prmt(R, m->A, 0x3214);
+      G = ((m->fz & 0xFFu) ? 1u : 0u) | m->fc << 8 | (m->fn & 0x80u) << 16 | m->fv << 25;
+      return done();
+    }
+    const uint32_t imm = (o & 3u) == 3u ? CTL_LAX : (o & 0xE0u) | ((o & 3u) == 1u ? 9u : o & 2u);  // the immediate form
+    return run(imm, v << 8, pn - pk);
+  };
+  // whether v to TIA register reg is more than a write of it: WSYNC, a rise of VSYNC (which ends the frame)
+  auto special = [&](uint32_t reg, uint32_t v) { return reg == 2u || (reg == 0u && (v & ~m->vsync_c & 2u)); };
+  auto tia = [&](uint32_t reg, uint32_t v, uint32_t t) {
+    if (reg == 0u) m->vsync_c = v;
+    if (reg == 1u) m->vblank_write(v);
+    queue();
+    m->push_at(reg << 8 | v, t + 1u);
+  };
+  // v to address a at the instruction's last cycle
+  auto store = [&](uint32_t a, uint32_t v) -> uint4 {
+    const uint32_t t = (pn >> 16) - 1u;
+    v &= 0xFFu;
+    if (is_ram(a)) ram(a) = (uint8_t)v;
+    else if (a & 0x1000u) m->hotspot(a & 0xFFFu);
+    else if (a & 0x80u) fc_riot_write(io, a, v, 76ull * m->l0c + t);
+    else if (special(a & 0x3Fu, v)) return no;
+    else tia(a & 0x3Fu, v, t);
+    return done();
+  };
+  // a read-modify-write of RAM or a TIA register (operation o >> 5: shifts, DEC, INC): the result to r
+  auto modify = [&](uint32_t o, uint32_t a, uint32_t &r) -> bool {
+    if (!is_ram(a) && (a & 0x1080u)) return false;
+    const uint32_t t = (pn >> 16) - 1u, reg = a & 0x3Fu;
+    if (!is_ram(a) && reg <= 2u) return false;
+    const uint32_t v = value(a, t - 2u), cin = G >> 8 & 1u;
+    uint32_t cout = cin;
+    switch (o >> 5) {
+      case 0: r = v << 1; cout = v >> 7; break;
+      case 1: r = v << 1 | cin; cout = v >> 7; break;
+      case 2: r = v >> 1; cout = v & 1u; break;
+      case 3: r = v >> 1 | cin << 7; cout = v & 1u; break;
+      case 6: r = v - 1u; break;
+      default: r = v + 1u; break;
+    }
+    r &= 0xFFu;
+    if (is_ram(a)) {
+      ram(a) = (uint8_t)r;
+    } else {
+      tia(reg, v, t - 1u);
+      tia(reg, r, t);
+    }
+    G = (G & ~FL_C) | cout << 8;
+    return true;
+  };
+  // the pointer in RAM that ea is the address of, to sum (base: without the index)
+  auto pointer = [&]() -> bool {
+    if (ea < 0x80u || ea == 0xFFu) return false;
+    base = ram(ea) | ram(ea + 1u) << 8;
+    sum = base + ((opcode & 0x10u) ? R >> 16 & 0xFFu : 0u);
+    return true;
+  };
+  uint32_t sp = m->SP;  // pulls, calls and returns outside RAM are the general decoder's
+  switch (kind) {
+    case QK_PTR: {
+      if (!pointer()) return no;
+      const uint32_t entry = CTL_N + (opcode >> 4);
+      const uint4 g = ctl(entry, 3);
+      ea = sum & 0x1FFFu;
+      if (sm8(OFF_REG + ea) & g.x & live) return run(entry, opcode | base << 8, d.z);
+      pn += ((base ^ sum) & g.z) << 8;
+      return (g.x & RG_OUT) ? store(ea, R) : operate(opcode, value(ea, (pn >> 16) - 1u));
+    }
+    case QK_SUM:
+      if (d.y == 0) return operate(opcode & ~2u, rec >> 8 & 0xFFu);  // immediate ($EB too)
+      pn += ((base ^ sum) & f.z) << 8;
+      return operate(opcode, value(ea, (pn >> 16) - 1u));
+    case QK_MEM: {
+      pn += ((base ^ sum) & f.z) << 8;
+      if (f.x & RG_OUT) return store(ea, (opcode & 3u) == 1u ? R : (opcode & 2u) ? R >> 8 : R >> 16);
+      if (f.x & RG_WRAM) {
+        uint32_t r;
+        if (!modify(opcode, ea, r)) return no;
+        nz(r);
+        return done();
+      }
+      // a timer wait loop: its idle iterations retire with the read that ends them
+      if (opcode == 0xADu && m->idle) {
+        const uint32_t then = m->rom(m->bank * 4096u + ((pk + 3u) & 0xFFFu));
+        pn += (m->idle_forward(rec, then, pk & 0xFFFFu, pk >> 16) - (pk >> 16)) << 16;
+      }
+      const uint32_t v = value(ea, (pn >> 16) - 1u);
+      if (pn - pk < 0x100000u) return operate(opcode, v);
+      R = prmt(R, v, 0x3214);
+      nz(v);
+      return done();
+    }
+    case QK_BIT: {
+      const uint32_t v = value(ea, (pn >> 16) - 1u);
+      G = (G & FL_C) | ((R & v & 0xFFu) ? 1u : 0u) | (v & 0x80u) << 16 | (v & 0x40u) << 25;
+      return done();
+    }
+    case QK_PUSH: {
+      const uint32_t p = (G >> 16 & 0x80u) | (G >> 25 & 0x40u) | 0x30u | fdi | ((G & FL_Z) ? 0u : 2u) | (G >> 8 & 1u);
+      const uint4 r = store(0x100u | sp, (opcode & 0x40u) ? R : p);
+      if (r.w) m->SP = (sp - 1u) & 0xFFu;
+      return r;
+    }
+    case QK_PULL: {
+      if (sp < 0x7Fu || sp == 0xFFu) return no;
+      m->SP = ++sp;
+      const uint32_t v = ram(sp);
+      if (opcode & 0x40u) {
+        R = prmt(R, v, 0x3214);
+        nz(v);
+      } else {
+        G = ((v & 2u) ? 0u : 1u) | (v & 1u) << 8 | (v & 0x80u) << 16 | (v & 0x40u) << 25;
+        m->fdi = v & 0x0Cu;
+      }
+      return done();
+    }
+    case QK_JSR:
+      if (sp < 0x81u) return no;
+      ram(sp) = (uint8_t)((pk + 2u) >> 8);
+      ram(sp - 1u) = (uint8_t)(pk + 2u);
+      m->SP = sp - 2u;
+      pn = prmt(rec, pn, 0x7621);
+      return done();
+    case QK_RTS:
+      if (sp < 0x7Fu || sp >= 0xFEu) return no;
+      m->SP = sp += 2u;
+      pn = prmt((ram(sp - 1u) | ram(sp) << 8) + 1u, pn, 0x7610);
+      return done();
+    case QK_REG:
+      switch (opcode) {
+        case 0xBA: R = prmt(R, sp, 0x3240); nz(sp); break;
+        case 0x9A: m->SP = R >> 8 & 0xFFu; break;
+        case 0x58: m->fdi = fdi & ~0x04u; break;
+        case 0x78: m->fdi = fdi | 0x04u; break;
+        case 0xD8: m->fdi = fdi & ~0x08u; break;
+        default: m->fdi = fdi | 0x08u; break;
+      }
+      return done();
+    case QK_COMBO: {
+      if ((opcode & 0x0Fu) == 3u && !pointer()) return no;
+      const uint32_t a = sum & ((opcode & 0x0Fu) == 3u ? 0x1FFFu : d.y), op = opcode >> 5;
+      if (op == 5u) {  // LAX
+        pn += ((base ^ sum) & f.z) << 8;
+        return operate(opcode, value(a, (pn >> 16) - 1u));
+      }
+      if (op == 4u) return store(a, R & (R >> 8));  // SAX
+      // the memory operation, then the accumulator's with its result as an immediate operand
+      uint32_t r;
+      if (((op == 3u || op == 7u) && (fdi & 0x08u)) || !modify(opcode, a, r)) return no;
+      return run((opcode & 0xE0u) | 9u, r << 8, d.z);
+    }
+    case QK_AND: {  // ANC, ALR, SBX: what they set from A and the operand
+      const uint32_t b = rec >> 8 & 0xFFu;
+      uint32_t r, cout;
+      if (opcode == 0xCBu) {
+        const uint32_t ax = R & (R >> 8) & 0xFFu;
+        r = (ax - b) & 0xFFu;
+        cout = ax >= b ? 1u : 0u;
+        R = prmt(R, r, 0x3240);
+      } else {
+        r = R & b & 0xFFu;
+        cout = opcode == 0x4Bu ? r & 1u : r >> 7;
+        if (opcode == 0x4Bu) r >>= 1;
+        R = prmt(R, r, 0x3214);
+      }
+      nz(r);
+      G = (G & ~FL_C) | cout << 8;
+      return done();
+    }
+    case QK_NOP:  // the operand's read changes nothing but at a hotspot
+      if (ea & 0x1000u) m->hotspot(ea & 0xFFFu);
+      pn += ((base ^ sum) & f.z) << 8;
+      return done();
+    default: return no;
+  }
 }
 
 template <bool SPLIT>
@@ -1145,31 +1395,43 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
   // start at or after that cycle, in the high half, over FFFF.  qi: queue
   // position, and the instructions retired since the last service in the high
   // half.  bk, bf: the bank's words, for data at 4 * (bus address) and for the
-  // fetch.  run: all ones, or 0 while the lane waits.
-  uint32_t R, G, pk, nl, qi, bk, bf, run;
+  // fetch.  live: the accesses that the lane may make in the loop (RG_*).
+  // run: live, or 0 while the lane waits.
+  uint32_t R, G, pk, nl, qi, bk, bf, live, run;
   uint32_t rec;
   uint4 c, d, e, f;  // control words 0-3, 4-7, 8-11, 12-15
   bool active = true;
   auto word_at = [&](uint32_t p) { return lds_const(mad(p & 0xFFFu, k4, bf)); };
-  auto control = [&](uint32_t w, uint4 &c_, uint4 &d_, uint4 &e_, uint4 &f_) {
-    const uint32_t a = mad(w & 0xFFu, unit * 16u, ctl);
+  auto control = [&](uint32_t entry, uint4 &c_, uint4 &d_, uint4 &e_, uint4 &f_) {
+    const uint32_t a = mad(entry, unit * 16u, ctl);
     c_ = lds_const4<0>(a);
     d_ = lds_const4<CTL_TABLE>(a);
     e_ = lds_const4<2 * CTL_TABLE>(a);
     f_ = lds_const4<3 * CTL_TABLE>(a);
+  };
+  auto mode = [&] { live = fdi & 0x08u ? RG_DECIMAL : ~0u; };
+  auto banked = [&] {
+    bk = o.rom + bank * 16384u - 0x4000u;
+    bf = smb + o.rom + bank * 16384u;
+  };
+  auto line = [&] { nl = (((pk >> 16) + 75u) / 76u * 76u) << 16 | 0xFFFFu; };
+  // the instruction at pk, and whether the loop may run it
+  auto next = [&] {
+    rec = word_at(pk);
+    run = ((pk & 0x1000u) == 0) | (rec >= REC_BAD) | ((pk >> 16) >= cap) ? 0u : live;
+    control(rec & 0xFFu, c, d, e, f);
   };
   // the console's fields to the loop's registers, and the next instruction
   auto enter = [&](bool stay) {
     R = A | X << 8 | Y << 16 | 0xFF000000u;
     G = ((fz & 0xFFu) ? 1u : 0u) | fc << 8 | (fn & 0x80u) << 16 | fv << 25;
     pk = (PC & 0xFFFFu) | min(kf, 0xFFFFu) << 16;
-    nl = ((min(kf, 0xFFFFu) + 75u) / 76u * 76u) << 16 | 0xFFFFu;
+    line();
     qi = qtail & 0xFFu;
-    bk = o.rom + bank * 16384u - 0x4000u;
-    bf = smb + o.rom + bank * 16384u;
-    rec = word_at(pk);
-    run = stay | ((pk & 0x1000u) == 0) | (rec >= REC_BAD) | (kf >= cap) | ((fdi & 0x08u) != 0) ? 0u : ~0u;
-    control(rec, c, d, e, f);
+    banked();
+    mode();
+    next();
+    if (stay) run = 0;
   };
   auto leave = [&] {
     A = R & 0xFF; X = (R >> 8) & 0xFF; Y = (R >> 16) & 0xFF;
@@ -1179,11 +1441,10 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
     qtail += (qi & 0xFFFFu) - (qtail & 0xFFu);
     instret += qi >> 16;
   };
-  enter(jam != 0);
-  uint32_t held = 0, act = wmask;
-  for (;;) {
+  // n.value rounds of the hot loop, one block of code
+  auto batch = [&](auto n) {
 #pragma unroll
-    for (uint32_t r = 0; r < BATCH; ++r) {
+    for (uint32_t r = 0; r < n.value; ++r) {
       // --- next instruction (branches and JMP abs: the sum is the target and the cycle)
       const uint32_t pn = mad(pk, k1, d.z);
       const uint32_t base = prmt(rec, pn, c.x);
@@ -1201,7 +1462,7 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
       const uint32_t y = prmt(sm8(at), sum, d.x);
       const uint32_t x = prmt(R, y, c.z);
       uint4 cn, dn, en, fn;  // the next instruction's control words, on their way while this one is computed
-      control(nrec, cn, dn, en, fn);
+      control(nrec & 0xFFu, cn, dn, en, fn);
       // --- result, of x and y ^ e.y
       const uint32_t xo = lop3<0x96>(x, y, e.y);
       const uint32_t raw = mad(lop3<0x60>(x, y, e.y), e.z, mad(xo, f.y, prmt(G, k1, e.w)));
@@ -1212,7 +1473,8 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
       // events past another lap's bit: the lap's complement is bit 15 of -qi * 1024 - 1024
       const uint32_t ev = mad(ea, k256, s) | (mad(qi, unit * (0u - EV_LAP / QLEN), 0u - EV_LAP / QLEN) & EV_LAP);
       if (out) vsm32(mad(qi & (QLEN - 1), k4, o.q)) = prmt(ev, pnext, 0x7610);
-      if (pnext > nl) nl = mad(k256, 76u << 8, nl);       // one step: no instruction is longer than a line
+      // one step: no instruction is longer than a line (a waiting lane's is set again when it is served)
+      if (pnext > nl) nl = mad(k256, 76u << 8, nl);
       if (put & RG_WSYNC) pnext = prmt(pnext, nl, 0x7610);  // on to the next line's first cycle
       const bool done = put != 0;  // in single statements: a block of them would become a branch
       const uint32_t gn = (G & ~e.x) | (prmt(s, lop3<0x14>(x, s, xo), FL_SEL) & e.x);  // V: (x ^ s) & ~(x ^ y)
@@ -1223,26 +1485,81 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
       if (out) qi = mad(k1, k1, qi);
       // bit 31: no instruction word there, the PC outside the cartridge, the line cap
       const uint32_t stop = nrec | mad(pnext, unit * 0xFFF80000u, 0xFFF80000u) | mad(pnext, 0u - unit, (cap << 16) - 1u);
-      run = !done | ((int)stop < 0) ? 0u : ~0u;
+      run = !done | ((int)stop < 0) ? 0u : live;
       rec = nrec; c = cn; d = dn; e = en; f = fn;
     }
+  };
+  enter(jam != 0);
+  uint32_t held = 0, act = wmask;
+  for (;;) {
+    batch(Rounds<BATCH>{});
     // --- service: waiting lanes, and queues without room for another batch
     rounds += BATCH;
     const bool full = ((qi - qhead_seen) & 0xFFu) > QLEN - BATCH;
     uint32_t m = __ballot_sync(wmask, ((run == 0) | full) & active);
     if (m == 0) continue;
     m = __ballot_sync(wmask, (run == 0) & active);
-    if (m != 0 && (m == act || ++held > 1)) {
+    if (m != 0 && (m == act || (held += BATCH) > HOLD)) {
       held = 0;
-      const uint32_t r0 = ++rounds;
-      if (active && run == 0) {
-        leave();
-        active = fc_service<SPLIT, Hook>(this, &hook);
-        enter(!active);
+      bool slow;
+      for (;;) {
+        slow = active & (run == 0);  // not served yet
+        if (slow) {
+          rec = word_at(pk);
+          const uint32_t kind = sm8(OFF_DEC + DEC_QUICK + (rec & 0xFFu));
+          const bool other = (kind == QK_NONE) | (rec >= REC_BAD) | ((pk & 0x1000u) == 0) | ((pk >> 16) >= cap);
+          if (!other & (kind == QK_PTR)) {  // the common case, a third of a call's time
+            const uint32_t z = (rec >> 8) + ((rec & 0x10u) ? 0u : R >> 8) & 0xFFu, za = ramb + 4u * z;
+            const uint32_t w = (rec & 0xFFu) | sm8(za) << 8 | sm8(za + 4u) << 16;
+            control(CTL_N + (rec >> 4 & 0xFu), c, d, e, f);
+            const uint32_t at = ((w >> 8) + prmt(R, w, c.y)) & 0x1FFFu;
+            if ((z >= 0x80u) & (z != 0xFFu) & ((sm8(OFF_REG + at) & f.x & live) != 0)) {
+              rec = w;
+              run = live;
+              line();
+              slow = false;
+            }
+          }
+          if (!other & slow) {
+            const uint4 r = fc_quick<SPLIT>(this, R, G, pk, rec, kind, qi);
+            if (r.w & QS_SYNC) qi = (qi & 0xFFFF0000u) | (qtail & 0xFFu);
+            banked();
+            if (r.w & QS_DONE) {
+              R = r.x; G = r.y; pk = r.z;
+              line();
+              qi += 1u << 16;
+              mode();
+              next();
+              slow = false;
+            } else if (r.w & QS_RUN) {
+              rec = r.x; G = r.y;
+              control(r.w >> 8, c, d, e, f);
+              d.z = r.z;
+              run = live;
+              line();
+              slow = false;
+            }
+            if ((r.w & QS_SYNC) && jam) run = 0;  // the TIA side stalled
+          }
+        }
+        // lanes in step with one another, all served: most likely they soon wait together again.  The single-warp
+        // form, whose rounds are not the longer part of a step, is 7 % slower with the second copy of the loop.
+        if (!SPLIT || m != act) break;
+        if (__any_sync(wmask, slow | (active & (((qi - qhead_seen) & 0xFFu) > QLEN - BRIEF)))) break;
+        batch(Rounds<BRIEF>{});
+        rounds += BRIEF;
+        if (__any_sync(wmask, active & (run != 0))) break;
       }
-      rounds = r0 + __reduce_max_sync(wmask, rounds - r0);  // a lane's further decoder passes hold up the others
-      act = __ballot_sync(wmask, active);
-      if (act == 0) break;
+      if (__any_sync(wmask, slow)) {
+        ++rounds;
+        if (slow) {
+          leave();
+          active = fc_service<SPLIT, Hook>(this, &hook);
+          enter(!active);
+        }
+        act = __ballot_sync(wmask, active);
+        if (act == 0) break;
+      }
     }
     // room for a batch of events
     if constexpr (SPLIT) {
