@@ -49,16 +49,18 @@ SM_COUNT, SMSP_PER_SM, SM_MAX_MHZ = 152, 4, 2070.0
 # A shape captured on another workload is used with its source named; a shape
 # never captured reports achieved = null.
 INTERP_CAPTURES = {
-    # (kernel, envs per warp, opcode dispatch, config): (warp-inst per executed 6502 instruction, DRAM bytes per env-step)
-    ("k_interp_split", 32, 1, 3): (1412574931 / 433986434, (31363840 + 456011776) / 32768),
-    ("k_interp_split", 32, 1, 2): (272340736 / 94164973, (1458432 + 9803264) / 4096),
+    # (kernel, envs per warp, config): (warp-inst per executed 6502 instruction, DRAM bytes per env-step)
+    ("k_interp_split", 32, 3): (1412574931 / 433986434, (31363840 + 456011776) / 32768),
+    ("k_interp_split", 32, 2): (272340736 / 94164973, (1458432 + 9803264) / 4096),
 }
 # Algorithmic bytes of the fused rasterise + preprocess kernel per env-step,
-# besides 4 bytes per logged TIA write: band snapshots and record counts of the
-# two rendered frames (2 x 105 x 48 + 2 x 8), the three older stack planes read from the
-# ring, the 84x84x4 stack written out, the new plane written to the ring and
-# the ring head.
-FUSED_FIXED_BYTES_PER_ENV_STEP = 2 * 105 * 48 + 2 * 8 + 3 * 7056 + 4 * 7056 + 7056 + 1
+# besides 4 bytes per logged TIA write: record counts of the two rendered
+# frames (2 x 8), the three older stack planes read from the ring, the 84x84x4
+# stack written out, the new plane written to the ring and the ring head.  The
+# band snapshots of the two frames, which only this way of painting reads, are
+# reported beside it.
+FUSED_FIXED_BYTES_PER_ENV_STEP = 2 * 8 + 3 * 7056 + 4 * 7056 + 7056 + 1
+FUSED_SNAPSHOT_BYTES_PER_ENV_STEP = 2 * 105 * 48
 # Warp instructions per env-step of the fused kernel (it is bound by issue,
 # not HBM), from the same captures: smsp__inst_executed.sum / env-steps.
 FUSED_WARP_INST_PER_ENV_STEP = {3: 1220170065 / 32768, 2: 129733917 / 4096}
@@ -90,7 +92,7 @@ def parse(argv=None):
     p.add_argument("--warps-per-frame", type=int, default=0)
     p.add_argument("--tia-warps", type=int, default=0, choices=[0, 1, 2])
     p.add_argument("--grouping", type=int, default=0, choices=[0, 1, 2])
-    p.add_argument("--dispatch", type=int, default=0, choices=[0, 1, 2])
+    p.add_argument("--dispatch", type=int, default=0, choices=[0, 1, 2], help="passed on; every value runs the same code")
     p.add_argument("--divergence", action="store_true",
                    help="divergence study: frames/s and lane efficiency per window of steps from one shared "
                         "start state per cartridge, beside a run from the usual random start states and the oracle "
@@ -449,7 +451,7 @@ def profile_pass(env, do_step, acts, flush):
     return env.profile_read(), instr / k, logrec / k, rounds / k
 
 
-def interp_roofline(prof, instr_per_step, kernel, lanes, dispatch, config, n_envs, frameskip):
+def interp_roofline(prof, instr_per_step, kernel, lanes, config, n_envs, frameskip):
     """Issue-slot roofline of the interpreter (plain integer and control work:
     no tensor-core or FLOP peak applies)."""
     ms, n = prof.get("interpreter", (0.0, 0))
@@ -457,13 +459,13 @@ def interp_roofline(prof, instr_per_step, kernel, lanes, dispatch, config, n_env
         return None
     dur = ms / n / 1000.0
     peak = SM_COUNT * SMSP_PER_SM * SM_MAX_MHZ * 1e6 / 1e9
-    cap = INTERP_CAPTURES.get((kernel, lanes, dispatch, config))
-    src = f"ncu capture of {kernel}, {lanes} envs/warp, dispatch {dispatch}, this workload"
+    cap = INTERP_CAPTURES.get((kernel, lanes, config))
+    src = f"ncu capture of {kernel}, {lanes} envs/warp, this workload"
     if cap is None:
-        other = [(k, v) for k, v in INTERP_CAPTURES.items() if k[:3] == (kernel, lanes, dispatch)]
+        other = [(k, v) for k, v in INTERP_CAPTURES.items() if k[:2] == (kernel, lanes)]
         if other:
             cap = other[0][1]
-            src = f"ncu capture of {kernel}, {lanes} envs/warp, dispatch {dispatch}, workload config {other[0][0][3]}"
+            src = f"ncu capture of {kernel}, {lanes} envs/warp, workload config {other[0][0][2]}"
     ach = cap[0] * instr_per_step / dur / 1e9 if cap else None
     return {"bound": "alu", "kernel": kernel, "achieved": ach, "peak": peak, "unit": "Gwarp-inst/s",
             "frac": (ach / peak) if ach else None, "traffic": cap[1] * n_envs if cap else None,
@@ -490,6 +492,7 @@ def fused_roofline(prof, logrec_per_step, config, n_envs):
     issue_peak = SM_COUNT * SMSP_PER_SM * SM_MAX_MHZ * 1e6 / 1e9
     return {"bound": "hbm", "kernel": "fused_raster_preprocess", "achieved": ach, "peak": peak, "unit": "GB/s",
             "frac": ach / peak, "traffic": tb * n_envs if tb else None, "algorithmic_bytes_per_env_step": per_step,
+            "snapshot_bytes_per_env_step": FUSED_SNAPSHOT_BYTES_PER_ENV_STEP,
             "launch_ms": dur * 1000.0,
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured copy)" if hbm else "fallback 6.8 TB/s",
             # what binds it in practice: issue slots (same method as the interpreter's roofline)
@@ -574,7 +577,7 @@ def divergence_run(args, w, rank):
             ins = sum(c[0] for c in cnt[a:a + win])
             rnd = sum(c[2] for c in cnt[a:a + win])
             out.append({"steps": [a, a + win], "frames_per_s": w.n_envs * w.frameskip * win / t,
-                        "lockstep_lane_efficiency": ins / rnd if rnd else None,
+                        "lane_efficiency": ins / rnd if rnd else None,
                         "m6502_inst_per_env_frame": ins / (w.n_envs * w.frameskip * win)})
         return out, shape
 
@@ -609,7 +612,7 @@ def divergence_run(args, w, rank):
 
 def shape_dict(shape):
     """launch_shape() as named fields (the grouping word also carries the
-    compact-dispatch flag, 4)."""
+    configuration's dispatch, 4 for 2; it chooses nothing)."""
     e, b, wpf, grid, tia, g = shape
     return {"envs_per_warp": e, "envs_per_block": b, "warps_per_frame": wpf, "grid": grid, "tia_warps": tia,
             "grouping": g & 3, "dispatch": 2 if g & 4 else 1}
@@ -762,11 +765,10 @@ def main(argv=None):
         e2e = {"value": frames_all / dt, "unit": "frames/s", "h2d_bytes_per_step": int(ha[0].numel()),
                "d2h_bytes_per_step": int(ho.numel() + hr.numel() * 4 + hd.numel()),
                "p50_step_ms": hp50, "p99_step_ms": hp99}
-    roof = interp_roofline(prof, instr, kern, shape[0], shape_dict(shape)["dispatch"], args.config, w.n_envs,
-                           w.frameskip)
+    roof = interp_roofline(prof, instr, kern, shape[0], args.config, w.n_envs, w.frameskip)
     if roof and lane_rounds:
         # instructions per lane and issue round: the fraction of a warp's lanes that make progress in a round
-        roof["lockstep_lane_efficiency"] = instr / lane_rounds
+        roof["lane_efficiency"] = instr / lane_rounds
     roof2 = fused_roofline(prof, logrec, args.config, w.n_envs)
     kernels = {k: {"ms_per_launch": v[0] / max(1, v[1]), "launches": v[1]} for k, v in prof.items()}
     env.close()
