@@ -99,7 +99,7 @@ typedef struct {
                              banked cartridge; 0 = autotune */
     int dispatch;         /* batched form: 0, 1 or 2.  Kept for callers: it chose between two opcode switches;
                              the interpreter's hot loop has no switch any more, and every value runs the same
-                             code (launch_shape reports 2 as before) */
+                             code (launch_shape adds 4 to grouping for 2) */
     int idle_skip;        /* batched form: 1 = a RIOT-timer wait loop (LDA INTIM at PC, BNE back to PC) retires
                              the iterations that read a nonzero timer value at once (cycles and instruction
                              counts advanced exactly; same results), 0 = every iteration runs.  Default 1;
@@ -299,7 +299,8 @@ ATARI_API int atari_env_get_cache(atari_env *env, void *d_dst, atari_stream stre
  * iterations of a RIOT-timer wait loop that the batched form retires at once,
  * see idle_skip, are not counted), TIA
  * log records written, and issue rounds summed over the envs (each
- * env counts the rounds its warp issued, so instructions / lane_rounds is
+ * env counts the rounds its warp issued, those in which waiting lanes are
+ * served beside the loop among them, so instructions / lane_rounds is
  * the fraction of a warp's lanes that execute per round: the emulated-
  * instruction SIMT efficiency the paper's divergence discussion in Section 4
  * is about; 0 in the plain form, which counts no rounds).  Host

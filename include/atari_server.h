@@ -78,8 +78,9 @@ ATARI_API size_t atari_server_footprint(int slots, int tick_envs, int n_roms, co
  * the largest that fits budget_bytes, capped by max_slots.  The tick buffers
  * are sized for max_tick_envs.  Everything is allocated here, and nothing on
  * the device is allocated per request.  A cfg without an envs_per_warp /
- * envs_per_block choice gets 32 envs per warp, 128 per block.  Returns
- * ATARI_ENOMEM when not even one env fits the budget. */
+ * envs_per_block choice gets 32 envs per warp, 64 per block, and without a
+ * tia_warps choice paired TIA warps.  Returns ATARI_ENOMEM when not even one
+ * env fits the budget. */
 ATARI_API int atari_server_create(const uint8_t *const *roms, const size_t *rom_sizes, const atari_rom_meta *meta,
                                   int n_roms, const atari_config *cfg, const uint8_t *luma,
                                   const atari_server_config *scfg, atari_server **out);

@@ -1107,10 +1107,10 @@ struct FastConsoleT {
   // instruction's words are loaded before this one's result is computed; eight
   // warps on an SM are bound by the integer pipe, two cycles an instruction,
   // which is why sums, shifts left and counters are multiply-adds.  One round:
-  // 157 cycles with one warp on an SM, 284 with eight (208 and 365 with the
-  // control words loaded at the round's end, V in a register of its own, the
-  // branch's condition in three operations, RAM addressed apart from the
-  // cartridge and regions of 32 bytes).  What it does not take (fc_quick, and the
+  // 157 cycles with one warp on an SM, 284 with eight (with the control words
+  // loaded at the round's end, V in a register of its own, the branch's
+  // condition in three operations, RAM addressed apart from the cartridge and
+  // regions of 32 bytes: 208 and 365).  What it does not take (fc_quick, and the
   // general decoder for the rest) stops the lane in front of the instruction;
   // after every BATCH rounds the lanes that wait are looked at, and served
   // together.
@@ -1503,7 +1503,8 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
       held = 0;
       bool slow;
       for (;;) {
-        slow = active & (run == 0);  // not served yet
+        ++rounds;  // in which each waiting lane's instruction is served
+        slow = active & (run == 0);
         if (slow) {
           rec = word_at(pk);
           const uint32_t kind = sm8(OFF_DEC + DEC_QUICK + (rec & 0xFFu));
@@ -1551,7 +1552,6 @@ __device__ __forceinline__ void FastConsoleT<SPLIT>::run(Hook &hook) {
         if (__any_sync(wmask, active & (run != 0))) break;
       }
       if (__any_sync(wmask, slow)) {
-        ++rounds;
         if (slow) {
           leave();
           active = fc_service<SPLIT, Hook>(this, &hook);

@@ -8,14 +8,13 @@
 // column, 32 columns per operation; the planes turn into pixels eight columns
 // at a time, with a byte permute that picks from the four class colours.
 //
-// The former kernel had a warp walk the rows with one lane per column: all 32
-// lanes applied every record to 32 copies of the registers, 182,482
-// warp-instructions per env-step on the banked workload, at two thirds of the
-// issue slots.  Painting, maximum and resampling of 32768 envs went from 7.1
-// to 2.4 ms with it, of 4096 sprite envs from 0.85 to 0.27 ms.  Keeping each
-// object's mask and rebuilding only what a write staled: 2.17 and 0.24 ms.
-// Warps that resample their own rows, a fifth warp for the kept planes and one
-// copy of the code for both frames: 1.97 and 0.22 ms.
+// Painting, maximum and resampling of 32768 banked envs take 1.94 ms, of 4096
+// sprite envs 0.22 ms, 37,237 warp-instructions per env-step, at half of the
+// issue slots.  With a lane per column instead (every lane applies every record
+// to its own copy of the registers): 182,482 warp-instructions, 7.1 and 0.85 ms.
+// With every object's mask rebuilt for every piece of a row: 2.4 and 0.27 ms;
+// with the whole block resampling after a barrier and the kept planes copied by
+// the painting warps: 2.17 and 0.24 ms.
 #pragma once
 #include <cstdint>
 
