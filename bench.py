@@ -50,8 +50,8 @@ SM_COUNT, SMSP_PER_SM, SM_MAX_MHZ = 152, 4, 2070.0
 # never captured reports achieved = null.
 INTERP_CAPTURES = {
     # (kernel, envs per warp, config): (warp-inst per executed 6502 instruction, DRAM bytes per env-step)
-    ("k_interp_split", 32, 3): (1412574931 / 433986434, (31363840 + 456011776) / 32768),
-    ("k_interp_split", 32, 2): (272340736 / 94164973, (1458432 + 9803264) / 4096),
+    ("k_interp_split", 32, 3): (1384003528 / 433986434, (32122624 + 456944640) / 32768),
+    ("k_interp_split", 32, 2): (269669960 / 94164973, (1462784 + 9739776) / 4096),
 }
 # Algorithmic bytes of the fused rasterise + preprocess kernel per env-step,
 # besides 4 bytes per logged TIA write: record counts of the two rendered

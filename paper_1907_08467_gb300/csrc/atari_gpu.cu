@@ -366,7 +366,7 @@ __device__ void step_env(Console<Mem> &m, uint8_t *st, int i, const StepArgs &a,
 // branches one after another, so a warp of one env is the faster while few
 // enough envs are there (ms a step at 1, 2, 4, 8, 32 lanes: 22, 30, 38, 52, 79
 // for 1024 sprite envs, 46, 60, 74, 80, 84 for 4096).  Its 72 registers let 28
-// warps on an SM, so from 4257 envs on a part of them runs after the others (43
+// warps on an SM, so from 4257 envs on a part of them runs after the others (44
 // ms at 4256, 73 at 4864), which full warps still do not reach there (91); with
 // many more envs the issue slots are full and full warps win (281, 277, 239, 199,
 // 165 for 32768 banked envs).  The line is 32 envs an SM, 4864.
