@@ -534,7 +534,7 @@ struct EnvOff {
 // (address - 0x80) for every address below the cartridge's and looks at the
 // value only when the address is RAM's; the cartridge (16 KB at least) behind
 // the RAM and the tables before it keep those loads inside the block's memory.
-constexpr uint32_t OFF_REG = 0, OFF_DEC = OFF_REG + REGION_BYTES, OFF_CTL = OFF_DEC + DEC_CTL, 
+constexpr uint32_t OFF_REG = 0, OFF_DEC = OFF_REG + REGION_BYTES, OFF_CTL = OFF_DEC + DEC_CTL,
                    OFF_RAM = OFF_DEC + DEC_BYTES;
 static_assert(OFF_RAM % 16 == 0 && OFF_RAM >= 0x4000u, "aligned; rom - 0x4000 and ram - 0x200 stay offsets");
 __host__ __device__ inline uint32_t ram_part(uint32_t envs) { return ((envs + 3) / 4 * RAM_GROUP + 15) / 16 * 16; }
